@@ -34,6 +34,11 @@ struct LimbTab {
   const ulonglong2* WL;         // [7][N/8]
   const ulonglong2* IWL;        // [7][N/8]
   u32* chk;                     // device check words (read by the checked kernel build only)
+  // double-precision ring products (d2mhe_fft.cuh): residues split at 2^fft_h, the high part's results rounded by
+  // adding fft_magic to fraction bits that fft_fmask clears, the constants of fft_sum
+  double fft_magic;
+  u64 fft_k0;
+  u32 fft_h, fft_fmask;
 };
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,459 @@
+// Block-level pieces of the double-precision ring products (see d2mhe_fft.cuh): transforms of one
+// polynomial held in the registers of a thread block, tensor memory as the home of the transform that
+// stays with the block, and the rounding to residues.
+#pragma once
+#include "d2mhe_fft.cuh"
+#include "d2mhe_kernels_common.cuh"
+
+namespace {
+
+// GR groups of TG = 16 R threads, n = 256 R GR points, 16 per thread; COLS columns r = tg + c TG of R points each
+// in pass C (tg = thread of the group).  CTAS: thread blocks per SM, 512 threads of 128 registers in all.
+template <int LOGN>
+struct FftGeo {
+  static constexpr int R = LOGN == 12 ? 8 : 16, GR = LOGN == 14 ? 2 : 1;
+  static constexpr int TG = 16 * R, T = TG * GR, NG = 256 * R, n = NG * GR, COLS = 16 / R;
+  static constexpr int CTAS = 512 / T;
+  // Shared memory: per group NG complex numbers in rows of 256 (kC) with a stride of 271, which leaves room for the
+  // 16 x 17 layout of the exchange inside a row; the low part's results (a word and a byte for each of 2n).
+  static constexpr int RS = 271;
+  static constexpr size_t ex_bytes = (size_t)GR * R * RS * 16, stash_bytes = (size_t)n * 10;
+  static constexpr size_t smem_bytes = ex_bytes + stash_bytes + 16;
+  // Words of tensor memory per thread for one transform, and columns for `k` of them: warp w of a block
+  // reaches the lanes 32 (w mod 4) .. + 31 only, so warps w, w + 4, .. share lanes and split the columns.
+  static constexpr int WORDS = 64;
+  __host__ __device__ static constexpr u32 tmem_cols(int k) { return (u32)(WORDS * k * (T / 128)); }
+};
+
+// the block's shared memory and this thread's place in it
+template <int LOGN>
+struct FftSmem {
+  using G = FftGeo<LOGN>;
+  double2* ex;     // of this thread's group
+  double2* other;  // of the other group (GR = 2)
+  u32 *words, *bytes, *slot;
+  u32 tg;
+  __device__ __forceinline__ FftSmem() {
+    const u32 g = group();
+    tg = G::GR > 1 ? threadIdx.x % G::TG : threadIdx.x;
+    double2* base = reinterpret_cast<double2*>(smem_raw);
+    ex = base + g * (G::R * G::RS);
+    other = base + (1u - g) * (G::R * G::RS);
+    words = reinterpret_cast<u32*>(smem_raw + G::ex_bytes);
+    bytes = words + 2 * G::n;
+    slot = bytes + G::n / 2;
+  }
+  __device__ __forceinline__ u32 group() const { return G::GR > 1 ? threadIdx.x / G::TG : 0u; }
+  __device__ __forceinline__ void group_sync() const {
+    if (G::GR == 1)
+      __syncthreads();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(1u + group()), "n"(G::TG) : "memory");
+  }
+};
+
+// ---- tensor memory --------------------------------------------------------------------------------
+// One warp allocates; every thread then owns `words` 32-bit words at the returned address.
+__device__ __forceinline__ void tmem_alloc(u32* slot_smem, u32 cols) {
+  const u32 a = (u32)__cvta_generic_to_shared(slot_smem);
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(a), "r"(cols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_free(u32 base, u32 cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols));
+}
+__device__ __forceinline__ u32 tmem_thread_base(u32 base, u32 words) {
+  const u32 w = threadIdx.x >> 5;
+  return base + ((w & 3u) << 21) + (w >> 2) * words;
+}
+__device__ __forceinline__ void tmem_store4(u32 addr, const cpx (&c)[4]) {
+  u32 w[16];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    w[4 * i] = (u32)__double2loint(c[i].r), w[4 * i + 1] = (u32)__double2hiint(c[i].r);
+    w[4 * i + 2] = (u32)__double2loint(c[i].i), w[4 * i + 3] = (u32)__double2hiint(c[i].i);
+  }
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(addr),
+      "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]),
+      "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_store_done() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// issues the load of four points; the words are valid after tmem_wait
+struct TmemQuad {
+  u32 w[16];
+  __device__ __forceinline__ void issue(u32 addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]),
+          "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
+        : "r"(addr));
+  }
+  // ties the words to a wait issued before: nothing that uses them can move above it
+  __device__ __forceinline__ void get(cpx (&c)[4]) {
+    asm volatile("" : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7]),
+                      "+r"(w[8]), "+r"(w[9]), "+r"(w[10]), "+r"(w[11]), "+r"(w[12]), "+r"(w[13]), "+r"(w[14]), "+r"(w[15]));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      c[i].r = __hiloint2double((int)w[4 * i + 1], (int)w[4 * i]);
+      c[i].i = __hiloint2double((int)w[4 * i + 3], (int)w[4 * i + 2]);
+    }
+  }
+};
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ---- exchanges through shared memory: 16-byte accesses, eight lanes to a wavefront ----------------------------------
+// Inside the 16 threads of a row: element k of lane a goes to element a of lane k, through a 16 x 17 layout (both
+// directions without bank conflicts, constant offsets).  Rows belong to one warp: no block barrier.
+template <int LOGN>
+__device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+  using G = FftGeo<LOGN>;
+  const u32 l16 = sm.tg & 15u;
+  double2* e = sm.ex + (sm.tg >> 4) * G::RS;
+  static_for<16>([&](auto k_) {
+    constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
+    e[l16 + k * 17] = make_double2(xr[i], xi[i]);
+  });
+  __syncwarp();
+  static_for<16>([&](auto k_) {
+    constexpr int k = brev_c<16>(decltype(k_)::value);  // in the order in which the next pass uses them
+    const double2 t = e[l16 * 17 + k];
+    xr[k] = t.x;
+    xi[k] = t.y;
+  });
+  __syncwarp();
+}
+// the 16 results of a row pass -> row-major, and back; own rows only
+template <int LOGN>
+__device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN>& sm, const double* xr, const double* xi) {
+  double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
+  static_for<16>([&](auto k_) {
+    constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
+    e[16 * k] = make_double2(xr[i], xi[i]);
+  });
+}
+template <int LOGN>
+__device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+  const double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
+  static_for<16>([&](auto k_) {
+    constexpr int k = brev_c<16>(decltype(k_)::value);
+    const double2 t = e[16 * k];
+    xr[k] = t.x;
+    xi[k] = t.y;
+  });
+}
+template <int LOGN>
+__device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN>& sm, const double* xr, const double* xi) {
+  using G = FftGeo<LOGN>;
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c)
+    static_for<G::R>([&](auto k_) {
+      constexpr int k = decltype(k_)::value, i = brev_c<G::R>(k);
+      sm.ex[sm.tg + k * G::RS + c * G::TG] = make_double2(xr[c * G::R + i], xi[c * G::R + i]);
+    });
+}
+template <int LOGN>
+__device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+  using G = FftGeo<LOGN>;
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c)
+    static_for<G::R>([&](auto k_) {
+      constexpr int k = brev_c<G::R>(decltype(k_)::value);
+      const double2 t = sm.ex[sm.tg + k * G::RS + c * G::TG];
+      xr[c * G::R + k] = t.x;
+      xi[c * G::R + k] = t.y;
+    });
+}
+
+// A 16-byte load that stays where it is written (a prefetch into registers that have just become free, or a
+// table entry that is read again in every transform instead of living in registers).
+__device__ __forceinline__ cpx ld_here(const double2* p) {
+  cpx c;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(c.r), "=d"(c.i) : "l"(p));
+  return c;
+}
+__device__ __forceinline__ cpx ld_cpx(const double2* p) {
+  const double2 t = __ldg(p);
+  return cpx{t.x, t.y};
+}
+
+// psi^-j of digit jC = JC of a column: tw * e^(-i pi JC / 2R) (one group), e^(-i pi JC / 4R) (first of two) or
+// e^(3 i pi JC / 4R) (second of two; psi_1 = e^(-3 i pi / 4 NG)).
+template <int LOGN, int JC>
+__device__ __forceinline__ cpx fft_twist(const cpx tw, u32 group) {
+  using G = FftGeo<LOGN>;
+  if constexpr (JC == 0) return tw;
+  if constexpr (G::GR == 1) {
+    constexpr int a = -32 * JC / G::R;
+    return cmul(tw, cpx{root_c<a>(), root_s<a>()});
+  } else {
+    const cpx r0{root_c<-JC>(), root_s<-JC>()}, r1{root_c<3 * JC>(), root_s<3 * JC>()};
+    return cmul(tw, group ? r1 : r0);
+  }
+}
+
+// Forward transform.  in(j): the coefficients j and j + n as a complex number, j < n.  Leaves
+// Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
+template <int LOGN, class In>
+__device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
+  using G = FftGeo<LOGN>;
+  constexpr int R = G::R;
+  const u32 g = sm.group();
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c) {
+    const u32 r = sm.tg + (u32)(c * G::TG);
+    const cpx t = ld_cpx(ft.twist + 256 * g + r);
+    static_for<R>([&](auto j_) {
+      constexpr int j = decltype(j_)::value;
+      cpx z = in(r + 256u * (u32)j);
+      if constexpr (G::GR == 2) {  // z_j +- q z_(j + n/2)
+        const cpx y = in(r + 256u * (u32)j + G::NG);
+        const double h = g ? -root_c<16>() : root_c<16>();
+        z = cpx{D2MHE_FMA(h, y.r - y.i, z.r), D2MHE_FMA(h, y.r + y.i, z.i)};
+      }
+      const cpx p = fft_twist<LOGN, j>(t, g);
+      z = cmul(z, cpx{p.r, -p.i});
+      xr[c * R + j] = z.r;
+      xi[c * R + j] = z.i;
+    });
+    fft_eval<R, 1, 0>(xr + c * R, xi + c * R, TwNone());
+  }
+  __syncthreads();  // previous users of ex are done
+  fft_put_cols<LOGN>(sm, xr, xi);
+  sm.group_sync();
+  fft_get_rows<LOGN>(sm, xr, xi);
+  const u32 l16 = sm.tg & 15u, row = sm.tg >> 4;
+  {
+    const cpx t[2] = {ld_cpx(ft.fwd2 + row), ld_cpx(ft.fwd2 + R + row)};
+    fft_eval<16, 1, 0>(xr, xi, TwDerived<16, 1>(t));
+  }
+  __syncwarp();  // the rows have been read by their own warp only
+  fft_swap_row<LOGN>(sm, xr, xi);
+  {
+    const u32 k = row + (u32)R * l16;
+    const cpx t[2] = {ld_cpx(ft.fwd3 + k), ld_cpx(ft.fwd3 + 16 * R + k)};
+    fft_eval<16, 1, 0>(xr, xi, TwDerived<16, 1>(t));
+  }
+}
+
+// A transform in tensor memory: four points (k, k + 8, k + 4, k + 12) after one another, as fft_product4 takes them.
+__device__ __forceinline__ void fft_to_tmem(u32 addr, const double* xr, const double* xi) {
+  static_for<4>([&](auto q_) {
+    cpx c[4];
+    static_for<4>([&](auto i_) {
+      constexpr int k = brev_c<16>(decltype(q_)::value + 4 * brev_c<4>(decltype(i_)::value));
+      c[i_.value] = cpx{xr[k], xi[k]};
+    });
+    tmem_store4(addr + q_.value * 16, c);
+  });
+}
+
+// A stored transform (a row of n points): point kA of a thread in slot kA T + thread.
+template <int LOGN>
+__device__ __forceinline__ void fft_load(const double2* row, double* xr, double* xi) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const cpx s = ld_here(row + threadIdx.x + k * FftGeo<LOGN>::T);
+    xr[k] = s.r;
+    xi[k] = s.i;
+  }
+}
+template <int LOGN>
+__device__ __forceinline__ void fft_store(double2* row, const double* xr, const double* xi, double scale) {
+  static_for<16>([&](auto k_) {
+    constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
+    row[threadIdx.x + k * FftGeo<LOGN>::T] = make_double2(xr[i] * scale, xi[i] * scale);
+  });
+}
+
+// Products of the points in registers with a transform in tensor memory (with the first two stages of pass A).
+__device__ __forceinline__ void fft_product_tmem(u32 addr, double* xr, double* xi) {
+  TmemQuad buf[2];
+  buf[0].issue(addr);
+  static_for<4>([&](auto q_) {
+    constexpr int q = decltype(q_)::value;
+    tmem_wait();
+    cpx c[4];
+    buf[q & 1].get(c);
+    if constexpr (q + 1 < 4) buf[(q + 1) & 1].issue(addr + (q + 1) * 16);
+    fft_product4<-1>(xr, xi, q, c);
+  });
+}
+
+// Inverse transform of what the products left, up to the twist: digit jC of column r = tg + c TG is left in
+// x[c R + brev(jC)]; tw: the columns' twist.  before_last(): called ahead of the arithmetic of pass C.
+// Table entries are fetched a pass ahead of their use (they come from L2 as often as not).
+template <int LOGN, class Hook>
+__device__ __forceinline__ void fft_inverse(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi,
+                                            cpx (&tw)[FftGeo<LOGN>::COLS], Hook before_last) {
+  using G = FftGeo<LOGN>;
+  const cpx t2[2] = {ld_here(ft.inv2 + (sm.tg & 15u)), ld_here(ft.inv2 + 16 + (sm.tg & 15u))};
+  fft_eval<16, -1, 2>(xr, xi, TwNone());
+  __syncthreads();  // previous users of ex are done
+  fft_swap_row<LOGN>(sm, xr, xi);
+  cpx t[G::COLS][2];
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) t[c][i] = ld_here(ft.inv3 + 256 * i + sm.tg + c * G::TG);
+  fft_eval<16, -1, 0>(xr, xi, TwDerived<16, -1>(t2));
+  fft_put_rows<LOGN>(sm, xr, xi);
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c) tw[c] = ld_here(ft.twist + 256 * sm.group() + sm.tg + c * G::TG);
+  sm.group_sync();
+  fft_get_cols<LOGN>(sm, xr, xi);
+  before_last();
+#pragma unroll
+  for (int c = 0; c < G::COLS; ++c) fft_eval<G::R, -1, 0>(xr + c * G::R, xi + c * G::R, TwDerived<G::R, -1>(t[c]));
+}
+
+// Result number i of a thread (below 32) belongs to this coefficient.
+template <int LOGN>
+__device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN>& sm, int i) {
+  using G = FftGeo<LOGN>;
+  if (G::GR == 2) return sm.tg + 256u * (8u * sm.group() + (u32)(i & 7)) + 4096u * (u32)(i >> 3);
+  if (G::R == 8) return sm.tg + 128u * (u32)(i >> 4) + 256u * (u32)(i & 15);
+  return sm.tg + 256u * (u32)i;
+}
+// The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
+// eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4], a, b) with v = bits of
+// M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.  x[a] and x[b] are free
+// afterwards.
+template <int LOGN, class Out>
+__device__ __forceinline__ void fft_results(const FftSmem<LOGN>& sm, const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr,
+                                            double* xi, double magic, Out out) {
+  using G = FftGeo<LOGN>;
+  constexpr int R = G::R;
+  if constexpr (G::GR == 1) {
+    // portion: digits j, j + 1 of a column; results (column c) i = 2R c + j, + 1 (real) and + R (imaginary)
+    static_for<8>([&](auto m_) {
+      constexpr int m = decltype(m_)::value, c = 2 * m / R, j = 2 * m % R, i0 = c * R + brev_c<R>(j), i1 = c * R + brev_c<R>(j + 1);
+      const cpx p0 = fft_twist<LOGN, j>(tw[c], 0), p1 = fft_twist<LOGN, j + 1>(tw[c], 0);
+      u64 v[4];
+      v[0] = (u64)__double_as_longlong(__fma_rn(xr[i0], p0.r, __fma_rn(-xi[i0], p0.i, magic)));
+      v[1] = (u64)__double_as_longlong(__fma_rn(xr[i1], p1.r, __fma_rn(-xi[i1], p1.i, magic)));
+      v[2] = (u64)__double_as_longlong(__fma_rn(xr[i0], p0.i, __fma_rn(xi[i0], p0.r, magic)));
+      v[3] = (u64)__double_as_longlong(__fma_rn(xr[i1], p1.i, __fma_rn(xi[i1], p1.r, magic)));
+      out(m_, std::integral_constant<int, 2 * R * c + j>{}, std::integral_constant<int, R>{}, v,
+          std::integral_constant<int, i0>{}, std::integral_constant<int, i1>{});
+    });
+  } else {
+    // Group g finishes the digits 8 g .. 8 g + 7 and sends the others; column r of ex is this thread's own until the
+    // block barrier.  z_j = y0 + y1, z_(j + 4096) = (y0 - y1) e^(-i pi / 4); the group signs make both sides equal.
+    const u32 g = sm.group();
+    static_for<16>([&](auto j_) {
+      constexpr int j = decltype(j_)::value, i = brev_c<16>(j);
+      const cpx z = cmul(cpx{xr[i], xi[i]}, fft_twist<LOGN, j>(tw[0], g));
+      xr[i] = z.r;
+      xi[i] = z.i;
+    });
+    static_for<8>([&](auto j_) {
+      constexpr int j = decltype(j_)::value, lo = brev_c<16>(j), hi = brev_c<16>(j + 8);
+      sm.ex[sm.tg + j * G::RS] = g ? make_double2(xr[lo], xi[lo]) : make_double2(xr[hi], xi[hi]);
+      if (g) xr[lo] = xr[hi], xi[lo] = xi[hi];
+    });
+    __syncthreads();
+    const double s = g ? -root_c<16>() : root_c<16>();
+    static_for<8>([&](auto j_) {
+      constexpr int j = decltype(j_)::value, lo = brev_c<16>(j), hi = brev_c<16>(j + 8);
+      const double2 o = sm.other[sm.tg + j * G::RS];
+      const double dr = xr[lo] - o.x, di = xi[lo] - o.y;  // group 1: the negative, undone by s
+      u64 v[4];
+      v[0] = (u64)__double_as_longlong((xr[lo] + o.x) + magic);
+      v[1] = (u64)__double_as_longlong(__fma_rn(s, dr + di, magic));
+      v[2] = (u64)__double_as_longlong((xi[lo] + o.y) + magic);
+      v[3] = (u64)__double_as_longlong(__fma_rn(s, di - dr, magic));
+      out(j_, j_, std::integral_constant<int, 0>{}, v, std::integral_constant<int, lo>{}, std::integral_constant<int, hi>{});
+    });
+  }
+}
+// number (fft_coef's i) of result B of the portion whose first is I0: one group: I0, I0 + 1, I0 + R, I0 + R + 1;
+// two groups: I0 + 8 B
+template <int I0, int RR, int B>
+__device__ __forceinline__ constexpr int fft_result_number() {
+  return RR ? I0 + (B & 1) + (B >> 1) * RR : I0 + 8 * B;
+}
+
+// The low part's result V_lo (|V_lo| < 2^39) waits for the high part as a word and a byte: with 8 fraction bits
+// V_lo + 2^39 is bytes 1 .. 5 of the rounded value.
+#define D2MHE_FFT_MAGIC_LO (1.5 * 17592186044416.0 + 549755813888.0 + 0.5) /* 1.5 * 2^44 + 2^39 + 1/2 */
+__device__ __forceinline__ u32 lo_word(u64 bits) { return __byte_perm((u32)bits, (u32)(bits >> 32), 0x4321); }
+__device__ __forceinline__ u32 lo_bytes(u64 a, u64 b, u64 c, u64 d) {  // byte 5 of four rounded values
+  return __byte_perm(__byte_perm((u32)(a >> 32), (u32)(b >> 32), 0x0051),
+                     __byte_perm((u32)(c >> 32), (u32)(d >> 32), 0x0051), 0x5410);
+}
+
+// 64 p + V_lo + 2^h V_hi + e0 - 19, below 130 p.  word, bytes: what fft_finish kept, byte I of `bytes`; hi: the rounded
+// high part with f fraction bits, f = 32 - (b - h) and p = 2^b - d: its low word holds V_hi mod 2^(b-h) above the
+// fraction, its high word floor(V_hi / 2^(b-h)) plus a constant, which counts multiples of 2^b = d (mod p).
+// The constants are collected in fft_k0.
+template <int I>
+__device__ __forceinline__ u64 fft_sum(u32 word, u32 bytes, u64 hi, u32 e0, const LimbTab& lt) {
+  u32 hl, hh;
+  split64(hi, hl, hh);
+  u64 s = madwide(hl & lt.fft_fmask, 1u << lt.sf_shift, lt.fft_k0 + e0);
+  s = madwide(hh, lt.sf_d, s);
+  return s + join64(word, __byte_perm(bytes, 0, 0x4440 | I));
+}
+
+// Noise bytes (e + 19) of a polynomial, 32 per thread in the order of fft_coef: 16-byte slots [2][T].
+template <int LOGN>
+struct FftNoise {
+  u32 w[8];
+  __device__ __forceinline__ void load(const uint4* poly) {
+    // volatile: a plain load is moved down to its first use, and its latency costs 7-12 % of the share kernel
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                 : "l"(poly + threadIdx.x));
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(poly + threadIdx.x + FftGeo<LOGN>::T));
+  }
+  template <int I>
+  __device__ __forceinline__ u32 get() const {
+    return __byte_perm(w[I / 4], 0, 0x4440 | (I % 4));
+  }
+};
+
+// The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
+// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  next: the
+// stored transform whose points are fetched into the registers that become free.  (One copy of the code for both
+// parts: two copies share subexpressions, and 300 bytes of them were spilled.)
+template <int LOGN, class Store>
+__device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
+                                           double* xr, double* xi, bool high, const double2* next,
+                                           const FftNoise<LOGN>& nz, Store store) {
+  using G = FftGeo<LOGN>;
+  const double magic = high ? lt.fft_magic : D2MHE_FFT_MAGIC_LO;
+  fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4], auto a_, auto b_) {
+    constexpr int m = decltype(m_)::value, a = decltype(a_)::value, b = decltype(b_)::value;
+    u32* w = sm.words + threadIdx.x + 4 * m * G::T;
+    u32* wb = sm.bytes + threadIdx.x + m * G::T;
+    if (high) {
+      const u32 bytes = *wb;
+      static_for<4>([&](auto q_) {
+        constexpr int q = decltype(q_)::value, i = fft_result_number<decltype(i_)::value, decltype(rr_)::value, q>();
+        store(fft_coef<LOGN>(sm, i), fft_sum<q>(w[q * G::T], bytes, v[q], nz.template get<i>(), lt));
+      });
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i * G::T] = lo_word(v[i]);
+      *wb = lo_bytes(v[0], v[1], v[2], v[3]);
+    }
+    const cpx s0 = ld_here(next + threadIdx.x + a * G::T), s1 = ld_here(next + threadIdx.x + b * G::T);
+    xr[a] = s0.r, xi[a] = s0.i;
+    xr[b] = s1.r, xi[b] = s1.i;
+  });
+}
+
+__device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer
+  return __hiloint2double(0x43300000, v ^ (int)0x80000000u) - __hiloint2double(0x43300000, (int)0x80000000u);
+}
+// part `half` of coefficients j and j + n of a residue row
+__device__ __forceinline__ cpx fft_split_pair(const u64* row, u32 j, u32 n, u32 half, const LimbTab& lt) {
+  int a0, a1, b0, b1;
+  fft_split(__ldg(row + j), lt.p, lt.fft_h, a0, a1);
+  fft_split(__ldg(row + j + n), lt.p, lt.fft_h, b0, b1);
+  return cpx{small_to_double(half ? a1 : a0), small_to_double(half ? b1 : b0)};
+}
+
+}  // namespace

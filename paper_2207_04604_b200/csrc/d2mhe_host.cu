@@ -1,6 +1,7 @@
 // Host side of the C ABI: parameter validation, table construction, argument checks,
 // index staging and the chunked whole-round driver.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -230,6 +231,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   // floor(q/t) mod q_l: q = Delta t + (q mod t)  =>  Delta = -(q mod t) t^-1 (mod q_l)
   const u64 q_mod_t = q_mod(t);
 
+  bool fft_ok = logn >= 12 && logn <= 14;
   bool all_special = true;  // every prime is 2^b - d with b >= 32, d < 2^32 and 256 d < 2^b
   for (u32 l = 0; l < L; ++l) {
     const u64 p = c->moduli[l];
@@ -267,6 +269,18 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     T.sf_d = special ? (u32)gap : 0;
     T.sf_shift = special ? bits - 32 : 0;
     if (!special) all_special = false;
+    // Double-precision products (bounds: d2mhe_fft.cuh): the low part has h <= 40 - log2 N bits, the high part at most 28;
+    // its results keep f = 32 - (bits - h) fraction bits.
+    T.fft_h = std::min((bits + 1) / 2, 40 - logn);
+    if (!special || bits - T.fft_h > 28) {
+      fft_ok = false;
+    } else {
+      const u32 f = 32 - (bits - T.fft_h);
+      T.fft_fmask = ~((1u << f) - 1u);
+      T.fft_magic = 1.5 * (double)((u64)1 << (52 - f)) + 0.5;
+      const u64 h0 = ((u64)(1075 - f) << 20) + ((u64)1 << 19);  // high word of the magic number
+      T.fft_k0 = 64 * p - ((u64)1 << 39) - D2MHE_GAUSS_B - gap * h0;
+    }
 
     const u64 psi = c->roots[l], psi_inv = h_inv(psi, p);
     std::vector<u64> pw(n), ipw(n);
@@ -380,6 +394,37 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     // (q-1)/2 mod t = (q mod t - 1) * 2^-1 mod t   (t odd)
     rt.half_mod_t = h_mul((q_mod_t + t - 1) % t, h_inv(2, t), t);
     rt.qinv_mod_t = h_inv(q_mod_t, t);
+  }
+
+  // double-precision ring products
+  if (fft_ok && all_special) {
+    const u32 groups = logn == 14 ? 2 : 1, m = n / 2 / groups, R = m / 256;
+    // e^(2 pi i num / den), in extended precision before the rounding to double
+    auto root = [](double num, double den) {
+      const long double a = 6.283185307179586476925286766559005768L * (long double)num / (long double)den;
+      return make_double2((double)cosl(a), (double)sinl(a));
+    };
+    std::vector<double2> tw(256 * groups), f2(2 * R), f3(2 * (m / 16)), i2(32), i3(512);
+    for (u32 r = 0; r < 256; ++r) {
+      tw[r] = root(-(double)r, groups == 1 ? 4.0 * m : 8.0 * m);
+      if (groups == 2) tw[256 + r] = root(3.0 * r, 8.0 * m);
+    }
+    for (u32 i = 0; i < 2; ++i) {
+      for (u32 k = 0; k < R; ++k) f2[R * i + k] = root(k << (2 * i), 16.0 * R);
+      for (u32 k = 0; k < m / 16; ++k) f3[m / 16 * i + k] = root(k << (2 * i), m);
+      for (u32 k = 0; k < 16; ++k) i2[16 * i + k] = root(-(double)(k << (2 * i)), 256.0);
+      for (u32 k = 0; k < 256; ++k) i3[256 * i + k] = root(-(double)(k << (2 * i)), m);
+    }
+    const std::vector<double2>* src[5] = {&tw, &f2, &f3, &i2, &i3};
+    const double2** dst[5] = {&c->view.fft.twist, &c->view.fft.fwd2, &c->view.fft.fwd3, &c->view.fft.inv2,
+                              &c->view.fft.inv3};
+    for (int i = 0; i < 5; ++i) {
+      *dst[i] = dev_upload(c, *src[i], &err);
+      if (err != cudaSuccess) return fail_cuda(c, err);
+    }
+    c->view.s_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
+    c->view.fft_on = 1;
   }
 
   // key storage
@@ -632,6 +677,11 @@ d2mhe_status d2mhe_keygen_share(d2mhe_ctx* c, const u32* parties, u32 n_parties)
       if (e != cudaSuccess) return fail_staged(c, sg, e);
       c->launches += 1;
     }
+  }
+  if (c->view.fft_on) {
+    e = L_(fft_secret)(c->view, c->stream, sg.dev[0], n_parties, TAG_SECRET, c->view.s_fft);
+    if (e != cudaSuccess) return fail_staged(c, sg, e);
+    c->launches += 1;
   }
   for (u32 i = 0; i < n_parties; ++i) c->has_share[parties[i]] = true;
   return release_slot(c, sg);

@@ -27,6 +27,15 @@ struct RoundTab {
   u64 qinv_mod_t;          // q^-1 mod t
 };
 
+// Twiddle factors of the double-precision ring products: groups of m = 256 R points (w_k = e^(2 pi i / k)).
+struct FftTab {
+  const double2* twist;  // [groups][256]  psi_g^-r: psi = e^(i pi / 2m), or psi_0 = e^(i pi / 4m) and psi_1 = e^(-3 i pi / 4m)
+  const double2* fwd2;   // [2][R]         w_(16R)^(4^i k)
+  const double2* fwd3;   // [2][m/16]      w_m^(4^i k)
+  const double2* inv2;   // [2][16]        w_256^(-4^i k)
+  const double2* inv3;   // [2][256]       w_m^(-4^i r)
+};
+
 // The per-limb constants travel as a kernel parameter (constant bank): indexed by the
 // CTA-uniform limb number they are read through the uniform datapath instead of occupying
 // vector registers in every thread.
@@ -54,6 +63,10 @@ struct DevView {
   // {residue out of Montgomery form, its 32-bit Shoup companion}
   u64* s32;       // [K][L][N]
   u64* pk32;      // [2][L][N]
+  // ring products in double precision (set when the sizes are inside the bounds of d2mhe_fft.cuh)
+  u32 fft_on;
+  FftTab fft;
+  double2* s_fft;  // [K][n]  transforms of s_k, times 1/n
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
@@ -187,7 +200,11 @@ cudaError_t check_selftest(const DevView& v, cudaStream_t s); \
 cudaError_t sample_encrypt_noise(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 ct_first, u32 n_cts, \
                                  u32 unit_first, u32 n_units, u32* out); \
 cudaError_t sample_share_noise(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
-                               u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out); \
+                               u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out, \
+                               bool fft); \
+cudaError_t share_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev, \
+                      u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares); \
+cudaError_t fft_secret(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 n_parties, u32 tag, double2* dst); \
 cudaError_t make_tab32(const DevView& v, cudaStream_t s, const u64* src, u64* dst, size_t rows); \
 cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \
                       u32 ct_first, u32 n_cts, const u32* plain, u32* ct, void* scratch, size_t scratch_bytes, \

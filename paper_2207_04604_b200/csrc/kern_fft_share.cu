@@ -1,0 +1,111 @@
+// Decryption shares h = s_k c_1 + e by double-precision FFT (see d2mhe_fft.cuh and DevView::fft_on).
+#include <algorithm>
+
+#include "d2mhe_fft_block.cuh"
+
+namespace {
+
+// One thread block = one (recipient, ciphertext, limb); it walks over the parties of the list.
+// What bounds it: the double-precision pipe and the issue slots around it (about 50 double-precision and 45 other
+// instructions per complex point and part), then shared memory (two exchanges per transform).  The transforms of
+// both parts of c_1 stay in tensor memory (all 256 KB of an SM: 32 bytes per point), where neither the load/store
+// pipe nor L2 sees them again; the key's transform does not depend on the limb (8 N bytes per party, L2) and is
+// fetched into the registers that the end of the previous transform frees.  The rounded low part waits in shared
+// memory, thread by thread, for the high part.
+// grid = n_units * L * split; party a belongs to block a mod split of its unit.
+template <int LOGN>
+__global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
+    k_share_fft(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ agg,
+                const u32* __restrict__ parties, u32 n_parties, u32 n_cts, u32 unit_first,
+                const uint4* __restrict__ noise, u64* __restrict__ shares, u32 split) {
+  using G = FftGeo<LOGN>;
+  constexpr int n = G::n;
+  const u32 part = blockIdx.x % split, rest = blockIdx.x / split;
+  const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
+  if (part >= n_parties) return;
+  const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
+  const LimbTab& lt = lp.limbs[l];
+  const FftSmem<LOGN> sm;
+  if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
+  __syncthreads();
+  const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
+  const size_t row = (size_t)l * v.n, poly = (size_t)v.L * v.n;
+  const u64* c1 = agg + ((size_t)unit * 2 + 1) * poly + row;
+  double xr[16], xi[16];
+#pragma unroll 1
+  for (u32 half = 0; half < 2; ++half) {
+    fft_forward<LOGN>(sm, v.fft, xr, xi, [&](u32 j) {
+      if (!D2MHE_CHK(v.chk, j + n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
+      return fft_split_pair(c1, j, n, half, lt);
+    });
+    fft_to_tmem(tm + half * G::WORDS, xr, xi);
+  }
+  tmem_store_done();
+  // the stored transform of a party's key; a party number that fails the check reads row 0
+  auto key_of = [&](u32 a) {
+    u32 party = parties[a];
+    if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY)) party = 0;
+    return v.s_fft + (size_t)party * n;
+  };
+  const double2* key = key_of(part);
+  fft_load<LOGN>(key, xr, xi);
+  u32 a = part;
+  bool high = false;
+#pragma unroll 1
+  while (a < n_parties) {
+    // after a low part the same key again, then the next party's (the last fetch is not used)
+    const double2* next = high && a + split < n_parties ? key_of(a + split) : key;
+    u64* out = shares + (((size_t)irec * n_parties + a) * n_cts + cl) * poly + row;
+    FftNoise<LOGN> nz;
+    cpx tw[G::COLS];
+    fft_product_tmem(tm + (high ? G::WORDS : 0), xr, xi);
+    fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
+      if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16);
+    });
+    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, next, nz, [&](u32 j, u64 s) {
+      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) out[j] = canon8<true>(s, lt);
+    });
+    key = next;
+    if (high) a += split;
+    high = !high;
+  }
+  __syncthreads();
+  if (tid < 32) tmem_free(tbase, G::tmem_cols(2));
+}
+
+template <int LOGN>
+cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
+                         u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
+  using G = FftGeo<LOGN>;
+  cudaError_t e = set_smem(k_share_fft<LOGN>, G::smem_bytes);
+  if (e != cudaSuccess) return e;
+  // Parties of a unit over `split` blocks, each of which transforms c_1 for itself: the split with the
+  // shortest schedule, counted in part transforms (2 forward + 2 per share) over whole waves of blocks.
+  const u32 resident = v.sms * G::CTAS, base = n_units * v.L;
+  u32 split = 1;
+  u64 best = ~0ull;
+  for (u32 c = 1; c <= std::min(n_parties, 16u); ++c) {
+    const u64 waves = ((u64)base * c + resident - 1) / resident, per = (n_parties + c - 1) / c;
+    const u64 cost = waves * (2 + 2 * per);
+    if (cost < best) best = cost, split = c;
+  }
+  k_share_fft<LOGN><<<base * split, G::T, G::smem_bytes, s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
+                                                              reinterpret_cast<const uint4*>(noise), shares, split);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+namespace D2MHE_LAUNCH_NS {
+
+cudaError_t share_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
+                      u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
+  switch (v.logn) {
+    case 12: return launch_share<12>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    case 13: return launch_share<13>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    case 14: return launch_share<14>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace D2MHE_LAUNCH_NS

@@ -319,7 +319,7 @@ cudaError_t partial_decrypt32(const DevView& v, const LimbParams& lp, cudaStream
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
     cudaError_t e = sample_share_noise(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
-                                       reinterpret_cast<u32*>(scratch));
+                                       reinterpret_cast<u32*>(scratch), false);
     if (e != cudaSuccess) return e;
     e = pdec32_units(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu,
                      reinterpret_cast<const signed char*>(scratch), shares);

@@ -1231,3 +1231,39 @@ def test_checked_build_reports_a_violation_without_losing_the_context(d2):
     plain.sync()
     assert plain.debug_last_device_check() == [0, 0, 0, 0]
     plain.close()
+
+
+# ----------------------------------------------------------------------------------
+# ring products in double precision
+# ----------------------------------------------------------------------------------
+
+
+@pytest.mark.parametrize("log2_n,bits,L,K", [
+    (12, 33, 4, 1), (12, 36, 3, 3), (12, 56, 2, 17), (13, 41, 2, 2), (13, 54, 1, 5), (13, 55, 2, 4), (13, 56, 2, 3),
+    (14, 48, 2, 3), (14, 54, 2, 2), (14, 55, 2, 2),
+])
+def test_share_products_at_the_limits_of_the_split(d2, log2_n, bits, L, K):
+    """Residues at the ends of both parts of the split, in all coefficients and mixed; 56 bits at N = 8192 and 55 bits at
+    N = 16384 are just outside the range of the double-precision products."""
+    moduli = wl.ntt_primes(bits, 2 << log2_n, L)
+    n, parties = 1 << log2_n, list(range(K))
+    ctx = d2.Context(log2_n, moduli, K, seed=77)
+    o = make_oracle(log2_n, moduli, seed=77)
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    o.collective_pk(parties)
+    rng = np.random.default_rng(log2_n * 100 + bits)
+    h = min((bits + 1) // 2, 40 - log2_n)
+    agg = np.zeros((1, 3, 2, L, n), dtype=np.uint64)
+    for l, p in enumerate(moduli):
+        top = ((1 << (h - 1)) - 1) + (((p // 2) >> h) - 1 << h)  # both parts near their largest values
+        edge = np.array([0, 1, p - 1, (p - 1) // 2, (p + 1) // 2, 1 << (h - 1), (1 << (h - 1)) - 1, p - (1 << (h - 1)),
+                         top, p - top], dtype=np.uint64)
+        agg[0, 0, 1, l] = rng.choice(edge, n)
+        agg[0, 1, 1, l] = top
+        agg[0, 2, 1, l] = rng.integers(0, p, n, dtype=np.uint64)
+    shares = ctx.empty_u64(1, K, 3, L, n)
+    ctx.partial_decrypt(d2.from_u64_numpy(agg, ctx.device), [K - 1], parties, 5, 3, shares)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(shares), o.partial_decrypt(agg, [K - 1], parties, 5))
+    ctx.close()

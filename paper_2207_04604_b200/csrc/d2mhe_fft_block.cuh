@@ -166,8 +166,8 @@ __device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN>& sm, double* xr
     });
 }
 
-// A 16-byte load that stays where it is written (a prefetch into registers that have just become free, or a
-// table entry that is read again in every transform instead of living in registers).
+// A 16-byte load that stays where it is written (a table entry that is read again in every transform instead of
+// living in registers, or a batch of loads that is issued as a whole).
 __device__ __forceinline__ cpx ld_here(const double2* p) {
   cpx c;
   asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(c.r), "=d"(c.i) : "l"(p));
@@ -317,9 +317,8 @@ __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN>& sm, int i) {
   return sm.tg + 256u * (u32)i;
 }
 // The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
-// eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4], a, b) with v = bits of
-// M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.  x[a] and x[b] are free
-// afterwards.
+// eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4]) with v = bits of
+// M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.
 template <int LOGN, class Out>
 __device__ __forceinline__ void fft_results(const FftSmem<LOGN>& sm, const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr,
                                             double* xi, double magic, Out out) {
@@ -335,8 +334,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN>& sm, const cpx (
       v[1] = (u64)__double_as_longlong(__fma_rn(xr[i1], p1.r, __fma_rn(-xi[i1], p1.i, magic)));
       v[2] = (u64)__double_as_longlong(__fma_rn(xr[i0], p0.i, __fma_rn(xi[i0], p0.r, magic)));
       v[3] = (u64)__double_as_longlong(__fma_rn(xr[i1], p1.i, __fma_rn(xi[i1], p1.r, magic)));
-      out(m_, std::integral_constant<int, 2 * R * c + j>{}, std::integral_constant<int, R>{}, v,
-          std::integral_constant<int, i0>{}, std::integral_constant<int, i1>{});
+      out(m_, std::integral_constant<int, 2 * R * c + j>{}, std::integral_constant<int, R>{}, v);
     });
   } else {
     // Group g finishes the digits 8 g .. 8 g + 7 and sends the others; column r of ex is this thread's own until the
@@ -364,7 +362,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN>& sm, const cpx (
       v[1] = (u64)__double_as_longlong(__fma_rn(s, dr + di, magic));
       v[2] = (u64)__double_as_longlong((xi[lo] + o.y) + magic);
       v[3] = (u64)__double_as_longlong(__fma_rn(s, di - dr, magic));
-      out(j_, j_, std::integral_constant<int, 0>{}, v, std::integral_constant<int, lo>{}, std::integral_constant<int, hi>{});
+      out(j_, j_, std::integral_constant<int, 0>{}, v);
     });
   }
 }
@@ -415,17 +413,15 @@ struct FftNoise {
 };
 
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
-// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  next: the
-// stored transform whose points are fetched into the registers that become free.  (One copy of the code for both
-// parts: two copies share subexpressions, and 300 bytes of them were spilled.)
+// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  (One copy of
+// the code for both parts: two copies share subexpressions, and 300 bytes of them were spilled.)
 template <int LOGN, class Store>
 __device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
-                                           double* xr, double* xi, bool high, const double2* next,
-                                           const FftNoise<LOGN>& nz, Store store) {
+                                           double* xr, double* xi, bool high, const FftNoise<LOGN>& nz, Store store) {
   using G = FftGeo<LOGN>;
   const double magic = high ? lt.fft_magic : D2MHE_FFT_MAGIC_LO;
-  fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4], auto a_, auto b_) {
-    constexpr int m = decltype(m_)::value, a = decltype(a_)::value, b = decltype(b_)::value;
+  fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4]) {
+    constexpr int m = decltype(m_)::value;
     u32* w = sm.words + threadIdx.x + 4 * m * G::T;
     u32* wb = sm.bytes + threadIdx.x + m * G::T;
     if (high) {
@@ -439,9 +435,6 @@ __device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTa
       for (int i = 0; i < 4; ++i) w[i * G::T] = lo_word(v[i]);
       *wb = lo_bytes(v[0], v[1], v[2], v[3]);
     }
-    const cpx s0 = ld_here(next + threadIdx.x + a * G::T), s1 = ld_here(next + threadIdx.x + b * G::T);
-    xr[a] = s0.r, xi[a] = s0.i;
-    xr[b] = s1.r, xi[b] = s1.i;
   });
 }
 

@@ -9,9 +9,11 @@ namespace {
 // What bounds it: the double-precision pipe and the issue slots around it (about 50 double-precision and 45 other
 // instructions per complex point and part), then shared memory (two exchanges per transform).  The transforms of
 // both parts of c_1 stay in tensor memory (all 256 KB of an SM: 32 bytes per point), where neither the load/store
-// pipe nor L2 sees them again; the key's transform does not depend on the limb (8 N bytes per party, L2) and is
-// fetched into the registers that the end of the previous transform frees.  The rounded low part waits in shared
-// memory, thread by thread, for the high part.
+// pipe nor L2 sees them again; the key's transform does not depend on the limb (8 N bytes per party) and comes from
+// L2, or from L1 when the other block of the SM has just read it.  (Fetching it point by point into the registers that
+// the end of the previous transform frees was slower: 46.8 k instead of 40.0 k clocks per share and limb at N = 16384,
+// 18.5 k instead of 17.3 k at N = 8192.)  The rounded low part waits in shared memory, thread by thread, for the high
+// part.  The shares are written with a streaming hint, so that the keys stay in L2.
 // grid = n_units * L * split; party a belongs to block a mod split of its unit.
 template <int LOGN>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
@@ -48,22 +50,21 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     return v.s_fft + (size_t)party * n;
   };
   const double2* key = key_of(part);
-  fft_load<LOGN>(key, xr, xi);
   u32 a = part;
   bool high = false;
 #pragma unroll 1
   while (a < n_parties) {
-    // after a low part the same key again, then the next party's (the last fetch is not used)
-    const double2* next = high && a + split < n_parties ? key_of(a + split) : key;
+    const double2* next = high && a + split < n_parties ? key_of(a + split) : key;  // the address, a part ahead
     u64* out = shares + (((size_t)irec * n_parties + a) * n_cts + cl) * poly + row;
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
+    fft_load<LOGN>(key, xr, xi);
     fft_product_tmem(tm + (high ? G::WORDS : 0), xr, xi);
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
       if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16);
     });
-    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, next, nz, [&](u32 j, u64 s) {
-      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) out[j] = canon8<true>(s, lt);
+    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
+      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
     });
     key = next;
     if (high) a += split;

@@ -180,6 +180,11 @@ struct GaussTab {
   u64 cdt[D2MHE_CDT_LEN];
   unsigned short lut[256];
 };
+// For the sampling kernels: the count for the top 12 bits of a draw, bit 7 set when the bucket holds a threshold.
+struct __align__(16) GaussFast {
+  unsigned char lut[4096];
+  u64 cdt[D2MHE_CDT_LEN];
+};
 __device__ __forceinline__ int gauss_from_r(const GaussTab& g, u64 r) {
   u32 e = g.lut[r >> 56];
   u32 base = e & 0xffu, inside = e >> 8;

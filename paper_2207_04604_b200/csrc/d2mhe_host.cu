@@ -337,6 +337,20 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     }
     c->view.gauss = dev_upload(c, g, &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
+    std::vector<GaussFast> f(1);
+    for (int k = 0; k < D2MHE_CDT_LEN; ++k) f[0].cdt[k] = kGaussCdt[k];
+    for (u32 b = 0; b < 4096; ++b) {
+      const u64 lo = (u64)b << 52, hi = lo | (((u64)1 << 52) - 1);
+      u32 base = 0, inside = 0;
+      for (int k = 0; k < D2MHE_CDT_LEN; ++k)
+        if (kGaussCdt[k] <= lo)
+          ++base;
+        else if (kGaussCdt[k] <= hi)
+          ++inside;
+      f[0].lut[b] = (unsigned char)(base | (inside ? 0x80 : 0));
+    }
+    c->view.gauss_fast = dev_upload(c, f, &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
   }
 
   // plaintext-modulus transforms

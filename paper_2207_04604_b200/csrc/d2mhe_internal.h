@@ -47,6 +47,7 @@ struct LimbParams {
 struct DevView {
   const LimbTab* limbs;
   const GaussTab* gauss;
+  const GaussFast* gauss_fast;
   PlainTab plain;
   RoundTab round;
   u64 seed;
@@ -70,6 +71,14 @@ struct DevView {
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
+
+// What is sampled for a share or ciphertext, in order: stream tags (TAG_ENC_U is ternary, the others Gaussian).
+struct SampleKinds {
+  u32 n, tag0, tag1, tag2;
+};
+static const SampleKinds kSampleShare = {1, TAG_DEC_ERR, 0, 0};
+static const SampleKinds kSampleEncrypt = {3, TAG_ENC_U, TAG_ENC_E0, TAG_ENC_E1};
+static const SampleKinds kSampleConvert = {3, TAG_CONV_MU, TAG_CONV_E0, TAG_CONV_E1};
 
 // ---- host-side context (shared by the translation units that implement the C ABI) ----
 #include <vector>
@@ -197,11 +206,9 @@ cudaError_t secret_product(const DevView& v, const LimbParams& lp, cudaStream_t 
 cudaError_t muladd(const DevView& v, cudaStream_t s, const u64* a, const u64* b, const u64* c, \
                    u64* d, u32 batch); \
 cudaError_t check_selftest(const DevView& v, cudaStream_t s); \
-cudaError_t sample_encrypt_noise(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 ct_first, u32 n_cts, \
-                                 u32 unit_first, u32 n_units, u32* out); \
-cudaError_t sample_share_noise(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
-                               u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out, \
-                               bool fft); \
+cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
+                           u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds, \
+                           bool fft_order, void* out); \
 cudaError_t share_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev, \
                       u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares); \
 cudaError_t fft_secret(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 n_parties, u32 tag, double2* dst); \

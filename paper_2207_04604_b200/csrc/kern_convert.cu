@@ -75,32 +75,9 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 }
 
 // mu_k, e_{0,k}, e_{1,k} of a conversion share do not depend on the limb: like the noise of the
-// decryption shares they are sampled once per share by a kernel of its own, one byte per
+// decryption shares they are sampled once per share by a kernel of its own (kern_sample.cu), one byte per
 // coefficient, into scratch memory that the caller of the launcher lends ([mu | e_0 | e_1], N bytes
 // each, per (recipient, ciphertext) unit and party), so the share kernel needs no clusters.
-// grid = ceil(n_units * n_parties * 3 * N / 4 / 256); one thread = four samples = one packed word.
-__global__ void __launch_bounds__(256)
-    k_sample_convert_noise(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties,
-                           u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units,
-                           u32* __restrict__ out) {
-  __shared__ GaussTab gt;
-  load_gauss(&gt, v.gauss);
-  const u32 words = v.n >> 2;
-  const size_t total = (size_t)n_units * n_parties * 3 * words;
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= total) return;  // the last block is ragged
-  const u32 w = (u32)(e % words), which = (u32)((e / words) % 3);
-  const size_t share = e / (3 * (size_t)words);
-  const u32 a = (u32)(share % n_parties), unit = unit_first + (u32)(share / n_parties);
-  const u32 party = parties[a], recipient = recipients[unit / n_cts];
-  if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) return;
-  const Stream st(v.seed, which == 0 ? TAG_CONV_MU : which == 1 ? TAG_CONV_E0 : TAG_CONV_E1, ct_first + unit % n_cts,
-                  party, recipient);
-  u32 pack = 0;
-#pragma unroll
-  for (u32 b = 0; b < 4; ++b) pack |= ((u32)gauss_from_r(gt, st.draw64(4 * w + b)) & 0xffu) << (8 * b);
-  out[e] = pack;
-}
 
 // Conversion shares (Eq. 2): (h_0, h_1) = (s_k c_1 + mu_k p_{0,i} + e_{0,k}, mu_k p_{1,i} + e_{1,k}).
 // grid = n_units * L; units unit_first .. unit_first + n_units - 1 of the (recipient, ciphertext) grid.
@@ -252,10 +229,8 @@ cudaError_t convert_share(const DevView& v, const LimbParams& lp, cudaStream_t s
   per_batch = whole_wave_batch(v, per_batch, n_units, v.L);
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    const size_t words = (size_t)nu * per_unit / 4;
-    k_sample_convert_noise<<<(unsigned)((words + 255) / 256), 256, 0, s>>>(
-        v, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, reinterpret_cast<u32*>(scratch));
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
+                                   kSampleConvert, false, scratch);
     if (e != cudaSuccess) return e;
     e = convert_share_units(v, lp, s, agg, recipients_dev, parties_dev, n_parties, n_cts, first, nu,
                             reinterpret_cast<const u32*>(scratch), shares);

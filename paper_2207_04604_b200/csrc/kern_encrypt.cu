@@ -5,34 +5,10 @@
 
 namespace {
 
-// u, e_0 and e_1 do not depend on the limb: a kernel of its own samples them once per (party,
+// u, e_0 and e_1 do not depend on the limb: a kernel of its own (kern_sample.cu) samples them once per (party,
 // ciphertext), one byte per coefficient, into scratch memory that the caller of the launcher lends
 // ([u | e_0 | e_1], N bytes each), and the encryption kernel stages them in shared memory.  No
 // thread-block clusters: every CTA is placed freely.
-// grid = ceil(n_units * 3 * N / 4 / 256); one thread = four samples = one packed word.
-__global__ void __launch_bounds__(256)
-    k_sample_encrypt_noise(DevView v, const u32* __restrict__ parties, u32 ct_first, u32 n_cts, u32 unit_first,
-                           u32 n_units, u32* __restrict__ small) {
-  __shared__ GaussTab gt;
-  load_gauss(&gt, v.gauss);
-  const u32 words = v.n >> 2;
-  const size_t total = (size_t)n_units * 3 * words;
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= total) return;
-  const u32 w = (u32)(e % words), which = (u32)((e / words) % 3), unit = unit_first + (u32)(e / (3 * (size_t)words));
-  const u32 party = parties[unit / n_cts], c = ct_first + unit % n_cts;
-  if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY)) return;
-  const Stream st(v.seed, which == 0 ? TAG_ENC_U : which == 1 ? TAG_ENC_E0 : TAG_ENC_E1, c, party, 0);
-  u32 pack = 0;
-  if (which == 0) {
-#pragma unroll
-    for (u32 b = 0; b < 4; ++b) pack |= ((u32)st.ternary(4 * w + b) & 0xffu) << (8 * b);
-  } else {
-#pragma unroll
-    for (u32 b = 0; b < 4; ++b) pack |= ((u32)gauss_from_r(gt, st.draw64(4 * w + b)) & 0xffu) << (8 * b);
-  }
-  small[e] = pack;
-}
 
 // grid = n_units * L * split; units unit_first .. unit_first + n_units - 1 of the (party, ciphertext) grid.
 // NTT(u) is parked in the output row of c_1 (re-read for both components, overwritten by
@@ -103,15 +79,6 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 
 namespace D2MHE_LAUNCH_NS {
 
-// u, e_0, e_1 of units unit_first .. unit_first + n_units - 1 into out ([u | e_0 | e_1], N bytes each, per unit)
-cudaError_t sample_encrypt_noise(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 ct_first, u32 n_cts,
-                                 u32 unit_first, u32 n_units, u32* out) {
-  const size_t words = (size_t)n_units * 3 * v.n / 4;
-  k_sample_encrypt_noise<<<(unsigned)((words + 255) / 256), 256, 0, s>>>(v, parties_dev, ct_first, n_cts, unit_first,
-                                                                        n_units, out);
-  return cudaGetLastError();
-}
-
 // The split variant serves calls of a few thread blocks, where the latency of one block's transforms is
 // what counts: at N = 4096 it runs with one octet per thread and round (512 threads per polynomial).
 #undef D2MHE_DISPATCH_G12
@@ -143,7 +110,7 @@ cudaError_t encrypt(const DevView& v, const LimbParams& lp, cudaStream_t s, cons
   per_batch = whole_wave_batch(v, per_batch, n_units, v.L);
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    cudaError_t e = sample_encrypt_noise(v, s, parties_dev, ct_first, n_cts, first, nu, reinterpret_cast<u32*>(scratch));
+    cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, false, scratch);
     if (e != cudaSuccess) return e;
     e = encrypt_units(v, lp, s, first, nu, reinterpret_cast<const u32*>(scratch), plain, ct);
     if (e != cudaSuccess) return e;

@@ -28,49 +28,10 @@ __device__ __forceinline__ u64 mont_lazy_sf(u64 a, u64 b, u64 p, u64 pinv, u32 d
 }
 
 // The noise polynomial e of a share does not depend on the limb.  It is sampled once per share by a
-// kernel of its own (Philox + table inversion, one byte per coefficient, into scratch memory that
-// the caller of the launcher lends), so the share kernel needs no thread-block clusters: every CTA
-// is placed freely and spends its time on the transforms.  (A variant that sampled inside the share
-// kernel and spread the samples over a cluster of the limbs' CTAs was 3 % slower at N = 8192 and
-// 8 % at N = 16384, where clusters of one-CTA-per-SM blocks also leave SMs idle.)
-//
-// grid = ceil(n_units * n_parties * N / 4 / (256 * wpt)); one packed word = four samples, wpt words per thread.
-// noise[(u * n_parties + a) * N + j], u = unit - unit_first, unit = irec * n_cts + cl.
-// fft != 0 (the double-precision share kernel): the bytes of a share are e + 19, 32 for each of T = N / 32 threads in
-// the order of fft_coef, as 16-byte slots [2][T].
-__global__ void __launch_bounds__(256)
-    k_sample_share_noise(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties,
-                         u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units,
-                         u32* __restrict__ noise, u32 wpt, u32 fft) {
-  __shared__ GaussTab gt;
-  load_gauss(&gt, v.gauss);
-  const u32 words = v.n >> 2;
-  const size_t total = (size_t)n_units * n_parties * words;
-#pragma unroll 1
-  for (u32 it = 0; it < wpt; ++it) {  // several words per thread: the table load above is paid once
-    const size_t e = ((size_t)blockIdx.x * wpt + it) * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const u32 w = (u32)(e % words);
-    const size_t share = e / words;
-    const u32 a = (u32)(share % n_parties), unit = unit_first + (u32)(share / n_parties);
-    const u32 party = parties[a], recipient = recipients[unit / n_cts];
-    if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) continue;
-    const Stream se(v.seed, TAG_DEC_ERR, ct_first + unit % n_cts, party, recipient);
-    u32 pack = 0, j0 = 4 * w, step = 1;
-    int bias = 0;
-    if (fft) {
-      const u32 t = (w >> 2) & ((v.n >> 5) - 1), m = (w & 3u) + (w >= (v.n >> 3) ? 4u : 0u);  // word m of thread t
-      j0 = v.logn == 14   ? (t & 255u) + 2048u * (t >> 8) + 1024u * (m & 1u) + 4096u * (m >> 1)
-           : v.logn == 13 ? t + 1024u * m
-                          : t + 128u * (m >> 2) + 1024u * (m & 3u);
-      step = 256;
-      bias = D2MHE_GAUSS_B;
-    }
-#pragma unroll
-    for (u32 b = 0; b < 4; ++b) pack |= ((u32)(gauss_from_r(gt, se.draw64(j0 + b * step)) + bias) & 0xffu) << (8 * b);
-    noise[e] = pack;
-  }
-}
+// kernel of its own (kern_sample.cu: one byte per coefficient, into scratch memory that the caller of the launcher
+// lends), so the share kernel needs no thread-block clusters: every CTA is placed freely and spends its time on the
+// transforms.  (A variant that sampled inside the share kernel and spread the samples over a cluster of the limbs'
+// CTAs was 3 % slower at N = 8192 and 8 % at N = 16384, where clusters of one-CTA-per-SM blocks also leave SMs idle.)
 
 // grid = n_units * L * split; units unit_first .. unit_first + n_units - 1 of the (recipient, ciphertext)
 // grid.  split > 1 (chosen by the launcher when the grid would otherwise leave most SMs idle) gives the
@@ -144,19 +105,6 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 
 namespace D2MHE_LAUNCH_NS {
 
-// the noise of the shares of units unit_first .. unit_first + n_units - 1: N bytes per (unit, party)
-cudaError_t sample_share_noise(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
-                               u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out,
-                               bool fft) {
-  const size_t words = (size_t)n_units * n_parties * v.n / 4;
-  // four words per thread once the grid is several waves deep (the table load and its barrier are then paid
-  // once per 4096 samples); small calls keep one word per thread: their latency is what counts
-  const u32 wpt = words >= (size_t)256 * 4 * 8 * v.sms * 2 ? 4u : 1u;
-  k_sample_share_noise<<<(unsigned)((words + 256 * (size_t)wpt - 1) / (256 * (size_t)wpt)), 256, 0, s>>>(
-      v, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, n_units, out, wpt, fft ? 1u : 0u);
-  return cudaGetLastError();
-}
-
 #undef D2MHE_EXTRA_TARGS
 #define D2MHE_EXTRA_TARGS , false
 static cudaError_t pdec_units_plain(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg,
@@ -210,8 +158,8 @@ cudaError_t partial_decrypt_scratch(const DevView& v, const LimbParams& lp, cuda
   per_batch = whole_wave_batch(v, per_batch, n_units, v.L);
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    cudaError_t e = sample_share_noise(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
-                                       reinterpret_cast<u32*>(scratch), v.fft_on != 0);
+    cudaError_t e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
+                                   kSampleShare, v.fft_on != 0, scratch);
     if (e != cudaSuccess) return e;
     e = v.fft_on ? share_fft(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu, scratch, shares)
                  : pdec_pre_units(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu,

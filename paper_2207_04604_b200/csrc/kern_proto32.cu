@@ -284,7 +284,7 @@ cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, co
   if (per_batch == 0) return cudaErrorInvalidValue;
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    cudaError_t e = sample_encrypt_noise(v, s, parties_dev, ct_first, n_cts, first, nu, reinterpret_cast<u32*>(scratch));
+    cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, false, scratch);
     if (e != cudaSuccess) return e;
     e = encrypt32_units(v, lp, s, first, nu, reinterpret_cast<const u32*>(scratch), plain, ct);
     if (e != cudaSuccess) return e;
@@ -318,8 +318,8 @@ cudaError_t partial_decrypt32(const DevView& v, const LimbParams& lp, cudaStream
   }
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    cudaError_t e = sample_share_noise(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
-                                       reinterpret_cast<u32*>(scratch), false);
+    cudaError_t e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
+                                   kSampleShare, false, scratch);
     if (e != cudaSuccess) return e;
     e = pdec32_units(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu,
                      reinterpret_cast<const signed char*>(scratch), shares);

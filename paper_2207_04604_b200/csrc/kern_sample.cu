@@ -1,0 +1,109 @@
+// Small samples drawn ahead of the protocol kernels: error polynomials, u and mu_k, one byte per coefficient.
+#include <algorithm>
+
+#include "d2mhe_kernels_common.cuh"
+
+namespace {
+
+// A discrete Gaussian sample is a count of the thresholds at or below a 64-bit draw.  The table gives the count for
+// the top 12 bits; bit 7 marks the 0.9 % of the buckets that hold a threshold, where the exact thresholds decide.
+// (With 8 bits, one bucket in eight: nearly every warp walked the thresholds.)
+__device__ __forceinline__ u32 gauss_count(const GaussFast& g, u32 o0, u32 o1, u32 cnt) {
+  const u64 r = ((u64)o0 << 32) | o1;
+  cnt &= 0x7fu;
+  while (cnt < D2MHE_CDT_LEN && r >= g.cdt[cnt]) ++cnt;
+  return cnt;
+}
+
+// Polynomial number p of this launch: sample kind tag[p % n_tags] of share p / n_tags; N bytes each, one after
+// another.  A share is a (unit, party) pair (recipients != null) or a (party, ciphertext) unit.  A thread block works
+// on one polynomial, so all of the counter but the coefficient is uniform over the block and the first two of the ten
+// Philox rounds cost half.  What bounds it: the integer multiplier (17 widening multiplications per sample).
+// ORDER = 0: byte j is the sample of coefficient j, signed.  ORDER = 12, 13, 14 (log2 N): samples + 19 in the order in
+// which the threads of the double-precision kernels of that size need them (fft_coef): 32 for each of T = N / 32
+// threads, as 16-byte slots [2][T].
+// grid = polynomials * segs; a block draws words / segs packed words of its polynomial.
+// Measured at N = 8192, 32 M samples: 154 us with a block-independent kernel and an 8-bit table, 110 us now.
+template <int ORDER>
+__global__ void __launch_bounds__(256)
+    k_sample_streams(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties, u32 n_parties,
+                     u32 ct_first, u32 n_cts, u32 unit_first, SampleKinds kinds, u32 segs, u32* __restrict__ out) {
+  __shared__ GaussFast gt;
+  for (u32 i = threadIdx.x; i < sizeof(GaussFast) / 16; i += blockDim.x)
+    reinterpret_cast<uint4*>(&gt)[i] = __ldg(reinterpret_cast<const uint4*>(v.gauss_fast) + i);
+  __syncthreads();
+  const u32 poly = blockIdx.x / segs, seg = blockIdx.x % segs;
+  const u32 which = poly % kinds.n, share = poly / kinds.n;
+  const u32 tag = which == 0 ? kinds.tag0 : which == 1 ? kinds.tag1 : kinds.tag2;
+  const u32 unit = unit_first + (recipients ? share / n_parties : share);
+  const u32 party = recipients ? parties[share % n_parties] : parties[unit / n_cts];
+  const u32 recipient = recipients ? recipients[unit / n_cts] : 0u;
+  if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) return;
+  const u32 c1 = ct_first + unit % n_cts, c2 = party | (recipient << 16), k0 = (u32)v.seed, k1 = (u32)(v.seed >> 32);
+  const u32 words = v.n >> 2, per = words / segs;
+  u32* dst = out + (size_t)poly * words;
+#pragma unroll 1
+  for (u32 w = seg * per + threadIdx.x; w < (seg + 1) * per; w += blockDim.x) {
+    u32 j0 = 4 * w;
+    constexpr u32 step = ORDER ? 256u : 1u;
+    if (ORDER) {
+      constexpr u32 T = (1u << ORDER) / 32u;
+      const u32 t = (w >> 2) & (T - 1), m = (w & 3u) + 4u * (w / (ORDER ? 4u * T : 1u));  // word m of thread t
+      j0 = ORDER == 14   ? (t & 255u) + 2048u * (t >> 8) + 1024u * (m & 1u) + 4096u * (m >> 1)
+           : ORDER == 13 ? t + 1024u * m
+                         : t + 128u * (m >> 2) + 1024u * (m & 3u);
+    }
+    u32 o0[4], o1[4], e[4];
+#pragma unroll
+    for (u32 b = 0; b < 4; ++b) {
+      u32 o2, o3;
+      philox4x32_10(k0, k1, j0 + b * step, c1, c2, tag, o0[b], o1[b], o2, o3);
+    }
+    if (tag == TAG_ENC_U) {
+#pragma unroll
+      for (u32 b = 0; b < 4; ++b) e[b] = __umulhi(o0[b], 3u) + (D2MHE_GAUSS_B - 1);
+    } else {
+#pragma unroll
+      for (u32 b = 0; b < 4; ++b) e[b] = gt.lut[o0[b] >> 20];
+      if ((e[0] | e[1] | e[2] | e[3]) & 0x80u) {
+#pragma unroll
+        for (u32 b = 0; b < 4; ++b)
+          if (e[b] & 0x80u) e[b] = gauss_count(gt, o0[b], o1[b], e[b]);
+      }
+    }
+    u32 pack = e[0] | (e[1] << 8) | (e[2] << 16) | (e[3] << 24);
+    if (!ORDER) pack = __vsub4(pack, 0x01010101u * D2MHE_GAUSS_B);
+    dst[w] = pack;
+  }
+}
+
+}  // namespace
+
+namespace D2MHE_LAUNCH_NS {
+
+cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
+                           u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds,
+                           bool fft_order, void* out) {
+  const u32 words = v.n >> 2, threads = std::max(32u, std::min(words, 256u));
+  const size_t polys = (size_t)n_units * (recipients_dev ? n_parties : 1u) * kinds.n;
+  // Eight words per thread, so that the table is fetched once for 8192 samples (2 % over two words on the share call);
+  // when that does not fill the GPU (eight blocks per SM), down to one word per thread.
+  u32 segs = std::max(1u, words / (8 * threads));
+  while (segs * 2 * threads <= words && polys * segs < (size_t)8 * v.sms) segs *= 2;
+  const unsigned grid = (unsigned)(polys * segs);
+  u32* o = reinterpret_cast<u32*>(out);
+  switch (fft_order ? v.logn : 0) {
+#define D2MHE_SAMPLE(ORDER_)                                                                                         \
+  k_sample_streams<ORDER_><<<grid, threads, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first, n_cts,       \
+                                                    unit_first, kinds, segs, o)
+    case 0: D2MHE_SAMPLE(0); break;
+    case 12: D2MHE_SAMPLE(12); break;
+    case 13: D2MHE_SAMPLE(13); break;
+    case 14: D2MHE_SAMPLE(14); break;
+    default: return cudaErrorInvalidValue;
+#undef D2MHE_SAMPLE
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace D2MHE_LAUNCH_NS

@@ -193,22 +193,21 @@ __device__ __forceinline__ cpx fft_twist(const cpx tw, u32 group) {
   }
 }
 
-// Forward transform.  in(j): the coefficients j and j + n as a complex number, j < n.  Leaves
-// Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
+// Forward transform.  in(c, jC, h): the coefficients j and j + n as a complex number, j = r + 256 jC + h n/2 with
+// r = tg + c TG (h = 0 for one group).  Leaves Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
 template <int LOGN, class In>
-__device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
+__device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
   using G = FftGeo<LOGN>;
   constexpr int R = G::R;
   const u32 g = sm.group();
-#pragma unroll
-  for (int c = 0; c < G::COLS; ++c) {
-    const u32 r = sm.tg + (u32)(c * G::TG);
-    const cpx t = ld_cpx(ft.twist + 256 * g + r);
+  static_for<G::COLS>([&](auto c_) {
+    constexpr int c = decltype(c_)::value;
+    const cpx t = ld_cpx(ft.twist + 256 * g + sm.tg + (u32)(c * G::TG));
     static_for<R>([&](auto j_) {
       constexpr int j = decltype(j_)::value;
-      cpx z = in(r + 256u * (u32)j);
+      cpx z = in(c_, j_, std::integral_constant<int, 0>{});
       if constexpr (G::GR == 2) {  // z_j +- q z_(j + n/2)
-        const cpx y = in(r + 256u * (u32)j + G::NG);
+        const cpx y = in(c_, j_, std::integral_constant<int, 1>{});
         const double h = g ? -root_c<16>() : root_c<16>();
         z = cpx{D2MHE_FMA(h, y.r - y.i, z.r), D2MHE_FMA(h, y.r + y.i, z.i)};
       }
@@ -218,7 +217,7 @@ __device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTa
       xi[c * R + j] = z.i;
     });
     fft_eval<R, 1, 0>(xr + c * R, xi + c * R, TwNone());
-  }
+  });
   __syncthreads();  // previous users of ex are done
   fft_put_cols<LOGN>(sm, xr, xi);
   sm.group_sync();
@@ -237,12 +236,33 @@ __device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTa
   }
 }
 
+// in(j): the same by coefficient number, j < n
+template <int LOGN, class In>
+__device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
+  using G = FftGeo<LOGN>;
+  fft_forward_at<LOGN>(sm, ft, xr, xi, [&](auto c_, auto j_, auto h_) {
+    return in(sm.tg + (u32)(c_.value * G::TG + 256 * j_.value + h_.value * G::NG));
+  });
+}
+
 // A transform in tensor memory: four points (k, k + 8, k + 4, k + 12) after one another, as fft_product4 takes them.
 __device__ __forceinline__ void fft_to_tmem(u32 addr, const double* xr, const double* xi) {
   static_for<4>([&](auto q_) {
     cpx c[4];
     static_for<4>([&](auto i_) {
       constexpr int k = brev_c<16>(decltype(q_)::value + 4 * brev_c<4>(decltype(i_)::value));
+      c[i_.value] = cpx{xr[k], xi[k]};
+    });
+    tmem_store4(addr + q_.value * 16, c);
+  });
+}
+
+// the same for the points of a stored transform as fft_load leaves them
+__device__ __forceinline__ void fft_loaded_to_tmem(u32 addr, const double* xr, const double* xi) {
+  static_for<4>([&](auto q_) {
+    cpx c[4];
+    static_for<4>([&](auto i_) {
+      constexpr int k = decltype(q_)::value + 4 * brev_c<4>(decltype(i_)::value);
       c[i_.value] = cpx{xr[k], xi[k]};
     });
     tmem_store4(addr + q_.value * 16, c);

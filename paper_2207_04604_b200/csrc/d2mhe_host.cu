@@ -438,6 +438,8 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     }
     c->view.s_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
+    c->view.pk_fft = dev_alloc<double2>(c, 4 * (size_t)L * (n / 2), &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
     c->view.fft_on = 1;
   }
 
@@ -719,6 +721,11 @@ d2mhe_status d2mhe_collective_pk(d2mhe_ctx* c, const u32* parties, u32 n_parties
   c->launches += 1;
   if (c->view.pk32) {
     e = L_(make_tab32)(c->view, c->stream, c->view.pk_mont, c->view.pk32, 2 * (size_t)c->view.L);
+    if (e != cudaSuccess) return fail_staged(c, sg, e);
+    c->launches += 1;
+  }
+  if (c->view.fft_on) {
+    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, 2 * c->view.L, c->view.pk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
   }
@@ -1332,10 +1339,11 @@ static d2mhe_status round_impl(d2mhe_ctx* c, const int32_t* values, bool host_io
           return e;
       }
       unsigned char* noise = reinterpret_cast<unsigned char*>(shares + (size_t)K * S * cc * polyw);
-      const size_t noise_bytes = round_noise_bytes_per_ct(c) * cc;  // first u, e_0, e_1, later the shares' noise
+      const size_t noise_bytes = round_noise_bytes_per_ct(c) * cc;
       u32 enc_launches = 0;
-      if ((e = L_(encrypt)(c->view, c->limb_params, s, sg.dev[0], K, ct_first + done, cc, plain, ct, noise,
-                           noise_bytes, &enc_launches)) != cudaSuccess)
+      // what the encryption samples ahead goes where the shares and their noise will be
+      if ((e = L_(encrypt)(c->view, c->limb_params, s, sg.dev[0], K, ct_first + done, cc, plain, ct, shares,
+                           (size_t)K * S * cc * polyw * sizeof(u64) + noise_bytes, &enc_launches)) != cudaSuccess)
         return e;
       if ((e = L_(aggregate)(c->view, s, ct, cc, sg.dev[2], sg.dev[3], K, agg)) != cudaSuccess) return e;
       u32 pdec_launches = 0;

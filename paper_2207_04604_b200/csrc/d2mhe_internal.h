@@ -67,7 +67,8 @@ struct DevView {
   // ring products in double precision (set when the sizes are inside the bounds of d2mhe_fft.cuh)
   u32 fft_on;
   FftTab fft;
-  double2* s_fft;  // [K][n]  transforms of s_k, times 1/n
+  double2* s_fft;   // [K][n]        transforms of s_k, times 1/n
+  double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
@@ -211,6 +212,11 @@ cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipien
                            bool fft_order, void* out); \
 cudaError_t share_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev, \
                       u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares); \
+cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 ct_first, \
+                        u32 n_cts, u32 n_units, const u32* plain, u64* ct, void* scratch, size_t scratch_bytes, \
+                        u32* launches); \
+cudaError_t fft_samples(const DevView& v, cudaStream_t s, const void* src, u32 stride, u32 polys, double2* dst); \
+cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst); \
 cudaError_t fft_secret(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 n_parties, u32 tag, double2* dst); \
 cudaError_t make_tab32(const DevView& v, cudaStream_t s, const u64* src, u64* dst, size_t rows); \
 cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \

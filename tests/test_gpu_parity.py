@@ -1267,3 +1267,23 @@ def test_share_products_at_the_limits_of_the_split(d2, log2_n, bits, L, K):
     ctx.sync()
     assert np.array_equal(d2.to_u64_numpy(shares), o.partial_decrypt(agg, [K - 1], parties, 5))
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,C", [(12, 54, 1, 75), (12, 36, 3, 40), (13, 55, 1, 1), (13, 54, 3, 50), (14, 54, 1, 3), (14, 50, 5, 31)])
+def test_encrypt_sizes_against_oracle(d2, log2_n, bits, L, C):
+    """One and two thread blocks per ciphertext and limb, calls of part of a wave and of more than one; plaintext
+    coefficients at both ends of their range."""
+    moduli = wl.ntt_primes(bits, 2 << log2_n, L)
+    ctx = d2.Context(log2_n, moduli, 2, seed=78)
+    o = make_oracle(log2_n, moduli, seed=78)
+    ctx.keygen_share([0, 1])
+    ctx.collective_pk([0, 1])
+    pk = o.collective_pk([0, 1])
+    rng = np.random.default_rng(C)
+    plain = rng.integers(0, T, (1, C, 1 << log2_n)).astype(np.uint32)
+    plain[0, 0, ::2] = T - 1
+    ct = ctx.empty_u64(1, C, 2, L, 1 << log2_n)
+    ctx.encrypt([1], 9, C, d2.from_u32_numpy(plain, ctx.device), ct)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(ct), o.encrypt(pk, [1], 9, plain))
+    ctx.close()

@@ -23,6 +23,9 @@
 // four fraction bits and rounds twice (1/16), and 0.41 + 1/16 < 1/2: the rounded value IS the integer.  (Seen:
 // 2^-14 with random and with extreme c, 2^-10 with s = all ones.)  The low part has h <= 40 - log2 N bits, so that
 // its product fits 40 bits for any c and s.
+// Conversion adds the product of a public key (uniform: |p|_2 is sqrt(3) smaller) with a Gaussian mu (|M_k| 3.9 times
+// larger): there the 2-norm bound is 1.4, and what is relied on is that the error is spread, as rounding errors are: it
+// would take a tenth of its square on one of the 16384 coefficients to reach 1/2 (seen: 2^-13).
 //
 // Organisation.  A group of 16 R threads (R = 8 or 16) transforms 256 R points, 16 of them in a thread's registers.
 // Index digits k = kC + R kB + 16 R kA, j = jA + 16 jB + 256 jC:
@@ -260,6 +263,27 @@ D2MHE_HD void fft_product4(double* xr, double* xi, int k, const cpx (&c)[4]) {
   xi[i3] = D2MHE_FMA(2.0, x2.i, -xi[i2]);
   fft_bfly_one(xr[i0], xi[i0], xr[i2], xi[i2]);
   fft_bfly_i<SGN>(xr[i1], xi[i1], xr[i3], xi[i3]);
+}
+
+D2MHE_HD cpx cmul_add(cpx a, cpx b, cpx c) {
+  return cpx{D2MHE_FMA(-a.i, b.i, D2MHE_FMA(a.r, b.r, c.r)), D2MHE_FMA(a.i, b.r, D2MHE_FMA(a.r, b.i, c.i))};
+}
+// The same for the sums c x + a b of two products each.
+template <int SGN>
+D2MHE_HD void fft_product4_sum(double* xr, double* xi, int k, const cpx (&c)[4], const cpx (&a)[4], const cpx (&b)[4]) {
+  const int at[4] = {k, k + 8, k + 4, k + 12};
+#pragma unroll
+  for (int h = 0; h < 4; h += 2) {
+    const int i = at[h], j = at[h + 1];
+    const cpx x = cmul_add(a[h], b[h], cmul(c[h], cpx{xr[i], xi[i]}));
+    const cpx y = cmul_add(a[h + 1], b[h + 1], cmul_add(c[h + 1], cpx{xr[j], xi[j]}, x));
+    xr[i] = y.r;
+    xi[i] = y.i;
+    xr[j] = D2MHE_FMA(2.0, x.r, -y.r);
+    xi[j] = D2MHE_FMA(2.0, x.i, -y.i);
+  }
+  fft_bfly_one(xr[k], xi[k], xr[k + 4], xi[k + 4]);
+  fft_bfly_i<SGN>(xr[k + 8], xi[k + 8], xr[k + 12], xi[k + 12]);
 }
 
 // The split of a residue c in [0, p): centred, low part in [-2^(h-1), 2^(h-1)), high part the rest.

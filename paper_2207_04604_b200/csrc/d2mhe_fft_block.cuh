@@ -301,6 +301,38 @@ __device__ __forceinline__ void fft_product_tmem(u32 addr, double* xr, double* x
   });
 }
 
+// The same with a stored transform instead of the one in tensor memory.
+template <int LOGN>
+__device__ __forceinline__ void fft_product_row(const double2* row, double* xr, double* xi) {
+  static_for<4>([&](auto q_) {
+    constexpr int q = decltype(q_)::value;
+    cpx c[4];
+    static_for<4>([&](auto i_) {
+      c[i_.value] = ld_cpx(row + threadIdx.x + (q + 4 * brev_c<4>(decltype(i_)::value)) * FftGeo<LOGN>::T);
+    });
+    fft_product4<-1>(xr, xi, q, c);
+  });
+}
+// Sums of two products: registers by tensor memory, and two stored transforms.
+template <int LOGN>
+__device__ __forceinline__ void fft_product_sum(u32 addr, const double2* row_a, const double2* row_b, double* xr,
+                                                double* xi) {
+  static_for<4>([&](auto q_) {
+    constexpr int q = decltype(q_)::value;
+    TmemQuad quad;
+    quad.issue(addr + q * 16);
+    cpx a[4], b[4], c[4];
+    static_for<4>([&](auto i_) {
+      constexpr int k = q + 4 * brev_c<4>(decltype(i_)::value);
+      a[i_.value] = ld_cpx(row_a + threadIdx.x + k * FftGeo<LOGN>::T);
+      b[i_.value] = ld_cpx(row_b + threadIdx.x + k * FftGeo<LOGN>::T);
+    });
+    tmem_wait();
+    quad.get(c);
+    fft_product4_sum<-1>(xr, xi, q, c, a, b);
+  });
+}
+
 // Inverse transform of what the products left, up to the twist: digit jC of column r = tg + c TG is left in
 // x[c R + brev(jC)]; tw: the columns' twist.  before_last(): called ahead of the arithmetic of pass C.
 // Table entries are fetched a pass ahead of their use (they come from L2 as often as not).
@@ -432,12 +464,33 @@ struct FftNoise {
   }
 };
 
+struct FftNoNoise {
+  template <int I>
+  __device__ __forceinline__ u32 get() const {
+    return D2MHE_GAUSS_B;
+  }
+};
+
+// How many thread blocks share the parties of a unit, each of which transforms c_1 for itself: the split with the
+// shortest schedule, counted in part transforms (2 forward + per_party for each party) over whole waves of blocks.
+inline u32 fft_party_split(const DevView& v, u32 base, u32 ctas, u32 n_parties, u32 per_party) {
+  const u32 resident = v.sms * ctas;
+  u32 split = 1;
+  u64 best = ~0ull;
+  for (u32 c = 1; c <= n_parties && c <= 16u; ++c) {
+    const u64 waves = ((u64)base * c + resident - 1) / resident, per = (n_parties + c - 1) / c;
+    const u64 cost = waves * (2 + per_party * per);
+    if (cost < best) best = cost, split = c;
+  }
+  return split;
+}
+
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
 // High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  (One copy of
 // the code for both parts: two copies share subexpressions, and 300 bytes of them were spilled.)
-template <int LOGN, class Store>
+template <int LOGN, class Noise, class Store>
 __device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
-                                           double* xr, double* xi, bool high, const FftNoise<LOGN>& nz, Store store) {
+                                           double* xr, double* xi, bool high, const Noise& nz, Store store) {
   using G = FftGeo<LOGN>;
   const double magic = high ? lt.fft_magic : D2MHE_FFT_MAGIC_LO;
   fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4]) {

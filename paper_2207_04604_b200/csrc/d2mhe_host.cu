@@ -440,6 +440,10 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
     c->view.pk_fft = dev_alloc<double2>(c, 4 * (size_t)L * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
+    c->view.usk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
+    c->view.upk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
     c->view.fft_on = 1;
   }
 
@@ -470,7 +474,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
     const size_t per_sm = logn == 12 ? 4 : logn == 13 ? 2 : 1;  // resident blocks of the transform kernels
     const size_t units = (2 * (size_t)sms * per_sm + L - 1) / L;
-    const size_t want = units * P.num_parties * 6 * n;
+    const size_t want = units * P.num_parties * (c->view.fft_on ? 11 : 6) * n;
     c->noise_scratch_bytes = std::min(kNoiseScratchMaxBytes, std::max(kNoiseScratchBytes, (want + 255) / 256 * 256));
   }
   c->noise_scratch = dev_alloc<unsigned char>(c, c->noise_scratch_bytes, &err);
@@ -725,7 +729,8 @@ d2mhe_status d2mhe_collective_pk(d2mhe_ctx* c, const u32* parties, u32 n_parties
     c->launches += 1;
   }
   if (c->view.fft_on) {
-    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, 2 * c->view.L, c->view.pk_fft);
+    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, nullptr, 2 * c->view.L,
+                     c->view.pk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
   }
@@ -1037,6 +1042,14 @@ d2mhe_status d2mhe_user_keygen(d2mhe_ctx* c, const u32* users, u32 n_users, uint
   cudaError_t e = L_(user_keygen)(c->view, c->limb_params, c->stream, sg.dev[0], n_users);
   if (e != cudaSuccess) return fail_staged(c, sg, e);
   c->launches += 1;
+  if (c->view.fft_on) {
+    e = L_(fft_secret)(c->view, c->stream, sg.dev[0], n_users, TAG_USER_SECRET, c->view.usk_fft);
+    if (e == cudaSuccess)
+      e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.upk_coef, sg.dev[0], n_users * 2 * c->view.L,
+                       c->view.upk_fft);
+    if (e != cudaSuccess) return fail_staged(c, sg, e);
+    c->launches += 2;
+  }
   const size_t pk_words = 2 * (size_t)c->view.L * c->view.n;
   if (pk_out_dev) {
     for (u32 i = 0; i < n_users; ++i) {

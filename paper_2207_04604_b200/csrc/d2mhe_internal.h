@@ -69,6 +69,8 @@ struct DevView {
   FftTab fft;
   double2* s_fft;   // [K][n]        transforms of s_k, times 1/n
   double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n
+  double2* usk_fft;  // [K][n]            the same of the users' own keys
+  double2* upk_fft;  // [K][2][L][2][n]
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
@@ -79,6 +81,7 @@ struct SampleKinds {
 };
 static const SampleKinds kSampleShare = {1, TAG_DEC_ERR, 0, 0};
 static const SampleKinds kSampleEncrypt = {3, TAG_ENC_U, TAG_ENC_E0, TAG_ENC_E1};
+static const SampleKinds kSampleBoot = {2, TAG_BOOT_E0, TAG_BOOT_E1, 0};
 static const SampleKinds kSampleConvert = {3, TAG_CONV_MU, TAG_CONV_E0, TAG_CONV_E1};
 
 // ---- host-side context (shared by the translation units that implement the C ABI) ----
@@ -216,7 +219,20 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
                         u32 n_cts, u32 n_units, const u32* plain, u64* ct, void* scratch, size_t scratch_bytes, \
                         u32* launches); \
 cudaError_t fft_samples(const DevView& v, cudaStream_t s, const void* src, u32 stride, u32 polys, double2* dst); \
-cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst); \
+cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, const u32* users_dev, \
+                     u32 rows, double2* dst); \
+cudaError_t convert_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, \
+                        const u32* recipients_dev, u32 n_rec, const u32* parties_dev, u32 n_parties, u32 ct_first, \
+                        u32 n_cts, u64* shares, void* scratch, size_t scratch_bytes, u32* launches); \
+cudaError_t boot_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* recipients_dev, \
+                     u32 n_rec, const u32* parties_dev, u32 n_parties, u32 ct_first, u32 n_cts, u64* shares, \
+                     void* scratch, size_t scratch_bytes, u32* launches); \
+cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
+                         u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out); \
+cudaError_t sample_alpha(const DevView& v, cudaStream_t s, const u32* recipients_dev, u32 ct_first, u32 n_cts, \
+                         u32 unit_first, u32 n_units, u64* out); \
+cudaError_t secret_product_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* ct, \
+                               const u32* users_dev, u32 n_users, u32 n_cts, u64* prod); \
 cudaError_t fft_secret(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 n_parties, u32 tag, double2* dst); \
 cudaError_t make_tab32(const DevView& v, cudaStream_t s, const u64* src, u64* dst, size_t rows); \
 cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \

@@ -223,6 +223,12 @@ cudaError_t convert_share(const DevView& v, const LimbParams& lp, cudaStream_t s
                           u32 ct_first, u32 n_cts, u64* shares, void* scratch, size_t scratch_bytes, u32* launches) {
   const size_t per_unit = (size_t)n_parties * 3 * v.n;
   const u32 n_units = n_rec * n_cts;
+  // double-precision products; lists of parties too long for their samples take the modular transforms
+  if (v.fft_on && launches && scratch_bytes >= (size_t)n_parties * 11 * v.n) {
+    *launches = 0;
+    return convert_fft(v, lp, s, agg, recipients_dev, n_rec, parties_dev, n_parties, ct_first, n_cts, shares, scratch,
+                       scratch_bytes, launches);
+  }
   u32 per_batch = (u32)std::min<size_t>(scratch_bytes / per_unit, n_units);
   if (launches) *launches = 0;
   if (per_batch == 0) return cudaErrorInvalidValue;
@@ -252,6 +258,7 @@ cudaError_t convert_combine(const DevView& v, cudaStream_t s, const u64* agg, co
 
 cudaError_t secret_product(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* ct,
                            const u32* users_dev, u32 n_users, u32 n_cts, u64* prod) {
+  if (v.fft_on) return secret_product_fft(v, lp, s, ct, users_dev, n_users, n_cts, prod);
   D2MHE_DISPATCH(k_secret_product, v, n_users * n_cts * v.L, s, v, lp, ct, users_dev, n_cts, prod);
 }
 

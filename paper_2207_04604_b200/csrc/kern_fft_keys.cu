@@ -56,20 +56,28 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   fft_store<LOGN>(dst + (size_t)blockIdx.x * G::n, xr, xi, 1.0);
 }
 
-// Both parts of residue rows, times 1/n.   grid = rows * 2; limb of row r = r mod L; dst: [rows][2][n]
+// Both parts of residue rows, times 1/n.   grid = rows * 2; limb of row r = r mod L; src: [..][N], dst: [..][2][n].
+// users != null: row r is row r mod 2L of user users[r / 2L].
 template <int LOGN>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
-    k_fft_rows(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ src, double2* __restrict__ dst) {
+    k_fft_rows(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ src, const u32* __restrict__ users,
+               double2* __restrict__ dst) {
   using G = FftGeo<LOGN>;
-  const u32 half = blockIdx.x & 1u, r = blockIdx.x >> 1;
+  const u32 half = blockIdx.x & 1u;
+  size_t r = blockIdx.x >> 1;
+  if (users) {
+    const u32 user = users[r / (2 * v.L)];
+    if (!D2MHE_CHK(v.chk, user, v.K, SITE_PARTY)) return;
+    r = (size_t)user * 2 * v.L + r % (2 * v.L);
+  }
   const LimbTab& lt = lp.limbs[r % v.L];
-  const u64* row = src + (size_t)r * v.n;
+  const u64* row = src + r * v.n;
   double xr[16], xi[16];
   fft_forward<LOGN>(FftSmem<LOGN>(), v.fft, xr, xi, [&](u32 j) {
     if (!D2MHE_CHK(v.chk, j + G::n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
     return fft_split_pair(row, j, G::n, half, lt);
   });
-  fft_store<LOGN>(dst + (size_t)blockIdx.x * G::n, xr, xi, 1.0 / (double)G::n);
+  fft_store<LOGN>(dst + (2 * r + half) * G::n, xr, xi, 1.0 / (double)G::n);
 }
 
 // KERNEL<LOGN> with the exchange area as its shared memory
@@ -102,9 +110,10 @@ cudaError_t fft_samples(const DevView& v, cudaStream_t s, const void* src, u32 s
   D2MHE_FFT_DISPATCH(k_fft_samples, polys, v, reinterpret_cast<const uint4*>(src), stride, dst)
 }
 
-// src: rows of N residues; dst: [rows][2][n]
-cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst) {
-  D2MHE_FFT_DISPATCH(k_fft_rows, rows * 2, v, lp, src, dst)
+// src: rows of N residues (of the listed users: 2L rows each); dst: [rows][2][n]
+cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, const u32* users_dev, u32 rows,
+                     double2* dst) {
+  D2MHE_FFT_DISPATCH(k_fft_rows, rows * 2, v, lp, src, users_dev, dst)
 }
 
 }  // namespace D2MHE_LAUNCH_NS

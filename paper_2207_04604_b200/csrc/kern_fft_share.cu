@@ -15,7 +15,9 @@ namespace {
 // 18.5 k instead of 17.3 k at N = 8192.)  The rounded low part waits in shared memory, thread by thread, for the high
 // part.  The shares are written with a streaming hint, so that the keys stay in L2.
 // grid = n_units * L * split; party a belongs to block a mod split of its unit.
-template <int LOGN>
+// OWN: the products c_1 sk_i with user i's own key instead (parties: the users of the units' rows, one to a unit, no
+// noise), as BFV.Decrypt needs them.
+template <int LOGN, bool OWN>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_share_fft(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ agg,
                 const u32* __restrict__ parties, u32 n_parties, u32 n_cts, u32 unit_first,
@@ -45,9 +47,9 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   tmem_store_done();
   // the stored transform of a party's key; a party number that fails the check reads row 0
   auto key_of = [&](u32 a) {
-    u32 party = parties[a];
+    u32 party = parties[OWN ? irec : a];
     if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY)) party = 0;
-    return v.s_fft + (size_t)party * n;
+    return (OWN ? v.usk_fft : v.s_fft) + (size_t)party * n;
   };
   const double2* key = key_of(part);
   u32 a = part;
@@ -56,12 +58,13 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   while (a < n_parties) {
     const double2* next = high && a + split < n_parties ? key_of(a + split) : key;  // the address, a part ahead
     u64* out = shares + (((size_t)irec * n_parties + a) * n_cts + cl) * poly + row;
-    FftNoise<LOGN> nz;
+    typename std::conditional<OWN, FftNoNoise, FftNoise<LOGN>>::type nz;
     cpx tw[G::COLS];
     fft_load<LOGN>(key, xr, xi);
     fft_product_tmem(tm + (high ? G::WORDS : 0), xr, xi);
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
-      if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16);
+      if constexpr (!OWN)
+        if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16);
     });
     fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
@@ -74,23 +77,14 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   if (tid < 32) tmem_free(tbase, G::tmem_cols(2));
 }
 
-template <int LOGN>
+template <int LOGN, bool OWN>
 cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
                          u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_share_fft<LOGN>, G::smem_bytes);
+  cudaError_t e = set_smem(k_share_fft<LOGN, OWN>, G::smem_bytes);
   if (e != cudaSuccess) return e;
-  // Parties of a unit over `split` blocks, each of which transforms c_1 for itself: the split with the
-  // shortest schedule, counted in part transforms (2 forward + 2 per share) over whole waves of blocks.
-  const u32 resident = v.sms * G::CTAS, base = n_units * v.L;
-  u32 split = 1;
-  u64 best = ~0ull;
-  for (u32 c = 1; c <= std::min(n_parties, 16u); ++c) {
-    const u64 waves = ((u64)base * c + resident - 1) / resident, per = (n_parties + c - 1) / c;
-    const u64 cost = waves * (2 + 2 * per);
-    if (cost < best) best = cost, split = c;
-  }
-  k_share_fft<LOGN><<<base * split, G::T, G::smem_bytes, s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
+  const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 2);
+  k_share_fft<LOGN, OWN><<<n_units * v.L * split, G::T, G::smem_bytes, s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
                                                               reinterpret_cast<const uint4*>(noise), shares, split);
   return cudaGetLastError();
 }
@@ -102,9 +96,21 @@ namespace D2MHE_LAUNCH_NS {
 cudaError_t share_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
                       u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   switch (v.logn) {
-    case 12: return launch_share<12>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
-    case 13: return launch_share<13>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
-    case 14: return launch_share<14>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    case 12: return launch_share<12, false>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    case 13: return launch_share<13, false>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    case 14: return launch_share<14, false>(v, lp, s, agg, parties_dev, n_parties, n_cts, unit_first, n_units, noise, shares);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// prod[i, c] = c_1 sk_i, canonical, for users[i] and ct[i, c]
+cudaError_t secret_product_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* ct,
+                               const u32* users_dev, u32 n_users, u32 n_cts, u64* prod) {
+  const u32 n_units = n_users * n_cts;
+  switch (v.logn) {
+    case 12: return launch_share<12, true>(v, lp, s, ct, users_dev, 1, n_cts, 0, n_units, nullptr, prod);
+    case 13: return launch_share<13, true>(v, lp, s, ct, users_dev, 1, n_cts, 0, n_units, nullptr, prod);
+    case 14: return launch_share<14, true>(v, lp, s, ct, users_dev, 1, n_cts, 0, n_units, nullptr, prod);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -77,9 +77,70 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// M_k uniform mod t by rejection on bitlen(t)-bit draws, N words per share.  Half of the draws are rejected for
+// t = 65537, and a warp that waits for the last lane of every coefficient needs six draws each; here a thread goes on to
+// its next coefficient as soon as one is accepted, and only the end of its 16 is waited for (three draws each).
+// grid = shares * segs, 16 coefficients per thread, or N / blockDim.x in one block where that is less.
+__global__ void __launch_bounds__(256)
+    k_sample_masks(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties, u32 n_parties,
+                   u32 ct_first, u32 n_cts, u32 unit_first, u32 segs, u32* __restrict__ out) {
+  const u32 share = blockIdx.x / segs, seg = blockIdx.x % segs;
+  const u32 unit = unit_first + share / n_parties, party = parties[share % n_parties], recipient = recipients[unit / n_cts];
+  if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) return;
+  const Stream st(v.seed, TAG_BOOT_MASK, ct_first + unit % n_cts, party, recipient);
+  const u64 t = v.round.t;
+  u64 tmask = 1;
+  while (tmask <= t) tmask <<= 1;
+  tmask -= 1;
+  const u32 per = v.n / segs, end = (seg + 1) * per;
+  u32* dst = out + (size_t)share * v.n;
+  u32 j = seg * per + threadIdx.x, attempt = 0;
+  while (j < end) {
+    u64 r = st.draw64(j, attempt);
+    r = attempt < 255 ? r & tmask : r % t;  // the rule of uniform_mod
+    if (r < t) {
+      dst[j] = (u32)r;
+      j += blockDim.x;
+      attempt = 0;
+    } else {
+      ++attempt;
+    }
+  }
+}
+
+// The common polynomial alpha of every unit, all limbs: [units][L][N].
+__global__ void __launch_bounds__(256)
+    k_sample_alpha(DevView v, const u32* __restrict__ recipients, u32 ct_first, u32 n_cts, u32 unit_first, u32 rows,
+                   u64* __restrict__ out) {
+  const size_t total = (size_t)rows << v.logn, stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
+    const u32 j = (u32)(e & (v.n - 1)), row = (u32)(e >> v.logn), l = row % v.L, unit = unit_first + row / v.L;
+    const u32 recipient = recipients[unit / n_cts];
+    if (!D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) continue;
+    const Stream st(v.seed, TAG_BOOT_ALPHA, ct_first + unit % n_cts, l, recipient);
+    out[e] = uniform_mod(st, j, v.limbs[l].p, v.limbs[l].mask);
+  }
+}
+
 }  // namespace
 
 namespace D2MHE_LAUNCH_NS {
+
+cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
+                         u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out) {
+  const u32 threads = std::max(32u, std::min(v.n, 256u)), segs = std::max(1u, v.n / (16 * threads));
+  k_sample_masks<<<n_units * n_parties * segs, threads, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first,
+                                                                n_cts, unit_first, segs, out);
+  return cudaGetLastError();
+}
+
+cudaError_t sample_alpha(const DevView& v, cudaStream_t s, const u32* recipients_dev, u32 ct_first, u32 n_cts,
+                         u32 unit_first, u32 n_units, u64* out) {
+  const size_t total = (size_t)n_units * v.L * v.n;
+  const u32 blocks = (u32)std::min<size_t>((total + 255) / 256, (size_t)v.sms * 32);
+  k_sample_alpha<<<blocks, 256, 0, s>>>(v, recipients_dev, ct_first, n_cts, unit_first, n_units * v.L, out);
+  return cudaGetLastError();
+}
 
 cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
                            u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds,

@@ -1287,3 +1287,36 @@ def test_encrypt_sizes_against_oracle(d2, log2_n, bits, L, C):
     ctx.sync()
     assert np.array_equal(d2.to_u64_numpy(ct), o.encrypt(pk, [1], 9, plain))
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,K,C", [(12, 56, 2, 3, 2), (13, 55, 2, 2, 1), (13, 36, 3, 5, 2), (14, 54, 2, 2, 1)])
+def test_conversion_and_refresh_products_against_oracle(d2, log2_n, bits, L, K, C):
+    """Every share of both calls on rings whose products run in double precision; c_1 holds values at the ends of both
+    parts of the split."""
+    moduli = wl.ntt_primes(bits, 2 << log2_n, L)
+    n, parties = 1 << log2_n, list(range(K))
+    ctx = d2.Context(log2_n, moduli, K, seed=79)
+    o = make_oracle(log2_n, moduli, seed=79)
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    o.collective_pk(parties)
+    pk_dev = ctx.empty_u64(K, 2, L, n)
+    ctx.user_keygen(parties, pk_dev)
+    pk_users = np.stack([o.user_pk(i) for i in parties])
+    assert np.array_equal(d2.to_u64_numpy(pk_dev), pk_users)
+    rng = np.random.default_rng(bits)
+    h = min((bits + 1) // 2, 40 - log2_n)
+    agg = np.zeros((K, C, 2, L, n), dtype=np.uint64)
+    for l, p in enumerate(moduli):
+        agg[:, :, :, l] = rng.integers(0, p, (K, C, 2, n), dtype=np.uint64)
+        agg[0, 0, 1, l, ::3] = rng.choice(np.array([0, p - 1, (p - 1) // 2, (p + 1) // 2, 1 << (h - 1)], dtype=np.uint64),
+                                          agg[0, 0, 1, l, ::3].size)
+    dagg = d2.from_u64_numpy(agg, ctx.device)
+    shares = ctx.empty_u64(K, K, C, 2, L, n)
+    ctx.convert_share(dagg, parties, parties, 3, C, shares)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(shares), o.convert_share(agg, pk_users, parties, parties, 3))
+    ctx.bootstrap_share(dagg, parties, parties, 3, C, shares)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(shares), o.boot_share(agg, parties, parties, 3))
+    ctx.close()

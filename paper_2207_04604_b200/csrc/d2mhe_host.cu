@@ -380,6 +380,35 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
     pt.IW = dev_upload(c, IW, &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
+    if (logn >= 12 && logn <= 14) {
+      // twiddles of the packing kernels, pass by pass: the lowest address bit and the stages of a pass as in PackGeo
+      std::vector<uint2> enc, dec;
+      const u32 r0 = logn % 4 ? logn % 4 : 4, T = n / 16;
+      for (u32 i = 0; i < (logn + 3) / 4; ++i) {
+        const u32 B = i == 0 ? logn - 4 : logn - r0 - 4 * i, lanes = 1u << B, his = T >> B;
+        const size_t e0 = enc.size(), d0 = dec.size();
+        enc.resize(e0 + 15 * (size_t)lanes, make_uint2(0, 0));
+        dec.resize(d0 + 15 * (size_t)his, make_uint2(0, 0));
+        for (u32 e = 0; e < 4; ++e) {
+          const u32 beta = B + 3 - e, s = logn - 1 - beta, m = 1u << s;  // address bit, log2 span / groups
+          for (u32 d = 0; d < (8u >> e); ++d)
+            for (u32 a0 = 0; a0 < lanes; ++a0) {
+              const u64 w = ipw[(2 * (d * lanes + a0) + 1) << s];
+              enc[e0 + (size_t)(16 - (16 >> e) + d) * lanes + a0] = make_uint2((u32)w, sh32(w));
+            }
+          for (u32 d = 0; d < (1u << e); ++d)
+            for (u32 x = 0; x < his; ++x) {
+              const u32 hi = B == 0 ? h_brv(x, logn - 4) : x;
+              const u64 w = pw[h_brv(m + ((hi << e) | d), logn)];
+              dec[d0 + (size_t)((1u << e) - 1 + d) * his + x] = make_uint2((u32)w, sh32(w));
+            }
+        }
+      }
+      pt.enc_tw = dev_upload(c, enc, &err);
+      if (err != cudaSuccess) return fail_cuda(c, err);
+      pt.dec_tw = dev_upload(c, dec, &err);
+      if (err != cudaSuccess) return fail_cuda(c, err);
+    }
     pt.ninv = (u32)h_inv(n % t, t);
     pt.ninv_sh = sh32(pt.ninv);
   }

@@ -16,6 +16,8 @@ struct PlainTab {
   u32 half;            // (t-1)/2
   const uint2* W;      // [N] psi_t^brv(i) as {w, floor(w 2^32 / t)}
   const uint2* IW;     // [N] inverses
+  const uint2* enc_tw; // the same by passes (kern_pack.cu), N = 4096 .. 16384
+  const uint2* dec_tw;
 };
 
 // Constants of the exact scale-and-round (mixed-radix conversion).
@@ -174,6 +176,10 @@ cudaError_t int_probe(const DevView& v, const LimbParams& lp, cudaStream_t s, u3
 cudaError_t export_secret(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* key, signed char* out); \
 cudaError_t encode(const DevView& v, cudaStream_t s, const int32_t* values, u32 n_cts, u32* plain); \
 cudaError_t decode(const DevView& v, cudaStream_t s, const u32* plain, u32 n_cts, int32_t* values); \
+cudaError_t encode16(const DevView& v, cudaStream_t s, const int32_t* values, u32 n_groups, u32 group, \
+                     size_t group_stride, u32* plain); \
+cudaError_t decode16(const DevView& v, cudaStream_t s, const u32* plain, u32 n_groups, u32 group, size_t group_stride, \
+                     int32_t* values); \
 cudaError_t encode_strided(const DevView& v, cudaStream_t s, const int32_t* values, u32 n_groups, u32 group, \
                            size_t group_stride, u32* plain); \
 cudaError_t decode_strided(const DevView& v, cudaStream_t s, const u32* plain, u32 n_groups, u32 group, \

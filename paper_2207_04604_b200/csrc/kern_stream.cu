@@ -320,6 +320,7 @@ cudaError_t combine32(const DevView& v, cudaStream_t s, const u32* agg, const u3
 // (elements); plain: [n_groups * group, N] contiguous
 cudaError_t encode_strided(const DevView& v, cudaStream_t s, const int32_t* values, u32 n_groups, u32 group,
                            size_t group_stride, u32* plain) {
+  if (v.logn >= 12 && v.logn <= 14) return encode16(v, s, values, n_groups, group, group_stride, plain);
   const size_t smem = (size_t)v.n * 4;
   cudaError_t e = set_smem(k_encode, smem);
   if (e != cudaSuccess) return e;
@@ -333,6 +334,7 @@ cudaError_t encode(const DevView& v, cudaStream_t s, const int32_t* values, u32 
 
 cudaError_t decode_strided(const DevView& v, cudaStream_t s, const u32* plain, u32 n_groups, u32 group,
                            size_t group_stride, int32_t* values) {
+  if (v.logn >= 12 && v.logn <= 14) return decode16(v, s, plain, n_groups, group, group_stride, values);
   const size_t smem = (size_t)v.n * 4;
   cudaError_t e = set_smem(k_decode, smem);
   if (e != cudaSuccess) return e;

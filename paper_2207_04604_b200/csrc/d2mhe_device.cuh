@@ -25,6 +25,9 @@ struct LimbTab {
   u64 mask;                     // 2^bitlen(q_l) - 1, for the rejection sampler
   u64 rmod, rmod_sh;            // 2^64 mod q_l: leaves Montgomery form; builds Shoup companions
   u32 red_shift, red_mul;       // bitlen(q_l) - 1 and floor(2^(bitlen + 15) / q_l): small-quotient reduction
+  u64 crt, crt_sh;              // (q / q_l)^-1 mod q_l
+  u64 frac;                     // floor(t 2^(F + b) / q_l), b = bitlen(q_l): see k_combine
+  u32 frac_shift;               // 64 - b
   u32 sf_d, sf_shift;           // q_l = 2^b - sf_d with b = 32 + sf_shift (set when b >= 32 and sf_d < 2^32)
   const ulonglong2* W;          // [N] forward twiddles psi^brv(i) as {w, floor(w 2^64 / q_l)}
   const ulonglong2* IW;         // [N] their inverses

@@ -231,6 +231,10 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   // floor(q/t) mod q_l: q = Delta t + (q mod t)  =>  Delta = -(q mod t) t^-1 (mod q_l)
   const u64 q_mod_t = q_mod(t);
 
+  u32 t_bits = 0;
+  for (u64 x = t; x; x >>= 1) ++t_bits;
+  const u32 frac_bits = 59 - t_bits;  // 24 terms below 2^(F + t_bits) fit 64 bits
+  c->view.round.frac_bits = frac_bits;
   bool fft_ok = logn >= 12 && logn <= 14;
   bool all_special = true;  // every prime is 2^b - d with b >= 32, d < 2^32 and 256 d < 2^b
   for (u32 l = 0; l < L; ++l) {
@@ -271,6 +275,23 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (!special) all_special = false;
     // Double-precision products (bounds: d2mhe_fft.cuh): the low part has h <= 40 - log2 N bits, the high part at most 28;
     // its results keep f = 32 - (bits - h) fraction bits.
+    {
+      u64 others = 1;  // q / q_l mod q_l
+      for (u32 m = 0; m < L; ++m)
+        if (m != l) others = h_mul(others, c->moduli[m] % p, p);
+      T.crt = h_inv(others, p);
+      T.crt_sh = h_shoup(T.crt, p);
+      // floor(t 2^(F + b) / p) bit by bit (t 2^(F + b) has up to 120 bits)
+      u64 rem = 0, quo = 0;
+      for (u32 i = 0; i < frac_bits + bits + 32; ++i) {
+        const u32 pos = frac_bits + bits + 31 - i;  // bit of t 2^(F + b)
+        rem = 2 * rem + (pos >= frac_bits + bits ? (t >> (pos - frac_bits - bits)) & 1 : 0);
+        quo = 2 * quo + (rem >= p ? 1 : 0);
+        if (rem >= p) rem -= p;
+      }
+      T.frac = quo;
+      T.frac_shift = 64 - bits;
+    }
     T.fft_h = std::min((bits + 1) / 2, 40 - logn);
     if (!special || bits - T.fft_h > 28) {
       fft_ok = false;

@@ -27,6 +27,7 @@ struct RoundTab {
   u64 t, t_sh;             // t and floor(2^64 / t)
   u64 half_mod_t;          // (q-1)/2 mod t
   u64 qinv_mod_t;          // q^-1 mod t
+  u32 frac_bits;           // fraction bits F of the fixed-point sum of t y_l / q_l
 };
 
 // Twiddle factors of the double-precision ring products: groups of m = 256 R points (w_k = e^(2 pi i / k)).

@@ -71,74 +71,117 @@ __global__ void __launch_bounds__(256)
 }
 
 // ---------------------------------------------------------------------------
-// Combine + exact scale-and-round.  One thread per coefficient.
-//   v_l = c_0 + sum_k h_k mod q_l;  w'_l = t v_l + (q-1)/2 mod q_l;
-//   mixed-radix digits d_i of w' in [0,q);  w' mod t = sum d_i prod_{j<i} q_j mod t;
-//   x = ((q-1)/2 - w') q^-1 mod t  =  round(t v / q) mod t.
-// grid = (n_rec * n_cts, N / 256)
+// Combine + exact scale-and-round.
+//   v_l = c_0 + sum_k h_k mod q_l;  y_l = v_l (q / q_l)^-1 mod q_l;
+//   t v / q = sum_l t y_l / q_l  (mod t),  x = round(that) mod t.
+// Every term is rounded down to F fraction bits (59 - bitlen(t): 42 for t = 65537), two units low at most, so the sum
+// is at most 2L units low, and x is exact unless the fraction of sum + 1/2 lies within 2L units below a whole number:
+// then (once in 2^38 for random input, never for a ciphertext with noise to spare) the mixed-radix conversion below
+// decides.  L + 1 products per coefficient instead of L (L + 7) / 2 and no array of digits: the kernel is left with its
+// loads.  (The digits for every coefficient, one coefficient per thread: 48 us for 70 units of 10 shares at N = 8192,
+// L = 4 and 73 us for 40 of one share at N = 16384, L = 8; 42 and 46 us now.)
+// grid = (n_rec * n_cts, N / 64), 32 L threads.
 // ---------------------------------------------------------------------------
-// Up to 8 limbs the kernel is held to 32 registers (a few spilled words) so that 8 CTAs = 2048 threads
-// are resident per SM: the share streams need the loads in flight more than the registers
-// (measured: -13 % at N = 16384, L = 8, 20 shares; -2 % at N = 8192, L = 4, 10 shares).
-// W = u64, or u32 for the 32-bit-word messages (same arithmetic on the loaded residues).
-template <int LMAX, class W>
-__global__ void __launch_bounds__(256, LMAX <= 8 ? 8 : 3)
-    k_combine(DevView v, const W* __restrict__ agg, const W* __restrict__ shares, u32 n_shares,
-              u32 share_comps, u32 n_cts, u32* __restrict__ plain) {
-  const u32 unit = blockIdx.x, irec = unit / n_cts, cl = unit % n_cts;
-  const u32 j = blockIdx.y * blockDim.x + threadIdx.x;
-  if (j >= v.n) return;
+
+// mixed-radix (Garner) digits d_i of w' = t v + (q-1)/2 in [0, q);  w' mod t = sum d_i prod_{j<i} q_j mod t;
+// x = ((q-1)/2 - w') q^-1 mod t.  acc(l): v_l, any 64-bit representative.
+template <class Acc>
+__device__ __noinline__ u32 round_exact(const DevView& v, Acc acc) {
   const u32 L = v.L;
-  if (!D2MHE_CHK(v.chk, L, (u32)LMAX + 1u, SITE_LIMB)) return;
+  u64 d[D2MHE_MAX_LIMBS];
+  const u64 t = v.round.t, tsh = v.round.t_sh;
+  u64 sum = 0;
+  for (u32 i = 0; i < L; ++i) {
+    const LimbTab* lt = v.limbs + i;
+    u64 tmp = addmod(shoup_full(acc(i), lt->tmod, lt->tmod_sh, lt->p), lt->half, lt->p);
+    for (u32 j = 0; j < i; ++j) {
+      const ulonglong2 gi = __ldg(v.round.ginv + i * L + j);
+      tmp = shoup_full(tmp + lt->cq - d[j], gi.x, gi.y, lt->p);
+    }
+    d[i] = tmp;
+    sum = shoup_full(sum + shoup_full(tmp, 1, tsh, t) * v.round.prefix_mod_t[i], 1, tsh, t);
+  }
+  const u64 diff = v.round.half_mod_t + t - sum;  // in (0, 2t)
+  return (u32)shoup_full(diff * v.round.qinv_mod_t, 1, tsh, t);
+}
+
+template <class W>
+struct Pair2;
+template <>
+struct Pair2<u64> {
+  typedef ulonglong2 type;
+};
+template <>
+struct Pair2<u32> {
+  typedef uint2 type;
+};
+
+// W = u64, or u32 for the 32-bit-word messages (same arithmetic on the loaded residues).
+// One warp per limb: a thread sums the shares of two coefficients of its limb, all of its loads independent of one
+// another, and the block adds up the limbs' terms through shared memory.  (All limbs in one thread, one after another,
+// had too few loads in flight: 59 us for the 70 units above.)
+template <class W>
+__global__ void __launch_bounds__(32 * D2MHE_MAX_LIMBS)
+    k_combine(const __grid_constant__ DevView v, const W* __restrict__ agg, const W* __restrict__ shares, u32 n_shares,
+              u32 share_comps, u32 n_cts, u32* __restrict__ plain) {
+  typedef typename Pair2<W>::type P2;
+  __shared__ u64 terms[D2MHE_MAX_LIMBS][64];
+  const u32 unit = blockIdx.x, irec = unit / n_cts, cl = unit % n_cts;
+  const u32 lane = threadIdx.x & 31u, wl = threadIdx.x >> 5, L = v.L, j0 = blockIdx.y * 64u, jj = j0 + 2 * lane;
   const size_t poly = (size_t)L * v.n;
   const W* c0 = agg + (size_t)unit * 2 * poly;
+  const W* sh = shares + ((size_t)irec * n_shares * n_cts + cl) * share_comps * poly;
+  const size_t kstride = (size_t)n_cts * share_comps * poly;
+  // primes below 2^57 and fewer than 120 shares: the plain 64-bit sum cannot overflow and the multiplication by the
+  // CRT factor reduces any 64-bit value, so the loads are all independent
   const bool lazy = (v.wide != 0 || sizeof(W) == 4) && n_shares < 120;
-  u64 d[LMAX];
+  if (jj < v.n && D2MHE_CHK(v.chk, wl, L, SITE_LIMB)) {
+    const LimbTab* lt = v.limbs + wl;
+    const u64 p = lt->p, w = lt->crt, ws = lt->crt_sh, fr = lt->frac;
+    const u32 fs = lt->frac_shift;
+    const size_t at = (size_t)wl * v.n + jj;
+    const P2 c = __ldg(reinterpret_cast<const P2*>(c0 + at));
+    u64 a0 = c.x, a1 = c.y;
+    const W* s = sh + at;
+    if (lazy) {
+      // ten shares at a time, predicated, so that the loads of a remainder are in flight together too
+      for (u32 k0 = 0; k0 < n_shares; k0 += 10) {
+        P2 h[10];
 #pragma unroll
-  for (int l = 0; l < LMAX; ++l) {
-    if (l < (int)L) {
-      const LimbTab* lt = v.limbs + l;
-      const u64 p = lt->p;
-      u64 acc = __ldg(c0 + (size_t)l * v.n + j);
-      const W* sh = shares + ((size_t)irec * n_shares * n_cts + cl) * share_comps * poly + (size_t)l * v.n + j;
-      const size_t kstride = (size_t)n_cts * share_comps * poly;
-      if (lazy) {
-        // primes below 2^57 and fewer than 120 shares: the plain 64-bit sum cannot overflow and the
-        // multiplication by t below reduces any 64-bit value, so the loads are all independent
-#pragma unroll 8
-        for (u32 k = 0; k < n_shares; ++k) acc += __ldg(sh + k * kstride);
-      } else {
-        for (u32 k = 0; k < n_shares; ++k) acc = addmod(acc, __ldg(sh + k * kstride), p);
+        for (u32 k = 0; k < 10; ++k) {
+          h[k].x = 0, h[k].y = 0;
+          if (k0 + k < n_shares) h[k] = __ldg(reinterpret_cast<const P2*>(s + (k0 + k) * kstride));
+        }
+#pragma unroll
+        for (u32 k = 0; k < 10; ++k) a0 += h[k].x, a1 += h[k].y;
       }
-      d[l] = addmod(shoup_full(acc, lt->tmod, lt->tmod_sh, p), lt->half, p);
-    }
-  }
-  // mixed-radix (Garner) digits in place: d_i <- ((w'_i - d_0) q_0^-1 - d_1) q_1^-1 ... mod q_i
-#pragma unroll
-  for (int i = 1; i < LMAX; ++i) {
-    if (i < (int)L) {
-      const LimbTab* lt = v.limbs + i;
-      const u64 p = lt->p, cq = lt->cq;
-      u64 tmp = d[i];
-#pragma unroll
-      for (int jj = 0; jj < i; ++jj) {
-        const ulonglong2 gi = __ldg(v.round.ginv + i * L + jj);
-        tmp = shoup_full(tmp + cq - d[jj], gi.x, gi.y, p);
+    } else {
+#pragma unroll 4
+      for (u32 k = 0; k < n_shares; ++k) {
+        const P2 h = __ldg(reinterpret_cast<const P2*>(s + k * kstride));
+        a0 = addmod(a0, h.x, p);
+        a1 = addmod(a1, h.y, p);
       }
-      d[i] = tmp;
     }
+    terms[wl][2 * lane] = mulhi_u64(shoup_full(a0, w, ws, p) << fs, fr);
+    terms[wl][2 * lane + 1] = mulhi_u64(shoup_full(a1, w, ws, p) << fs, fr);
   }
-  const u64 t = v.round.t, tsh = v.round.t_sh;
-  u64 acc = 0;
-#pragma unroll
-  for (int i = 0; i < LMAX; ++i) {
-    if (i < (int)L) {
-      const u64 di = shoup_full(d[i], 1, tsh, t);  // d_i mod t
-      acc = shoup_full(acc + di * v.round.prefix_mod_t[i], 1, tsh, t);
-    }
+  __syncthreads();
+  for (u32 i = threadIdx.x; i < 64u && j0 + i < v.n; i += blockDim.x) {
+    const u32 F = v.round.frac_bits;
+    u64 sum = (u64)1 << (F - 1);
+    for (u32 l = 0; l < L; ++l) sum += terms[l][i];
+    u32 x = (u32)shoup_full(sum >> F, 1, v.round.t_sh, v.round.t);
+    if ((sum & (((u64)1 << F) - 1)) >= ((u64)1 << F) - 2 * L)
+      x = round_exact(v, [&](u32 l) {
+        const size_t at = (size_t)l * v.n + j0 + i;
+        const u64 p = v.limbs[l].p;
+        u64 acc = c0[at];
+        for (u32 k = 0; k < n_shares; ++k) acc = addmod(acc, sh[k * kstride + at], p);
+        return acc;
+      });
+    plain[(size_t)unit * v.n + j0 + i] = x;
   }
-  const u64 diff = v.round.half_mod_t + t - acc;  // in (0, 2t)
-  plain[(size_t)unit * v.n + j] = (u32)shoup_full(diff * v.round.qinv_mod_t, 1, tsh, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -298,13 +341,8 @@ cudaError_t aggregate(const DevView& v, cudaStream_t s, const u64* ct, u32 n_cts
 template <class W>
 static cudaError_t combine_words(const DevView& v, cudaStream_t s, const W* agg, const W* shares, u32 n_rec,
                                  u32 n_shares, u32 share_comps, u32 n_cts, u32* plain) {
-  dim3 grid(n_rec * n_cts, (v.n + 255) / 256);
-  if (v.L <= 4)
-    k_combine<4, W><<<grid, 256, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
-  else if (v.L <= 8)
-    k_combine<8, W><<<grid, 256, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
-  else
-    k_combine<D2MHE_MAX_LIMBS, W><<<grid, 256, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
+  dim3 grid(n_rec * n_cts, (v.n + 63) / 64);
+  k_combine<W><<<grid, 32 * v.L, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
   return cudaGetLastError();
 }
 cudaError_t combine(const DevView& v, cudaStream_t s, const u64* agg, const u64* shares, u32 n_rec,

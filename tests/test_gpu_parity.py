@@ -6,7 +6,7 @@ import torch
 
 from paper_2207_04604_b200 import workloads as wl
 
-from common import T, make_oracle, psi_t_for, small_moduli
+from common import T, from_big, make_oracle, psi_t_for, q_of, small_moduli
 
 pytestmark = pytest.mark.gpu
 
@@ -1319,4 +1319,36 @@ def test_conversion_and_refresh_products_against_oracle(d2, log2_n, bits, L, K, 
     ctx.bootstrap_share(dagg, parties, parties, 3, C, shares)
     ctx.sync()
     assert np.array_equal(d2.to_u64_numpy(shares), o.boot_share(agg, parties, parties, 3))
+    ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,t", [(5, 30, 7, T), (6, 36, 3, T), (5, 54, 8, T), (4, 60, 24, T), (6, 54, 1, T), (5, 54, 4, (1 << 30) - 35),
+                                            (5, 36, 2, 97)])
+def test_rounding_on_both_sides_of_every_kind_of_boundary(d2, log2_n, bits, L, t):
+    """Values whose scaled quotient t v / q lies a fraction t / q or less to either side of m + 1/2 (where the fixed-point sum
+    cannot decide), a few fixed-point units away, and in the middle, against rounding of the big integers."""
+    moduli = small_moduli(log2_n, bits, L)
+    n, K = 1 << log2_n, 2
+    q = q_of(moduli)
+    ctx = d2.Context(log2_n, moduli, K, seed=80, plain_modulus=t)
+    ctx.keygen_share([0, 1])
+    ctx.collective_pk([0, 1])
+    rng = np.random.default_rng(bits)
+    vs = []
+    ulp = q >> (59 - t.bit_length())  # one fixed-point unit of t v / q is about ulp / t in v
+    for i in range(n):
+        m = int(rng.integers(0, t)) if i > 3 else (0, t - 1, 1, t // 2)[i]
+        base = (2 * m + 1) * q // (2 * t)
+        off = (0, 1, -1, 2, ulp // t, -ulp // t, (2 * L + 1) * ulp // t, -(2 * L + 1) * ulp // t, q // (3 * t), -q // (3 * t))[i % 10]
+        vs.append((base + off) % q)
+    half = [int(rng.integers(0, 1 << 62)) * (q >> 62) % q for _ in range(n)]  # split over c_0 and two shares
+    third = [int(rng.integers(0, 1 << 62)) * (q >> 62) % q for _ in range(n)]
+    agg = np.zeros((1, 1, 2, L, n), dtype=np.uint64)
+    agg[0, 0, 0] = from_big([(v - a - b) % q for v, a, b in zip(vs, half, third)], moduli)
+    shares = np.stack([from_big(half, moduli), from_big(third, moduli)]).reshape(1, 2, 1, L, n)
+    out = ctx.empty_u32(1, 1, n)
+    ctx.combine_decrypt(d2.from_u64_numpy(agg, ctx.device), d2.from_u64_numpy(shares, ctx.device), 1, 2, 1, out)
+    ctx.sync()
+    want = [((2 * t * v + q) // (2 * q)) % t for v in vs]
+    assert d2.to_u32_numpy(out)[0, 0].tolist() == want
     ctx.close()

@@ -864,8 +864,8 @@ d2mhe_status d2mhe_aggregate(d2mhe_ctx* c, const uint64_t* ct_dev, u32 n_rows, u
   const size_t counts[2] = {(size_t)n_out + 1, nnz ? (size_t)nnz : 1};
   d2mhe_status st = stage_indices(c, arrays, counts, 2, &sg);
   if (st != D2MHE_OK) return st;
-  cudaError_t e = L_(aggregate)(c->view, c->stream, reinterpret_cast<const u64*>(ct_dev), n_cts,
-                                          sg.dev[0], sg.dev[1], n_out, reinterpret_cast<u64*>(agg_dev));
+  cudaError_t e = L_(aggregate)(c->view, c->stream, reinterpret_cast<const u64*>(ct_dev), n_rows, n_cts,
+                                          sg.dev[0], sg.dev[1], n_out, nnz, reinterpret_cast<u64*>(agg_dev));
   if (e != cudaSuccess) return fail_staged(c, sg, e);
   c->launches += 1;
   return release_slot(c, sg);
@@ -1015,7 +1015,7 @@ d2mhe_status d2mhe_aggregate32(d2mhe_ctx* c, const uint32_t* ct_dev, u32 n_rows,
   const size_t counts[2] = {(size_t)n_out + 1, nnz ? (size_t)nnz : 1};
   d2mhe_status st = stage_indices(c, arrays, counts, 2, &sg);
   if (st != D2MHE_OK) return st;
-  cudaError_t e = L_(aggregate32)(c->view, c->stream, ct_dev, n_cts, sg.dev[0], sg.dev[1], n_out, agg_dev);
+  cudaError_t e = L_(aggregate32)(c->view, c->stream, ct_dev, n_rows, n_cts, sg.dev[0], sg.dev[1], n_out, nnz, agg_dev);
   if (e != cudaSuccess) return fail_staged(c, sg, e);
   c->launches += 1;
   return release_slot(c, sg);
@@ -1408,7 +1408,7 @@ static d2mhe_status round_impl(d2mhe_ctx* c, const int32_t* values, bool host_io
       if ((e = L_(encrypt)(c->view, c->limb_params, s, sg.dev[0], K, ct_first + done, cc, plain, ct, shares,
                            (size_t)K * S * cc * polyw * sizeof(u64) + noise_bytes, &enc_launches)) != cudaSuccess)
         return e;
-      if ((e = L_(aggregate)(c->view, s, ct, cc, sg.dev[2], sg.dev[3], K, agg)) != cudaSuccess) return e;
+      if ((e = L_(aggregate)(c->view, s, ct, K, cc, sg.dev[2], sg.dev[3], K, nnz, agg)) != cudaSuccess) return e;
       u32 pdec_launches = 0;
       if ((e = L_(partial_decrypt_scratch)(c->view, c->limb_params, s, agg, sg.dev[0], K, sg.dev[1], S,
                                            ct_first + done, cc, shares, noise, noise_bytes, &pdec_launches)) !=

@@ -188,8 +188,10 @@ cudaError_t decode_strided(const DevView& v, cudaStream_t s, const u32* plain, u
 cudaError_t encrypt(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \
                     u32 ct_first, u32 n_cts, const u32* plain, u64* ct, void* scratch, size_t scratch_bytes, \
                     u32* launches); \
-cudaError_t aggregate(const DevView& v, cudaStream_t s, const u64* ct, u32 n_cts, \
-                      const u32* offsets_dev, const u32* rows_dev, u32 n_out, u64* agg); \
+cudaError_t aggregate(const DevView& v, cudaStream_t s, const u64* ct, u32 n_rows, u32 n_cts, \
+                      const u32* offsets_dev, const u32* rows_dev, u32 n_out, u32 nnz, u64* agg); \
+cudaError_t aggregate_columns32(const DevView& v, cudaStream_t s, const u32* ct, u32 n_rows, u32 n_cts, \
+                                const u32* offsets_dev, const u32* rows_dev, u32 n_out, u32 nnz, u32* agg, bool* done); \
 cudaError_t partial_decrypt_scratch(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, \
                                     const u32* recipients_dev, u32 n_rec, const u32* parties_dev, \
                                     u32 n_parties, u32 ct_first, u32 n_cts, u64* shares, void* scratch, \
@@ -245,8 +247,8 @@ cudaError_t make_tab32(const DevView& v, cudaStream_t s, const u64* src, u64* ds
 cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \
                       u32 ct_first, u32 n_cts, const u32* plain, u32* ct, void* scratch, size_t scratch_bytes, \
                       u32* launches); \
-cudaError_t aggregate32(const DevView& v, cudaStream_t s, const u32* ct, u32 n_cts, const u32* offsets_dev, \
-                        const u32* rows_dev, u32 n_out, u32* agg); \
+cudaError_t aggregate32(const DevView& v, cudaStream_t s, const u32* ct, u32 n_rows, u32 n_cts, const u32* offsets_dev, \
+                        const u32* rows_dev, u32 n_out, u32 nnz, u32* agg); \
 cudaError_t partial_decrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, \
                               const u32* recipients_dev, u32 n_rec, const u32* parties_dev, u32 n_parties, \
                               u32 ct_first, u32 n_cts, u32* shares, void* scratch, size_t scratch_bytes, \

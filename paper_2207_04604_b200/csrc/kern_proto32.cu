@@ -293,8 +293,11 @@ cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, co
   return cudaSuccess;
 }
 
-cudaError_t aggregate32(const DevView& v, cudaStream_t s, const u32* ct, u32 n_cts, const u32* offsets_dev,
-                        const u32* rows_dev, u32 n_out, u32* agg) {
+cudaError_t aggregate32(const DevView& v, cudaStream_t s, const u32* ct, u32 n_rows, u32 n_cts, const u32* offsets_dev,
+                        const u32* rows_dev, u32 n_out, u32 nnz, u32* agg) {
+  bool done = false;
+  const cudaError_t e = aggregate_columns32(v, s, ct, n_rows, n_cts, offsets_dev, rows_dev, n_out, nnz, agg, &done);
+  if (e != cudaSuccess || done) return e;
   const size_t ct_quads = (size_t)v.L * v.n / 2;
   u32 by = (u32)((ct_quads + 255) / 256);
   if (by > 32768) by = 32768;

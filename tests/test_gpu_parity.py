@@ -1352,3 +1352,36 @@ def test_rounding_on_both_sides_of_every_kind_of_boundary(d2, log2_n, bits, L, t
     want = [((2 * t * v + q) // (2 * q)) % t for v in vs]
     assert d2.to_u32_numpy(out)[0, 0].tolist() == want
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,n_rows,n_out,n_cts", [(3, 36, 5, 7, 2), (8, 54, 9, 40, 120), (9, 60, 6, 5, 60), (10, 54, 70, 9, 30), (8, 30, 7, 7, 210),
+                                                           (12, 54, 3, 66, 7)])
+def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_rows, n_out, n_cts):
+    """Lists that name every row more often than there are rows (columns in shared memory), and too many rows for it;
+    empty lists, one entry, one list of 200 entries, residues at their largest."""
+    L = 3
+    moduli = small_moduli(log2_n, bits, L)
+    ctx = d2.Context(log2_n, moduli, 2, seed=81)
+    rng = np.random.default_rng(n_out)
+    lens = rng.integers(0, 2 * n_rows // n_out + 6, n_out)
+    lens[0], lens[1], lens[2] = 0, 1, 200
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint32)
+    rows = rng.integers(0, n_rows, offsets[-1]).astype(np.uint32)
+    rows[1:] = np.where(rng.random(offsets[-1] - 1) < 0.3, n_rows - 1, rows[1:])
+    ct = np.stack([wl.random_polys(moduli, log2_n, n_cts * 2, seed=r) for r in range(n_rows)]).reshape(n_rows, n_cts, 2, L, 1 << log2_n)
+    ct[n_rows - 1] = (np.array(moduli, dtype=np.uint64) - 1)[None, None, :, None]
+    want = np.zeros((n_out, n_cts, 2, L, 1 << log2_n), dtype=object)
+    for i in range(n_out):
+        for r in rows[offsets[i]:offsets[i + 1]]:
+            want[i] += ct[r].astype(object)
+    want = (want % np.array(moduli, dtype=object)[None, None, None, :, None]).astype(np.uint64)
+    agg = ctx.empty_u64(n_out, n_cts, 2, L, 1 << log2_n)
+    ctx.aggregate(d2.from_u64_numpy(ct, ctx.device), n_rows, n_cts, offsets, rows, agg)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(agg), want)
+    if bits <= 30:
+        agg32 = ctx.empty_u32(n_out, n_cts, 2, L, 1 << log2_n)
+        ctx.aggregate32(d2.from_u32_numpy(ct.astype(np.uint32), ctx.device), n_rows, n_cts, offsets, rows, agg32)
+        ctx.sync()
+        assert np.array_equal(d2.to_u32_numpy(agg32).astype(np.uint64), want)
+    ctx.close()

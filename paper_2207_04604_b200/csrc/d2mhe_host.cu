@@ -122,23 +122,37 @@ struct DeviceGuard {
   }
 };
 
+// Device memory of the context.  Blocks up to 1 MiB (the dozens of tables) share 8 MiB allocations: one cudaMalloc per
+// table was a good part of d2mhe_create.
+void* dev_bytes(d2mhe_ctx* c, size_t bytes, cudaError_t* err) {
+  const size_t chunk = (size_t)8 << 20;
+  bytes = (std::max<size_t>(bytes, 16) + 255) / 256 * 256;
+  const bool small = bytes <= ((size_t)1 << 20);
+  void* d = nullptr;
+  *err = cudaSuccess;
+  if (!small || bytes > c->arena_left) {
+    *err = cudaMalloc(&d, small ? chunk : bytes);
+    if (*err != cudaSuccess) return nullptr;
+    c->allocs.push_back(d);
+    if (!small) return d;
+    c->arena = reinterpret_cast<unsigned char*>(d);
+    c->arena_left = chunk;
+  }
+  d = c->arena;
+  c->arena += bytes;
+  c->arena_left -= bytes;
+  return d;
+}
 template <class T>
 T* dev_upload(d2mhe_ctx* c, const std::vector<T>& h, cudaError_t* err) {
-  void* d = nullptr;
-  size_t bytes = std::max<size_t>(h.size() * sizeof(T), 16);
-  *err = cudaMalloc(&d, bytes);
+  void* d = dev_bytes(c, h.size() * sizeof(T), err);
   if (*err != cudaSuccess) return nullptr;
-  c->allocs.push_back(d);
   if (!h.empty()) *err = cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
   return reinterpret_cast<T*>(d);
 }
 template <class T>
 T* dev_alloc(d2mhe_ctx* c, size_t count, cudaError_t* err) {
-  void* d = nullptr;
-  *err = cudaMalloc(&d, std::max<size_t>(count * sizeof(T), 16));
-  if (*err != cudaSuccess) return nullptr;
-  c->allocs.push_back(d);
-  return reinterpret_cast<T*>(d);
+  return reinterpret_cast<T*>(dev_bytes(c, count * sizeof(T), err));
 }
 
 d2mhe_status fail_cuda(d2mhe_ctx* c, cudaError_t e) {
@@ -524,7 +538,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
     const size_t per_sm = logn == 12 ? 4 : logn == 13 ? 2 : 1;  // resident blocks of the transform kernels
     const size_t units = (2 * (size_t)sms * per_sm + L - 1) / L;
-    const size_t want = units * P.num_parties * (c->view.fft_on ? 11 : 6) * n;
+    const size_t want = units * (P.num_parties * 6 + (c->view.fft_on ? 8 * L : 0)) * n;  // alpha of the refresh: 8 N L bytes a unit
     c->noise_scratch_bytes = std::min(kNoiseScratchMaxBytes, std::max(kNoiseScratchBytes, (want + 255) / 256 * 256));
   }
   c->noise_scratch = dev_alloc<unsigned char>(c, c->noise_scratch_bytes, &err);

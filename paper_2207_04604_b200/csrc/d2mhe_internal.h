@@ -123,6 +123,8 @@ struct d2mhe_ctx {
   DevView view;
   LimbParams limb_params;
   std::vector<void*> allocs;        // device allocations to free
+  unsigned char* arena = nullptr;   // rest of the last allocation that small blocks share
+  size_t arena_left = 0;
   std::vector<bool> has_share;
   std::vector<bool> has_user_key;
   std::vector<u32> pk_parties;      // party set of the last collective_pk

@@ -42,7 +42,12 @@ struct LimbTab {
   double fft_magic;
   u64 fft_k0;
   u32 fft_h, fft_fmask;
+  // the same on 32-bit words (kern_fft32.cu): floor(2^46 / q_l), a multiple of q_l and the constants of the rounding
+  u32 fft32_mu;
+  u64 fft32_k;
 };
+#define D2MHE_FFT32_F 6  // fraction bits of a rounded product
+#define D2MHE_FFT32_MAGIC (1.5 * 70368744177664.0 + 0.5) /* 1.5 * 2^46 + 1/2 */
 
 // ---------------------------------------------------------------------------
 // Checked build.  Compiled with D2MHE_CHECKED every kernel tests the indices it is about to use

@@ -25,8 +25,8 @@ struct FftGeo {
   __host__ __device__ static constexpr u32 tmem_cols(int k) { return (u32)(WORDS * k * (T / 128)); }
 };
 
-// the block's shared memory and this thread's place in it
-template <int LOGN>
+// the block's shared memory and this thread's place in it (STASH: with room for the low part's results)
+template <int LOGN, bool STASH = true>
 struct FftSmem {
   using G = FftGeo<LOGN>;
   double2* ex;     // of this thread's group
@@ -41,7 +41,7 @@ struct FftSmem {
     other = base + (1u - g) * (G::R * G::RS);
     words = reinterpret_cast<u32*>(smem_raw + G::ex_bytes);
     bytes = words + 2 * G::n;
-    slot = bytes + G::n / 2;
+    slot = STASH ? bytes + G::n / 2 : words;
   }
   __device__ __forceinline__ u32 group() const { return G::GR > 1 ? threadIdx.x / G::TG : 0u; }
   __device__ __forceinline__ void group_sync() const {
@@ -106,8 +106,8 @@ __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.syn
 // ---- exchanges through shared memory: 16-byte accesses, eight lanes to a wavefront ----------------------------------
 // Inside the 16 threads of a row: element k of lane a goes to element a of lane k, through a 16 x 17 layout (both
 // directions without bank conflicts, constant offsets).  Rows belong to one warp: no block barrier.
-template <int LOGN>
-__device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   using G = FftGeo<LOGN>;
   const u32 l16 = sm.tg & 15u;
   double2* e = sm.ex + (sm.tg >> 4) * G::RS;
@@ -125,16 +125,16 @@ __device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN>& sm, double* xr
   __syncwarp();
 }
 // the 16 results of a row pass -> row-major, and back; own rows only
-template <int LOGN>
-__device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN>& sm, const double* xr, const double* xi) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN, STASH>& sm, const double* xr, const double* xi) {
   double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
     constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
     e[16 * k] = make_double2(xr[i], xi[i]);
   });
 }
-template <int LOGN>
-__device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   const double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
     constexpr int k = brev_c<16>(decltype(k_)::value);
@@ -143,8 +143,8 @@ __device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN>& sm, double* xr
     xi[k] = t.y;
   });
 }
-template <int LOGN>
-__device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN>& sm, const double* xr, const double* xi) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN, STASH>& sm, const double* xr, const double* xi) {
   using G = FftGeo<LOGN>;
 #pragma unroll
   for (int c = 0; c < G::COLS; ++c)
@@ -153,8 +153,8 @@ __device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN>& sm, const doub
       sm.ex[sm.tg + k * G::RS + c * G::TG] = make_double2(xr[c * G::R + i], xi[c * G::R + i]);
     });
 }
-template <int LOGN>
-__device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN>& sm, double* xr, double* xi) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   using G = FftGeo<LOGN>;
 #pragma unroll
   for (int c = 0; c < G::COLS; ++c)
@@ -195,8 +195,8 @@ __device__ __forceinline__ cpx fft_twist(const cpx tw, u32 group) {
 
 // Forward transform.  in(c, jC, h): the coefficients j and j + n as a complex number, j = r + 256 jC + h n/2 with
 // r = tg + c TG (h = 0 for one group).  Leaves Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
-template <int LOGN, class In>
-__device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
+template <int LOGN, bool STASH, class In>
+__device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi, In in) {
   using G = FftGeo<LOGN>;
   constexpr int R = G::R;
   const u32 g = sm.group();
@@ -237,8 +237,8 @@ __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN>& sm, const Ff
 }
 
 // in(j): the same by coefficient number, j < n
-template <int LOGN, class In>
-__device__ __forceinline__ void fft_forward(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi, In in) {
+template <int LOGN, bool STASH, class In>
+__device__ __forceinline__ void fft_forward(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi, In in) {
   using G = FftGeo<LOGN>;
   fft_forward_at<LOGN>(sm, ft, xr, xi, [&](auto c_, auto j_, auto h_) {
     return in(sm.tg + (u32)(c_.value * G::TG + 256 * j_.value + h_.value * G::NG));
@@ -336,8 +336,8 @@ __device__ __forceinline__ void fft_product_sum(u32 addr, const double2* row_a, 
 // Inverse transform of what the products left, up to the twist: digit jC of column r = tg + c TG is left in
 // x[c R + brev(jC)]; tw: the columns' twist.  before_last(): called ahead of the arithmetic of pass C.
 // Table entries are fetched a pass ahead of their use (they come from L2 as often as not).
-template <int LOGN, class Hook>
-__device__ __forceinline__ void fft_inverse(const FftSmem<LOGN>& sm, const FftTab& ft, double* xr, double* xi,
+template <int LOGN, bool STASH, class Hook>
+__device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi,
                                             cpx (&tw)[FftGeo<LOGN>::COLS], Hook before_last) {
   using G = FftGeo<LOGN>;
   const cpx t2[2] = {ld_here(ft.inv2 + (sm.tg & 15u)), ld_here(ft.inv2 + 16 + (sm.tg & 15u))};
@@ -361,8 +361,8 @@ __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN>& sm, const FftTa
 }
 
 // Result number i of a thread (below 32) belongs to this coefficient.
-template <int LOGN>
-__device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN>& sm, int i) {
+template <int LOGN, bool STASH>
+__device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN, STASH>& sm, int i) {
   using G = FftGeo<LOGN>;
   if (G::GR == 2) return sm.tg + 256u * (8u * sm.group() + (u32)(i & 7)) + 4096u * (u32)(i >> 3);
   if (G::R == 8) return sm.tg + 128u * (u32)(i >> 4) + 256u * (u32)(i & 15);
@@ -371,8 +371,8 @@ __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN>& sm, int i) {
 // The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
 // eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4]) with v = bits of
 // M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.
-template <int LOGN, class Out>
-__device__ __forceinline__ void fft_results(const FftSmem<LOGN>& sm, const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr,
+template <int LOGN, bool STASH, class Out>
+__device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr,
                                             double* xi, double magic, Out out) {
   using G = FftGeo<LOGN>;
   constexpr int R = G::R;
@@ -483,6 +483,12 @@ inline u32 fft_party_split(const DevView& v, u32 base, u32 ctas, u32 n_parties, 
     if (cost < best) best = cost, split = c;
   }
   return split;
+}
+
+// How many thread blocks share the two components of a ciphertext: two when that is no more work for the slowest SM.
+inline u32 fft_component_split(const DevView& v, u32 base, u32 ctas) {
+  const u32 resident = v.sms * ctas;
+  return (2 * base + resident - 1) / resident < 2 * ((base + resident - 1) / resident) ? 2 : 1;
 }
 
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.

@@ -249,7 +249,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   for (u64 x = t; x; x >>= 1) ++t_bits;
   const u32 frac_bits = 59 - t_bits;  // 24 terms below 2^(F + t_bits) fit 64 bits
   c->view.round.frac_bits = frac_bits;
-  bool fft_ok = logn >= 12 && logn <= 14;
+  bool fft_ok = logn >= 12 && logn <= 14, fft32_ok = fft_ok && c->narrow;
   bool all_special = true;  // every prime is 2^b - d with b >= 32, d < 2^32 and 256 d < 2^b
   for (u32 l = 0; l < L; ++l) {
     const u64 p = c->moduli[l];
@@ -315,6 +315,14 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
       T.fft_magic = 1.5 * (double)((u64)1 << (52 - f)) + 0.5;
       const u64 h0 = ((u64)(1075 - f) << 20) + ((u64)1 << 19);  // high word of the magic number
       T.fft_k0 = 64 * p - ((u64)1 << 39) - D2MHE_GAUSS_B - gap * h0;
+    }
+
+    if (bits < 17 || bits > 30 || logn + bits > 43) {
+      fft32_ok = false;
+    } else {
+      T.fft32_mu = (u32)(((u64)1 << 46) / p);
+      const u64 b0 = ((u64)(1075 - D2MHE_FFT32_F) << 52) + ((u64)1 << 51);  // the magic number without its half
+      T.fft32_k = ((((u64)1 << 44) + p - 1) / p) * p - D2MHE_GAUSS_B - (b0 >> D2MHE_FFT32_F);
     }
 
     const u64 psi = c->roots[l], psi_inv = h_inv(psi, p);
@@ -475,7 +483,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   }
 
   // double-precision ring products
-  if (fft_ok && all_special) {
+  if ((fft_ok && all_special) || fft32_ok) {
     const u32 groups = logn == 14 ? 2 : 1, m = n / 2 / groups, R = m / 256;
     // e^(2 pi i num / den), in extended precision before the rounding to double
     auto root = [](double num, double den) {
@@ -504,11 +512,14 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
     c->view.pk_fft = dev_alloc<double2>(c, 4 * (size_t)L * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
+    c->view.fft32_on = fft32_ok ? 1 : 0;
+    c->view.fft_on = fft32_ok ? 0 : 1;
+  }
+  if (c->view.fft_on) {
     c->view.usk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
     c->view.upk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
-    c->view.fft_on = 1;
   }
 
   // key storage
@@ -762,7 +773,7 @@ d2mhe_status d2mhe_keygen_share(d2mhe_ctx* c, const u32* parties, u32 n_parties)
       c->launches += 1;
     }
   }
-  if (c->view.fft_on) {
+  if (c->view.fft_on || c->view.fft32_on) {
     e = L_(fft_secret)(c->view, c->stream, sg.dev[0], n_parties, TAG_SECRET, c->view.s_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
@@ -792,9 +803,10 @@ d2mhe_status d2mhe_collective_pk(d2mhe_ctx* c, const u32* parties, u32 n_parties
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
   }
-  if (c->view.fft_on) {
-    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, nullptr, 2 * c->view.L,
-                     c->view.pk_fft);
+  if (c->view.fft_on || c->view.fft32_on) {
+    e = c->view.fft_on ? L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, nullptr, 2 * c->view.L,
+                                      c->view.pk_fft)
+                       : L_(fft_rows32)(c->view, c->limb_params, c->stream, c->view.pk_coef, 2 * c->view.L, c->view.pk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
   }

@@ -68,10 +68,11 @@ struct DevView {
   u64* s32;       // [K][L][N]
   u64* pk32;      // [2][L][N]
   // ring products in double precision (set when the sizes are inside the bounds of d2mhe_fft.cuh)
-  u32 fft_on;
+  u32 fft_on;    // the 64-bit calls
+  u32 fft32_on;  // the 32-bit-word calls
   FftTab fft;
   double2* s_fft;   // [K][n]        transforms of s_k, times 1/n
-  double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n
+  double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n (fft32_on: [2][L][n], whole)
   double2* usk_fft;  // [K][n]            the same of the users' own keys
   double2* upk_fft;  // [K][2][L][2][n]
   u32* range_flag;
@@ -232,6 +233,11 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
 cudaError_t fft_samples(const DevView& v, cudaStream_t s, const void* src, u32 stride, u32 polys, double2* dst); \
 cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, const u32* users_dev, \
                      u32 rows, double2* dst); \
+cudaError_t share32_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, const u32* parties_dev, \
+                        u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u32* shares); \
+cudaError_t encrypt32_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, u32 unit_first, u32 n_units, \
+                          const double2* u_fft, const void* noise, const u32* plain, u32* ct); \
+cudaError_t fft_rows32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst); \
 cudaError_t convert_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, \
                         const u32* recipients_dev, u32 n_rec, const u32* parties_dev, u32 n_parties, u32 ct_first, \
                         u32 n_cts, u64* shares, void* scratch, size_t scratch_bytes, u32* launches); \

@@ -56,10 +56,8 @@ cudaError_t launch_encrypt(const DevView& v, const LimbParams& lp, cudaStream_t 
   using G = FftGeo<LOGN>;
   cudaError_t e = set_smem(k_encrypt_fft<LOGN>, G::smem_bytes);
   if (e != cudaSuccess) return e;
-  // one block per component when that takes no more than half of the waves' time again
-  const u32 resident = v.sms * G::CTAS, base = n_units * v.L;
-  const u32 split = (2 * base + resident - 1) / resident < 2 * ((base + resident - 1) / resident) ? 2 : 1;
-  k_encrypt_fft<LOGN><<<base * split, G::T, G::smem_bytes, s>>>(v, lp, unit_first, u_fft,
+  const u32 split = fft_component_split(v, n_units * v.L, G::CTAS);
+  k_encrypt_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes, s>>>(v, lp, unit_first, u_fft,
                                                                 reinterpret_cast<const uint4*>(noise), plain, ct, split);
   return cudaGetLastError();
 }

@@ -276,7 +276,9 @@ cudaError_t make_tab32(const DevView& v, cudaStream_t s, const u64* src, u64* ds
 cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties,
                       u32 ct_first, u32 n_cts, const u32* plain, u32* ct, void* scratch, size_t scratch_bytes,
                       u32* launches) {
-  const size_t per_unit = 3 * (size_t)v.n;
+  // double-precision products: 8 N bytes of scratch more per unit, for the transform of u
+  const bool fft = v.fft32_on && scratch_bytes >= 11 * (size_t)v.n;
+  const size_t per_unit = (fft ? 11 : 3) * (size_t)v.n;
   const u32 n_units = n_parties * n_cts;
   u32 per_batch = (u32)std::min<size_t>(scratch_bytes / per_unit, n_units);
   if (per_batch > 1) per_batch &= ~1u;  // whole pairs per batch
@@ -284,11 +286,18 @@ cudaError_t encrypt32(const DevView& v, const LimbParams& lp, cudaStream_t s, co
   if (per_batch == 0) return cudaErrorInvalidValue;
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
-    cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, false, scratch);
+    unsigned char* small = reinterpret_cast<unsigned char*>(scratch) + (fft ? (size_t)nu * 8 * v.n : 0);
+    cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, fft, small);
     if (e != cudaSuccess) return e;
-    e = encrypt32_units(v, lp, s, first, nu, reinterpret_cast<const u32*>(scratch), plain, ct);
+    if (fft) {
+      double2* u_fft = reinterpret_cast<double2*>(scratch);
+      e = fft_samples(v, s, small, 3, nu, u_fft);
+      if (e == cudaSuccess) e = encrypt32_fft(v, lp, s, first, nu, u_fft, small, plain, ct);
+    } else {
+      e = encrypt32_units(v, lp, s, first, nu, reinterpret_cast<const u32*>(small), plain, ct);
+    }
     if (e != cudaSuccess) return e;
-    if (launches) *launches += 2;
+    if (launches) *launches += fft ? 3 : 2;
   }
   return cudaSuccess;
 }
@@ -322,10 +331,11 @@ cudaError_t partial_decrypt32(const DevView& v, const LimbParams& lp, cudaStream
   for (u32 first = 0; first < n_units; first += per_batch) {
     const u32 nu = std::min(per_batch, n_units - first);
     cudaError_t e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu,
-                                   kSampleShare, false, scratch);
+                                   kSampleShare, v.fft32_on != 0, scratch);
     if (e != cudaSuccess) return e;
-    e = pdec32_units(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu,
-                     reinterpret_cast<const signed char*>(scratch), shares);
+    e = v.fft32_on ? share32_fft(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu, scratch, shares)
+                   : pdec32_units(v, lp, s, agg, parties_dev, n_parties, n_cts, first, nu,
+                                  reinterpret_cast<const signed char*>(scratch), shares);
     if (e != cudaSuccess) return e;
     if (launches) *launches += 2;
   }

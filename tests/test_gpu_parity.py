@@ -1385,3 +1385,33 @@ def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_r
         ctx.sync()
         assert np.array_equal(d2.to_u32_numpy(agg32).astype(np.uint64), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,K,C", [(12, 30, 3, 3, 2), (12, 20, 5, 17, 1), (13, 30, 2, 4, 3), (13, 17, 2, 2, 1), (14, 29, 2, 2, 1),
+                                               (14, 30, 2, 2, 1)])
+def test_32_bit_products_at_the_limits(d2, log2_n, bits, L, K, C):
+    """Shares of extreme and uniform residues and ciphertexts of extreme plaintexts on 32-bit words; 30 bits at N = 16384 is just
+    outside the range of the double-precision products."""
+    moduli = wl.ntt_primes(bits, 2 << log2_n, L)
+    n, parties, t = 1 << log2_n, list(range(K)), 97
+    ctx = d2.Context(log2_n, moduli, K, seed=82, plain_modulus=t)
+    o = make_oracle(log2_n, moduli, seed=82, t=t)
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    pk = o.collective_pk(parties)
+    rng = np.random.default_rng(bits)
+    agg = np.zeros((1, 3, 2, L, n), dtype=np.uint64)
+    for l, p in enumerate(moduli):
+        agg[0, 0, 1, l] = rng.choice(np.array([0, 1, p - 1, (p - 1) // 2, (p + 1) // 2], dtype=np.uint64), n)
+        agg[0, 1, 1, l] = (p - 1) // 2
+        agg[0, 2, 1, l] = rng.integers(0, p, n, dtype=np.uint64)
+    shares = ctx.empty_u32(1, K, 3, L, n)
+    ctx.partial_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), [K - 1], parties, 5, 3, shares)
+    plain = rng.integers(0, t, (K, C, n)).astype(np.uint32)
+    plain[0, 0, ::2] = t - 1
+    ct = ctx.empty_u32(K, C, 2, L, n)
+    ctx.encrypt32(parties, 9, C, d2.from_u32_numpy(plain, ctx.device), ct)
+    ctx.sync()
+    assert np.array_equal(d2.to_u32_numpy(shares).astype(np.uint64), o.partial_decrypt(agg, [K - 1], parties, 5))
+    assert np.array_equal(d2.to_u32_numpy(ct).astype(np.uint64), o.encrypt(pk, parties, 9, plain))
+    ctx.close()

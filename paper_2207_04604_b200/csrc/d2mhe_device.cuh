@@ -359,7 +359,9 @@ __device__ __forceinline__ u64 reduce_small(u64 x, const Mod& m) {
 // residues of the same prime below 2^30 (two polynomials transformed side by side with the
 // same twiddles), each half with Harvey's lazy butterflies in 32-bit arithmetic: one high and
 // two low multiplies per butterfly instead of five and four.
-enum : int { MODE_STRICT = 0, MODE_WIDE = 1, MODE_PAIR = 2 };
+// 3 = primes below 2^60 that are not WIDE: sixteen p fit a word, so a round of three stages needs four (forward) or six
+// (inverse) small-quotient reductions of an octet instead of twelve conditional subtractions.
+enum : int { MODE_STRICT = 0, MODE_WIDE = 1, MODE_PAIR = 2, MODE_LAZY60 = 3 };
 
 __device__ __forceinline__ u32 csub32(u32 x, u32 p) { return min(x, x - p); }  // x - p wraps above x when x < p
 // y*w mod p in [0, 2p) for any 32-bit y, given ws = floor(w 2^32 / p), p < 2^31
@@ -393,7 +395,7 @@ __device__ __forceinline__ void ct_bfly(u64& X, u64& Y, const ulonglong2 w, cons
     return;
   }
   constexpr bool WIDE = MODE == MODE_WIDE;
-  const u64 x = WIDE ? X : csub(X, m.fourp);
+  const u64 x = WIDE || MODE == MODE_LAZY60 ? X : csub(X, m.fourp);
   const u64 t = WIDE ? shoup_approx_sf(Y, w.x, w.y, m.sf_d, m.sf_shift) : shoup_approx(Y, w.x, w.y, m.np);  // [0,4p)
   X = x + t;
   Y = x - t + m.fourp;
@@ -407,15 +409,23 @@ __device__ __forceinline__ void gs_bfly(u64& X, u64& Y, const ulonglong2 w, cons
   }
   constexpr bool WIDE = MODE == MODE_WIDE;
   const u64 s = X + Y;
-  const u64 d = X - Y + (WIDE ? c : m.fourp);
-  X = WIDE ? s : csub(s, m.fourp);
+  const u64 d = X - Y + (WIDE ? c : MODE == MODE_LAZY60 ? m.fourp << 1 : m.fourp);
+  X = WIDE || MODE == MODE_LAZY60 ? s : csub(s, m.fourp);
   Y = WIDE ? shoup_approx_sf(d, w.x, w.y, m.sf_d, m.sf_shift) : shoup_approx(d, w.x, w.y, m.np);
 }
 
 // three (or fewer) forward stages on an octet; m = groups at the first stage, i = group index
+// LAZY60: the first stage's X operands are brought below 3p here; outputs are below 3p + 4p per stage.
+template <int WIDE>
+__device__ __forceinline__ void fwd_reduce(u64 (&x)[8], const Mod& md) {
+  if (WIDE == MODE_LAZY60)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = reduce_small(x[k], md);
+}
 template <int WIDE>
 __device__ __forceinline__ void fwd_octet(u64 (&x)[8], const ulonglong2* __restrict__ W, u32 m,
                                           u32 i, int nst, const Mod& md) {
+  fwd_reduce<WIDE>(x, md);
   {
     const ulonglong2 w = tw_ld(W, m + i, md.tw_limit, md);
 #pragma unroll
@@ -440,6 +450,7 @@ __device__ __forceinline__ void fwd_octet(u64 (&x)[8], const ulonglong2* __restr
 template <int MODE>
 __device__ __forceinline__ void fwd_octet_last(u64 (&x)[8], const ulonglong2* __restrict__ WL, u32 oc,
                                                u32 i, const Mod& md) {
+  fwd_reduce<MODE>(x, md);
   {
     const ulonglong2 w = tw_ld(WL, i, md.twl_limit, md);
 #pragma unroll
@@ -458,6 +469,18 @@ __device__ __forceinline__ void fwd_octet_last(u64 (&x)[8], const ulonglong2* __
     ct_bfly<MODE>(x[2 * r], x[2 * r + 1], w, md);
   }
 }
+// LAZY60: with inputs below 4p the first two inverse stages leave x0, x4 below 16p, x1, x5 below 8p and the rest below 4p;
+// x0 and x4 are brought below 3p before the third, and x0 .. x3 (then below 16p) after it.
+template <int MODE>
+__device__ __forceinline__ void inv_reduce_mid(u64 (&x)[8], const Mod& md) {
+  if (MODE == MODE_LAZY60) x[0] = reduce_small(x[0], md), x[4] = reduce_small(x[4], md);
+}
+template <int MODE>
+__device__ __forceinline__ void inv_reduce_end(u64 (&x)[8], const Mod& md) {
+  if (MODE == MODE_LAZY60)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = reduce_small(x[k], md);
+}
 template <int MODE>
 __device__ __forceinline__ void inv_octet_first(u64 (&x)[8], const ulonglong2* __restrict__ IWL, u32 oc,
                                                 u32 i, const Mod& md, bool reduce0 = true) {
@@ -474,12 +497,14 @@ __device__ __forceinline__ void inv_octet_first(u64 (&x)[8], const ulonglong2* _
     gs_bfly<MODE>(x[4], x[6], w1, md, c32);
     gs_bfly<MODE>(x[5], x[7], w1, md, c32);
   }
+  inv_reduce_mid<MODE>(x, md);
   {
     const ulonglong2 w = tw_ld(IWL, i, md.twl_limit, md);
 #pragma unroll
     for (int k = 0; k < 4; ++k) gs_bfly<MODE>(x[k], x[k + 4], w, md, c64);
   }
   if (MODE == MODE_WIDE && reduce0) x[0] = reduce_small(x[0], md);
+  inv_reduce_end<MODE>(x, md);
 }
 
 // Inverse stages on an octet whose inputs are all below 16p (WIDE) / 4p (otherwise).
@@ -503,12 +528,14 @@ __device__ __forceinline__ void inv_octet(u64 (&x)[8], const ulonglong2* __restr
     gs_bfly<MODE>(x[4], x[6], w1, md, c32);
     gs_bfly<MODE>(x[5], x[7], w1, md, c32);
   }
+  if (nst >= 3) inv_reduce_mid<MODE>(x, md);
   {
     const ulonglong2 w = tw_ld(IW, m + i, md.tw_limit, md);
 #pragma unroll
     for (int k = 0; k < 4; ++k) gs_bfly<MODE>(x[k], x[k + 4], w, md, c64);
   }
   if (MODE == MODE_WIDE && reduce0) x[0] = reduce_small(x[0], md);
+  inv_reduce_end<MODE>(x, md);
 }
 
 // Brings the outputs of the last inverse round below 4p.  After a full round the bounds are

@@ -547,7 +547,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     int sms = 0;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (err != cudaSuccess) return fail_cuda(c, err);
-    const size_t per_sm = logn == 12 ? 4 : logn == 13 ? 2 : 1;  // resident blocks of the transform kernels
+    const size_t per_sm = logn == 11 || logn == 12 ? 4 : logn == 13 ? 2 : 1;  // resident blocks of the transform kernels
     const size_t units = (2 * (size_t)sms * per_sm + L - 1) / L;
     const size_t want = units * (P.num_parties * 6 + (c->view.fft_on ? 8 * L : 0)) * n;  // alpha of the refresh: 8 N L bytes a unit
     c->noise_scratch_bytes = std::min(kNoiseScratchMaxBytes, std::max(kNoiseScratchBytes, (want + 255) / 256 * 256));
@@ -571,6 +571,9 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   c->view.L = L;
   c->view.K = P.num_parties;
   c->view.wide = all_special ? 1 : 0;
+  c->view.below60 = 1;
+  for (u32 l = 0; l < L; ++l)
+    if (c->moduli[l] >= ((u64)1 << 60)) c->view.below60 = 0;
   for (u32 l = 0; l < L; ++l)
     if (c->moduli[l] >= ((u64)1 << 56)) c->view.wide = 0;  // 130 p (a lazily grown value plus its additive terms) must fit 64 bits
 

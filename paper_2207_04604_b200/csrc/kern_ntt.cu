@@ -3,7 +3,7 @@
 
 namespace {
 
-template <int LOGN, int G, bool WIDE>
+template <int LOGN, int G, int WIDE>
 __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
     k_ntt_fwd(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys) {
   const u32 l = blockIdx.x % v.L;
@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
       });
 }
 
-template <int LOGN, int G, bool WIDE>
+template <int LOGN, int G, int WIDE>
 __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
     k_ntt_inv(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys) {
   const u32 l = blockIdx.x % v.L;
@@ -44,9 +44,9 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 // coefficients o + k * 4096 (coalesced across threads; every thread uses the same 2^SA - 1
 // twiddles).  After it the array is 2^SA independent blocks of 4096, each finished by the
 // shared-memory engine with the twiddles of its sub-tree (pass B).  The inverse runs B then A.
-// Between the passes values are lazily reduced (below 8p); pass A always uses the
-// one-conditional-subtraction butterflies, which are valid for every prime below 2^61.
-template <int SA, bool INV>
+// Between the passes values are lazily reduced: below 8p with one conditional subtraction per butterfly (MODE_STRICT);
+// WIDE primes take 16 stages without any; below 2^60 (LAZY60) three stages fit and the fourth's operands are reduced.
+template <int SA, bool INV, int MODE>
 __global__ void __launch_bounds__(256)
     k_ntt_strided(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys) {
   constexpr int R = 1 << SA;
@@ -67,7 +67,11 @@ __global__ void __launch_bounds__(256)
       for (int i = 0; i < m; ++i) {
         const ulonglong2 w = __ldg(lt.W + m + i);
 #pragma unroll
-        for (int j = 0; j < half; ++j) ct_bfly<false>(x[i * 2 * half + j], x[i * 2 * half + j + half], w, md);
+        for (int j = 0; j < half; ++j) {
+          u64& X = x[i * 2 * half + j];
+          if (MODE == MODE_LAZY60 && s == 3) X = reduce_small(X, md);  // p, 5p, 9p, 13p before the stages
+          ct_bfly<MODE>(X, x[i * 2 * half + j + half], w, md);
+        }
       }
     }
 #pragma unroll
@@ -80,8 +84,12 @@ __global__ void __launch_bounds__(256)
       for (int i = 0; i < m; ++i) {
         const ulonglong2 w = __ldg(lt.IW + m + i);
 #pragma unroll
-        for (int j = 0; j < half; ++j)
-          gs_bfly<false>(x[i * 2 * half + j], x[i * 2 * half + j + half], w, md, 0);
+        for (int j = 0; j < half; ++j) {
+          u64 &X = x[i * 2 * half + j], &Y = x[i * 2 * half + j + half];
+          // sums double from 4p: WIDE adds what they have reached; LAZY60 (8p) brings both below 3p from the second on
+          if (MODE == MODE_LAZY60 && s < SA - 1) X = reduce_small(X, md), Y = reduce_small(Y, md);
+          gs_bfly<MODE>(X, Y, w, md, md.fourp << (SA - 1 - s));
+        }
       }
     }
 #pragma unroll
@@ -90,7 +98,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // Pass B: block b of polynomial-limb r; grid = batch * L * 2^soff.
-template <int LOGN, int G, bool WIDE>
+template <int LOGN, int G, int WIDE>
 __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
     k_ntt_fwd_blk(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys, u32 soff) {
   const u32 b = blockIdx.x & ((1u << soff) - 1), r = blockIdx.x >> soff;
@@ -105,7 +113,7 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
       },
       soff, b);
 }
-template <int LOGN, int G, bool WIDE>
+template <int LOGN, int G, int WIDE>
 __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
     k_ntt_inv_blk(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys, u32 soff) {
   const u32 b = blockIdx.x & ((1u << soff) - 1), r = blockIdx.x >> soff;
@@ -130,39 +138,76 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 
 namespace D2MHE_LAUNCH_NS {
 
+static int ntt_mode(const DevView& v) { return v.wide ? MODE_WIDE : v.below60 ? MODE_LAZY60 : MODE_STRICT; }
+
 static cudaError_t ntt_two_pass(const DevView& v, const LimbParams& lp, cudaStream_t s, u64* polys,
                                 u32 batch, bool inverse) {
   const u32 soff = v.logn - 12, rows = batch * v.L;
   const size_t smem = poly_bytes(4096);
   const u32 grid_a = rows * 16;
   const u32 grid_b = rows << soff, threads = ntt_threads(4096, D2MHE_G12);
-  cudaError_t e;
-#define D2MHE_STRIDED(SA_, INV_) k_ntt_strided<SA_, INV_><<<grid_a, 256, 0, s>>>(v, lp, polys)
-  if (!inverse) {
-    if (soff == 3) D2MHE_STRIDED(3, false); else D2MHE_STRIDED(4, false);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (v.wide)
-      e = launch_clustered(k_ntt_fwd_blk<12, D2MHE_G12, true>, grid_b, threads, smem, s, 1, v, lp, polys, soff);
-    else
-      e = launch_clustered(k_ntt_fwd_blk<12, D2MHE_G12, false>, grid_b, threads, smem, s, 1, v, lp, polys, soff);
-    return e;
-  }
-  if (v.wide)
-    e = launch_clustered(k_ntt_inv_blk<12, D2MHE_G12, true>, grid_b, threads, smem, s, 1, v, lp, polys, soff);
+  const int mode = ntt_mode(v);
+  cudaError_t e = cudaSuccess;
+#define D2MHE_STRIDED(INV_, MODE_)                                              \
+  do {                                                                          \
+    if (soff == 3)                                                              \
+      k_ntt_strided<3, INV_, MODE_><<<grid_a, 256, 0, s>>>(v, lp, polys);       \
+    else                                                                        \
+      k_ntt_strided<4, INV_, MODE_><<<grid_a, 256, 0, s>>>(v, lp, polys);       \
+    e = cudaGetLastError();                                                     \
+  } while (0)
+#define D2MHE_BLOCKS(KERNEL, MODE_) \
+  e = launch_clustered(KERNEL<12, D2MHE_G12, MODE_>, grid_b, threads, smem, s, 1, v, lp, polys, soff)
+#define D2MHE_TWO_PASS(MODE_)                 \
+  do {                                        \
+    if (!inverse) {                           \
+      D2MHE_STRIDED(false, MODE_);            \
+      if (e != cudaSuccess) return e;         \
+      D2MHE_BLOCKS(k_ntt_fwd_blk, MODE_);     \
+    } else {                                  \
+      D2MHE_BLOCKS(k_ntt_inv_blk, MODE_);     \
+      if (e != cudaSuccess) return e;         \
+      D2MHE_STRIDED(true, MODE_);             \
+    }                                         \
+  } while (0)
+  if (mode == MODE_WIDE)
+    D2MHE_TWO_PASS(MODE_WIDE);
+  else if (mode == MODE_LAZY60)
+    D2MHE_TWO_PASS(MODE_LAZY60);
   else
-    e = launch_clustered(k_ntt_inv_blk<12, D2MHE_G12, false>, grid_b, threads, smem, s, 1, v, lp, polys, soff);
-  if (e != cudaSuccess) return e;
-  if (soff == 3) D2MHE_STRIDED(3, true); else D2MHE_STRIDED(4, true);
+    D2MHE_TWO_PASS(MODE_STRICT);
 #undef D2MHE_STRIDED
-  return cudaGetLastError();
+#undef D2MHE_BLOCKS
+#undef D2MHE_TWO_PASS
+  return e;
 }
+
+// one-pass sizes: the instantiation for the ring degree and the arithmetic mode
+#define D2MHE_NTT_MODE(KERNEL, LOGN_, G_)                                                                      \
+  do {                                                                                                         \
+    const u32 grid = batch * v.L, threads = ntt_threads(v.n, G_);                                              \
+    const size_t smem = poly_bytes(v.n);                                                                       \
+    if (mode == MODE_WIDE) return launch_clustered(KERNEL<LOGN_, G_, MODE_WIDE>, grid, threads, smem, s, 1, v, lp, polys);   \
+    if (mode == MODE_LAZY60)                                                                                   \
+      return launch_clustered(KERNEL<LOGN_, G_, MODE_LAZY60>, grid, threads, smem, s, 1, v, lp, polys);        \
+    return launch_clustered(KERNEL<LOGN_, G_, MODE_STRICT>, grid, threads, smem, s, 1, v, lp, polys);          \
+  } while (0)
+#define D2MHE_NTT_SIZE(KERNEL)                                 \
+  switch (v.logn) {                                            \
+    case 11: D2MHE_NTT_MODE(KERNEL, 11, 1);                    \
+    case 12: D2MHE_NTT_MODE(KERNEL, 12, D2MHE_G12);            \
+    case 13: D2MHE_NTT_MODE(KERNEL, 13, D2MHE_G13);            \
+    case 14: D2MHE_NTT_MODE(KERNEL, 14, D2MHE_G14);            \
+    default: D2MHE_NTT_MODE(KERNEL, 0, 1);                     \
+  }
 
 cudaError_t ntt(const DevView& v, const LimbParams& lp, cudaStream_t s, u64* polys, u32 batch, bool inverse) {
   if (v.logn > 14) return ntt_two_pass(v, lp, s, polys, batch, inverse);
+  const int mode = ntt_mode(v);
   if (inverse) {
-    D2MHE_DISPATCH(k_ntt_inv, v, batch * v.L, s, v, lp, polys);
+    D2MHE_NTT_SIZE(k_ntt_inv)
   } else {
-    D2MHE_DISPATCH(k_ntt_fwd, v, batch * v.L, s, v, lp, polys);
+    D2MHE_NTT_SIZE(k_ntt_fwd)
   }
 }
 

@@ -39,6 +39,8 @@ def _brv(n_bits):
     (9, 60, 2, 2), (10, 36, 3, 2), (11, 54, 2, 2), (12, 36, 3, 5), (12, 60, 4, 3),
     (13, 54, 4, 3), (13, 60, 1, 7), (14, 54, 8, 2), (14, 60, 3, 3),
     (15, 60, 2, 2), (15, 50, 3, 1), (16, 60, 3, 2), (16, 54, 1, 3),
+    (11, 60, 2, 3), (11, 61, 1, 2), (12, 61, 2, 2), (13, 57, 2, 3), (14, 61, 1, 2), (15, 61, 1, 2), (15, 54, 2, 1), (16, 61, 2, 1),
+    (16, 58, 1, 1),
 ])
 def test_ntt_forward_inverse_against_oracle(d2, log2_n, bits, L, batch):
     moduli = wl.ntt_primes(bits, 1 << 17, L) if bits >= 50 else small_moduli(log2_n, bits, L)

@@ -33,7 +33,7 @@ namespace {
 constexpr int ntt_default_g(int logn) { return logn == 12 ? D2MHE_G12 : logn == 13 ? D2MHE_G13 : logn == 14 ? D2MHE_G14 : 1; }
 constexpr int ntt_minb_ct(int logn, int g) {
   return g != ntt_default_g(logn) ? 2
-                                  : logn == 12 ? D2MHE_MINB12 : logn == 13 ? D2MHE_MINB13 : logn == 14 ? D2MHE_MINB14 : 1;
+                                  : logn == 11 ? 4 : logn == 12 ? D2MHE_MINB12 : logn == 13 ? D2MHE_MINB13 : logn == 14 ? D2MHE_MINB14 : 1;
 }
 
 // Shared-memory layout of the transform kernels: [GaussTab][polynomial].
@@ -240,6 +240,9 @@ cudaError_t launch_clustered(void (*kernel)(KArgs...), u32 grid, u32 threads, si
     const size_t smem_ = poly_bytes(n_, extra);                                                \
     const bool wide_ = (view).wide != 0;                                                       \
     switch (logn_) {                                                                           \
+      case 11:                                                                                 \
+        D2MHE_LAUNCH_W(KERNEL, 11, 1, wide_, grid, stream, cs, __VA_ARGS__);                   \
+        break;                                                                                 \
       case 12:                                                                                 \
         D2MHE_LAUNCH_W(KERNEL, 12, D2MHE_DISPATCH_G12, wide_, grid, stream, cs, __VA_ARGS__);  \
         break;                                                                                 \

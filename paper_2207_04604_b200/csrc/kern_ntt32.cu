@@ -115,6 +115,7 @@ namespace D2MHE_LAUNCH_NS {
 
 cudaError_t ntt32(const DevView& v, const LimbParams& lp, cudaStream_t s, u32* polys, u32 batch, bool inverse) {
   switch (v.logn) {
+    case 11: return launch_ntt32<11, 1>(v, lp, s, polys, batch, inverse);
     case 12: return launch_ntt32<12, D2MHE_G12>(v, lp, s, polys, batch, inverse);
     case 13: return launch_ntt32<13, D2MHE_G13>(v, lp, s, polys, batch, inverse);
     case 14: return launch_ntt32<14, D2MHE_G14>(v, lp, s, polys, batch, inverse);

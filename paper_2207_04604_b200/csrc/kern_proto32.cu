@@ -242,6 +242,7 @@ cudaError_t launch_pdec32(const DevView& v, const LimbParams& lp, cudaStream_t s
 
 #define D2MHE_DISPATCH32(FN, ...)                                        \
   switch (v.logn) {                                                      \
+    case 11: return FN<11, 1>(__VA_ARGS__);                              \
     case 12: return FN<12, D2MHE_G12>(__VA_ARGS__);                      \
     case 13: return FN<13, D2MHE_G13>(__VA_ARGS__);                      \
     case 14: return FN<14, D2MHE_G14>(__VA_ARGS__);                      \

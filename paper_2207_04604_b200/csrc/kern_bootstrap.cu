@@ -84,7 +84,8 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 }
 
 // ct' = (Lambda x + sum_k eta_{1,k}, alpha) with x the rounded plaintext of c_0 + eta_0.
-// grid = (n_rec * n_cts, chunks); one residue per thread and iteration.
+// grid = (n_rec * n_cts, chunks); a pair of residues per thread and iteration.  Bound by HBM (8 N L bytes of every
+// share): the loads of five shares are in flight before the first is added.
 __global__ void __launch_bounds__(256)
     k_boot_finish(DevView v, const u32* __restrict__ x, const u64* __restrict__ shares,
                   const u32* __restrict__ recipients, u32 n_shares, u32 ct_first, u32 n_cts,
@@ -92,17 +93,32 @@ __global__ void __launch_bounds__(256)
   const u32 unit = blockIdx.x, irec = unit / n_cts, cl = unit % n_cts;
   const u32 recipient = recipients[irec];
   if (!D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) return;
-  const size_t poly = (size_t)v.L * v.n;
-  for (size_t e = (size_t)blockIdx.y * blockDim.x + threadIdx.x; e < poly; e += (size_t)gridDim.y * blockDim.x) {
-    const u32 l = (u32)(e >> v.logn), j = (u32)(e & (v.n - 1));
+  const size_t pairs = (size_t)v.L * v.n / 2, stride = (size_t)n_cts * 2 * pairs;  // stride: from share to share
+  const ulonglong2* eta = reinterpret_cast<const ulonglong2*>(shares) + (((size_t)irec * n_shares * n_cts + cl) * 2 + 1) * pairs;
+  const uint2* xs = reinterpret_cast<const uint2*>(x) + (size_t)unit * (v.n / 2);
+  ulonglong2* o = reinterpret_cast<ulonglong2*>(out) + (size_t)unit * 2 * pairs;
+  for (size_t e = (size_t)blockIdx.y * blockDim.x + threadIdx.x; e < pairs; e += (size_t)gridDim.y * blockDim.x) {
+    const u32 l = (u32)((2 * e) >> v.logn), j = (u32)((2 * e) & (v.n - 1));
     const LimbTab* lt = v.limbs + l;
     const u64 p = lt->p;
-    u64 acc = csub(shoup_u32(x[(size_t)unit * v.n + j], lt->delta, lt->delta_sh, lt->np), p);
-    for (u32 k = 0; k < n_shares; ++k)
-      acc = addmod(acc, __ldg(shares + ((((size_t)irec * n_shares + k) * n_cts + cl) * 2 + 1) * poly + e), p);
-    out[(size_t)unit * 2 * poly + e] = acc;
+    const uint2 xv = __ldg(xs + (j >> 1));
+    ulonglong2 acc = make_ulonglong2(csub(shoup_u32(xv.x, lt->delta, lt->delta_sh, lt->np), p),
+                                     csub(shoup_u32(xv.y, lt->delta, lt->delta_sh, lt->np), p));
+    const ulonglong2* src = eta + e;
+    for (u32 k = 0; k < n_shares; k += 5) {
+      ulonglong2 h[5];
+#pragma unroll
+      for (u32 i = 0; i < 5; ++i)
+        h[i] = k + i < n_shares ? __ldcs(src + (k + i) * stride) : make_ulonglong2(0, 0);
+#pragma unroll
+      for (u32 i = 0; i < 5; ++i) {
+        acc.x = addmod(acc.x, h[i].x, p);
+        acc.y = addmod(acc.y, h[i].y, p);
+      }
+    }
+    o[e] = acc;
     const Stream sa(v.seed, TAG_BOOT_ALPHA, ct_first + cl, l, recipient);
-    out[(size_t)unit * 2 * poly + poly + e] = uniform_mod(sa, j, p, lt->mask);
+    o[pairs + e] = make_ulonglong2(uniform_mod(sa, j, p, lt->mask), uniform_mod(sa, j + 1, p, lt->mask));
   }
 }
 
@@ -153,8 +169,8 @@ cudaError_t boot_share(const DevView& v, const LimbParams& lp, cudaStream_t s, c
 
 cudaError_t boot_finish(const DevView& v, cudaStream_t s, const u32* x, const u64* shares,
                         const u32* recipients_dev, u32 n_rec, u32 n_shares, u32 ct_first, u32 n_cts, u64* out) {
-  const size_t poly = (size_t)v.L * v.n;
-  u32 by = (u32)((poly + 255) / 256);
+  const size_t pairs = (size_t)v.L * v.n / 2;
+  u32 by = (u32)((pairs + 255) / 256);
   if (by > 32768) by = 32768;
   dim3 grid(n_rec * n_cts, by);
   k_boot_finish<<<grid, 256, 0, s>>>(v, x, shares, recipients_dev, n_shares, ct_first, n_cts, out);

@@ -78,13 +78,17 @@ __global__ void __launch_bounds__(256)
 }
 
 // M_k uniform mod t by rejection on bitlen(t)-bit draws, N words per share.  Half of the draws are rejected for
-// t = 65537, and a warp that waits for the last lane of every coefficient needs six draws each; here a thread goes on to
-// its next coefficient as soon as one is accepted, and only the end of its 16 is waited for (three draws each).
-// grid = shares * segs, 16 coefficients per thread, or N / blockDim.x in one block where that is less.
-__global__ void __launch_bounds__(256)
+// t = 65537, so what counts is that no lane waits for another's redraw: a warp draws once for each of its coefficients,
+// packs the numbers of the rejected ones into a list in shared memory and goes over the list again, 32 at a time, until
+// it is empty.  512 coefficients take 31 full draws and about five partly filled ones, where lanes that walk over 16
+// coefficients of their own wait for the slowest of the 32 (46 draws).  The attempt is uniform over the warp.
+// grid = shares * segs; each warp of a block has per <= MASKS_PER_WARP coefficients.
+constexpr u32 MASKS_PER_WARP = 512;
+__global__ void __launch_bounds__(128)
     k_sample_masks(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties, u32 n_parties,
-                   u32 ct_first, u32 n_cts, u32 unit_first, u32 segs, u32* __restrict__ out) {
-  const u32 share = blockIdx.x / segs, seg = blockIdx.x % segs;
+                   u32 ct_first, u32 n_cts, u32 unit_first, u32 segs, u32 per, u32* __restrict__ out) {
+  __shared__ unsigned short lists[4][MASKS_PER_WARP];
+  const u32 share = blockIdx.x / segs, seg = blockIdx.x % segs, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const u32 unit = unit_first + share / n_parties, party = parties[share % n_parties], recipient = recipients[unit / n_cts];
   if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) return;
   const Stream st(v.seed, TAG_BOOT_MASK, ct_first + unit % n_cts, party, recipient);
@@ -92,19 +96,32 @@ __global__ void __launch_bounds__(256)
   u64 tmask = 1;
   while (tmask <= t) tmask <<= 1;
   tmask -= 1;
-  const u32 per = v.n / segs, end = (seg + 1) * per;
-  u32* dst = out + (size_t)share * v.n;
-  u32 j = seg * per + threadIdx.x, attempt = 0;
-  while (j < end) {
-    u64 r = st.draw64(j, attempt);
-    r = attempt < 255 ? r & tmask : r % t;  // the rule of uniform_mod
-    if (r < t) {
-      dst[j] = (u32)r;
-      j += blockDim.x;
-      attempt = 0;
-    } else {
-      ++attempt;
+  const u32 first = (seg * (blockDim.x >> 5) + warp) * per;
+  u32* dst = out + (size_t)share * v.n + first;
+  unsigned short* list = lists[warp];
+  u32 count = per;
+#pragma unroll 1
+  for (u32 attempt = 0; count; ++attempt) {  // the draw of attempt 255 is taken mod t: the list is empty after it
+    u32 left = 0;
+#pragma unroll 1
+    for (u32 b = 0; b < count; b += 32) {
+      const u32 at = b + lane;
+      bool again = false;
+      u32 j = at;
+      if (at < count) {
+        if (attempt) j = list[at];
+        u64 r = st.draw64(first + j, attempt);
+        r = attempt < 255 ? r & tmask : r % t;  // the rule of uniform_mod
+        again = r >= t;
+        if (!again) dst[j] = (u32)r;
+      }
+      // packed in place: left <= b, and what stands below b + 32 has been read
+      const u32 votes = __ballot_sync(0xffffffffu, again);
+      if (again) list[left + __popc(votes & ((1u << lane) - 1u))] = (unsigned short)j;
+      left += __popc(votes);
     }
+    __syncwarp();
+    count = left;
   }
 }
 
@@ -128,9 +145,9 @@ namespace D2MHE_LAUNCH_NS {
 
 cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
                          u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out) {
-  const u32 threads = std::max(32u, std::min(v.n, 256u)), segs = std::max(1u, v.n / (16 * threads));
-  k_sample_masks<<<n_units * n_parties * segs, threads, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first,
-                                                                n_cts, unit_first, segs, out);
+  const u32 per = std::min(v.n, MASKS_PER_WARP), warps = std::min(v.n / per, 4u), segs = v.n / (per * warps);
+  k_sample_masks<<<n_units * n_parties * segs, 32 * warps, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first,
+                                                                   n_cts, unit_first, segs, per, out);
   return cudaGetLastError();
 }
 

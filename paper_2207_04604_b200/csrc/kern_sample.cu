@@ -81,9 +81,10 @@ __global__ void __launch_bounds__(256)
 // t = 65537, so what counts is that no lane waits for another's redraw: a warp draws once for each of its coefficients,
 // packs the numbers of the rejected ones into a list in shared memory and goes over the list again, 32 at a time, until
 // it is empty.  512 coefficients take 31 full draws and about five partly filled ones, where lanes that walk over 16
-// coefficients of their own wait for the slowest of the 32 (46 draws).  The attempt is uniform over the warp.  Bound by the integer
-// multiplier and the logic pipe beside it, as above.  10.6 M masks mod 65537: 91 us (107 us with both words of every draw, 125 us without the lists); with 64
-// coefficients at a time, two draws to a lane, 20 % slower (the partly filled draws double).
+// coefficients of their own wait for the slowest of the 32 (46 draws).  The attempt is uniform over the warp.
+// Bound by the integer multiplier and the logic pipe beside it, as above.  10.6 M masks mod 65537: 91 us (107 us with
+// both words of every draw, 125 us without the lists); with 64 coefficients at a time, two draws to a lane, 20 % slower
+// (twice as many partly filled draws).
 // grid = shares * segs; each warp of a block has per <= MASKS_PER_WARP coefficients.
 constexpr u32 MASKS_PER_WARP = 512;
 __global__ void __launch_bounds__(128)

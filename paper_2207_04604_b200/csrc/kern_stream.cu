@@ -70,23 +70,28 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// The same with every ciphertext read once: a thread keeps its 16 bytes of all n_rows ciphertexts of index c in shared
-// memory (a column of its own: no barrier but the one that publishes the lists) and adds them up list by list.  What the
-// kernel above spends its time on is one L2 read per list entry (70 sums of five at N = 8192, L = 4: 26.6 -> 20.4 us;
-// MNIST-shaped round 527 -> 504 us).  Chosen when the lists together name more rows than there are, the columns of 128
-// threads fit half of an SM's shared memory, and there are four blocks for every SM (a tiny round is 2 us slower).
-// grid = (n_cts, ciphertext bytes / 16 / 128); shared memory: columns [n_rows][128], then offsets and rows.
-template <class W>
-__global__ void __launch_bounds__(128)
+// The same with every ciphertext read once: a block keeps COLS columns of 16 bytes of all n_rows ciphertexts of index c in
+// shared memory and adds them up list by list.  What the kernel above spends its time on is one L2 read per list entry
+// (70 sums of five at N = 8192, L = 4: 26.6 -> 20.4 us; MNIST-shaped round 527 -> 504 us).  The sums are a chain of
+// shared-memory reads (entry, then residues), and columns of many rows leave room for few threads to hide it, so GROUPS
+// groups of COLS threads share the columns and each takes every GROUPS-th list (N = 16384, L = 8, one group of 128 ->
+// four of 32: 20 rows, lists of 7, 11 indices 227 -> 207 us; 50 rows, lists of 9, four indices 363 -> 223 us).
+// Chosen when the lists together name more rows than there are, the columns of four blocks fit an SM's shared memory
+// (200 rows, columns of two blocks: 349 us against 242 without columns; 100 rows: 231 against 262), and there are
+// 512 columns for every SM (a tiny round is 2 us slower).
+// grid = (n_cts, ciphertext bytes / 16 / COLS); shared memory: columns [n_rows][COLS], then offsets and rows.
+template <class W, u32 COLS, u32 GROUPS>
+__global__ void __launch_bounds__(COLS * GROUPS)
     k_aggregate_columns(DevView v, const W* __restrict__ ct, u32 n_rows, u32 n_cts, const u32* __restrict__ offsets,
                         const u32* __restrict__ rows, u32 n_out, u32 nnz, W* __restrict__ agg) {
   constexpr u32 PER = 16 / sizeof(W);  // residues per vector
-  uint4* col = reinterpret_cast<uint4*>(smem_raw) + threadIdx.x;
-  u32* off = reinterpret_cast<u32*>(smem_raw + (size_t)n_rows * 128 * 16);
+  const u32 tx = threadIdx.x % COLS, group = threadIdx.x / COLS;
+  uint4* col = reinterpret_cast<uint4*>(smem_raw) + tx;
+  u32* off = reinterpret_cast<u32*>(smem_raw + (size_t)n_rows * COLS * 16);
   u32* lst = off + n_out + 1;
-  for (u32 i = threadIdx.x; i <= n_out; i += 128) off[i] = offsets[i];
-  for (u32 i = threadIdx.x; i < nnz; i += 128) lst[i] = rows[i];
-  const u32 c = blockIdx.x, vecs = 2 * v.L * v.n / PER, e = blockIdx.y * 128 + threadIdx.x;
+  for (u32 i = threadIdx.x; i <= n_out; i += COLS * GROUPS) off[i] = offsets[i];
+  for (u32 i = threadIdx.x; i < nnz; i += COLS * GROUPS) lst[i] = rows[i];
+  const u32 c = blockIdx.x, vecs = 2 * v.L * v.n / PER, e = blockIdx.y * COLS + tx;
   const u32 l = ((e * PER) >> v.logn) % v.L;
   const bool in = e < vecs;
   const uint4* src = reinterpret_cast<const uint4*>(ct) + (size_t)c * vecs + e;
@@ -94,8 +99,9 @@ __global__ void __launch_bounds__(128)
     // global -> shared without passing through registers: all rows in flight at once
     const u32 dst = (u32)__cvta_generic_to_shared(col);
 #pragma unroll 4
-    for (u32 r = 0; r < n_rows; ++r)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + r * 2048), "l"(src + (size_t)r * n_cts * vecs)
+    for (u32 r = group; r < n_rows; r += GROUPS)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + r * (COLS * 16)),
+                   "l"(src + (size_t)r * n_cts * vecs)
                    : "memory");
     asm volatile("cp.async.wait_all;" ::: "memory");
   }
@@ -103,7 +109,7 @@ __global__ void __launch_bounds__(128)
   if (!in) return;
   const u64 p = v.limbs[l].p, one_sh = v.limbs[l].one_sh;
   uint4* out = reinterpret_cast<uint4*>(agg) + (size_t)c * vecs + e;
-  for (u32 i = 0; i < n_out; ++i) {
+  for (u32 i = group; i < n_out; i += GROUPS) {
     const u32 beg = off[i], end = off[i + 1];
     uint4 o;
     if (sizeof(W) == 8) {
@@ -112,7 +118,7 @@ __global__ void __launch_bounds__(128)
       for (u32 a = beg; a < end; ++a) {
         const u32 r = lst[a];
         if (!D2MHE_CHK(v.chk, r, n_rows, SITE_PARTY)) continue;
-        const uint4 x = col[r * 128];
+        const uint4 x = col[r * COLS];
         a0 += join64(x.x, x.y);
         a1 += join64(x.z, x.w);
         if (!lazy) a0 = csub(a0, p), a1 = csub(a1, p);
@@ -125,7 +131,7 @@ __global__ void __launch_bounds__(128)
       for (u32 a = beg; a < end; ++a) {
         const u32 r = lst[a];
         if (!D2MHE_CHK(v.chk, r, n_rows, SITE_PARTY)) continue;
-        const uint4 x = col[r * 128];
+        const uint4 x = col[r * COLS];
         o.x += x.x, o.y += x.y, o.z += x.z, o.w += x.w;
         o.x = min(o.x, o.x - q), o.y = min(o.y, o.y - q), o.z = min(o.z, o.z - q), o.w = min(o.w, o.w - q);
       }
@@ -395,14 +401,17 @@ cudaError_t muladd(const DevView& v, cudaStream_t s, const u64* a, const u64* b,
 template <class W>
 static cudaError_t columns_launch(const DevView& v, cudaStream_t s, const W* ct, u32 n_rows, u32 n_cts,
                                   const u32* offsets_dev, const u32* rows_dev, u32 n_out, u32 nnz, W* agg, bool* done) {
-  const size_t smem = (size_t)n_rows * 128 * 16 + ((size_t)n_out + 1 + nnz) * 4;
-  const u32 blocks = (u32)((2 * (size_t)v.L * v.n * sizeof(W) / 16 + 127) / 128);
-  *done = nnz > n_rows && smem <= 112 * 1024 && blocks <= 65535 && (size_t)n_cts * blocks >= 4 * (size_t)v.sms;
+  // groups of 32 threads but for few rows (N = 8192, L = 4, one group of 128 / four of 32: 9 rows 43.0 / 48.1 us, 10 rows
+  // 41.0 / 43.9, 13 rows 41.0 / 39.8, 16 rows 56.0 / 51.2, 30 rows 73.7 / 51.2)
+  const u32 cols = n_rows < 12 ? 128 : 32;
+  const size_t smem = (size_t)n_rows * cols * 16 + ((size_t)n_out + 1 + nnz) * 4;
+  const u32 blocks = (u32)((2 * (size_t)v.L * v.n * sizeof(W) / 16 + cols - 1) / cols);
+  *done = nnz > n_rows && smem <= 56 * 1024 && blocks <= 65535 && (size_t)n_cts * blocks * cols >= 512 * (size_t)v.sms;
   if (!*done) return cudaSuccess;
-  cudaError_t e = set_smem(k_aggregate_columns<W>, smem);
+  const auto kernel = cols == 128 ? k_aggregate_columns<W, 128, 1> : k_aggregate_columns<W, 32, 4>;
+  cudaError_t e = set_smem(kernel, smem);
   if (e != cudaSuccess) return e;
-  k_aggregate_columns<W><<<dim3(n_cts, blocks), 128, smem, s>>>(v, ct, n_rows, n_cts, offsets_dev, rows_dev, n_out, nnz,
-                                                               agg);
+  kernel<<<dim3(n_cts, blocks), 128, smem, s>>>(v, ct, n_rows, n_cts, offsets_dev, rows_dev, n_out, nnz, agg);
   return cudaGetLastError();
 }
 // neighbour sums by columns where that is the better kernel (*done)

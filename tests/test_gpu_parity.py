@@ -1357,7 +1357,8 @@ def test_rounding_on_both_sides_of_every_kind_of_boundary(d2, log2_n, bits, L, t
 
 
 @pytest.mark.parametrize("log2_n,bits,n_rows,n_out,n_cts", [(3, 36, 5, 7, 2), (8, 54, 9, 40, 120), (9, 60, 6, 5, 60), (10, 54, 70, 9, 30), (8, 30, 7, 7, 210),
-                                                           (12, 54, 3, 66, 7)])
+                                                           (12, 54, 3, 66, 7), (9, 54, 11, 9, 60), (9, 54, 12, 9, 60), (9, 30, 13, 6, 120),
+                                                           (9, 54, 111, 5, 60)])
 def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_rows, n_out, n_cts):
     """Lists that name every row more often than there are rows (columns in shared memory), and too many rows for it;
     empty lists, one entry, one list of 200 entries, residues at their largest."""

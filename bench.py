@@ -107,32 +107,41 @@ def algorithmic_bytes(cfg, n_cts):
     }
 
 
-# Integer roofline of the transform-bearing kernels.  The scarce unit is the 32-bit integer
-# multiply-add pipe.  Its rate is MEASURED in every run by the library's register-only loops
-# (d2mhe_debug_int_throughput: mad.lo.u32, mad.wide.u32, mad.hi.u32, and the engine's butterfly)
-# and the roofline's peak is the measured mad.lo rate in lane operations ("slots") per second;
-# 148 SMs x 64 lanes x 1.965 GHz (unit counts and maximum clock) is printed beside it.  A widening
-# or high-half multiply occupies the pipe for two slots (the measured rates say so).  Algorithmic
-# slots: one lazy Shoup butterfly = 5 widening/high + 3 low multiplies = 13 slots (the primes of
-# every configuration are 2^b - d with small d, which turns a fourth low multiply into a shift);
-# a transform = (N/2) log2 N butterflies; a pointwise product = 14; one Philox4x32-10 call = 20
-# widening multiplies = 40 slots (one call serves all L limbs).
-IMAD_LANES_PER_SM = 64
+# Rooflines of the transform-bearing kernels.  The protocol kernels form their ring products by
+# double-precision FFT, and the scarce unit is the double-precision pipe: 64 lanes per SM and clock,
+# 148 SMs, 1.965 GHz (unit counts and maximum clock).  Algorithmic operations (a fused multiply-add
+# counts one) per complex point, N/2 points: radix-2 stages with the twiddle fused, 3 each; 4 for the
+# twist of either end; an inverse transform also 4 for the product and 2 for the rounding.  A 54-bit
+# residue is two parts, each with an inverse transform; a residue below 2^30 is one.
+# The stand-alone transforms stay on the integer multiply-add pipe, whose rate is MEASURED in every
+# run by the library's register-only loops (d2mhe_debug_int_throughput: mad.lo.u32, mad.wide.u32,
+# mad.hi.u32, and the engine's butterfly): the peak is the measured mad.lo rate in lane operations
+# ("slots") per second.  A widening or high-half multiply occupies the pipe for two slots (the
+# measured rates say so), so one lazy Shoup butterfly = 5 widening/high + 3 low multiplies = 13 slots
+# (the primes of every configuration are 2^b - d with small d, which turns a fourth low multiply into
+# a shift).
+LANES_PER_SM = 64
 NUM_SMS = 148
 SM_MAX_HZ = 1.965e9
-IMAD_PEAK_UNIT_COUNTS = NUM_SMS * IMAD_LANES_PER_SM * SM_MAX_HZ
+LANE_PEAK_UNIT_COUNTS = NUM_SMS * LANES_PER_SM * SM_MAX_HZ  # of either pipe
 SLOTS_PER_BUTTERFLY = 13
 
 
-def algorithmic_mad_slots(cfg, n_cts):
-    K, S, L, n = cfg.num_parties, cfg.num_parties, cfg.num_limbs, cfg.n
-    transform = SLOTS_PER_BUTTERFLY * (n // 2) * cfg.log2_n   # slots per limb-transform
+def fft_ops(cfg):
+    """Double-precision operations of a forward and of an inverse transform (with its product and rounding)."""
+    points, stages = cfg.n // 2, 3 * (cfg.log2_n - 1)
+    return points * (stages + 4), points * (stages + 10)
+
+
+def algorithmic_fp64_ops(cfg, n_cts):
+    K, S, L = cfg.num_parties, cfg.num_parties, cfg.num_limbs
     units = K * n_cts
+    fwd, inv = fft_ops(cfg)
     return {
-        # NTT(u) + 2 inverse transforms, 2 pointwise products, Lambda*m (10 slots) per limb; 3 samples per coefficient
-        "encrypt": units * (L * (3 * transform + n * (2 * 14 + 10)) + 3 * 40 * n),
-        # NTT(c1) once, then per share: pointwise product + inverse transform per limb, one sample per coefficient
-        "partial_decrypt": units * (L * (transform + S * (transform + 14 * n)) + S * 40 * n),
+        # the transform of u once for all limbs, then two components times two parts per limb
+        "encrypt": units * (fwd + L * 4 * inv),
+        # both parts of c_1 once per limb, then two parts for every share
+        "partial_decrypt": units * L * (2 * fwd + S * 2 * inv),
     }
 
 
@@ -140,7 +149,7 @@ def algorithmic_mad_slots(cfg, n_cts):
 # from the ncu captures under profiles/ (taken on a few ciphertext indices of the configuration and
 # scaled by the units of a launch: the traffic is the shares written plus c_1 and the noise bytes
 # read, all proportional to the units).  None when the kernel has changed since the capture.
-NCU_TRAFFIC_BYTES_PER_UNIT = {("resnet18-K50", "partial_decrypt"): (589769984 + 5258257000) / 100.0}
+NCU_TRAFFIC_BYTES_PER_UNIT = {}
 
 
 def measure_int_peak(ctx):
@@ -154,7 +163,7 @@ def measure_int_peak(ctx):
            "mul_hi_per_s": mul_hi,
            "slots_per_mad_wide": lo / wide if wide else None, "slots_per_mad_hi": lo / hi if hi else None,
            "slots_per_mul_wide": lo / mul_wide if mul_wide else None, "slots_per_mul_hi": lo / mul_hi if mul_hi else None,
-           "unit_count_peak_per_s": IMAD_PEAK_UNIT_COUNTS,
+           "unit_count_peak_per_s": LANE_PEAK_UNIT_COUNTS,
            "mad_lo_warp_instr_per_clk_per_sm_at_max_clock": lo / 32 / NUM_SMS / SM_MAX_HZ}
     try:
         bf = max(ctx.debug_int_throughput(3, 2048) for _ in range(3))
@@ -487,11 +496,9 @@ def ntt_microbench(ctx, cfg, dev, stream, flush):
 def convert_bootstrap_bench(ctx, cfg, dev, stream, flush, offsets, rows, seed):
     """MBFV.Convert to the recipients' own keys (+ BFV.Decrypt) and MBFV.Bootstrap on the first few
     ciphertext indices of the workload, all K recipients and share holders: CUDA-event time per call
-    and the share calls' fraction of the integer roofline (slots counted as for the decryption shares:
-    Convert = NTT(c_1) once, then per share NTT(mu_k), two inverse transforms, three pointwise
-    products per limb and three samples per coefficient; Bootstrap = NTT(c_1), NTT(alpha) and L
-    samples per coefficient once, then per share two inverse transforms, two products and Lambda M_k
-    per limb and three samples per coefficient)."""
+    and the share calls' fraction of the double-precision roofline (Convert: both parts of c_1 once per
+    limb, mu_k once per share, then two components times two parts per share and limb; Bootstrap: both
+    parts of c_1 and alpha once per limb, then the same)."""
     import torch
 
     K, L, n = cfg.num_parties, cfg.num_limbs, cfg.n
@@ -544,14 +551,14 @@ def convert_bootstrap_bench(ctx, cfg, dev, stream, flush, offsets, rows, seed):
     ctx.partial_decrypt(conv, parties, parties, 0, cc, sh1)
     ctx.combine_decrypt(conv, sh1, K, K, cc, out_plain)
     check("Bootstrap")
-    T = SLOTS_PER_BUTTERFLY * (n // 2) * cfg.log2_n
+    fwd, inv = fft_ops(cfg)
     units, S = K * cc, K
-    slots_conv = units * (L * (T + S * (3 * T + 3 * 14 * n)) + S * 3 * 40 * n)
-    slots_boot = units * (L * (2 * T + 40 * n + S * (2 * T + 2 * 14 * n + 10 * n)) + S * 3 * 40 * n)
+    ops_conv = units * (L * (2 * fwd + S * 4 * inv) + S * fwd)
+    ops_boot = units * L * (4 * fwd + S * 4 * inv)
     return {"cts": cc, "units": units,
             "convert_share_ms": t_cs, "convert_combine_ms": t_cc, "decrypt_ms": t_cd,
             "bootstrap_share_ms": t_bs, "bootstrap_combine_ms": t_bc,
-            "convert_share_slots": slots_conv, "bootstrap_share_slots": slots_boot,
+            "convert_share_fp64_ops": ops_conv, "bootstrap_share_fp64_ops": ops_boot,
             "share_bytes": units * S * 2 * 8 * n * L}
 
 
@@ -608,15 +615,13 @@ def narrow_round_bench(args, local_rank):
 
     ms32, per32 = run(True)
     ms64, per64 = run(False)
-    lo = max(ctx.debug_int_throughput(0, 4096) for _ in range(3))
-    t32 = 4 * (n // 2) * cfg.log2_n  # one high and two low multiplies per 32-bit butterfly
-    slots_pdec = K * C * (L * (t32 + K * (t32 + 4 * n)) + K * 40 * n)
+    fwd, inv = fft_ops(cfg)
+    ops_pdec = K * C * L * (fwd + K * inv)  # one part: the residues are below 2^30
     coeffs = coeffs_of(cfg, 0, C)
     ctx.close()
     return {"config": config_dict(cfg), "note": "call by call on one stream; not the headline (its primes are not the benchmark's)",
             "words32": {"ms_per_round": ms32, "value": coeffs / (ms32 * 1e-3), "unit": UNIT, "calls_ms": per32,
-                        "partial_decrypt_alu_frac": slots_pdec / (per32["partial_decrypt"] * 1e-3) / lo,
-                        "slots_per_butterfly": 4},
+                        "partial_decrypt_fp64_frac": ops_pdec / (per32["partial_decrypt"] * 1e-3) / LANE_PEAK_UNIT_COUNTS},
             "words64_same_primes": {"ms_per_round": ms64, "value": coeffs / (ms64 * 1e-3), "unit": UNIT, "calls_ms": per64}}
 
 
@@ -669,7 +674,7 @@ def run_cuda(args, cfg):
         ab = algorithmic_bytes(cfg, C)
         per_call, serial_steps, n_chunks_total = res["per_call"], res["serial_steps"], res["n_chunks_total"]
         total_ms = sum(per_call.values())
-        slots = algorithmic_mad_slots(cfg, C)
+        fp64 = algorithmic_fp64_ops(cfg, C)
         ntt = res["ntt"]
         for k_ in ("forward", "inverse", "muladd") if ntt else ():
             ntt[k_ + "_frac_of_hbm"] = ntt[k_ + "_GBps"] / peak
@@ -677,7 +682,7 @@ def run_cuda(args, cfg):
             ntt[k_ + "_alu_frac"] = ntt[k_ + "_butterflies_per_s"] * SLOTS_PER_BUTTERFLY / imad_peak
         cb = res["convert_bootstrap"]
         for k_ in ("convert", "bootstrap") if cb else ():
-            cb[k_ + "_share_alu_frac"] = cb[k_ + "_share_slots"] / (cb[k_ + "_share_ms"] * 1e-3) / imad_peak
+            cb[k_ + "_share_fp64_frac"] = cb[k_ + "_share_fp64_ops"] / (cb[k_ + "_share_ms"] * 1e-3) / LANE_PEAK_UNIT_COUNTS
             cb[k_ + "_share_GBps"] = cb["share_bytes"] / 1e9 / (cb[k_ + "_share_ms"] * 1e-3)
         kernels = {}
         for name in STEP_CALLS:
@@ -686,8 +691,8 @@ def run_cuda(args, cfg):
                              "share": per_call[name] / total_ms if total_ms else None,
                              "algorithmic_GB": ab[name] / 1e9, "GBps": ab[name] / 1e9 / (ms * 1e-3) if ms else None,
                              "hbm_frac": ab[name] / 1e9 / (ms * 1e-3) / peak if ms else None}
-            if name in slots:
-                kernels[name]["alu_frac"] = slots[name] / (ms * 1e-3) / imad_peak if ms else None
+            if name in fp64:
+                kernels[name]["fp64_frac"] = fp64[name] / (ms * 1e-3) / LANE_PEAK_UNIT_COUNTS if ms else None
         kernels["aggregate"]["note"] = ("algorithmic bytes count every list's read of a ciphertext; the ciphertexts were "
                                         "just written and most of those reads hit L2, so this is not a DRAM roofline fraction")
         dominant = max(STEP_CALLS, key=lambda k_: per_call[k_])
@@ -697,14 +702,11 @@ def run_cuda(args, cfg):
         achieved = ab[dominant] / chunks_per_step / 1e9 / (dur_ms * 1e-3)
         per_unit = NCU_TRAFFIC_BYTES_PER_UNIT.get((cfg.name, dominant))
         traffic = per_unit * units_per_launch if per_unit else None
-        if dominant in slots:  # transform-bearing kernel: bound by the integer multiply-add pipe
-            got = slots[dominant] / chunks_per_step / (dur_ms * 1e-3)
-            roofline = {"bound": "alu", "kernel": dominant, "achieved": got / 1e12, "peak": imad_peak / 1e12,
-                        "unit": "T int32 multiply-add slots/s", "frac": got / imad_peak,
-                        "peak_source": "measured in this run: mad.lo.u32 lane operations/s of a register-only loop on "
-                                       "all SMs (d2mhe_debug_int_throughput); unit counts x maximum clock give %.2f"
-                                       % (IMAD_PEAK_UNIT_COUNTS / 1e12),
-                        "frac_of_unit_count_peak": got / IMAD_PEAK_UNIT_COUNTS,
+        if dominant in fp64:  # bound by the double-precision pipe and the issue slots around it
+            got = fp64[dominant] / chunks_per_step / (dur_ms * 1e-3)
+            roofline = {"bound": "alu", "kernel": dominant, "achieved": got / 1e12, "peak": LANE_PEAK_UNIT_COUNTS / 1e12,
+                        "unit": "T double-precision lane operations/s", "frac": got / LANE_PEAK_UNIT_COUNTS,
+                        "peak_source": "148 SMs x 64 lanes x 1.965 GHz (unit counts and maximum clock)",
                         "traffic": traffic, "avg_launch_ms": dur_ms, "avg_launch_mcycles": mcycles(dur_ms),
                         "units_per_launch": units_per_launch,
                         "launches_note": "one call = the sampling kernel (about 5 % of the time) followed by the "

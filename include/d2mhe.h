@@ -154,7 +154,7 @@ d2mhe_status d2mhe_aggregate(d2mhe_ctx* ctx, const uint64_t* ct_dev, uint32_t n_
  * recipients, parties: HOST arrays of indices < K.
  * The noise of the shares is sampled by a kernel of its own into the scratch buffer that the
  * context owns (one byte per share coefficient; as many (recipient, ciphertext) pairs per launch as
- * fit, rounded down to whole waves of thread blocks), so the call is one or more pairs of launches
+ * fit, rounded down to whole waves of thread blocks), so the call is one or more groups of launches
  * on the context's stream.
  * D2MHE_ERR_UNSUPPORTED if n_parties * N exceeds that buffer (d2mhe_convert_share and
  * d2mhe_bootstrap_share work the same way with 3 and 6 bytes per share coefficient).

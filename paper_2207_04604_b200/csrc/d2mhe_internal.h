@@ -166,9 +166,11 @@ struct d2mhe_ctx {
 #endif
 
 // Launchers (one per kernel or kernel sequence).  Notes: encrypt and partial_decrypt_scratch sample
-// u, e_0, e_1 / the shares' noise ahead into caller-lent scratch (at least 3 N / n_parties N bytes)
-// and report their number of launches, and so do convert_share (n_parties 3 N bytes) and boot_share
-// (n_parties 6 N bytes); combine sums the first of share_comps polynomials per
+// u, e_0, e_1 / the shares' noise ahead into caller-lent scratch (at least 3 N / n_parties N bytes; with
+// 11 N bytes encrypt takes the double-precision products, which keep the transform of u there too)
+// and report their number of launches, and so do convert_share (n_parties 3 N bytes, double precision from
+// n_parties 11 N) and boot_share (n_parties 6 N bytes, double precision from
+// n_parties 6 N + 8 N L); combine sums the first of share_comps polynomials per
 // (recipient, party, ciphertext); int_probe synchronises the stream; export_secret turns key rows
 // [L][N] (transform domain, Montgomery form) into int8 coefficients [L][N] (127 = not ternary);
 // check_selftest makes one thread of the checked build raise SITE_SELFTEST (no memory access).

@@ -263,6 +263,8 @@ cudaError_t launch_clustered(void (*kernel)(KArgs...), u32 grid, u32 threads, si
 #define D2MHE_DISPATCH(KERNEL, view, grid, stream, ...) \
   D2MHE_DISPATCH_EX(KERNEL, view, grid, stream, 0, 1, __VA_ARGS__)
 
+// Raises a kernel's limit of dynamic shared memory (one value per kernel and device): every caller of a kernel passes the
+// same `bytes`, or none above 48 KB, so that host threads cannot lower it for one another.
 template <class K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   if (bytes <= 48 * 1024) return cudaSuccess;

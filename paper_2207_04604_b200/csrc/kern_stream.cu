@@ -404,12 +404,14 @@ static cudaError_t columns_launch(const DevView& v, cudaStream_t s, const W* ct,
   // groups of 32 threads but for few rows (N = 8192, L = 4, one group of 128 / four of 32: 9 rows 43.0 / 48.1 us, 10 rows
   // 41.0 / 43.9, 13 rows 41.0 / 39.8, 16 rows 56.0 / 51.2, 30 rows 73.7 / 51.2)
   const u32 cols = n_rows < 12 ? 128 : 32;
-  const size_t smem = (size_t)n_rows * cols * 16 + ((size_t)n_out + 1 + nnz) * 4;
+  const size_t smem = (size_t)n_rows * cols * 16 + ((size_t)n_out + 1 + nnz) * 4, most = 56 * 1024;
   const u32 blocks = (u32)((2 * (size_t)v.L * v.n * sizeof(W) / 16 + cols - 1) / cols);
-  *done = nnz > n_rows && smem <= 56 * 1024 && blocks <= 65535 && (size_t)n_cts * blocks * cols >= 512 * (size_t)v.sms;
+  *done = nnz > n_rows && smem <= most && blocks <= 65535 && (size_t)n_cts * blocks * cols >= 512 * (size_t)v.sms;
   if (!*done) return cudaSuccess;
   const auto kernel = cols == 128 ? k_aggregate_columns<W, 128, 1> : k_aggregate_columns<W, 32, 4>;
-  cudaError_t e = set_smem(kernel, smem);
+  // The limit is one value per kernel and device: always the same one, so that a call with fewer rows on another host
+  // thread cannot lower it between this call's two steps.
+  cudaError_t e = set_smem(kernel, most);
   if (e != cudaSuccess) return e;
   kernel<<<dim3(n_cts, blocks), 128, smem, s>>>(v, ct, n_rows, n_cts, offsets_dev, rows_dev, n_out, nnz, agg);
   return cudaGetLastError();

@@ -1,5 +1,7 @@
 """GPU parity: every output of the CUDA library against the CPU oracle, bit for bit,
 through the C ABI (via the thin ctypes binding)."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -1388,6 +1390,37 @@ def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_r
         ctx.sync()
         assert np.array_equal(d2.to_u32_numpy(agg32).astype(np.uint64), want)
     ctx.close()
+
+
+def test_neighbour_sums_of_different_sizes_on_several_threads(d2):
+    """Four host threads, each with its own context, sum 91 to 102 rows at the same time: all need more than 48 KB of shared
+    memory, by different amounts, and the limit of a kernel is shared by all threads of the process."""
+    log2_n, n_cts, errors, calls = 8, 304, [], 4000
+    moduli = small_moduli(log2_n, 54, 1)
+
+    def work(n_rows, seed):
+        try:
+            ctx = d2.Context(log2_n, moduli, 2, seed=seed)
+            gen = torch.Generator(device=ctx.device).manual_seed(seed)
+            ct = torch.randint(0, moduli[0], (n_rows, n_cts, 2, 1, 1 << log2_n), dtype=torch.int64, device=ctx.device, generator=gen)
+            offsets = np.arange(n_rows + 1, dtype=np.uint32) * 9
+            rows = ((np.arange(n_rows)[:, None] + np.arange(9)[None, :]) % n_rows).astype(np.uint32).ravel()
+            agg = ctx.empty_u64(n_rows, n_cts, 2, 1, 1 << log2_n)
+            for _ in range(calls):
+                ctx.aggregate(ct, n_rows, n_cts, offsets, rows, agg)
+            ctx.sync()
+            want = sum(torch.roll(ct, -k, 0) for k in range(9)) % moduli[0]
+            assert torch.equal(agg, want)
+            ctx.close()
+        except BaseException as e:  # noqa: BLE001 - reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=a) for a in ((91, 1), (102, 2), (93, 3), (99, 4))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
 
 
 @pytest.mark.parametrize("log2_n,bits,L,K,C", [(12, 30, 3, 3, 2), (12, 20, 5, 17, 1), (13, 30, 2, 4, 3), (13, 17, 2, 2, 1), (14, 29, 2, 2, 1),

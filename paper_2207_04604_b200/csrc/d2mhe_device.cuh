@@ -7,6 +7,14 @@
 typedef unsigned long long u64;
 typedef unsigned int u32;
 
+// A residue in two parts: split at 2^h; the high part's results are rounded by adding `magic` to fraction bits that `fmask`
+// clears; k0 collects the constants of fft_sum.
+struct FftSplit {
+  double magic;
+  u64 k0;
+  u32 h, fmask;
+};
+
 // ---------------------------------------------------------------------------
 // Per-limb constants (one entry per RNS prime q_l), resident in global memory.
 // ---------------------------------------------------------------------------
@@ -37,11 +45,7 @@ struct LimbTab {
   const ulonglong2* WL;         // [7][N/8]
   const ulonglong2* IWL;        // [7][N/8]
   u32* chk;                     // device check words (read by the checked kernel build only)
-  // double-precision ring products (d2mhe_fft.cuh): residues split at 2^fft_h, the high part's results rounded by
-  // adding fft_magic to fraction bits that fft_fmask clears, the constants of fft_sum
-  double fft_magic;
-  u64 fft_k0;
-  u32 fft_h, fft_fmask;
+  FftSplit fft, fftc;           // double-precision ring products (d2mhe_fft.cuh): with ternary factors, and of Conversion
   // the same on 32-bit words (kern_fft32.cu): floor(2^46 / q_l), a multiple of q_l and the constants of the rounding
   u32 fft32_mu;
   u64 fft32_k;

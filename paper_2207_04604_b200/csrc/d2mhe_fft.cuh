@@ -4,28 +4,35 @@
 // coefficients is needed modulo X^N + 1 and p.  Both are integer polynomials, so the product can be formed over
 // the integers and reduced afterwards: c is centred and split, c = c_lo + 2^h c_hi, each part is multiplied with
 // s by a complex FFT of n = N/2 points in double precision, and the two integer results are rounded and
-// recombined modulo p.  The double-precision pipe of this GPU issues as many lanes per clock as its integer
-// multiplier (62 of 64 measured), but a complex radix-2 butterfly (two points = four coefficients, six fused
-// multiply-adds) stands for two modular butterflies of 15 multiplier slots each.
+// recombined modulo p.  The double-precision pipe of this GPU has as many lanes as its integer multiplier (64 per SM), but
+// a complex radix-2 butterfly (two points = four coefficients, six fused multiply-adds) stands for two modular
+// butterflies of 15 multiplier slots each.
 //
 // Exactness.  X^N + 1 = (X^n - i)(X^n + i), so with z_j = a_j + i a_(j+n) and psi = e^(i pi / 2n) the transform
 // is Z_k = sum_j z_j psi^j e^(2 pi i j k / n), and z_j = psi^-j / n sum_k Z_k e^(-2 pi i j k / n) recovers a product.
-// With u = 2^-53, a butterfly (X, Y) -> (X + wY, X - wY) computed as below has an error of at most 3.02 u times
-// the 2-norm of its outputs, plus the error of w (1 u for a table value or a constant, 4 u for its square, 3 u
-// more for a rotation by a constant); the rest of the operations are unitary up to scaling, so relative errors in
-// the 2-norm add up (Higham, Accuracy and Stability of Numerical Algorithms, ch. 24).  Counted over the stages:
-// 88 u per forward transform, 78 u for product and inverse, 254 u for a product.  A result coefficient is then
-// off by less than 256 u |c|_2 max_k |S_k|.
-//   |c|_2 <= 2^(m-1) sqrt(N) for EVERY part of m bits;
-//   max_k |S_k| < 6.5 sqrt(N) for a ternary s, except with probability below 2^-70 over the key (uniform ternary
-//   coefficients are sub-Gaussian with variance 2/3; 16 directions, n points).
-// Parts of at most 28 bits at N = 16384 stay below 0.41 (smaller rings: below 0.21); the rounding keeps at least
-// four fraction bits and rounds twice (1/16), and 0.41 + 1/16 < 1/2: the rounded value IS the integer.  (Seen:
-// 2^-14 with random and with extreme c, 2^-10 with s = all ones.)  The low part has h <= 40 - log2 N bits, so that
-// its product fits 40 bits for any c and s.
-// Conversion adds the product of a public key (uniform: |p|_2 is sqrt(3) smaller) with a Gaussian mu (|M_k| 3.9 times
-// larger): there the 2-norm bound is 1.4, and what is relied on is that the error is spread, as rounding errors are: it
-// would take a tenth of its square on one of the 16384 coefficients to reach 1/2 (seen: 2^-13).
+// The result has to be off by less than 1/2 minus the rounding below for EVERY residue polynomial c, so what is relied
+// on is the 2-norm only; with u = 2^-53:
+//   A stage's error is at most 2.94 u times the 2-norm of its outputs, plus the error of its twiddle factors: for a
+//     butterfly (X, Y) -> (X + wY = U, X - wY = V) as computed below, U is off by at most u ((1 + a) |U| + b |V|) and V by
+//     u |V| more, a = |3 + e^(2i arg w)| / 4, b = |1 - e^(2i arg w)| / 4.  Stages with w = 1 and i: u.
+//   All steps but these are unitary up to scaling, so relative errors in the 2-norm add up (Higham, Accuracy and Stability
+//     of Numerical Algorithms, ch. 24).  With the errors that the twiddle factors of this file have (0.6 to 2.6 u, computed
+//     and compared in the tests), forward, product and inverse together come to fft_error_units(log2 N) u.
+//   The two norms multiply as |C S|_2 <= |C|_2 max_k |S_k|.  That takes a bound for every single point of the key's
+//     transform and of its error.  A 2-norm bound gives none (n points share the error, one may have it all), so the
+//     transforms of keys are made in double-double arithmetic (kern_fft_keys.cu): every point is good to 1.2 u.
+//   |c|_2 <= 2^(m-1) sqrt(N) for a part of m bits, |u|_2 <= sqrt(N) for the ternary u of an encryption.
+//   max_k |S_k| < FFT_KEY_MAX sqrt(N) for a ternary s, but for a share of 2^-137 of all keys (uniform ternary
+//     coefficients are sub-Gaussian with variance 2/3; 32 directions, n points; there are 2^83 keys at most, for
+//     every seed and party).  max_k |P_k| < FFT_PK_MAX 2^m sqrt(N) for a uniform part of m bits of a public key, but for
+//     2^-111.  |mu|_2 < FFT_MU_NORM sqrt(N) for the Gaussian mu of Conversion, but for 2^-300.
+// fft_error, fft_error_pk and fft_error_conv below are these bounds; the host admits what stays below 1/2 with the
+// rounding, which keeps f >= 4 fraction bits and rounds once or twice (2^-f at most).  Shares and BFV.Decrypt: 0.22 + 1/16 at
+// N = 16384, smaller rings half of that; encryption 0.14; 32-bit words 0.44; Conversion 0.41 with parts of 27 bits.
+// (Seen: 2^-14 with random and with extreme c, 2^-10 with s = all ones.)
+// The low part has h <= 40 - log2 N bits, so that its product with a ternary factor fits 40 bits for any c.  Conversion
+// adds the product of the recipient's public key with mu, up to four times larger by the norms above: its low results
+// are kept in 44 bits, and its parts are halves, ceil(b / 2) bits each.
 //
 // Organisation.  A group of 16 R threads (R = 8 or 16) transforms 256 R points, 16 of them in a thread's registers.
 // Index digits k = kC + R kB + 16 R kA, j = jA + 16 jB + 256 jC:
@@ -152,6 +159,23 @@ D2MHE_HD constexpr int brev_c(int i) {
 #define D2MHE_FMA(a, b, c) std::fma((a), (b), (c))
 #endif
 
+// Error bounds (see above).
+#define FFT_KEY_MAX 8.5
+#define FFT_PK_MAX 2.75
+#define FFT_MU_NORM 4.0
+// |V| <= FFT_CONV_V N 2^(m-1) for a result of Conversion on parts of m bits: 1 for c s, FFT_MU_NORM for mu p
+#define FFT_CONV_V 5
+constexpr double fft_error_units(int logn) { return logn == 12 ? 91.0 : logn == 13 ? 101.0 : 107.0; }
+constexpr double fft_pow2(int e) { return e < 0 ? 1.0 / (double)(1ull << -e) : (double)(1ull << e); }
+// a part of m bits times a key; u times a part of a public key; the sum of Conversion (its product stage loses 5 u more on
+// c s and 3 u on mu p)
+constexpr double fft_error(int logn, int m) { return fft_error_units(logn) * FFT_KEY_MAX * fft_pow2(m - 1 + logn - 53); }
+constexpr double fft_error_pk(int logn, int m) { return fft_error_units(logn) * FFT_PK_MAX * fft_pow2(m + logn - 53); }
+constexpr double fft_error_conv(int logn, int m) {
+  return (fft_error_units(logn) + 5.0) * FFT_KEY_MAX * fft_pow2(m - 1 + logn - 53) +
+         (fft_error_units(logn) + 3.0) * FFT_MU_NORM * FFT_PK_MAX * fft_pow2(m + logn - 53);
+}
+
 // (X, Y) -> (X + w Y, X - w Y)
 D2MHE_HD void fft_bfly(double& xr, double& xi, double& yr, double& yi, double wr, double wi) {
   const double ur = D2MHE_FMA(-wi, yi, D2MHE_FMA(wr, yr, xr));
@@ -265,6 +289,20 @@ D2MHE_HD void fft_product4(double* xr, double* xi, int k, const cpx (&c)[4]) {
   fft_bfly_i<SGN>(xr[i1], xi[i1], xr[i3], xi[i3]);
 }
 
+// psi^-j of digit jC = JC of a column: tw * e^(-i pi JC / 2R) (one group), e^(-i pi JC / 4R) (first of two) or
+// e^(3 i pi JC / 4R) (second of two; psi_1 = e^(-3 i pi / 4 NG)).
+template <int R, int GR, int JC>
+D2MHE_HD cpx fft_twist(const cpx tw, unsigned group) {
+  if constexpr (JC == 0) return tw;
+  if constexpr (GR == 1) {
+    constexpr int a = -32 * JC / R;
+    return cmul(tw, cpx{root_c<a>(), root_s<a>()});
+  } else {
+    const cpx r0{root_c<-JC>(), root_s<-JC>()}, r1{root_c<3 * JC>(), root_s<3 * JC>()};
+    return cmul(tw, group ? r1 : r0);
+  }
+}
+
 D2MHE_HD cpx cmul_add(cpx a, cpx b, cpx c) {
   return cpx{D2MHE_FMA(-a.i, b.i, D2MHE_FMA(a.r, b.r, c.r)), D2MHE_FMA(a.i, b.r, D2MHE_FMA(a.r, b.i, c.i))};
 }
@@ -284,6 +322,57 @@ D2MHE_HD void fft_product4_sum(double* xr, double* xi, int k, const cpx (&c)[4],
   }
   fft_bfly_one(xr[k], xi[k], xr[k + 4], xi[k + 4]);
   fft_bfly_i<SGN>(xr[k + 8], xi[k + 8], xr[k + 12], xi[k + 12]);
+}
+
+// Double-double numbers h + l, |l| <= u |h| (Dekker; Knuth's sum, a fused product): relative errors of a few u^2.  The
+// single operations are spelled out: a sum that was contracted with the product before it would not be that sum.
+#ifdef __CUDA_ARCH__
+#define D2MHE_ADD(a, b) __dadd_rn((a), (b))
+#define D2MHE_MUL(a, b) __dmul_rn((a), (b))
+#else
+#define D2MHE_ADD(a, b) ((a) + (b))
+#define D2MHE_MUL(a, b) ((a) * (b))
+#endif
+struct alignas(16) dd {
+  double h, l;
+};
+struct ddc {
+  dd r, i;
+};
+D2MHE_HD dd dd_norm(double a, double b) {  // |a| >= |b|
+  const double s = D2MHE_ADD(a, b);
+  return dd{s, D2MHE_ADD(b, -D2MHE_ADD(s, -a))};
+}
+D2MHE_HD dd dd_add(dd a, dd b) {
+  const double s = D2MHE_ADD(a.h, b.h), t = D2MHE_ADD(s, -a.h);
+  const double e = D2MHE_ADD(D2MHE_ADD(a.h, -D2MHE_ADD(s, -t)), D2MHE_ADD(b.h, -t));
+  return dd_norm(s, D2MHE_ADD(e, D2MHE_ADD(a.l, b.l)));
+}
+D2MHE_HD dd dd_sub(dd a, dd b) { return dd_add(a, dd{-b.h, -b.l}); }
+D2MHE_HD dd dd_mul(dd a, dd b) {
+  const double p = D2MHE_MUL(a.h, b.h);
+  return dd_norm(p, D2MHE_FMA(a.h, b.l, D2MHE_FMA(a.l, b.h, D2MHE_FMA(a.h, b.h, -p))));
+}
+D2MHE_HD ddc dd_cadd(ddc a, ddc b) { return ddc{dd_add(a.r, b.r), dd_add(a.i, b.i)}; }
+D2MHE_HD ddc dd_csub(ddc a, ddc b) { return ddc{dd_sub(a.r, b.r), dd_sub(a.i, b.i)}; }
+D2MHE_HD ddc dd_cmul(ddc a, ddc b) {
+  return ddc{dd_sub(dd_mul(a.r, b.r), dd_mul(a.i, b.i)), dd_add(dd_mul(a.r, b.i), dd_mul(a.i, b.r))};
+}
+// e^(2 pi i k / order) for any k, from coarse[k / 256] and fine[k mod 256]; order: a power of two
+#define FFT_ROOT_FINE 256
+D2MHE_HD ddc dd_root(const ddc* coarse, const ddc* fine, unsigned order, unsigned k) {
+  k &= order - 1;
+  return dd_cmul(coarse[k / FFT_ROOT_FINE], fine[k % FFT_ROOT_FINE]);
+}
+// The table entry e^(2 pi i k / order), 64 bits of each part: the angle is brought below pi / 4 in whole numbers.
+inline ddc dd_root_entry(unsigned order, unsigned k) {
+  const unsigned quarter = order / 4, q = k / quarter, r = k % quarter;
+  const bool swap = r > quarter / 2;
+  const long double a = 6.283185307179586476925286766559005768L * (long double)(swap ? quarter - r : r) / (long double)order;
+  const long double c = swap ? sinl(a) : cosl(a), s = swap ? cosl(a) : sinl(a);
+  const long double x = q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s, y = q == 0 ? s : q == 1 ? c : q == 2 ? -s : -c;
+  const double xh = (double)x, yh = (double)y;
+  return ddc{dd{xh, (double)(x - xh)}, dd{yh, (double)(y - yh)}};
 }
 
 // The split of a residue c in [0, p): centred, low part in [-2^(h-1), 2^(h-1)), high part the rest.

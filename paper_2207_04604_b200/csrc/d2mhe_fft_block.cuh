@@ -15,23 +15,27 @@ struct FftGeo {
   static constexpr int TG = 16 * R, T = TG * GR, NG = 256 * R, n = NG * GR, COLS = 16 / R;
   static constexpr int CTAS = 512 / T;
   // Shared memory: per group NG complex numbers in rows of 256 (kC) with a stride of 271, which leaves room for the
-  // 16 x 17 layout of the exchange inside a row; the low part's results (a word and a byte for each of 2n).
+  // 16 x 17 layout of the exchange inside a row; the low part's results (stash: 0 none, 1 a word and a byte for each of
+  // 2n, 2 half a byte more).
   static constexpr int RS = 271;
-  static constexpr size_t ex_bytes = (size_t)GR * R * RS * 16, stash_bytes = (size_t)n * 10;
-  static constexpr size_t smem_bytes = ex_bytes + stash_bytes + 16;
+  static constexpr size_t ex_bytes = (size_t)GR * R * RS * 16;
+  __host__ __device__ static constexpr size_t smem_bytes(int stash) {
+    return ex_bytes + (stash ? (size_t)n * (9 + stash) : 0) + 16;
+  }
   // Words of tensor memory per thread for one transform, and columns for `k` of them: warp w of a block
   // reaches the lanes 32 (w mod 4) .. + 31 only, so warps w, w + 4, .. share lanes and split the columns.
   static constexpr int WORDS = 64;
   __host__ __device__ static constexpr u32 tmem_cols(int k) { return (u32)(WORDS * k * (T / 128)); }
 };
 
-// the block's shared memory and this thread's place in it (STASH: with room for the low part's results)
-template <int LOGN, bool STASH = true>
+// the block's shared memory and this thread's place in it (STASH: as in FftGeo::smem_bytes)
+template <int LOGN, int STASH = 1>
 struct FftSmem {
   using G = FftGeo<LOGN>;
   double2* ex;     // of this thread's group
   double2* other;  // of the other group (GR = 2)
   u32 *words, *bytes, *slot;
+  unsigned short* nibbles;
   u32 tg;
   __device__ __forceinline__ FftSmem() {
     const u32 g = group();
@@ -41,7 +45,8 @@ struct FftSmem {
     other = base + (1u - g) * (G::R * G::RS);
     words = reinterpret_cast<u32*>(smem_raw + G::ex_bytes);
     bytes = words + 2 * G::n;
-    slot = STASH ? bytes + G::n / 2 : words;
+    nibbles = reinterpret_cast<unsigned short*>(bytes + G::n / 2);
+    slot = reinterpret_cast<u32*>(smem_raw + G::smem_bytes(STASH) - 16);
   }
   __device__ __forceinline__ u32 group() const { return G::GR > 1 ? threadIdx.x / G::TG : 0u; }
   __device__ __forceinline__ void group_sync() const {
@@ -106,7 +111,7 @@ __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.syn
 // ---- exchanges through shared memory: 16-byte accesses, eight lanes to a wavefront ----------------------------------
 // Inside the 16 threads of a row: element k of lane a goes to element a of lane k, through a 16 x 17 layout (both
 // directions without bank conflicts, constant offsets).  Rows belong to one warp: no block barrier.
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   using G = FftGeo<LOGN>;
   const u32 l16 = sm.tg & 15u;
@@ -125,7 +130,7 @@ __device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN, STASH>& sm, dou
   __syncwarp();
 }
 // the 16 results of a row pass -> row-major, and back; own rows only
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN, STASH>& sm, const double* xr, const double* xi) {
   double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
@@ -133,7 +138,7 @@ __device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN, STASH>& sm, con
     e[16 * k] = make_double2(xr[i], xi[i]);
   });
 }
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   const double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
@@ -143,7 +148,7 @@ __device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN, STASH>& sm, dou
     xi[k] = t.y;
   });
 }
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN, STASH>& sm, const double* xr, const double* xi) {
   using G = FftGeo<LOGN>;
 #pragma unroll
@@ -153,7 +158,7 @@ __device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN, STASH>& sm, con
       sm.ex[sm.tg + k * G::RS + c * G::TG] = make_double2(xr[c * G::R + i], xi[c * G::R + i]);
     });
 }
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN, STASH>& sm, double* xr, double* xi) {
   using G = FftGeo<LOGN>;
 #pragma unroll
@@ -178,24 +183,9 @@ __device__ __forceinline__ cpx ld_cpx(const double2* p) {
   return cpx{t.x, t.y};
 }
 
-// psi^-j of digit jC = JC of a column: tw * e^(-i pi JC / 2R) (one group), e^(-i pi JC / 4R) (first of two) or
-// e^(3 i pi JC / 4R) (second of two; psi_1 = e^(-3 i pi / 4 NG)).
-template <int LOGN, int JC>
-__device__ __forceinline__ cpx fft_twist(const cpx tw, u32 group) {
-  using G = FftGeo<LOGN>;
-  if constexpr (JC == 0) return tw;
-  if constexpr (G::GR == 1) {
-    constexpr int a = -32 * JC / G::R;
-    return cmul(tw, cpx{root_c<a>(), root_s<a>()});
-  } else {
-    const cpx r0{root_c<-JC>(), root_s<-JC>()}, r1{root_c<3 * JC>(), root_s<3 * JC>()};
-    return cmul(tw, group ? r1 : r0);
-  }
-}
-
 // Forward transform.  in(c, jC, h): the coefficients j and j + n as a complex number, j = r + 256 jC + h n/2 with
 // r = tg + c TG (h = 0 for one group).  Leaves Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
-template <int LOGN, bool STASH, class In>
+template <int LOGN, int STASH, class In>
 __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi, In in) {
   using G = FftGeo<LOGN>;
   constexpr int R = G::R;
@@ -211,7 +201,7 @@ __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, c
         const double h = g ? -root_c<16>() : root_c<16>();
         z = cpx{D2MHE_FMA(h, y.r - y.i, z.r), D2MHE_FMA(h, y.r + y.i, z.i)};
       }
-      const cpx p = fft_twist<LOGN, j>(t, g);
+      const cpx p = fft_twist<G::R, G::GR, j>(t, g);
       z = cmul(z, cpx{p.r, -p.i});
       xr[c * R + j] = z.r;
       xi[c * R + j] = z.i;
@@ -237,7 +227,7 @@ __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, c
 }
 
 // in(j): the same by coefficient number, j < n
-template <int LOGN, bool STASH, class In>
+template <int LOGN, int STASH, class In>
 __device__ __forceinline__ void fft_forward(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi, In in) {
   using G = FftGeo<LOGN>;
   fft_forward_at<LOGN>(sm, ft, xr, xi, [&](auto c_, auto j_, auto h_) {
@@ -336,7 +326,7 @@ __device__ __forceinline__ void fft_product_sum(u32 addr, const double2* row_a, 
 // Inverse transform of what the products left, up to the twist: digit jC of column r = tg + c TG is left in
 // x[c R + brev(jC)]; tw: the columns' twist.  before_last(): called ahead of the arithmetic of pass C.
 // Table entries are fetched a pass ahead of their use (they come from L2 as often as not).
-template <int LOGN, bool STASH, class Hook>
+template <int LOGN, int STASH, class Hook>
 __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi,
                                             cpx (&tw)[FftGeo<LOGN>::COLS], Hook before_last) {
   using G = FftGeo<LOGN>;
@@ -361,7 +351,7 @@ __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, cons
 }
 
 // Result number i of a thread (below 32) belongs to this coefficient.
-template <int LOGN, bool STASH>
+template <int LOGN, int STASH>
 __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN, STASH>& sm, int i) {
   using G = FftGeo<LOGN>;
   if (G::GR == 2) return sm.tg + 256u * (8u * sm.group() + (u32)(i & 7)) + 4096u * (u32)(i >> 3);
@@ -371,7 +361,7 @@ __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN, STASH>& sm, int i) {
 // The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
 // eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4]) with v = bits of
 // M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.
-template <int LOGN, bool STASH, class Out>
+template <int LOGN, int STASH, class Out>
 __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr,
                                             double* xi, double magic, Out out) {
   using G = FftGeo<LOGN>;
@@ -380,7 +370,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     // portion: digits j, j + 1 of a column; results (column c) i = 2R c + j, + 1 (real) and + R (imaginary)
     static_for<8>([&](auto m_) {
       constexpr int m = decltype(m_)::value, c = 2 * m / R, j = 2 * m % R, i0 = c * R + brev_c<R>(j), i1 = c * R + brev_c<R>(j + 1);
-      const cpx p0 = fft_twist<LOGN, j>(tw[c], 0), p1 = fft_twist<LOGN, j + 1>(tw[c], 0);
+      const cpx p0 = fft_twist<G::R, G::GR, j>(tw[c], 0), p1 = fft_twist<G::R, G::GR, j + 1>(tw[c], 0);
       u64 v[4];
       v[0] = (u64)__double_as_longlong(__fma_rn(xr[i0], p0.r, __fma_rn(-xi[i0], p0.i, magic)));
       v[1] = (u64)__double_as_longlong(__fma_rn(xr[i1], p1.r, __fma_rn(-xi[i1], p1.i, magic)));
@@ -394,7 +384,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     const u32 g = sm.group();
     static_for<16>([&](auto j_) {
       constexpr int j = decltype(j_)::value, i = brev_c<16>(j);
-      const cpx z = cmul(cpx{xr[i], xi[i]}, fft_twist<LOGN, j>(tw[0], g));
+      const cpx z = cmul(cpx{xr[i], xi[i]}, fft_twist<G::R, G::GR, j>(tw[0], g));
       xr[i] = z.r;
       xi[i] = z.i;
     });
@@ -425,26 +415,31 @@ __device__ __forceinline__ constexpr int fft_result_number() {
   return RR ? I0 + (B & 1) + (B >> 1) * RR : I0 + 8 * B;
 }
 
-// The low part's result V_lo (|V_lo| < 2^39) waits for the high part as a word and a byte: with 8 fraction bits
-// V_lo + 2^39 is bytes 1 .. 5 of the rounded value.
+// The low part's result V_lo waits for the high part: with 8 fraction bits V_lo + 2^39 is bytes 1 .. 5 of the rounded
+// value (|V_lo| <= 2^39: ternary factors), V_lo + 2^43 is these and the low half of byte 6 (Conversion: below 2^43).
 #define D2MHE_FFT_MAGIC_LO (1.5 * 17592186044416.0 + 549755813888.0 + 0.5) /* 1.5 * 2^44 + 2^39 + 1/2 */
+#define D2MHE_FFT_MAGIC_LO44 (1.5 * 17592186044416.0 + 0.5)                /* 1.5 * 2^44 + 1/2 */
 __device__ __forceinline__ u32 lo_word(u64 bits) { return __byte_perm((u32)bits, (u32)(bits >> 32), 0x4321); }
 __device__ __forceinline__ u32 lo_bytes(u64 a, u64 b, u64 c, u64 d) {  // byte 5 of four rounded values
   return __byte_perm(__byte_perm((u32)(a >> 32), (u32)(b >> 32), 0x0051),
                      __byte_perm((u32)(c >> 32), (u32)(d >> 32), 0x0051), 0x5410);
 }
 
-// 64 p + V_lo + 2^h V_hi + e0 - 19, below 130 p.  word, bytes: what fft_finish kept, byte I of `bytes`; hi: the rounded
-// high part with f fraction bits, f = 32 - (b - h) and p = 2^b - d: its low word holds V_hi mod 2^(b-h) above the
-// fraction, its high word floor(V_hi / 2^(b-h)) plus a constant, which counts multiples of 2^b = d (mod p).
-// The constants are collected in fft_k0.
-template <int I>
-__device__ __forceinline__ u64 fft_sum(u32 word, u32 bytes, u64 hi, u32 e0, const LimbTab& lt) {
+// 64 p + V_lo + 2^h V_hi + e0 - 19, between 0 and 129 p: the multiples of d below add up to less than 61 p (d N / 2 with
+// ternary factors, where 256 d < 2^b is enough; FFT_CONV_V times that in Conversion, which the host tests).  low: V_lo plus
+// its offset; hi: the rounded high part with f fraction bits, f = 32 - (b - h) and p = 2^b - d: its low word holds
+// V_hi mod 2^(b-h) above the fraction, its high word floor(V_hi / 2^(b-h)) plus a constant, which counts multiples of
+// 2^b = d (mod p).  The constants are collected in k0.
+__device__ __forceinline__ u64 fft_sum(u64 low, u64 hi, u32 e0, const FftSplit& sp, const LimbTab& lt) {
   u32 hl, hh;
   split64(hi, hl, hh);
-  u64 s = madwide(hl & lt.fft_fmask, 1u << lt.sf_shift, lt.fft_k0 + e0);
+  u64 s = madwide(hl & sp.fmask, 1u << lt.sf_shift, sp.k0 + e0);
   s = madwide(hh, lt.sf_d, s);
-  return s + join64(word, __byte_perm(bytes, 0, 0x4440 | I));
+  return s + low;
+}
+
+__device__ __forceinline__ u32 lo_nibbles(u64 a, u64 b, u64 c, u64 d) {  // low half of byte 6 of four rounded values
+  return ((u32)(a >> 48) & 15u) | ((u32)(b >> 44) & 0xf0u) | ((u32)(c >> 40) & 0xf00u) | ((u32)(d >> 36) & 0xf000u);
 }
 
 // Noise bytes (e + 19) of a polynomial, 32 per thread in the order of fft_coef: 16-byte slots [2][T].
@@ -494,25 +489,30 @@ inline u32 fft_component_split(const DevView& v, u32 base, u32 ctas) {
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
 // High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  (One copy of
 // the code for both parts: two copies share subexpressions, and 300 bytes of them were spilled.)
-template <int LOGN, class Noise, class Store>
-__device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
-                                           double* xr, double* xi, bool high, const Noise& nz, Store store) {
+template <int LOGN, int STASH, class Noise, class Store>
+__device__ __forceinline__ void fft_finish(const FftSmem<LOGN, STASH>& sm, const LimbTab& lt, const FftSplit& sp,
+                                           const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr, double* xi, bool high,
+                                           const Noise& nz, Store store) {
   using G = FftGeo<LOGN>;
-  const double magic = high ? lt.fft_magic : D2MHE_FFT_MAGIC_LO;
+  const double magic = high ? sp.magic : STASH == 2 ? D2MHE_FFT_MAGIC_LO44 : D2MHE_FFT_MAGIC_LO;
   fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4]) {
     constexpr int m = decltype(m_)::value;
     u32* w = sm.words + threadIdx.x + 4 * m * G::T;
     u32* wb = sm.bytes + threadIdx.x + m * G::T;
+    unsigned short* wn = sm.nibbles + threadIdx.x + m * G::T;
     if (high) {
-      const u32 bytes = *wb;
+      const u32 bytes = *wb, nibbles = STASH == 2 ? *wn : 0u;
       static_for<4>([&](auto q_) {
         constexpr int q = decltype(q_)::value, i = fft_result_number<decltype(i_)::value, decltype(rr_)::value, q>();
-        store(fft_coef<LOGN>(sm, i), fft_sum<q>(w[q * G::T], bytes, v[q], nz.template get<i>(), lt));
+        u32 top = __byte_perm(bytes, 0, 0x4440 | q);
+        if (STASH == 2) top |= (q < 3 ? nibbles << (8 - 4 * (q < 3 ? q : 0)) : nibbles >> 4) & 0xf00u;
+        store(fft_coef<LOGN>(sm, i), fft_sum(join64(w[q * G::T], top), v[q], nz.template get<i>(), sp, lt));
       });
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i) w[i * G::T] = lo_word(v[i]);
       *wb = lo_bytes(v[0], v[1], v[2], v[3]);
+      if (STASH == 2) *wn = (unsigned short)lo_nibbles(v[0], v[1], v[2], v[3]);
     }
   });
 }
@@ -520,11 +520,11 @@ __device__ __forceinline__ void fft_finish(const FftSmem<LOGN>& sm, const LimbTa
 __device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer
   return __hiloint2double(0x43300000, v ^ (int)0x80000000u) - __hiloint2double(0x43300000, (int)0x80000000u);
 }
-// part `half` of coefficients j and j + n of a residue row
-__device__ __forceinline__ cpx fft_split_pair(const u64* row, u32 j, u32 n, u32 half, const LimbTab& lt) {
+// part `half` of coefficients j and j + n of a residue row mod p, split at 2^h
+__device__ __forceinline__ cpx fft_split_pair(const u64* row, u32 j, u32 n, u32 half, u64 p, u32 h) {
   int a0, a1, b0, b1;
-  fft_split(__ldg(row + j), lt.p, lt.fft_h, a0, a1);
-  fft_split(__ldg(row + j + n), lt.p, lt.fft_h, b0, b1);
+  fft_split(__ldg(row + j), p, h, a0, a1);
+  fft_split(__ldg(row + j + n), p, h, b0, b1);
   return cpx{small_to_double(half ? a1 : a0), small_to_double(half ? b1 : b0)};
 }
 

@@ -249,7 +249,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   for (u64 x = t; x; x >>= 1) ++t_bits;
   const u32 frac_bits = 59 - t_bits;  // 24 terms below 2^(F + t_bits) fit 64 bits
   c->view.round.frac_bits = frac_bits;
-  bool fft_ok = logn >= 12 && logn <= 14, fft32_ok = fft_ok && c->narrow;
+  bool fft_ok = logn >= 12 && logn <= 14, fft32_ok = fft_ok && c->narrow, conv_ok = fft_ok;
   bool all_special = true;  // every prime is 2^b - d with b >= 32, d < 2^32 and 256 d < 2^b
   for (u32 l = 0; l < L; ++l) {
     const u64 p = c->moduli[l];
@@ -287,8 +287,6 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     T.sf_d = special ? (u32)gap : 0;
     T.sf_shift = special ? bits - 32 : 0;
     if (!special) all_special = false;
-    // Double-precision products (bounds: d2mhe_fft.cuh): the low part has h <= 40 - log2 N bits, the high part at most 28;
-    // its results keep f = 32 - (bits - h) fraction bits.
     {
       u64 others = 1;  // q / q_l mod q_l
       for (u32 m = 0; m < L; ++m)
@@ -306,18 +304,29 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
       T.frac = quo;
       T.frac_shift = 64 - bits;
     }
-    T.fft_h = std::min((bits + 1) / 2, 40 - logn);
-    if (!special || bits - T.fft_h > 28) {
+    // Double-precision products (bounds: d2mhe_fft.cuh): the low part has h <= 40 - log2 N bits, the high part at most 28;
+    // its results keep f = 32 - (bits - h) fraction bits.  Conversion: halves.
+    // one split, its high part with f fraction bits: false when `error` (of its larger part) and the rounding reach 1/2
+    auto split = [&](FftSplit& sp, u32 h, u64 offset, double error) {
+      const u32 f = 32 - (bits - h);
+      sp.h = h;
+      sp.fmask = ~((1u << f) - 1u);
+      sp.magic = 1.5 * (double)((u64)1 << (52 - f)) + 0.5;
+      const u64 h0 = ((u64)(1075 - f) << 20) + ((u64)1 << 19);  // high word of the magic number
+      sp.k0 = 64 * p - offset - D2MHE_GAUSS_B - gap * h0;
+      return error + fft_pow2(-(int)std::min(f, 8u)) < 0.5;
+    };
+    const u32 h = std::min((bits + 1) / 2, 40 - logn), h_conv = (bits + 1) / 2, high = std::max(h, bits - h);
+    if (!special || logn > 14 || bits - h > 28) {
       fft_ok = false;
     } else {
-      const u32 f = 32 - (bits - T.fft_h);
-      T.fft_fmask = ~((1u << f) - 1u);
-      T.fft_magic = 1.5 * (double)((u64)1 << (52 - f)) + 0.5;
-      const u64 h0 = ((u64)(1075 - f) << 20) + ((u64)1 << 19);  // high word of the magic number
-      T.fft_k0 = 64 * p - ((u64)1 << 39) - D2MHE_GAUSS_B - gap * h0;
+      if (!split(T.fft, h, (u64)1 << 39, std::max(fft_error(logn, high), fft_error_pk(logn, high)))) fft_ok = false;
+      if (!split(T.fftc, h_conv, (u64)1 << 43, fft_error_conv(logn, h_conv)) ||
+          (u128)gap * FFT_CONV_V * (n / 2) > (u128)61 * p)
+        conv_ok = false;
     }
 
-    if (bits < 17 || bits > 30 || logn + bits > 43) {
+    if (bits < 17 || bits > 30 || std::max(fft_error(logn, bits), fft_error_pk(logn, bits)) + fft_pow2(-D2MHE_FFT32_F) >= 0.5) {
       fft32_ok = false;
     } else {
       T.fft32_mu = (u32)(((u64)1 << 46) / p);
@@ -501,6 +510,11 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
       for (u32 k = 0; k < 16; ++k) i2[16 * i + k] = root(-(double)(k << (2 * i)), 256.0);
       for (u32 k = 0; k < 256; ++k) i3[256 * i + k] = root(-(double)(k << (2 * i)), m);
     }
+    std::vector<ddc> roots;
+    for (u32 k = 0; k < 8 * m / FFT_ROOT_FINE; ++k) roots.push_back(dd_root_entry(8 * m, k * FFT_ROOT_FINE));
+    for (u32 k = 0; k < FFT_ROOT_FINE; ++k) roots.push_back(dd_root_entry(8 * m, k));
+    c->view.fft.roots = dev_upload(c, roots, &err);
+    if (err != cudaSuccess) return fail_cuda(c, err);
     const std::vector<double2>* src[5] = {&tw, &f2, &f3, &i2, &i3};
     const double2** dst[5] = {&c->view.fft.twist, &c->view.fft.fwd2, &c->view.fft.fwd3, &c->view.fft.inv2,
                               &c->view.fft.inv3};
@@ -518,7 +532,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   if (c->view.fft_on) {
     c->view.usk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
-    c->view.upk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), &err);
+    if (conv_ok) c->view.upk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), &err);
     if (err != cudaSuccess) return fail_cuda(c, err);
   }
 
@@ -807,9 +821,8 @@ d2mhe_status d2mhe_collective_pk(d2mhe_ctx* c, const u32* parties, u32 n_parties
     c->launches += 1;
   }
   if (c->view.fft_on || c->view.fft32_on) {
-    e = c->view.fft_on ? L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, nullptr, 2 * c->view.L,
-                                      c->view.pk_fft)
-                       : L_(fft_rows32)(c->view, c->limb_params, c->stream, c->view.pk_coef, 2 * c->view.L, c->view.pk_fft);
+    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.pk_coef, nullptr, 2 * c->view.L, c->view.fft32_on != 0,
+                     c->view.pk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;
   }
@@ -1123,11 +1136,14 @@ d2mhe_status d2mhe_user_keygen(d2mhe_ctx* c, const u32* users, u32 n_users, uint
   c->launches += 1;
   if (c->view.fft_on) {
     e = L_(fft_secret)(c->view, c->stream, sg.dev[0], n_users, TAG_USER_SECRET, c->view.usk_fft);
-    if (e == cudaSuccess)
-      e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.upk_coef, sg.dev[0], n_users * 2 * c->view.L,
-                       c->view.upk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
-    c->launches += 2;
+    c->launches += 1;
+  }
+  if (c->view.upk_fft) {
+    e = L_(fft_rows)(c->view, c->limb_params, c->stream, c->view.upk_coef, sg.dev[0], n_users * 2 * c->view.L, false,
+                     c->view.upk_fft);
+    if (e != cudaSuccess) return fail_staged(c, sg, e);
+    c->launches += 1;
   }
   const size_t pk_words = 2 * (size_t)c->view.L * c->view.n;
   if (pk_out_dev) {

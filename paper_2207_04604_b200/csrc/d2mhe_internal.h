@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "d2mhe_device.cuh"
+#include "d2mhe_fft.cuh"
 
 #define D2MHE_MAX_LIMBS 24
 #define D2MHE_MAX_SMEM_LOGN 14  // largest polynomial that fits one CTA's shared memory
@@ -37,6 +38,7 @@ struct FftTab {
   const double2* fwd3;   // [2][m/16]      w_m^(4^i k)
   const double2* inv2;   // [2][16]        w_256^(-4^i k)
   const double2* inv3;   // [2][256]       w_m^(-4^i r)
+  const ddc* roots;      // roots of unity of order 8m: every 256th, then the first 256 (dd_root)
 };
 
 // The per-limb constants travel as a kernel parameter (constant bank): indexed by the
@@ -75,7 +77,7 @@ struct DevView {
   double2* s_fft;   // [K][n]        transforms of s_k, times 1/n
   double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n (fft32_on: [2][L][n], whole)
   double2* usk_fft;  // [K][n]            the same of the users' own keys
-  double2* upk_fft;  // [K][2][L][2][n]
+  double2* upk_fft;  // [K][2][L][2][n]   (null: Conversion takes the modular transforms)
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
@@ -235,12 +237,11 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
                         u32* launches); \
 cudaError_t fft_samples(const DevView& v, cudaStream_t s, const void* src, u32 stride, u32 polys, double2* dst); \
 cudaError_t fft_rows(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, const u32* users_dev, \
-                     u32 rows, double2* dst); \
+                     u32 rows, bool whole, double2* dst); \
 cudaError_t share32_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, const u32* parties_dev, \
                         u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u32* shares); \
 cudaError_t encrypt32_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, u32 unit_first, u32 n_units, \
                           const double2* u_fft, const void* noise, const u32* plain, u32* ct); \
-cudaError_t fft_rows32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst); \
 cudaError_t convert_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, \
                         const u32* recipients_dev, u32 n_rec, const u32* parties_dev, u32 n_parties, u32 ct_first, \
                         u32 n_cts, u64* shares, void* scratch, size_t scratch_bytes, u32* launches); \

@@ -224,7 +224,7 @@ cudaError_t convert_share(const DevView& v, const LimbParams& lp, cudaStream_t s
   const size_t per_unit = (size_t)n_parties * 3 * v.n;
   const u32 n_units = n_rec * n_cts;
   // double-precision products; lists of parties too long for their samples take the modular transforms
-  if (v.fft_on && launches && scratch_bytes >= (size_t)n_parties * 11 * v.n) {
+  if (v.upk_fft && launches && scratch_bytes >= (size_t)n_parties * 11 * v.n) {
     *launches = 0;
     return convert_fft(v, lp, s, agg, recipients_dev, n_rec, parties_dev, n_parties, ct_first, n_cts, shares, scratch,
                        scratch_bytes, launches);

@@ -1,7 +1,6 @@
 // Encryption and decryption shares on 32-bit words by double-precision FFT (see d2mhe_fft.cuh): a residue below 2^30
 // is one part, so a product takes one transform instead of two, and nothing waits in shared memory.
-// Used when log2 N + bits <= 43: the 2-norm bound is 0.81 then, 0.47 for uniform residues (what c_1 and the public key
-// are); beyond that the argument given there for conversion applies.  Seen: below 2^-11.
+// Used when the error bound there allows it: log2 N + bits <= 43, where it is 0.44 for any residues.  Seen: below 2^-11.
 #include <algorithm>
 
 #include "d2mhe_fft_block.cuh"
@@ -22,7 +21,7 @@ __device__ __forceinline__ u32 fft_residue32(u64 bits, u32 e0, const LimbTab& lt
 
 // the end of an inverse transform: store(coefficient, value below 3p)
 template <int LOGN, class Store>
-__device__ __forceinline__ void fft_finish32(const FftSmem<LOGN, false>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
+__device__ __forceinline__ void fft_finish32(const FftSmem<LOGN, 0>& sm, const LimbTab& lt, const cpx (&tw)[FftGeo<LOGN>::COLS],
                                              double* xr, double* xi, const FftNoise<LOGN>& nz, Store store) {
   fft_results<LOGN>(sm, tw, xr, xi, D2MHE_FFT32_MAGIC, [&](auto, auto i_, auto rr_, const u64(&v)[4]) {
     static_for<4>([&](auto q_) {
@@ -34,7 +33,7 @@ __device__ __forceinline__ void fft_finish32(const FftSmem<LOGN, false>& sm, con
 
 template <int LOGN>
 constexpr size_t smem32() {
-  return FftGeo<LOGN>::smem_bytes - FftGeo<LOGN>::stash_bytes;
+  return FftGeo<LOGN>::smem_bytes(0);
 }
 
 // One thread block = one (recipient, ciphertext, limb) and its part of the parties; as k_share_fft.
@@ -52,7 +51,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p;
-  const FftSmem<LOGN, false> sm;
+  const FftSmem<LOGN, 0> sm;
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -100,7 +99,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p, delta = (u32)lt.delta, delta_sh = (u32)(lt.delta_sh >> 32);
-  const FftSmem<LOGN, false> sm;
+  const FftSmem<LOGN, 0> sm;
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -129,21 +128,6 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   if (tid < 32) tmem_free(tbase, G::tmem_cols(1));
 }
 
-// Whole residue rows (below 2^30), times 1/n.   grid = rows; limb of row r = r mod L; dst: [rows][n]
-template <int LOGN>
-__global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
-    k_fft_rows32(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ src, double2* __restrict__ dst) {
-  using G = FftGeo<LOGN>;
-  const LimbTab& lt = lp.limbs[blockIdx.x % v.L];
-  const u64* row = src + (size_t)blockIdx.x * v.n;
-  double xr[16], xi[16];
-  fft_forward<LOGN>(FftSmem<LOGN, false>(), v.fft, xr, xi, [&](u32 j) {
-    if (!D2MHE_CHK(v.chk, j + G::n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
-    return centred_pair((u32)row[j], (u32)row[j + G::n], lt);
-  });
-  fft_store<LOGN>(dst + (size_t)blockIdx.x * G::n, xr, xi, 1.0 / (double)G::n);
-}
-
 template <int LOGN>
 cudaError_t launch_share32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, const u32* parties_dev,
                            u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u32* shares) {
@@ -166,15 +150,6 @@ cudaError_t launch_encrypt32(const DevView& v, const LimbParams& lp, cudaStream_
       v, lp, unit_first, u_fft, reinterpret_cast<const uint4*>(noise), plain, ct, split);
   return cudaGetLastError();
 }
-template <int LOGN>
-cudaError_t launch_rows32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst) {
-  using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_fft_rows32<LOGN>, G::ex_bytes);
-  if (e != cudaSuccess) return e;
-  k_fft_rows32<LOGN><<<rows, G::T, G::ex_bytes, s>>>(v, lp, src, dst);
-  return cudaGetLastError();
-}
-
 #define D2MHE_BY_SIZE(FN, ...)                   \
   switch (v.logn) {                              \
     case 12: return FN<12>(__VA_ARGS__);         \
@@ -197,10 +172,4 @@ cudaError_t encrypt32_fft(const DevView& v, const LimbParams& lp, cudaStream_t s
                           const double2* u_fft, const void* noise, const u32* plain, u32* ct) {
   D2MHE_BY_SIZE(launch_encrypt32, v, lp, s, unit_first, n_units, u_fft, noise, plain, ct)
 }
-
-// src: rows of N residues; dst: [rows][n]
-cudaError_t fft_rows32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* src, u32 rows, double2* dst) {
-  D2MHE_BY_SIZE(launch_rows32, v, lp, s, src, rows, dst)
-}
-
 }  // namespace D2MHE_LAUNCH_NS

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   for (u32 half = 0; half < 2; ++half) {
     fft_forward<LOGN>(sm, v.fft, xr, xi, [&](u32 j) {
       if (!D2MHE_CHK(v.chk, j + n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
-      const cpx z = fft_split_pair(fixed, j, n, half, lt);
+      const cpx z = fft_split_pair(fixed, j, n, half, lt.p, lt.fft.h);
       return cpx{z.r * sign, z.i * sign};
     });
     fft_to_tmem(tm + half * G::WORDS, xr, xi);
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
       if (high) nz.load(noise + ((share * 2 + comp) * v.n) / 16);
     });
-    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
+    fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;
       const u64 dm = shoup_u32(__ldg(mask + j), lt.delta, lt.delta_sh, lt.np);  // Lambda M_k, below 2p
       __stcs(out + j, canon8<true>(s + (comp ? dm : lt.twop - dm), lt));
@@ -78,10 +78,10 @@ cudaError_t launch_boot(const DevView& v, const LimbParams& lp, cudaStream_t s, 
                         u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const u64* alpha, const void* noise,
                         const u32* masks, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_boot_fft<LOGN>, G::smem_bytes);
+  cudaError_t e = set_smem(k_boot_fft<LOGN>, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   const u32 split = fft_party_split(v, n_units * v.L * 2, G::CTAS, n_parties, 2);
-  k_boot_fft<LOGN><<<n_units * v.L * 2 * split, G::T, G::smem_bytes, s>>>(
+  k_boot_fft<LOGN><<<n_units * v.L * 2 * split, G::T, G::smem_bytes(1), s>>>(
       v, lp, agg, parties_dev, n_parties, n_cts, unit_first, alpha, reinterpret_cast<const uint4*>(noise), masks, shares,
       split);
   return cudaGetLastError();

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   u32 recipient = recipients[irec];
   if (!D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) recipient = 0;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN> sm;
+  const FftSmem<LOGN, 2> sm;
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   for (u32 half = 0; half < 2; ++half) {
     fft_forward<LOGN>(sm, v.fft, xr, xi, [&](u32 j) {
       if (!D2MHE_CHK(v.chk, j + n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
-      return fft_split_pair(c1, j, n, half, lt);
+      return fft_split_pair(c1, j, n, half, lt.p, lt.fftc.h);
     });
     fft_to_tmem(tm + half * G::WORDS, xr, xi);
   }
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
       if (high) nz.load(noise + ((share * 3 + 1 + comp) * v.n) / 16);
     });
-    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
+    fft_finish<LOGN>(sm, lt, lt.fftc, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
     });
     i = (i + 1) & 3u;
@@ -79,10 +79,10 @@ cudaError_t launch_convert(const DevView& v, const LimbParams& lp, cudaStream_t 
                            const u32* recipients_dev, const u32* parties_dev, u32 n_parties, u32 n_cts, u32 unit_first,
                            u32 n_units, const double2* mu_fft, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_convert_fft<LOGN>, G::smem_bytes);
+  cudaError_t e = set_smem(k_convert_fft<LOGN>, G::smem_bytes(2));
   if (e != cudaSuccess) return e;
   const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 4);
-  k_convert_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes, s>>>(
+  k_convert_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes(2), s>>>(
       v, lp, agg, recipients_dev, parties_dev, n_parties, n_cts, unit_first, mu_fft,
       reinterpret_cast<const uint4*>(noise), shares, split);
   return cudaGetLastError();

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
       if (high) nz.load(noise + (((size_t)ulocal * 3 + 1 + comp) * v.n) / 16);
     });
-    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
+    fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;
       if (comp == 0) s += shoup_u32(__ldg(m + j), lt.delta, lt.delta_sh, lt.np);  // Lambda m, below 2p
       out[j] = canon8<true>(s, lt);
@@ -54,10 +54,10 @@ template <int LOGN>
 cudaError_t launch_encrypt(const DevView& v, const LimbParams& lp, cudaStream_t s, u32 unit_first, u32 n_units,
                            const double2* u_fft, const void* noise, const u32* plain, u64* ct) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_encrypt_fft<LOGN>, G::smem_bytes);
+  cudaError_t e = set_smem(k_encrypt_fft<LOGN>, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   const u32 split = fft_component_split(v, n_units * v.L, G::CTAS);
-  k_encrypt_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes, s>>>(v, lp, unit_first, u_fft,
+  k_encrypt_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, unit_first, u_fft,
                                                                 reinterpret_cast<const uint4*>(noise), plain, ct, split);
   return cudaGetLastError();
 }

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   for (u32 half = 0; half < 2; ++half) {
     fft_forward<LOGN>(sm, v.fft, xr, xi, [&](u32 j) {
       if (!D2MHE_CHK(v.chk, j + n, v.n, SITE_LOAD)) return cpx{0.0, 0.0};
-      return fft_split_pair(c1, j, n, half, lt);
+      return fft_split_pair(c1, j, n, half, lt.p, lt.fft.h);
     });
     fft_to_tmem(tm + half * G::WORDS, xr, xi);
   }
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
       if constexpr (!OWN)
         if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16);
     });
-    fft_finish<LOGN>(sm, lt, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
+    fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
     });
     key = next;
@@ -81,10 +81,10 @@ template <int LOGN, bool OWN>
 cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
                          u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_share_fft<LOGN, OWN>, G::smem_bytes);
+  cudaError_t e = set_smem(k_share_fft<LOGN, OWN>, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 2);
-  k_share_fft<LOGN, OWN><<<n_units * v.L * split, G::T, G::smem_bytes, s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
+  k_share_fft<LOGN, OWN><<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
                                                               reinterpret_cast<const uint4*>(noise), shares, split);
   return cudaGetLastError();
 }

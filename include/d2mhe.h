@@ -79,7 +79,9 @@ typedef struct {
  * key storage, index staging, and the scratch for the samples that d2mhe_encrypt,
  * d2mhe_partial_decrypt, d2mhe_convert_share and d2mhe_bootstrap_share draw ahead of their kernels:
  * 64 MiB, or what two waves of thread blocks of the share kernels need for this parameter set, at
- * most 512 MiB; d2mhe_sample_scratch_bytes reports it).  *out is NULL on failure. */
+ * most 512 MiB; d2mhe_sample_scratch_bytes reports it).  Transforms of the keys that only make later calls
+ * faster are left out where they would take more than a sixteenth of the memory that is still free.
+ * *out is NULL on failure. */
 d2mhe_status d2mhe_create(const d2mhe_params* params, d2mhe_ctx** out);
 void d2mhe_destroy(d2mhe_ctx* ctx);
 /* Stream (a cudaStream_t passed as void*) on which later calls are enqueued; NULL = default. */

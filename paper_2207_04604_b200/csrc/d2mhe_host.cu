@@ -155,6 +155,19 @@ T* dev_alloc(d2mhe_ctx* c, size_t count, cudaError_t* err) {
   return reinterpret_cast<T*>(dev_bytes(c, count * sizeof(T), err));
 }
 
+// Tables that make calls faster but that they can do without: null when they would take more than a sixteenth of the
+// device memory that is still free, so that a context of very many parties fits wherever it would fit without them and
+// leaves its caller the memory for the messages.
+template <class T>
+T* dev_spare(d2mhe_ctx* c, size_t count) {
+  size_t free_bytes = 0, total = 0;
+  cudaError_t e = cudaMemGetInfo(&free_bytes, &total);
+  T* d = nullptr;
+  if (e == cudaSuccess && count * sizeof(T) <= free_bytes / 16) d = dev_alloc<T>(c, count, &e);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e == cudaSuccess ? d : nullptr;
+}
+
 d2mhe_status fail_cuda(d2mhe_ctx* c, cudaError_t e) {
   if (c) c->last_cuda = e;
   return D2MHE_ERR_CUDA;
@@ -491,8 +504,10 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     rt.qinv_mod_t = h_inv(q_mod_t, t);
   }
 
-  // double-precision ring products
-  if ((fft_ok && all_special) || fft32_ok) {
+  // double-precision ring products: twiddle factors here, keys after everything that the context cannot do without
+  c->view.fft32_on = fft32_ok ? 1 : 0;
+  c->view.fft_on = fft_ok && all_special && !fft32_ok ? 1 : 0;
+  if (c->view.fft_on || c->view.fft32_on) {
     const u32 groups = logn == 14 ? 2 : 1, m = n / 2 / groups, R = m / 256;
     // e^(2 pi i num / den), in extended precision before the rounding to double
     auto root = [](double num, double den) {
@@ -522,18 +537,6 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
       *dst[i] = dev_upload(c, *src[i], &err);
       if (err != cudaSuccess) return fail_cuda(c, err);
     }
-    c->view.s_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
-    if (err != cudaSuccess) return fail_cuda(c, err);
-    c->view.pk_fft = dev_alloc<double2>(c, 4 * (size_t)L * (n / 2), &err);
-    if (err != cudaSuccess) return fail_cuda(c, err);
-    c->view.fft32_on = fft32_ok ? 1 : 0;
-    c->view.fft_on = fft32_ok ? 0 : 1;
-  }
-  if (c->view.fft_on) {
-    c->view.usk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * (n / 2), &err);
-    if (err != cudaSuccess) return fail_cuda(c, err);
-    if (conv_ok) c->view.upk_fft = dev_alloc<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), &err);
-    if (err != cudaSuccess) return fail_cuda(c, err);
   }
 
   // key storage
@@ -616,6 +619,16 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   }
   err = cudaEventCreateWithFlags(&c->fork_event, cudaEventDisableTiming);
   if (err != cudaSuccess) return fail_cuda(c, err);
+
+  if (c->view.fft_on || c->view.fft32_on) {
+    c->view.s_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2));
+    c->view.pk_fft = c->view.s_fft ? dev_spare<double2>(c, 4 * (size_t)L * (n / 2)) : nullptr;
+    if (!c->view.pk_fft) c->view.fft_on = c->view.fft32_on = 0;
+  }
+  if (c->view.fft_on) {
+    c->view.usk_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2));
+    if (conv_ok) c->view.upk_fft = dev_spare<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2));
+  }
   return D2MHE_OK;
 }
 
@@ -1134,7 +1147,7 @@ d2mhe_status d2mhe_user_keygen(d2mhe_ctx* c, const u32* users, u32 n_users, uint
   cudaError_t e = L_(user_keygen)(c->view, c->limb_params, c->stream, sg.dev[0], n_users);
   if (e != cudaSuccess) return fail_staged(c, sg, e);
   c->launches += 1;
-  if (c->view.fft_on) {
+  if (c->view.usk_fft) {
     e = L_(fft_secret)(c->view, c->stream, sg.dev[0], n_users, TAG_USER_SECRET, c->view.usk_fft);
     if (e != cudaSuccess) return fail_staged(c, sg, e);
     c->launches += 1;

@@ -70,14 +70,15 @@ struct DevView {
   // {residue out of Montgomery form, its 32-bit Shoup companion}
   u64* s32;       // [K][L][N]
   u64* pk32;      // [2][L][N]
-  // ring products in double precision (set when the sizes are inside the bounds of d2mhe_fft.cuh)
+  // ring products in double precision (set when the sizes are inside the bounds of d2mhe_fft.cuh and the device has room
+  // for the keys; usk_fft and upk_fft, null without room, serve BFV.Decrypt and Conversion)
   u32 fft_on;    // the 64-bit calls
   u32 fft32_on;  // the 32-bit-word calls
   FftTab fft;
   double2* s_fft;   // [K][n]        transforms of s_k, times 1/n
   double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n (fft32_on: [2][L][n], whole)
   double2* usk_fft;  // [K][n]            the same of the users' own keys
-  double2* upk_fft;  // [K][2][L][2][n]   (null: Conversion takes the modular transforms)
+  double2* upk_fft;  // [K][2][L][2][n]
   u32* range_flag;
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };

@@ -258,7 +258,7 @@ cudaError_t convert_combine(const DevView& v, cudaStream_t s, const u64* agg, co
 
 cudaError_t secret_product(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* ct,
                            const u32* users_dev, u32 n_users, u32 n_cts, u64* prod) {
-  if (v.fft_on) return secret_product_fft(v, lp, s, ct, users_dev, n_users, n_cts, prod);
+  if (v.usk_fft) return secret_product_fft(v, lp, s, ct, users_dev, n_users, n_cts, prod);
   D2MHE_DISPATCH(k_secret_product, v, n_users * n_cts * v.L, s, v, lp, ct, users_dev, n_cts, prod);
 }
 

@@ -1,5 +1,6 @@
 """GPU parity: every output of the CUDA library against the CPU oracle, bit for bit,
 through the C ABI (via the thin ctypes binding)."""
+import gc
 import threading
 
 import numpy as np
@@ -1390,6 +1391,44 @@ def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_r
         ctx.sync()
         assert np.array_equal(d2.to_u32_numpy(agg32).astype(np.uint64), want)
     ctx.close()
+
+
+def test_context_fits_where_only_the_keys_themselves_fit(d2):
+    """With too little device memory for the transforms of 400 parties' keys beside the keys, a context is created all the
+    same and gives the same messages."""
+    log2_n, K, L = 12, 400, 2
+    moduli, n, parties = wl.ntt_primes(50, 2 << log2_n, L), 1 << log2_n, list(range(K))
+    agg = torch.randint(0, min(moduli), (1, 1, 2, L, n), dtype=torch.int64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    shares = [torch.empty((1, K, 1, 2, L, n), dtype=torch.int64, device="cuda") for _ in range(2)]
+
+    def messages(out):
+        ctx = d2.Context(log2_n, moduli, K, seed=83)
+        used = free - torch.cuda.mem_get_info()[0]
+        ctx.keygen_share(parties)
+        ctx.user_keygen([0])
+        ctx.convert_share(agg, [0], parties, 0, 1, out)
+        ctx.sync()
+        ctx.close()
+        return used
+
+    def settle():
+        gc.collect()
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    free = settle()
+    messages(shares[0])  # loads the kernels
+    free = settle()
+    used = messages(shares[0])
+    free = settle()
+    filler = torch.empty(free - used + (60 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        messages(shares[1])
+    finally:
+        del filler
+        settle()
+    assert torch.equal(shares[0], shares[1])
 
 
 def test_neighbour_sums_of_different_sizes_on_several_threads(d2):

@@ -9,7 +9,7 @@ import torch
 
 from paper_2207_04604_b200 import workloads as wl
 
-from common import T, from_big, make_oracle, psi_t_for, q_of, small_moduli
+from common import T, from_big, make_oracle, psi_t_for, q_of, small_moduli, to_big
 
 pytestmark = pytest.mark.gpu
 
@@ -1390,6 +1390,31 @@ def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_r
         ctx.aggregate32(d2.from_u32_numpy(ct.astype(np.uint32), ctx.device), n_rows, n_cts, offsets, rows, agg32)
         ctx.sync()
         assert np.array_equal(d2.to_u32_numpy(agg32).astype(np.uint64), want)
+    ctx.close()
+
+
+@pytest.mark.parametrize("bits,L,K", [(54, 2, 101), (54, 1, 130), (60, 2, 121), (30, 3, 119), (30, 2, 311)])
+def test_combination_of_many_shares(d2, bits, L, K):
+    """More shares than a plain sum may have, all residues at their largest in one half of the coefficients."""
+    log2_n, n = 4, 16
+    moduli = small_moduli(log2_n, bits, L)
+    q, rng = q_of(moduli), np.random.default_rng(K)
+    ctx = d2.Context(log2_n, moduli, K, seed=84)
+    ctx.keygen_share(list(range(K)))
+    ctx.collective_pk(list(range(K)))
+    top = np.array(moduli, dtype=np.uint64)[:, None] - 1
+    agg, shares = rng.integers(0, 1 << 62, (1, 1, 2, L, n), dtype=np.uint64) % (top + 1), rng.integers(0, 1 << 62, (1, K, 1, L, n), dtype=np.uint64) % (top + 1)
+    agg[..., : n // 2], shares[..., : n // 2] = top, top
+    total = agg[0, 0, 0].astype(object) + shares[0, :, 0].astype(object).sum(axis=0)
+    want = [((2 * T * v + q) // (2 * q)) % T for v in to_big(total, moduli)]
+    out = ctx.empty_u32(1, 1, n)
+    ctx.combine_decrypt(d2.from_u64_numpy(agg, ctx.device), d2.from_u64_numpy(shares, ctx.device), 1, K, 1, out)
+    ctx.sync()
+    assert d2.to_u32_numpy(out)[0, 0].tolist() == want
+    if bits <= 30:
+        ctx.combine_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), d2.from_u32_numpy(shares.astype(np.uint32), ctx.device), 1, K, 1, out)
+        ctx.sync()
+        assert d2.to_u32_numpy(out)[0, 0].tolist() == want
     ctx.close()
 
 

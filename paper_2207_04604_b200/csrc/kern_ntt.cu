@@ -46,6 +46,9 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
 // shared-memory engine with the twiddles of its sub-tree (pass B).  The inverse runs B then A.
 // Between the passes values are lazily reduced: below 8p with one conditional subtraction per butterfly (MODE_STRICT);
 // WIDE primes take 16 stages without any; below 2^60 (LAZY60) three stages fit and the fourth's operands are reduced.
+// Forward at N = 32768 (three stages) the conditional subtractions cost nothing and the kernel without them is the slower
+// one (444 rows mod 54-bit primes, both passes: 150.7 us with them, 153.8 without; inverse 153.2 / 142.4; N = 65536
+// forward 327 / 317): there WIDE primes take MODE_STRICT.
 template <int SA, bool INV, int MODE>
 __global__ void __launch_bounds__(256)
     k_ntt_strided(DevView v, const __grid_constant__ LimbParams lp, u64* __restrict__ polys) {
@@ -151,7 +154,8 @@ static cudaError_t ntt_two_pass(const DevView& v, const LimbParams& lp, cudaStre
 #define D2MHE_STRIDED(INV_, MODE_)                                              \
   do {                                                                          \
     if (soff == 3)                                                              \
-      k_ntt_strided<3, INV_, MODE_><<<grid_a, 256, 0, s>>>(v, lp, polys);       \
+      k_ntt_strided<3, INV_, !INV_ && MODE_ == MODE_WIDE ? MODE_STRICT : MODE_>  \
+          <<<grid_a, 256, 0, s>>>(v, lp, polys);                                \
     else                                                                        \
       k_ntt_strided<4, INV_, MODE_><<<grid_a, 256, 0, s>>>(v, lp, polys);       \
     e = cudaGetLastError();                                                     \

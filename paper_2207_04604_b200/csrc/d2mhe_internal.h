@@ -249,8 +249,9 @@ cudaError_t convert_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
 cudaError_t boot_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* recipients_dev, \
                      u32 n_rec, const u32* parties_dev, u32 n_parties, u32 ct_first, u32 n_cts, u64* shares, \
                      void* scratch, size_t scratch_bytes, u32* launches); \
-cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
-                         u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out); \
+cudaError_t sample_boot(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
+                        u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, bool fft_order, void* noise, \
+                        u32* masks, u32* launches); \
 cudaError_t sample_alpha(const DevView& v, cudaStream_t s, const u32* recipients_dev, u32 ct_first, u32 n_cts, \
                          u32 unit_first, u32 n_units, u64* out); \
 cudaError_t secret_product_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* ct, \

@@ -43,9 +43,14 @@ __global__ void __launch_bounds__(ntt_threads_ct(LOGN, G), ntt_minb_ct(LOGN, G))
     if (a >= 0) {
       __syncthreads();  // every thread is done with the previous share's samples
       const size_t share = (size_t)ulocal * n_parties + a;
-      for (u32 w = threadIdx.x; w < words; w += blockDim.x)
-        reinterpret_cast<u32*>(small)[w] = __ldg(noise + share * words + w);
-      for (u32 w = threadIdx.x; w < v.n; w += blockDim.x) mask[w] = __ldg(masks + share * v.n + w);
+      const u32 *src = noise + share * words, *src_m = masks + share * v.n - words;
+      if (LOGN == 0) {  // rings up to 1024: one round of loads instead of two (N = 16, 30 parties: 170 -> 156 us)
+        for (u32 w = threadIdx.x; w < words + v.n; w += blockDim.x)
+          reinterpret_cast<u32*>(small)[w] = __ldg((w < words ? src : src_m) + w);
+      } else {
+        for (u32 w = threadIdx.x; w < words; w += blockDim.x) reinterpret_cast<u32*>(small)[w] = __ldg(src + w);
+        for (u32 w = threadIdx.x; w < v.n; w += blockDim.x) mask[w] = __ldg(src_m + words + w);
+      }
       // the barrier that opens the first inverse transform publishes the copy
     }
     u64* h0 = a < 0 ? park : shares + ((((size_t)irec * n_parties + a) * n_cts + cl) * 2) * poly + row;
@@ -155,14 +160,14 @@ cudaError_t boot_share(const DevView& v, const LimbParams& lp, cudaStream_t s, c
     const u32 nu = std::min(per_batch, n_units - first);
     u32* masks = reinterpret_cast<u32*>(scratch);
     u32* noise = masks + (size_t)nu * n_parties * v.n;
-    cudaError_t e = sample_masks(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, masks);
-    if (e != cudaSuccess) return e;
-    e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, kSampleBoot, false, noise);
+    u32 sampling = 0;
+    cudaError_t e = sample_boot(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, false, noise, masks,
+                                &sampling);
     if (e != cudaSuccess) return e;
     e = boot_share_units(v, lp, s, agg, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, noise, masks,
                          shares);
     if (e != cudaSuccess) return e;
-    if (launches) *launches += 3;
+    if (launches) *launches += 1 + sampling;
   }
   return cudaSuccess;
 }

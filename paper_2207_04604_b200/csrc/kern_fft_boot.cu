@@ -108,9 +108,7 @@ cudaError_t boot_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, con
     unsigned char* noise = base + nu * (poly_bytes_ + (size_t)n_parties * 4 * v.n);
     cudaError_t e = sample_alpha(v, s, recipients_dev, ct_first, n_cts, first, nu, alpha);
     if (e != cudaSuccess) return e;
-    e = sample_masks(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, masks);
-    if (e != cudaSuccess) return e;
-    e = sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, kSampleBoot, true, noise);
+    e = sample_boot(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, first, nu, true, noise, masks, launches);
     if (e != cudaSuccess) return e;
     switch (v.logn) {
 #define D2MHE_BOOT(LOGN_)                                                                                          \
@@ -124,7 +122,7 @@ cudaError_t boot_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, con
       default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    *launches += 4;
+    *launches += 2;
   }
   return cudaSuccess;
 }

@@ -77,6 +77,52 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// The same in the order of the coefficients for rings below 256, whose polynomials do not fill a block: one word for each
+// thread and step, whatever polynomial it belongs to, and behind them (masks != null) the words M_k of every share, so that
+// a small refresh needs one launch.  A block for each polynomial cost 5 % on the shares of 400 parties at N = 64, and a
+// launch of its own for the masks 10 to 19 % of a small refresh.
+__global__ void __launch_bounds__(256)
+    k_sample_small(DevView v, const u32* __restrict__ recipients, const u32* __restrict__ parties, u32 n_parties,
+                   u32 ct_first, u32 n_cts, u32 unit_first, SampleKinds kinds, size_t shares, u32* __restrict__ out,
+                   u32* __restrict__ masks) {
+  __shared__ GaussFast gt;
+  for (u32 i = threadIdx.x; i < sizeof(GaussFast) / 16; i += blockDim.x)
+    reinterpret_cast<uint4*>(&gt)[i] = __ldg(reinterpret_cast<const uint4*>(v.gauss_fast) + i);
+  __syncthreads();
+  const size_t noise = shares * kinds.n << (v.logn - 2), total = noise + (masks ? shares << v.logn : 0);
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+    const bool mask = e >= noise;
+    const size_t poly = mask ? (e - noise) >> v.logn : e >> (v.logn - 2), share = mask ? poly : poly / kinds.n;
+    const u32 which = mask ? 3u : (u32)(poly % kinds.n);
+    const u32 tag = which == 0 ? kinds.tag0 : which == 1 ? kinds.tag1 : which == 2 ? kinds.tag2 : TAG_BOOT_MASK;
+    const u32 unit = unit_first + (u32)(recipients ? share / n_parties : share);
+    const u32 party = recipients ? parties[share % n_parties] : parties[unit / n_cts];
+    const u32 recipient = recipients ? recipients[unit / n_cts] : 0u;
+    if (!D2MHE_CHK(v.chk, party, v.K, SITE_PARTY) || !D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) continue;
+    const Stream st(v.seed, tag, ct_first + unit % n_cts, party, recipient);
+    if (mask) {
+      const u32 t = (u32)v.round.t;
+      masks[e - noise] = (u32)uniform_mod(st, (u32)(e - noise) & (v.n - 1), t, 0xffffffffu >> __clz(t));
+      continue;
+    }
+    const u32 j0 = 4 * ((u32)e & ((v.n >> 2) - 1));
+    u32 pack = 0;
+#pragma unroll
+    for (u32 b = 0; b < 4; ++b) {
+      int x;
+      if (tag == TAG_ENC_U) {
+        x = st.ternary(j0 + b);
+      } else {
+        const u64 r = st.draw64(j0 + b);
+        const u32 cnt = gt.lut[r >> 52];
+        x = (int)(cnt & 0x80u ? gauss_count(gt, (u32)(r >> 32), (u32)r, cnt) : cnt) - D2MHE_GAUSS_B;
+      }
+      pack |= ((u32)x & 0xffu) << (8 * b);
+    }
+    out[e] = pack;
+  }
+}
+
 // M_k uniform mod t by rejection on bitlen(t)-bit draws, N words per share.  Half of the draws are rejected for
 // t = 65537, so what counts is that no lane waits for another's redraw: a warp draws once for each of its coefficients,
 // packs the numbers of the rejected ones into a list in shared memory and goes over the list again, 32 at a time, until
@@ -144,7 +190,7 @@ __global__ void __launch_bounds__(256)
 
 namespace D2MHE_LAUNCH_NS {
 
-cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
+static cudaError_t sample_masks(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
                          u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, u32* out) {
   const u32 per = std::min(v.n, MASKS_PER_WARP), warps = std::min(v.n / per, 4u), segs = v.n / (per * warps);
   k_sample_masks<<<n_units * n_parties * segs, 32 * warps, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first,
@@ -160,10 +206,41 @@ cudaError_t sample_alpha(const DevView& v, cudaStream_t s, const u32* recipients
   return cudaGetLastError();
 }
 
+static cudaError_t sample_small(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
+                                u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds,
+                                void* out, u32* masks) {
+  const size_t shares = (size_t)n_units * (recipients_dev ? n_parties : 1u);
+  const size_t blocks = (shares * (kinds.n * (v.n >> 2) + (masks ? v.n : 0)) + 255) / 256;
+  const unsigned grid = (unsigned)std::min(blocks, std::max((size_t)8 * v.sms, blocks / 8));  // the table once per 8 words
+  k_sample_small<<<grid, 256, 0, s>>>(v, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, kinds, shares,
+                                      reinterpret_cast<u32*>(out), masks);
+  return cudaGetLastError();
+}
+
+// e_0, e_1 and M_k of a refresh, for the modular kernels in one launch unless there are enough masks (2^20) for the lists
+// of k_sample_masks to pay for theirs, and lists of 256 and more.  (N = 1024, ten parties: 40 indices, 4 M masks, one launch
+// 546 us, two 511; 4 parties, two indices 73 / 83 us; N = 64, 400 parties: 3.47 / 3.59 ms.)
+cudaError_t sample_boot(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, u32 n_parties,
+                        u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, bool fft_order, void* noise, u32* masks,
+                        u32* launches) {
+  if (v.n < 256 || (!fft_order && ((size_t)n_units * n_parties << v.logn) <= (size_t)1 << 20)) {
+    *launches += 1;
+    return sample_small(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, n_units, kSampleBoot, noise,
+                        masks);
+  }
+  *launches += 2;
+  const cudaError_t e = sample_masks(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, n_units, masks);
+  if (e != cudaSuccess) return e;
+  return sample_streams(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, n_units, kSampleBoot,
+                        fft_order, noise);
+}
+
 cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev,
                            u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds,
                            bool fft_order, void* out) {
-  const u32 words = v.n >> 2, threads = std::max(32u, std::min(words, 256u));
+  if (v.n < 256)
+    return sample_small(v, s, recipients_dev, parties_dev, n_parties, ct_first, n_cts, unit_first, n_units, kinds, out, nullptr);
+  const u32 words = v.n >> 2, threads = std::min(words, 256u);
   const size_t polys = (size_t)n_units * (recipients_dev ? n_parties : 1u) * kinds.n;
   // Eight words per thread, so that the table is fetched once for 8192 samples (2 % over two words on the share call);
   // when that does not fill the GPU (eight blocks per SM), down to one word per thread.

@@ -1393,6 +1393,39 @@ def test_neighbour_sums_with_repeated_empty_and_long_lists(d2, log2_n, bits, n_r
     ctx.close()
 
 
+@pytest.mark.parametrize("log2_n,bits,L,K,C", [(3, 30, 2, 5, 3), (7, 54, 1, 3, 41), (8, 60, 2, 3, 2), (10, 54, 1, 2, 3), (11, 54, 2, 3, 1)])
+def test_samples_on_both_sides_of_the_small_ring_kernel(d2, log2_n, bits, L, K, C):
+    """Ciphertexts and the shares of all three kinds on rings whose polynomials share a sampling block and on the first that
+    have blocks of their own."""
+    moduli = wl.ntt_primes(bits, max(16, 2 << log2_n), L)
+    n, parties = 1 << log2_n, list(range(K))
+    ctx = d2.Context(log2_n, moduli, K, seed=85)
+    o = make_oracle(log2_n, moduli, seed=85)
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    pk = o.collective_pk(parties)
+    ctx.user_keygen(parties)
+    pk_users = np.stack([o.user_pk(i) for i in parties])
+    rng = np.random.default_rng(log2_n)
+    plain = rng.integers(0, T, (K, C, n)).astype(np.uint32)
+    ct = ctx.empty_u64(K, C, 2, L, n)
+    ctx.encrypt(parties, 7, C, d2.from_u32_numpy(plain, ctx.device), ct)
+    ctx.sync()
+    want = o.encrypt(pk, parties, 7, plain)
+    assert np.array_equal(d2.to_u64_numpy(ct), want)
+    one, two = ctx.empty_u64(K, K, C, L, n), ctx.empty_u64(K, K, C, 2, L, n)
+    ctx.partial_decrypt(ct, parties, parties, 7, C, one)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(one), o.partial_decrypt(want, parties, parties, 7))
+    ctx.convert_share(ct, parties, parties, 7, C, two)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(two), o.convert_share(want, pk_users, parties, parties, 7))
+    ctx.bootstrap_share(ct, parties, parties, 7, C, two)
+    ctx.sync()
+    assert np.array_equal(d2.to_u64_numpy(two), o.boot_share(want, parties, parties, 7))
+    ctx.close()
+
+
 @pytest.mark.parametrize("bits,L,K", [(54, 2, 101), (54, 1, 130), (60, 2, 121), (30, 3, 119), (30, 2, 311)])
 def test_combination_of_many_shares(d2, bits, L, K):
     """More shares than a plain sum may have, all residues at their largest in one half of the coefficients."""

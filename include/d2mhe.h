@@ -159,7 +159,9 @@ d2mhe_status d2mhe_aggregate(d2mhe_ctx* ctx, const uint64_t* ct_dev, uint32_t n_
  * fit, rounded down to whole waves of thread blocks), so the call is one or more groups of launches
  * on the context's stream.
  * D2MHE_ERR_UNSUPPORTED if n_parties * N exceeds that buffer (d2mhe_convert_share and
- * d2mhe_bootstrap_share work the same way with 3 and 6 bytes per share coefficient).
+ * d2mhe_bootstrap_share work the same way with 3 and 6 bytes per share coefficient; where the products
+ * run in double precision and the buffer has room, Conversion uses 11 bytes per share coefficient and the
+ * refresh 6 and 8 L for each coefficient of a recipient's ciphertext).
  */
 d2mhe_status d2mhe_partial_decrypt(d2mhe_ctx* ctx, const uint64_t* agg_dev,
                                    const uint32_t* recipients, uint32_t n_rec,

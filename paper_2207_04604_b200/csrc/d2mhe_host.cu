@@ -560,13 +560,16 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
     if (err != cudaSuccess) return fail_cuda(c, err);
   }
   {
-    // two waves of thread blocks = 2 * resident / L (recipient, ciphertext) units of K shares each
+    // two waves of thread blocks = 2 * resident / L (recipient, ciphertext) units of K shares each, for the refresh: 6 N bytes
+    // a share and in double precision alpha, 8 N L a unit.  Conversion in double precision takes 11 N a share and fits
+    // fewer units; a buffer for two waves of its own was slower, its samples no longer fitting L2 (20 parties at N = 16384,
+    // L = 8, 40 units: 111 MB, one wave at a time 2699 us; 133 MB, two waves 2742 us).
     int sms = 0;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (err != cudaSuccess) return fail_cuda(c, err);
     const size_t per_sm = logn == 11 || logn == 12 ? 4 : logn == 13 ? 2 : 1;  // resident blocks of the transform kernels
     const size_t units = (2 * (size_t)sms * per_sm + L - 1) / L;
-    const size_t want = units * (P.num_parties * 6 + (c->view.fft_on ? 8 * L : 0)) * n;  // alpha of the refresh: 8 N L bytes a unit
+    const size_t want = units * (P.num_parties * 6 + (c->view.fft_on ? 8 * L : 0)) * n;
     c->noise_scratch_bytes = std::min(kNoiseScratchMaxBytes, std::max(kNoiseScratchBytes, (want + 255) / 256 * 256));
   }
   c->noise_scratch = dev_alloc<unsigned char>(c, c->noise_scratch_bytes, &err);

@@ -99,8 +99,8 @@ static const SampleKinds kSampleConvert = {3, TAG_CONV_MU, TAG_CONV_E0, TAG_CONV
 
 static const size_t kIdxSlotWords = (size_t)1 << 21;  // u32 words per staging slot (8 MiB)
 static const int kIdxSlots = 4;
-// Sample scratch of a context (for the single calls): 64 MiB, or what two waves of thread blocks of
-// the share kernel with the largest samples (MBFV.Bootstrap: 6 N bytes per share) need, up to 512 MiB.
+// Sample scratch of a context (for the single calls): 64 MiB, or what two waves of thread blocks of the share kernel with
+// the largest samples need (build_tables), up to 512 MiB.
 static const size_t kNoiseScratchBytes = (size_t)64 << 20;
 static const size_t kNoiseScratchMaxBytes = (size_t)512 << 20;
 #ifndef D2MHE_ROUND_LANES

@@ -919,19 +919,43 @@ def test_sample_batches_of_one_call_reproduce_separate_calls(d2):
     ctx.encrypt(parties, 7, C, plain, whole)
     shares = ctx.empty_u64(K, K, C, 1, n)
     ctx.partial_decrypt(whole, parties, parties, 7, C, shares)
-    # Batches are cut to whole waves of thread blocks (592 resident blocks of this kernel on a 148-SM
-    # device, one block per unit here).  The slices straddle the ends of the first batches under that
-    # rule and the ones a cut at the scratch size would give.
-    wave = 592
-    edges = {cap_enc // wave * wave, cap_enc, cap_sh // wave * wave, cap_sh}
-    firsts = sorted({0, C - 3} | {max(0, min(C - 5, e % C - 2)) for e in edges})
-    for first, cnt in [(f, 3 if f in (0, C - 3) else 5) for f in firsts]:
+    # every unit against calls that each fit one batch (11 N bytes a unit where the products run in double precision) and
+    # whose ends fall elsewhere
+    step = scratch // (11 * n) // K - 7
+    for first in range(0, C, step):
+        cnt = min(step, C - first)
         part = ctx.empty_u64(K, cnt, 2, 1, n)
         ctx.encrypt(parties, 7 + first, cnt, plain[:, first:first + cnt].contiguous(), part)
         assert torch.equal(part, whole[:, first:first + cnt])
         sh = ctx.empty_u64(K, K, cnt, 1, n)
         ctx.partial_decrypt(part, parties, parties, 7 + first, cnt, sh)
         assert torch.equal(sh, shares[:, :, first:first + cnt])
+    ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,K", [(12, 54, 1, 4), (14, 54, 2, 3), (11, 54, 1, 6), (13, 60, 1, 3)])
+def test_conversion_and_refresh_batches_reproduce_separate_calls(d2, log2_n, bits, L, K):
+    """Conversion and refresh shares of more units than the sample scratch holds, the last batch a ragged one, against calls
+    that each fit one batch; in double precision, where the scratch also holds transforms or alpha, and modular."""
+    moduli, n, parties, rec = wl.ntt_primes(bits, 2 << log2_n, L), 1 << log2_n, list(range(K)), [0, K - 1]
+    double = bits == 54 and log2_n > 11
+    ctx = d2.Context(log2_n, moduli, K, seed=12)
+    ctx.keygen_share(parties)
+    ctx.user_keygen(parties)
+    gen = torch.Generator(device=ctx.device).manual_seed(4)
+    scratch = ctx.sample_scratch_bytes()
+    for call, unit in ((ctx.convert_share, (11 if double else 3) * K * n), (ctx.bootstrap_share, (6 * K + (8 * L if double else 0)) * n)):
+        fit = scratch // unit  # units in one batch
+        C, step = fit * 13 // 20 | 1, fit // 2 - 3
+        agg = torch.randint(0, min(moduli), (2, C, 2, L, n), dtype=torch.int64, device=ctx.device, generator=gen)
+        whole = ctx.empty_u64(2, K, C, 2, L, n)
+        call(agg, rec, parties, 5, C, whole)
+        for first in range(0, C, step):
+            cnt = min(step, C - first)
+            part = ctx.empty_u64(2, K, cnt, 2, L, n)
+            call(agg[:, first:first + cnt].contiguous(), rec, parties, 5 + first, cnt, part)
+            assert torch.equal(part, whole[:, :, first:first + cnt])
+    ctx.sync()
     ctx.close()
 
 
@@ -1098,11 +1122,9 @@ def test_32_bit_calls_in_several_batches_reproduce_separate_calls(d2):
     ctx.encrypt32(parties, 3, C, plain, whole)
     shares = ctx.empty_u32(K, K, C, 1, n)
     ctx.partial_decrypt32(whole, parties, parties, 3, C, shares)
-    wave = 592  # resident thread blocks of this kernel on a 148-SM device; one block per pair of units
-    edges = {2 * (cap_enc // 2 // wave * wave), cap_enc, 2 * (cap_sh // 2 // wave * wave), cap_sh}
-    firsts = sorted({0, C - 3} | {max(0, min(C - 5, e % C - 2)) for e in edges})
-    for first in firsts:
-        cnt = 3 if first in (0, C - 3) else 5
+    step = scratch // (11 * n) // K - 8  # calls that each fit one batch
+    for first in range(0, C, step):
+        cnt = min(step, C - first)
         part = ctx.empty_u32(K, cnt, 2, 1, n)
         ctx.encrypt32(parties, 3 + first, cnt, plain[:, first:first + cnt].contiguous(), part)
         assert torch.equal(part, whole[:, first:first + cnt])

@@ -202,9 +202,9 @@ __global__ void __launch_bounds__(32 * D2MHE_MAX_LIMBS)
   const W* c0 = agg + (size_t)unit * 2 * poly;
   const W* sh = shares + ((size_t)irec * n_shares * n_cts + cl) * share_comps * poly;
   const size_t kstride = (size_t)n_cts * share_comps * poly;
-  // primes below 2^56: plain 64-bit sums of a hundred shares cannot overflow and the multiplication by the CRT factor
-  // reduces any 64-bit value
-  const bool lazy = v.wide != 0 || sizeof(W) == 4;
+  // primes below 2^56 and fewer than 120 shares: the plain 64-bit sum cannot overflow and the multiplication by the
+  // CRT factor reduces any 64-bit value, so the loads are all independent
+  const bool lazy = (v.wide != 0 || sizeof(W) == 4) && n_shares < 120;
   if (jj < v.n && D2MHE_CHK(v.chk, wl, L, SITE_LIMB)) {
     const LimbTab* lt = v.limbs + wl;
     const u64 p = lt->p, w = lt->crt, ws = lt->crt_sh, fr = lt->frac;
@@ -213,24 +213,24 @@ __global__ void __launch_bounds__(32 * D2MHE_MAX_LIMBS)
     const P2 c = __ldg(reinterpret_cast<const P2*>(c0 + at));
     u64 a0 = c.x, a1 = c.y;
     const W* s = sh + at;
-    // Ten shares at a time, predicated, so that the loads of a remainder are in flight together too (from 120 shares on four
-    // at a time, one reduction each: 130 recipients of 130 shares at N = 2048, L = 2 104 us, 91 us like this).
-    for (u32 k0 = 0; k0 < n_shares; k0 += 10) {
-      P2 h[10];
+    // Ten shares at a time, predicated, so that the loads of a remainder are in flight together too.  (Four at a time from 120
+    // shares on: 130 recipients of 130 shares at N = 2048, L = 2 100 us, 92 us like this.)
+    auto add = [&](auto sum) {
+      for (u32 k0 = 0; k0 < n_shares; k0 += 10) {
+        P2 h[10];
 #pragma unroll
-      for (u32 k = 0; k < 10; ++k) {
-        h[k].x = 0, h[k].y = 0;
-        if (k0 + k < n_shares) h[k] = __ldg(reinterpret_cast<const P2*>(s + (k0 + k) * kstride));
+        for (u32 k = 0; k < 10; ++k) {
+          h[k].x = 0, h[k].y = 0;
+          if (k0 + k < n_shares) h[k] = __ldg(reinterpret_cast<const P2*>(s + (k0 + k) * kstride));
+        }
+#pragma unroll
+        for (u32 k = 0; k < 10; ++k) a0 = sum(a0, h[k].x), a1 = sum(a1, h[k].y);
       }
-      if (lazy) {
-#pragma unroll
-        for (u32 k = 0; k < 10; ++k) a0 += h[k].x, a1 += h[k].y;
-        if (k0 % 100 == 90) a0 = shoup_full(a0, 1, lt->one_sh, p), a1 = shoup_full(a1, 1, lt->one_sh, p);
-      } else {
-#pragma unroll
-        for (u32 k = 0; k < 10; ++k) a0 = addmod(a0, h[k].x, p), a1 = addmod(a1, h[k].y, p);
-      }
-    }
+    };
+    if (lazy)
+      add([](u64 x, u64 y) { return x + y; });
+    else
+      add([p](u64 x, u64 y) { return addmod(x, y, p); });
     terms[wl][2 * lane] = mulhi_u64(shoup_full(a0, w, ws, p) << fs, fr);
     terms[wl][2 * lane + 1] = mulhi_u64(shoup_full(a1, w, ws, p) << fs, fr);
   }

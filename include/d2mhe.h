@@ -170,7 +170,7 @@ d2mhe_status d2mhe_partial_decrypt(d2mhe_ctx* ctx, const uint64_t* agg_dev,
 
 /*
  * Combine and decrypt (Sec. 4.2 item 3: c_0 + sum_k h_k; Sec. 3.2 item 5:
- * x = [ round(t/q [.]_q) ]_t, computed exactly in RNS by a mixed-radix conversion).
+ * x = [ round(t/q [.]_q) ]_t, computed exactly in RNS).
  * n_shares must equal the size of the party set of the last d2mhe_collective_pk.
  * agg_dev: [n_rec, n_cts, 2, L, N] (only c_0 is read);
  * shares_dev: [n_rec, n_shares, n_cts, L, N];  plain_dev: out [n_rec, n_cts, N] in [0,t).

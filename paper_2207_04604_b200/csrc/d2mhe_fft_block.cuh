@@ -36,8 +36,10 @@ struct FftSmem {
   double2* other;  // of the other group (GR = 2)
   u32 *words, *bytes, *slot;
   unsigned short* nibbles;
+  u32* chk;  // device check words (read by the checked kernel build only)
   u32 tg;
-  __device__ __forceinline__ FftSmem() {
+  __device__ __forceinline__ explicit FftSmem(u32* check_words) {
+    chk = check_words;
     const u32 g = group();
     tg = G::GR > 1 ? threadIdx.x % G::TG : threadIdx.x;
     double2* base = reinterpret_cast<double2*>(smem_raw);
@@ -47,6 +49,16 @@ struct FftSmem {
     bytes = words + 2 * G::n;
     nibbles = reinterpret_cast<unsigned short*>(bytes + G::n / 2);
     slot = reinterpret_cast<u32*>(smem_raw + G::smem_bytes(STASH) - 16);
+  }
+  // element i of the exchange area behind e
+  __device__ __forceinline__ void put(double2* e, u32 i, double r, double im) const {
+    if (D2MHE_CHK(chk, (u32)(e - reinterpret_cast<double2*>(smem_raw)) + i, G::GR * G::R * G::RS, SITE_STAGED))
+      e[i] = make_double2(r, im);
+  }
+  __device__ __forceinline__ double2 get(const double2* e, u32 i) const {
+    if (!D2MHE_CHK(chk, (u32)(e - reinterpret_cast<const double2*>(smem_raw)) + i, G::GR * G::R * G::RS, SITE_STAGED))
+      return make_double2(0.0, 0.0);
+    return e[i];
   }
   __device__ __forceinline__ u32 group() const { return G::GR > 1 ? threadIdx.x / G::TG : 0u; }
   __device__ __forceinline__ void group_sync() const {
@@ -118,12 +130,12 @@ __device__ __forceinline__ void fft_swap_row(const FftSmem<LOGN, STASH>& sm, dou
   double2* e = sm.ex + (sm.tg >> 4) * G::RS;
   static_for<16>([&](auto k_) {
     constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
-    e[l16 + k * 17] = make_double2(xr[i], xi[i]);
+    sm.put(e, l16 + k * 17, xr[i], xi[i]);
   });
   __syncwarp();
   static_for<16>([&](auto k_) {
     constexpr int k = brev_c<16>(decltype(k_)::value);  // in the order in which the next pass uses them
-    const double2 t = e[l16 * 17 + k];
+    const double2 t = sm.get(e, l16 * 17 + k);
     xr[k] = t.x;
     xi[k] = t.y;
   });
@@ -135,7 +147,7 @@ __device__ __forceinline__ void fft_put_rows(const FftSmem<LOGN, STASH>& sm, con
   double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
     constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
-    e[16 * k] = make_double2(xr[i], xi[i]);
+    sm.put(e, 16 * k, xr[i], xi[i]);
   });
 }
 template <int LOGN, int STASH>
@@ -143,7 +155,7 @@ __device__ __forceinline__ void fft_get_rows(const FftSmem<LOGN, STASH>& sm, dou
   const double2* e = sm.ex + (sm.tg >> 4) * FftGeo<LOGN>::RS + (sm.tg & 15u);
   static_for<16>([&](auto k_) {
     constexpr int k = brev_c<16>(decltype(k_)::value);
-    const double2 t = e[16 * k];
+    const double2 t = sm.get(e, 16 * k);
     xr[k] = t.x;
     xi[k] = t.y;
   });
@@ -155,7 +167,7 @@ __device__ __forceinline__ void fft_put_cols(const FftSmem<LOGN, STASH>& sm, con
   for (int c = 0; c < G::COLS; ++c)
     static_for<G::R>([&](auto k_) {
       constexpr int k = decltype(k_)::value, i = brev_c<G::R>(k);
-      sm.ex[sm.tg + k * G::RS + c * G::TG] = make_double2(xr[c * G::R + i], xi[c * G::R + i]);
+      sm.put(sm.ex, sm.tg + k * G::RS + c * G::TG, xr[c * G::R + i], xi[c * G::R + i]);
     });
 }
 template <int LOGN, int STASH>
@@ -165,7 +177,7 @@ __device__ __forceinline__ void fft_get_cols(const FftSmem<LOGN, STASH>& sm, dou
   for (int c = 0; c < G::COLS; ++c)
     static_for<G::R>([&](auto k_) {
       constexpr int k = brev_c<G::R>(decltype(k_)::value);
-      const double2 t = sm.ex[sm.tg + k * G::RS + c * G::TG];
+      const double2 t = sm.get(sm.ex, sm.tg + k * G::RS + c * G::TG);
       xr[c * G::R + k] = t.x;
       xi[c * G::R + k] = t.y;
     });
@@ -182,6 +194,15 @@ __device__ __forceinline__ cpx ld_cpx(const double2* p) {
   const double2 t = __ldg(p);
   return cpx{t.x, t.y};
 }
+// entry i of a table of `limit`
+template <int LOGN, int STASH>
+__device__ __forceinline__ cpx tw_cpx(const FftSmem<LOGN, STASH>& sm, const double2* table, u32 i, u32 limit) {
+  return D2MHE_CHK(sm.chk, i, limit, SITE_TWIDDLE) ? ld_cpx(table + i) : cpx{0.0, 0.0};
+}
+template <int LOGN, int STASH>
+__device__ __forceinline__ cpx tw_here(const FftSmem<LOGN, STASH>& sm, const double2* table, u32 i, u32 limit) {
+  return D2MHE_CHK(sm.chk, i, limit, SITE_TWIDDLE) ? ld_here(table + i) : cpx{0.0, 0.0};
+}
 
 // Forward transform.  in(c, jC, h): the coefficients j and j + n as a complex number, j = r + 256 jC + h n/2 with
 // r = tg + c TG (h = 0 for one group).  Leaves Z_k, k = kC + R kB + 16 R kA, in x[brev(kA)] of thread (kC, kB) of its group.
@@ -192,7 +213,7 @@ __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, c
   const u32 g = sm.group();
   static_for<G::COLS>([&](auto c_) {
     constexpr int c = decltype(c_)::value;
-    const cpx t = ld_cpx(ft.twist + 256 * g + sm.tg + (u32)(c * G::TG));
+    const cpx t = tw_cpx(sm, ft.twist, 256 * g + sm.tg + (u32)(c * G::TG), 256 * G::GR);
     static_for<R>([&](auto j_) {
       constexpr int j = decltype(j_)::value;
       cpx z = in(c_, j_, std::integral_constant<int, 0>{});
@@ -214,14 +235,14 @@ __device__ __forceinline__ void fft_forward_at(const FftSmem<LOGN, STASH>& sm, c
   fft_get_rows<LOGN>(sm, xr, xi);
   const u32 l16 = sm.tg & 15u, row = sm.tg >> 4;
   {
-    const cpx t[2] = {ld_cpx(ft.fwd2 + row), ld_cpx(ft.fwd2 + R + row)};
+    const cpx t[2] = {tw_cpx(sm, ft.fwd2, row, R), tw_cpx(sm, ft.fwd2, R + row, 2 * R)};
     fft_eval<16, 1, 0>(xr, xi, TwDerived<16, 1>(t));
   }
   __syncwarp();  // the rows have been read by their own warp only
   fft_swap_row<LOGN>(sm, xr, xi);
   {
     const u32 k = row + (u32)R * l16;
-    const cpx t[2] = {ld_cpx(ft.fwd3 + k), ld_cpx(ft.fwd3 + 16 * R + k)};
+    const cpx t[2] = {tw_cpx(sm, ft.fwd3, k, 16 * R), tw_cpx(sm, ft.fwd3, 16 * R + k, 32 * R)};
     fft_eval<16, 1, 0>(xr, xi, TwDerived<16, 1>(t));
   }
 }
@@ -260,20 +281,21 @@ __device__ __forceinline__ void fft_loaded_to_tmem(u32 addr, const double* xr, c
 }
 
 // A stored transform (a row of n points): point kA of a thread in slot kA T + thread.
-template <int LOGN>
-__device__ __forceinline__ void fft_load(const double2* row, double* xr, double* xi) {
+template <int LOGN, int STASH>
+__device__ __forceinline__ void fft_load(const FftSmem<LOGN, STASH>& sm, const double2* row, double* xr, double* xi) {
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const cpx s = ld_here(row + threadIdx.x + k * FftGeo<LOGN>::T);
+    const cpx s = tw_here(sm, row, threadIdx.x + k * FftGeo<LOGN>::T, FftGeo<LOGN>::n);
     xr[k] = s.r;
     xi[k] = s.i;
   }
 }
-template <int LOGN>
-__device__ __forceinline__ void fft_store(double2* row, const double* xr, const double* xi, double scale) {
+template <int LOGN, int STASH>
+__device__ __forceinline__ void fft_store(const FftSmem<LOGN, STASH>& sm, double2* row, const double* xr, const double* xi) {
   static_for<16>([&](auto k_) {
     constexpr int k = decltype(k_)::value, i = brev_c<16>(k);
-    row[threadIdx.x + k * FftGeo<LOGN>::T] = make_double2(xr[i] * scale, xi[i] * scale);
+    const u32 at = threadIdx.x + k * FftGeo<LOGN>::T;
+    if (D2MHE_CHK(sm.chk, at, FftGeo<LOGN>::n, SITE_STORE)) row[at] = make_double2(xr[i], xi[i]);
   });
 }
 
@@ -292,21 +314,21 @@ __device__ __forceinline__ void fft_product_tmem(u32 addr, double* xr, double* x
 }
 
 // The same with a stored transform instead of the one in tensor memory.
-template <int LOGN>
-__device__ __forceinline__ void fft_product_row(const double2* row, double* xr, double* xi) {
+template <int LOGN, int STASH>
+__device__ __forceinline__ void fft_product_row(const FftSmem<LOGN, STASH>& sm, const double2* row, double* xr, double* xi) {
   static_for<4>([&](auto q_) {
     constexpr int q = decltype(q_)::value;
     cpx c[4];
     static_for<4>([&](auto i_) {
-      c[i_.value] = ld_cpx(row + threadIdx.x + (q + 4 * brev_c<4>(decltype(i_)::value)) * FftGeo<LOGN>::T);
+      c[i_.value] = tw_cpx(sm, row, threadIdx.x + (q + 4 * brev_c<4>(decltype(i_)::value)) * FftGeo<LOGN>::T, FftGeo<LOGN>::n);
     });
     fft_product4<-1>(xr, xi, q, c);
   });
 }
 // Sums of two products: registers by tensor memory, and two stored transforms.
-template <int LOGN>
-__device__ __forceinline__ void fft_product_sum(u32 addr, const double2* row_a, const double2* row_b, double* xr,
-                                                double* xi) {
+template <int LOGN, int STASH>
+__device__ __forceinline__ void fft_product_sum(const FftSmem<LOGN, STASH>& sm, u32 addr, const double2* row_a,
+                                                const double2* row_b, double* xr, double* xi) {
   static_for<4>([&](auto q_) {
     constexpr int q = decltype(q_)::value;
     TmemQuad quad;
@@ -314,8 +336,8 @@ __device__ __forceinline__ void fft_product_sum(u32 addr, const double2* row_a, 
     cpx a[4], b[4], c[4];
     static_for<4>([&](auto i_) {
       constexpr int k = q + 4 * brev_c<4>(decltype(i_)::value);
-      a[i_.value] = ld_cpx(row_a + threadIdx.x + k * FftGeo<LOGN>::T);
-      b[i_.value] = ld_cpx(row_b + threadIdx.x + k * FftGeo<LOGN>::T);
+      a[i_.value] = tw_cpx(sm, row_a, threadIdx.x + k * FftGeo<LOGN>::T, FftGeo<LOGN>::n);
+      b[i_.value] = tw_cpx(sm, row_b, threadIdx.x + k * FftGeo<LOGN>::T, FftGeo<LOGN>::n);
     });
     tmem_wait();
     quad.get(c);
@@ -330,7 +352,7 @@ template <int LOGN, int STASH, class Hook>
 __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi,
                                             cpx (&tw)[FftGeo<LOGN>::COLS], Hook before_last) {
   using G = FftGeo<LOGN>;
-  const cpx t2[2] = {ld_here(ft.inv2 + (sm.tg & 15u)), ld_here(ft.inv2 + 16 + (sm.tg & 15u))};
+  const cpx t2[2] = {tw_here(sm, ft.inv2, sm.tg & 15u, 16), tw_here(sm, ft.inv2, 16 + (sm.tg & 15u), 32)};
   fft_eval<16, -1, 2>(xr, xi, TwNone());
   __syncthreads();  // previous users of ex are done
   fft_swap_row<LOGN>(sm, xr, xi);
@@ -338,11 +360,11 @@ __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, cons
 #pragma unroll
   for (int c = 0; c < G::COLS; ++c)
 #pragma unroll
-    for (int i = 0; i < 2; ++i) t[c][i] = ld_here(ft.inv3 + 256 * i + sm.tg + c * G::TG);
+    for (int i = 0; i < 2; ++i) t[c][i] = tw_here(sm, ft.inv3, 256 * i + sm.tg + c * G::TG, 256 * (i + 1));
   fft_eval<16, -1, 0>(xr, xi, TwDerived<16, -1>(t2));
   fft_put_rows<LOGN>(sm, xr, xi);
 #pragma unroll
-  for (int c = 0; c < G::COLS; ++c) tw[c] = ld_here(ft.twist + 256 * sm.group() + sm.tg + c * G::TG);
+  for (int c = 0; c < G::COLS; ++c) tw[c] = tw_here(sm, ft.twist, 256 * sm.group() + sm.tg + c * G::TG, 256 * G::GR);
   sm.group_sync();
   fft_get_cols<LOGN>(sm, xr, xi);
   before_last();
@@ -390,14 +412,14 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     });
     static_for<8>([&](auto j_) {
       constexpr int j = decltype(j_)::value, lo = brev_c<16>(j), hi = brev_c<16>(j + 8);
-      sm.ex[sm.tg + j * G::RS] = g ? make_double2(xr[lo], xi[lo]) : make_double2(xr[hi], xi[hi]);
+      sm.put(sm.ex, sm.tg + j * G::RS, g ? xr[lo] : xr[hi], g ? xi[lo] : xi[hi]);
       if (g) xr[lo] = xr[hi], xi[lo] = xi[hi];
     });
     __syncthreads();
     const double s = g ? -root_c<16>() : root_c<16>();
     static_for<8>([&](auto j_) {
       constexpr int j = decltype(j_)::value, lo = brev_c<16>(j), hi = brev_c<16>(j + 8);
-      const double2 o = sm.other[sm.tg + j * G::RS];
+      const double2 o = sm.get(sm.other, sm.tg + j * G::RS);
       const double dr = xr[lo] - o.x, di = xi[lo] - o.y;  // group 1: the negative, undone by s
       u64 v[4];
       v[0] = (u64)__double_as_longlong((xr[lo] + o.x) + magic);
@@ -446,7 +468,8 @@ __device__ __forceinline__ u32 lo_nibbles(u64 a, u64 b, u64 c, u64 d) {  // low 
 template <int LOGN>
 struct FftNoise {
   u32 w[8];
-  __device__ __forceinline__ void load(const uint4* poly) {
+  __device__ __forceinline__ void load(const uint4* poly, u32* chk) {
+    if (!D2MHE_CHK(chk, 16 * (threadIdx.x + FftGeo<LOGN>::T) + 15, 2 * FftGeo<LOGN>::n, SITE_LOAD)) return;
     // volatile: a plain load is moved down to its first use, and its latency costs 7-12 % of the share kernel
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
                  : "l"(poly + threadIdx.x));
@@ -500,6 +523,7 @@ __device__ __forceinline__ void fft_finish(const FftSmem<LOGN, STASH>& sm, const
     u32* w = sm.words + threadIdx.x + 4 * m * G::T;
     u32* wb = sm.bytes + threadIdx.x + m * G::T;
     unsigned short* wn = sm.nibbles + threadIdx.x + m * G::T;
+    if (!D2MHE_CHK(sm.chk, threadIdx.x + (4 * m + 3) * G::T, 2 * G::n, SITE_STAGED)) return;
     if (high) {
       const u32 bytes = *wb, nibbles = STASH == 2 ? *wn : 0u;
       static_for<4>([&](auto q_) {

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p;
-  const FftSmem<LOGN, 0> sm;
+  const FftSmem<LOGN, 0> sm(v.chk);
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     u32* out = shares + (((size_t)irec * n_parties + a) * n_cts + cl) * poly + row;
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
-    fft_load<LOGN>(key, xr, xi);
+    fft_load(sm, key, xr, xi);
     fft_product_tmem(tm, xr, xi);
-    fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] { nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16); });
+    fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] { nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16, v.chk); });
     fft_finish32<LOGN>(sm, lt, tw, xr, xi, nz, [&](u32 j, u32 x) {
       if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, csub32(csub32(x, p), p));
     });
@@ -99,12 +99,12 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p, delta = (u32)lt.delta, delta_sh = (u32)(lt.delta_sh >> 32);
-  const FftSmem<LOGN, 0> sm;
+  const FftSmem<LOGN, 0> sm(v.chk);
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
   double xr[16], xi[16];
-  fft_load<LOGN>(u_fft + (size_t)ulocal * n, xr, xi);
+  fft_load(sm, u_fft + (size_t)ulocal * n, xr, xi);
   fft_loaded_to_tmem(tm, xr, xi);
   tmem_store_done();
   const u32* m = plain + (size_t)unit * v.n;
@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     u32* out = ct + (((size_t)unit * 2 + comp) * v.L + l) * v.n;
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
-    fft_load<LOGN>(v.pk_fft + ((size_t)comp * v.L + l) * n, xr, xi);
+    fft_load(sm, v.pk_fft + ((size_t)comp * v.L + l) * n, xr, xi);
     fft_product_tmem(tm, xr, xi);
-    fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] { nz.load(noise + (((size_t)ulocal * 3 + 1 + comp) * v.n) / 16); });
+    fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] { nz.load(noise + (((size_t)ulocal * 3 + 1 + comp) * v.n) / 16, v.chk); });
     fft_finish32<LOGN>(sm, lt, tw, xr, xi, nz, [&](u32 j, u32 x) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;
       x = csub32(csub32(x, p), p);

@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN> sm;
+  const FftSmem<LOGN> sm(v.chk);
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
@@ -55,10 +55,10 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     const u32* mask = masks + share * v.n;
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
-    fft_load<LOGN>(key, xr, xi);
+    fft_load(sm, key, xr, xi);
     fft_product_tmem(tm + (high ? G::WORDS : 0), xr, xi);
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
-      if (high) nz.load(noise + ((share * 2 + comp) * v.n) / 16);
+      if (high) nz.load(noise + ((share * 2 + comp) * v.n) / 16, v.chk);
     });
     fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;

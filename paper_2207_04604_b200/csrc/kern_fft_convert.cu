@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   u32 recipient = recipients[irec];
   if (!D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) recipient = 0;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN, 2> sm;
+  const FftSmem<LOGN, 2> sm(v.chk);
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
@@ -55,14 +55,14 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
     if (comp == 0) {
-      fft_load<LOGN>(v.s_fft + (size_t)party * n, xr, xi);
-      fft_product_sum<LOGN>(tm + (high ? G::WORDS : 0), mu_fft + share * n, key, xr, xi);
+      fft_load(sm, v.s_fft + (size_t)party * n, xr, xi);
+      fft_product_sum(sm, tm + (high ? G::WORDS : 0), mu_fft + share * n, key, xr, xi);
     } else {
-      fft_load<LOGN>(mu_fft + share * n, xr, xi);
-      fft_product_row<LOGN>(key, xr, xi);
+      fft_load(sm, mu_fft + share * n, xr, xi);
+      fft_product_row(sm, key, xr, xi);
     }
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
-      if (high) nz.load(noise + ((share * 3 + 1 + comp) * v.n) / 16);
+      if (high) nz.load(noise + ((share * 3 + 1 + comp) * v.n) / 16, v.chk);
     });
     fft_finish<LOGN>(sm, lt, lt.fftc, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));

@@ -18,12 +18,12 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 part = blockIdx.x % split, rest = blockIdx.x / split;
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN> sm;
+  const FftSmem<LOGN> sm(v.chk);
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
   double xr[16], xi[16];
-  fft_load<LOGN>(u_fft + (size_t)ulocal * n, xr, xi);
+  fft_load(sm, u_fft + (size_t)ulocal * n, xr, xi);
   fft_loaded_to_tmem(tm, xr, xi);
   tmem_store_done();
   const u32* m = plain + (size_t)unit * v.n;
@@ -35,10 +35,10 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     u64* out = ct + (((size_t)unit * 2 + comp) * v.L + l) * v.n;
     FftNoise<LOGN> nz;
     cpx tw[G::COLS];
-    fft_load<LOGN>(v.pk_fft + (((size_t)comp * v.L + l) * 2 + (high ? 1 : 0)) * n, xr, xi);
+    fft_load(sm, v.pk_fft + (((size_t)comp * v.L + l) * 2 + (high ? 1 : 0)) * n, xr, xi);
     fft_product_tmem(tm, xr, xi);
     fft_inverse<LOGN>(sm, v.fft, xr, xi, tw, [&] {
-      if (high) nz.load(noise + (((size_t)ulocal * 3 + 1 + comp) * v.n) / 16);
+      if (high) nz.load(noise + (((size_t)ulocal * 3 + 1 + comp) * v.n) / 16, v.chk);
     });
     fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;

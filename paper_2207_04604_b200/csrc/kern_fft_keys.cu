@@ -48,7 +48,9 @@ __device__ __forceinline__ void fft_key(const DevView& v, u32 group, double2* __
   for (u32 i = threadIdx.x; i < m; i += KEY_THREADS) {  // point kA of thread (kC, kB)
     const u32 kA = i / G::TG, t = i % G::TG, k = (t >> 4) + (u32)G::R * ((t & 15u) + 16u * kA);
     const u32 at = __brev(k) >> (32 - LM);
-    row[kA * G::T + group * G::TG + t] = make_double2(re[at].h * scale, im[at].h * scale);
+    const u32 slot = kA * G::T + group * G::TG + t;
+    if (!D2MHE_CHK(v.chk, at, m, SITE_STAGED) || !D2MHE_CHK(v.chk, slot, G::n, SITE_STORE)) continue;
+    row[slot] = make_double2(re[at].h * scale, im[at].h * scale);
   }
 }
 
@@ -69,7 +71,7 @@ template <int LOGN>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_fft_samples(DevView v, const uint4* __restrict__ src, u32 stride, double2* __restrict__ dst) {
   using G = FftGeo<LOGN>;
-  const FftSmem<LOGN> sm;
+  const FftSmem<LOGN> sm(v.chk);
   const uint4* poly = src + (size_t)blockIdx.x * stride * (v.n / 16);
   // number i of thread t is coefficient fft_coef(i): a column's coefficients are this thread's, or (two groups) this
   // thread's and the one's at the same place of the other group
@@ -96,7 +98,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
       return cpx{value(i / 4, i & 3), value((i + G::R) / 4, i & 3)};
     }
   });
-  fft_store<LOGN>(dst + (size_t)blockIdx.x * G::n, xr, xi, 1.0);
+  fft_store(sm, dst + (size_t)blockIdx.x * G::n, xr, xi);
 }
 
 // Residue rows, limb r mod L of row r: both parts (PARTS = 2), or whole rows below 2^30 (PARTS = 1).

@@ -1164,9 +1164,10 @@ def test_32_bit_protocol_calls_refuse_wide_primes(d2):
 
 
 def test_checked_build_gives_the_same_messages_and_reports_nothing(d2):
-    """Every kernel of the checked build (index tests on coefficient, octet, shared-memory, twiddle and
+    """The checked build (index tests on coefficient, octet, shared-memory, twiddle and
     party indices) on a small ring, on configuration 1, on the conversion and refresh calls and on the
-    stand-alone transforms: the same bit-exact messages, and no violation recorded."""
+    stand-alone transforms: the same bit-exact messages, and no violation recorded.  The kernels compiled for
+    other sizes follow in the next test."""
     log2_n, K = 6, 3
     moduli = small_moduli(log2_n, 54, 2)
     ctx = d2.Context(log2_n, moduli, K, seed=5, flags=d2.FLAG_DEVICE_CHECKS)
@@ -1231,6 +1232,52 @@ def test_checked_build_gives_the_same_messages_and_reports_nothing(d2):
     assert np.array_equal(d2.to_u32_numpy(d32), p32)
     narrow.sync()
     narrow.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L", [(12, 54, 2), (13, 54, 2), (14, 54, 1), (11, 54, 2), (12, 30, 3), (13, 30, 2), (14, 29, 2)])
+def test_checked_build_on_every_size_of_the_compiled_kernels(d2, log2_n, bits, L):
+    """Every call of the protocol, checked against the plain build (whose messages other tests compare with the oracle) at the
+    sizes that have kernels of their own: double-precision products of one and two groups, 32-bit words, packing, and
+    enough columns for the neighbour sums in shared memory."""
+    K, n = 3, 1 << log2_n
+    C, parties = -(-(1 << 18) // (n * L)), list(range(K))  # 2^18 columns of 16 bytes
+    moduli = wl.ntt_primes(bits, 2 << log2_n, L)
+    offsets, rows = np.array([0, 3, 3, 6], dtype=np.uint32), np.array([0, 1, 2, 2, 0, 2], dtype=np.uint32)
+    values = torch.randint(-5000, 5001, (K, C, n), dtype=torch.int32, device="cuda", generator=torch.Generator("cuda").manual_seed(6))
+    seen = []
+    for flags in (0, d2.FLAG_DEVICE_CHECKS):
+        ctx = d2.Context(log2_n, moduli, K, seed=86, flags=flags)
+        ctx.keygen_share(parties)
+        ctx.collective_pk(parties)
+        out = []
+
+        def messages(empty, encrypt, aggregate, partial_decrypt, combine):
+            plain, sums = ctx.empty_u32(K, C, n), torch.empty_like(values)
+            ct, agg, shares = empty(K, C, 2, L, n), empty(K, C, 2, L, n), empty(K, K, C, L, n)
+            ctx.encode(values, K * C, plain)
+            encrypt(parties, 2, C, plain, ct)
+            aggregate(ct, K, C, offsets, rows, agg)
+            partial_decrypt(agg, parties, parties, 2, C, shares)
+            combine(agg, shares, K, K, C, plain)
+            ctx.decode(plain, K * C, sums)
+            out.extend([ct, agg, shares, sums])
+            return agg
+
+        agg = messages(ctx.empty_u64, ctx.encrypt, ctx.aggregate, ctx.partial_decrypt, ctx.combine_decrypt)
+        if bits <= 30:
+            messages(ctx.empty_u32, ctx.encrypt32, ctx.aggregate32, ctx.partial_decrypt32, ctx.combine_decrypt32)
+        ctx.user_keygen(parties)
+        agg = agg[:, :2].contiguous()
+        two, ct, plain = [ctx.empty_u64(K, K, 2, 2, L, n) for _ in range(2)], [ctx.empty_u64(K, 2, 2, L, n) for _ in range(2)], ctx.empty_u32(2, K, 2, n)
+        ctx.convert_share(agg, parties, parties, 2, 2, two[0])
+        ctx.convert_combine(agg, two[0], K, K, 2, ct[0])
+        ctx.decrypt(parties, ct[0], 2, ctx.empty_u64(K, 2, L, n), plain[0])
+        ctx.bootstrap_share(agg, parties, parties, 2, 2, two[1])
+        ctx.bootstrap_combine(agg, two[1], parties, K, 2, 2, plain[1], ct[1])
+        ctx.sync()  # raises if an index was out of its range
+        seen.append(out + two + ct + [plain])
+        ctx.close()
+    assert all(torch.equal(a, b) for a, b in zip(*seen))
 
 
 def test_checked_build_reports_a_violation_without_losing_the_context(d2):

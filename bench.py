@@ -691,7 +691,10 @@ def run_cuda(args, cfg):
                              "share": per_call[name] / total_ms if total_ms else None,
                              "algorithmic_GB": ab[name] / 1e9, "GBps": ab[name] / 1e9 / (ms * 1e-3) if ms else None,
                              "hbm_frac": ab[name] / 1e9 / (ms * 1e-3) / peak if ms else None}
-            if name in fp64:
+            # encryption calls of up to an eighth of the resident blocks at N = 4096 take the modular kernel
+            modular = (name == "encrypt" and cfg.log2_n == 12 and K * C * serial_steps / n_chunks_total * cfg.num_limbs * 8
+                       <= 4 * torch.cuda.get_device_properties(dev).multi_processor_count)
+            if name in fp64 and not modular:
                 kernels[name]["fp64_frac"] = fp64[name] / (ms * 1e-3) / LANE_PEAK_UNIT_COUNTS if ms else None
         kernels["aggregate"]["note"] = ("algorithmic bytes count every list's read of a ciphertext; the ciphertexts were "
                                         "just written and most of those reads hit L2, so this is not a DRAM roofline fraction")

@@ -159,11 +159,10 @@ T* dev_alloc(d2mhe_ctx* c, size_t count, cudaError_t* err) {
 // device memory that is still free, so that a context of very many parties fits wherever it would fit without them and
 // leaves its caller the memory for the messages.
 template <class T>
-T* dev_spare(d2mhe_ctx* c, size_t count) {
-  size_t free_bytes = 0, total = 0;
-  cudaError_t e = cudaMemGetInfo(&free_bytes, &total);
-  T* d = nullptr;
-  if (e == cudaSuccess && count * sizeof(T) <= free_bytes / 16) d = dev_alloc<T>(c, count, &e);
+T* dev_spare(d2mhe_ctx* c, size_t count, size_t free_bytes) {
+  if (count * sizeof(T) > free_bytes / 16) return nullptr;
+  cudaError_t e = cudaSuccess;
+  T* d = dev_alloc<T>(c, count, &e);
   if (e != cudaSuccess) (void)cudaGetLastError();
   return e == cudaSuccess ? d : nullptr;
 }
@@ -624,13 +623,15 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
   if (err != cudaSuccess) return fail_cuda(c, err);
 
   if (c->view.fft_on || c->view.fft32_on) {
-    c->view.s_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2));
-    c->view.pk_fft = c->view.s_fft ? dev_spare<double2>(c, 4 * (size_t)L * (n / 2)) : nullptr;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) (void)cudaGetLastError();
+    c->view.s_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2), free_bytes);
+    c->view.pk_fft = c->view.s_fft ? dev_spare<double2>(c, 4 * (size_t)L * (n / 2), free_bytes) : nullptr;
     if (!c->view.pk_fft) c->view.fft_on = c->view.fft32_on = 0;
-  }
-  if (c->view.fft_on) {
-    c->view.usk_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2));
-    if (conv_ok) c->view.upk_fft = dev_spare<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2));
+    if (c->view.fft_on) {
+      c->view.usk_fft = dev_spare<double2>(c, (size_t)P.num_parties * (n / 2), free_bytes);
+      if (conv_ok) c->view.upk_fft = dev_spare<double2>(c, (size_t)P.num_parties * 4 * L * (n / 2), free_bytes);
+    }
   }
   return D2MHE_OK;
 }

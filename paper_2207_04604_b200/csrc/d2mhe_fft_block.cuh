@@ -380,6 +380,25 @@ __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN, STASH>& sm, int i) {
   if (G::R == 8) return sm.tg + 128u * (u32)(i >> 4) + 256u * (u32)(i & 15);
   return sm.tg + 256u * (u32)i;
 }
+// fft_twist's constants of two groups, by group and digit.  Selected instead, they were kept across the loop and spilled:
+// shares at N = 16384 1868 us, Conversion 4505 us, with two copies of the end of a part, 1852 and 4247 us like this.
+static __device__ __constant__ double2 c_digit[32] = {
+    {1.0, 0.0}, {0.9987954562051724, -0.049067674327418015},
+    {0.9951847266721969, -0.0980171403295606}, {0.989176509964781, -0.14673047445536175},
+    {0.9807852804032304, -0.19509032201612828}, {0.970031253194544, -0.2429801799032639},
+    {0.9569403357322088, -0.2902846772544624}, {0.9415440651830208, -0.33688985339222005},
+    {0.9238795325112867, -0.3826834323650898}, {0.9039892931234433, -0.4275550934302821},
+    {0.881921264348355, -0.47139673682599764}, {0.8577286100002721, -0.5141027441932218},
+    {0.8314696123025452, -0.5555702330196022}, {0.8032075314806449, -0.5956993044924334},
+    {0.773010453362737, -0.6343932841636455}, {0.7409511253549591, -0.6715589548470184},
+    {1.0, 0.0}, {0.989176509964781, 0.14673047445536175},
+    {0.9569403357322088, 0.2902846772544624}, {0.9039892931234433, 0.4275550934302821},
+    {0.8314696123025452, 0.5555702330196022}, {0.7409511253549591, 0.6715589548470184},
+    {0.6343932841636455, 0.773010453362737}, {0.5141027441932218, 0.8577286100002721},
+    {0.3826834323650898, 0.9238795325112867}, {0.2429801799032639, 0.970031253194544},
+    {0.0980171403295606, 0.9951847266721969}, {-0.049067674327418015, 0.9987954562051724},
+    {-0.19509032201612828, 0.9807852804032304}, {-0.33688985339222005, 0.9415440651830208},
+    {-0.47139673682599764, 0.881921264348355}, {-0.5956993044924334, 0.8032075314806449}};
 // The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
 // eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4]) with v = bits of
 // M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.
@@ -404,9 +423,12 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     // Group g finishes the digits 8 g .. 8 g + 7 and sends the others; column r of ex is this thread's own until the
     // block barrier.  z_j = y0 + y1, z_(j + 4096) = (y0 - y1) e^(-i pi / 4); the group signs make both sides equal.
     const u32 g = sm.group();
+    u32 step = g;  // not known to be the same in every transform: the constants are read where they are used
+    asm volatile("" : "+r"(step));
     static_for<16>([&](auto j_) {
       constexpr int j = decltype(j_)::value, i = brev_c<16>(j);
-      const cpx z = cmul(cpx{xr[i], xi[i]}, fft_twist<G::R, G::GR, j>(tw[0], g));
+      const double2 c = c_digit[step * 16 + j];
+      const cpx z = cmul(cpx{xr[i], xi[i]}, cmul(tw[0], cpx{c.x, c.y}));
       xr[i] = z.r;
       xi[i] = z.i;
     });
@@ -509,36 +531,55 @@ inline u32 fft_component_split(const DevView& v, u32 base, u32 ctas) {
   return (2 * base + resident - 1) / resident < 2 * ((base + resident - 1) / resident) ? 2 : 1;
 }
 
+// Nothing computed from the columns' twist before this point is kept for after it (and the other way round).
+template <int COLS>
+__device__ __forceinline__ void fft_fence(const cpx (&tw)[COLS], cpx (&out)[COLS]) {
+#pragma unroll
+  for (int c = 0; c < COLS; ++c) {
+    out[c] = tw[c];
+    asm volatile("" : "+d"(out[c].r), "+d"(out[c].i));
+  }
+}
+
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
-// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  (One copy of
-// the code for both parts: two copies share subexpressions, and 300 bytes of them were spilled.)
+// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  Each part has a
+// copy of the code of its own, so that the loads and the arithmetic of several portions overlap (with one copy and a
+// branch in every portion the end of a high part took 5.3 k clocks of a transform's 10.2 k at N = 8192; refresh shares there
+// 1789 -> 1630 us, encryption at N = 16384 459 -> 353 us); the fences keep the copies from sharing subexpressions, 300 bytes
+// of which were spilled.
 template <int LOGN, int STASH, class Noise, class Store>
 __device__ __forceinline__ void fft_finish(const FftSmem<LOGN, STASH>& sm, const LimbTab& lt, const FftSplit& sp,
                                            const cpx (&tw)[FftGeo<LOGN>::COLS], double* xr, double* xi, bool high,
                                            const Noise& nz, Store store) {
   using G = FftGeo<LOGN>;
-  const double magic = high ? sp.magic : STASH == 2 ? D2MHE_FFT_MAGIC_LO44 : D2MHE_FFT_MAGIC_LO;
-  fft_results<LOGN>(sm, tw, xr, xi, magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4]) {
-    constexpr int m = decltype(m_)::value;
-    u32* w = sm.words + threadIdx.x + 4 * m * G::T;
-    u32* wb = sm.bytes + threadIdx.x + m * G::T;
-    unsigned short* wn = sm.nibbles + threadIdx.x + m * G::T;
-    if (!D2MHE_CHK(sm.chk, threadIdx.x + (4 * m + 3) * G::T, 2 * G::n, SITE_STAGED)) return;
-    if (high) {
-      const u32 bytes = *wb, nibbles = STASH == 2 ? *wn : 0u;
+  cpx t[G::COLS];
+  if (high) {
+    fft_fence(tw, t);
+    fft_results<LOGN>(sm, t, xr, xi, sp.magic, [&](auto m_, auto i_, auto rr_, const u64(&v)[4]) {
+      constexpr int m = decltype(m_)::value;
+      const u32* w = sm.words + threadIdx.x + 4 * m * G::T;
+      if (!D2MHE_CHK(sm.chk, threadIdx.x + (4 * m + 3) * G::T, 2 * G::n, SITE_STAGED)) return;
+      const u32 bytes = sm.bytes[threadIdx.x + m * G::T], nibbles = STASH == 2 ? sm.nibbles[threadIdx.x + m * G::T] : 0u;
       static_for<4>([&](auto q_) {
         constexpr int q = decltype(q_)::value, i = fft_result_number<decltype(i_)::value, decltype(rr_)::value, q>();
         u32 top = __byte_perm(bytes, 0, 0x4440 | q);
         if (STASH == 2) top |= (q < 3 ? nibbles << (8 - 4 * (q < 3 ? q : 0)) : nibbles >> 4) & 0xf00u;
         store(fft_coef<LOGN>(sm, i), fft_sum(join64(w[q * G::T], top), v[q], nz.template get<i>(), sp, lt));
       });
-    } else {
+    });
+  } else {
+    fft_fence(tw, t);
+    fft_results<LOGN>(sm, t, xr, xi, STASH == 2 ? D2MHE_FFT_MAGIC_LO44 : D2MHE_FFT_MAGIC_LO,
+                      [&](auto m_, auto, auto, const u64(&v)[4]) {
+      constexpr int m = decltype(m_)::value;
+      u32* w = sm.words + threadIdx.x + 4 * m * G::T;
+      if (!D2MHE_CHK(sm.chk, threadIdx.x + (4 * m + 3) * G::T, 2 * G::n, SITE_STAGED)) return;
 #pragma unroll
       for (int i = 0; i < 4; ++i) w[i * G::T] = lo_word(v[i]);
-      *wb = lo_bytes(v[0], v[1], v[2], v[3]);
-      if (STASH == 2) *wn = (unsigned short)lo_nibbles(v[0], v[1], v[2], v[3]);
-    }
-  });
+      sm.bytes[threadIdx.x + m * G::T] = lo_bytes(v[0], v[1], v[2], v[3]);
+      if (STASH == 2) sm.nibbles[threadIdx.x + m * G::T] = (unsigned short)lo_nibbles(v[0], v[1], v[2], v[3]);
+    });
+  }
 }
 
 __device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer

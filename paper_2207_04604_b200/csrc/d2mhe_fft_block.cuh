@@ -20,7 +20,7 @@ struct FftGeo {
   static constexpr int RS = 271;
   static constexpr size_t ex_bytes = (size_t)GR * R * RS * 16;
   __host__ __device__ static constexpr size_t smem_bytes(int stash) {
-    return ex_bytes + (stash ? (size_t)n * (9 + stash) : 0) + 16;
+    return ex_bytes + (stash ? (size_t)n * (9 + stash) : 0) + 16;  // + the word of tcgen05.alloc, one for a wait that ran out, and the barrier
   }
   // Words of tensor memory per thread for one transform, and columns for `k` of them: warp w of a block
   // reaches the lanes 32 (w mod 4) .. + 31 only, so warps w, w + 4, .. share lanes and split the columns.
@@ -38,8 +38,10 @@ struct FftSmem {
   unsigned short* nibbles;
   u32* chk;  // device check words (read by the checked kernel build only)
   u32 tg;
-  __device__ __forceinline__ explicit FftSmem(u32* check_words) {
-    chk = check_words;
+  u32 phase = 0;         // of the barrier in the last transform
+  bool announce = true;  // false: a block barrier instead (a constant in every kernel)
+  __device__ __forceinline__ explicit FftSmem(const DevView& v) {
+    chk = v.chk;
     const u32 g = group();
     tg = G::GR > 1 ? threadIdx.x % G::TG : threadIdx.x;
     double2* base = reinterpret_cast<double2*>(smem_raw);
@@ -59,6 +61,37 @@ struct FftSmem {
     if (!D2MHE_CHK(chk, (u32)(e - reinterpret_cast<const double2*>(smem_raw)) + i, G::GR * G::R * G::RS, SITE_STAGED))
       return make_double2(0.0, 0.0);
     return e[i];
+  }
+  // The exchange area is free for the next transform when every warp has read the last one's columns.  A warp arrives
+  // when it has, and waits only when it writes there again, most of a transform later: nothing stalls where a block
+  // barrier made every warp wait for the slowest one.  Shares at N = 8192 716 -> 679 us, at N = 16384 1852 -> 1709 us,
+  // Conversion at N = 16384 4247 -> 3888 us (1480 rows of ten parties); not in the encryption kernels, whose two to four
+  // transforms a block don't repay it (N = 8192: 152 us with block barriers, 161 us).
+  __device__ __forceinline__ void init() const {  // one thread, ahead of a block barrier
+    slot[1] = 0;
+    asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(bar()), "r"(G::T / 32) : "memory");
+  }
+  __device__ __forceinline__ u32 bar() const { return (u32)__cvta_generic_to_shared(slot) + 8; }
+  __device__ __forceinline__ void finish(const DevView& v) const {  // one thread, behind the last block barrier
+    if (slot[1]) atomicOr(v.range_flag, RANGE_FLAG_WAIT);
+  }
+  __device__ __forceinline__ void release() const {
+    if (!announce) return;
+    __syncwarp();
+    if ((threadIdx.x & 31u) == 0) asm volatile("{.reg .b64 t; mbarrier.arrive.shared.b64 t, [%0];}" ::"r"(bar()) : "memory");
+  }
+  // The wait has a limit (a second or more), after which the call is reported as failed (finish).
+  __device__ __forceinline__ void acquire() {
+    if (!announce) {
+      __syncthreads();
+      return;
+    }
+    u32 done = 0;
+    for (int i = 0; !done && i < (1 << 20); ++i)
+      asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
+                   : "=r"(done) : "r"(bar()), "r"(phase ^ 1u) : "memory");
+    if (!done) slot[1] = 1;
+    phase ^= 1u;
   }
   __device__ __forceinline__ u32 group() const { return G::GR > 1 ? threadIdx.x / G::TG : 0u; }
   __device__ __forceinline__ void group_sync() const {
@@ -349,12 +382,12 @@ __device__ __forceinline__ void fft_product_sum(const FftSmem<LOGN, STASH>& sm, 
 // x[c R + brev(jC)]; tw: the columns' twist.  before_last(): called ahead of the arithmetic of pass C.
 // Table entries are fetched a pass ahead of their use (they come from L2 as often as not).
 template <int LOGN, int STASH, class Hook>
-__device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi,
+__device__ __forceinline__ void fft_inverse(FftSmem<LOGN, STASH>& sm, const FftTab& ft, double* xr, double* xi,
                                             cpx (&tw)[FftGeo<LOGN>::COLS], Hook before_last) {
   using G = FftGeo<LOGN>;
   const cpx t2[2] = {tw_here(sm, ft.inv2, sm.tg & 15u, 16), tw_here(sm, ft.inv2, 16 + (sm.tg & 15u), 32)};
   fft_eval<16, -1, 2>(xr, xi, TwNone());
-  __syncthreads();  // previous users of ex are done
+  sm.acquire();  // previous users of ex are done
   fft_swap_row<LOGN>(sm, xr, xi);
   cpx t[G::COLS][2];
 #pragma unroll
@@ -367,6 +400,7 @@ __device__ __forceinline__ void fft_inverse(const FftSmem<LOGN, STASH>& sm, cons
   for (int c = 0; c < G::COLS; ++c) tw[c] = tw_here(sm, ft.twist, 256 * sm.group() + sm.tg + c * G::TG, 256 * G::GR);
   sm.group_sync();
   fft_get_cols<LOGN>(sm, xr, xi);
+  if (G::GR == 1) sm.release();
   before_last();
 #pragma unroll
   for (int c = 0; c < G::COLS; ++c) fft_eval<G::R, -1, 0>(xr + c * G::R, xi + c * G::R, TwDerived<G::R, -1>(t[c]));
@@ -442,6 +476,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     static_for<8>([&](auto j_) {
       constexpr int j = decltype(j_)::value, lo = brev_c<16>(j), hi = brev_c<16>(j + 8);
       const double2 o = sm.get(sm.other, sm.tg + j * G::RS);
+      if constexpr (j == 7) sm.release();
       const double dr = xr[lo] - o.x, di = xi[lo] - o.y;  // group 1: the negative, undone by s
       u64 v[4];
       v[0] = (u64)__double_as_longlong((xr[lo] + o.x) + magic);

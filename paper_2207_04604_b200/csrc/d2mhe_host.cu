@@ -765,7 +765,7 @@ d2mhe_status d2mhe_sync(d2mhe_ctx* c) {
   if (flag) {
     e = cudaMemset(c->view.range_flag, 0, sizeof(u32));
     if (e != cudaSuccess) return fail_cuda(c, e);
-    return D2MHE_ERR_RANGE;
+    return flag & RANGE_FLAG_WAIT ? D2MHE_ERR_DEVICE_CHECK : D2MHE_ERR_RANGE;
   }
   return D2MHE_OK;
 }
@@ -1516,7 +1516,7 @@ static d2mhe_status round_impl(d2mhe_ctx* c, const int32_t* values, bool host_io
       return fail_cuda(c, e);
     if (flag) {
       if ((e = cudaMemset(c->view.range_flag, 0, sizeof(u32))) != cudaSuccess) return fail_cuda(c, e);
-      return D2MHE_ERR_RANGE;
+      return flag & RANGE_FLAG_WAIT ? D2MHE_ERR_DEVICE_CHECK : D2MHE_ERR_RANGE;
     }
   }
   return D2MHE_OK;

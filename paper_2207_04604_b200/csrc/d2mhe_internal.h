@@ -48,6 +48,8 @@ struct LimbParams {
   LimbTab limbs[D2MHE_MAX_LIMBS];
 };
 
+enum : u32 { RANGE_FLAG_VALUE = 1 /* a value out of range */, RANGE_FLAG_WAIT = 2 /* a wait inside a kernel ran out */ };
+
 // Everything a kernel needs, passed by value.
 struct DevView {
   const LimbTab* limbs;
@@ -79,7 +81,7 @@ struct DevView {
   double2* pk_fft;  // [2][L][2][n]  both parts of p_0, p_1, times 1/n (fft32_on: [2][L][n], whole)
   double2* usk_fft;  // [K][n]            the same of the users' own keys
   double2* upk_fft;  // [K][2][L][2][n]
-  u32* range_flag;
+  u32* range_flag;  // bits RANGE_FLAG_*, read and cleared by d2mhe_sync
   u32* chk;       // four check words {site, index, limit, block} of the checked build
 };
 

@@ -51,7 +51,8 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p;
-  const FftSmem<LOGN, 0> sm(v.chk);
+  FftSmem<LOGN, 0> sm(v);
+  if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     key = next;
   }
   __syncthreads();
+  if (tid == 0) sm.finish(v);
   if (tid < 32) tmem_free(tbase, G::tmem_cols(1));
 }
 
@@ -99,7 +101,9 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   const u32 p = (u32)lt.p, delta = (u32)lt.delta, delta_sh = (u32)(lt.delta_sh >> 32);
-  const FftSmem<LOGN, 0> sm(v.chk);
+  FftSmem<LOGN, 0> sm(v);
+  sm.announce = false;
+  if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -125,6 +129,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     });
   }
   __syncthreads();
+  if (tid == 0) sm.finish(v);
   if (tid < 32) tmem_free(tbase, G::tmem_cols(1));
 }
 

@@ -21,7 +21,8 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN> sm(v.chk);
+  FftSmem<LOGN> sm(v);
+  if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     high = !high;
   }
   __syncthreads();
+  if (tid == 0) sm.finish(v);
   if (tid < 32) tmem_free(tbase, G::tmem_cols(2));
 }
 

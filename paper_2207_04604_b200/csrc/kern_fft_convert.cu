@@ -25,7 +25,8 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   u32 recipient = recipients[irec];
   if (!D2MHE_CHK(v.chk, recipient, v.K, SITE_PARTY)) recipient = 0;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN, 2> sm(v.chk);
+  FftSmem<LOGN, 2> sm(v);
+  if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(2));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, 2 * G::WORDS);
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     if (i == 0) a += split;
   }
   __syncthreads();
+  if (tid == 0) sm.finish(v);
   if (tid < 32) tmem_free(tbase, G::tmem_cols(2));
 }
 

@@ -18,7 +18,9 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 part = blockIdx.x % split, rest = blockIdx.x / split;
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
-  const FftSmem<LOGN> sm(v.chk);
+  FftSmem<LOGN> sm(v);
+  sm.announce = false;
+  if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
@@ -47,6 +49,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     });
   }
   __syncthreads();
+  if (tid == 0) sm.finish(v);
   if (tid < 32) tmem_free(tbase, G::tmem_cols(1));
 }
 

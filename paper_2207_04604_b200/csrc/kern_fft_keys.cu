@@ -71,7 +71,7 @@ template <int LOGN>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_fft_samples(DevView v, const uint4* __restrict__ src, u32 stride, double2* __restrict__ dst) {
   using G = FftGeo<LOGN>;
-  const FftSmem<LOGN> sm(v.chk);
+  const FftSmem<LOGN> sm(v);
   const uint4* poly = src + (size_t)blockIdx.x * stride * (v.n / 16);
   // number i of thread t is coefficient fft_coef(i): a column's coefficients are this thread's, or (two groups) this
   // thread's and the one's at the same place of the other group

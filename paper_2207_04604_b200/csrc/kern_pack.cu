@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(PackGeo<LOGN>::T)
       bad |= val > (int)pt.half || val < -(int)pt.half;
     }
     if (bad) {
-      atomicOr(v.range_flag, 1u);
+      atomicOr(v.range_flag, RANGE_FLAG_VALUE);
 #pragma unroll
       for (u32 c = 0; c < 16; ++c) z[c] = (u32)((int)z[c] % (int)t);
     }

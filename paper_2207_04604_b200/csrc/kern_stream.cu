@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(1024)
     const u32 pos = __brev(j) >> (32 - logn);
     if (D2MHE_CHK(v.chk, pos, n, SITE_STAGED)) sm[pos] = (u32)r;
   }
-  if (bad) atomicOr(v.range_flag, 1u);
+  if (bad) atomicOr(v.range_flag, RANGE_FLAG_VALUE);
   __syncthreads();
   u32 lt = 0;  // log2 of the butterfly span of the next stage
   for (; lt + 1 < logn; lt += 2) {

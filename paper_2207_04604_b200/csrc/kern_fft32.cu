@@ -37,15 +37,16 @@ constexpr size_t smem32() {
 }
 
 // One thread block = one (recipient, ciphertext, limb) and its part of the parties; as k_share_fft.
-// grid = n_units * L * split
-template <int LOGN>
+// grid: fft_deal, rows = n_units * L
+template <int LOGN, bool MIXED>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_share32_fft(DevView v, const __grid_constant__ LimbParams lp, const u32* __restrict__ agg,
                   const u32* __restrict__ parties, u32 n_parties, u32 n_cts, u32 unit_first,
-                  const uint4* __restrict__ noise, u32* __restrict__ shares, u32 split) {
+                  const uint4* __restrict__ noise, u32* __restrict__ shares, FftDeal deal) {
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
-  const u32 part = blockIdx.x % split, rest = blockIdx.x / split;
+  u32 part, split;
+  const u32 rest = fft_dealt<MIXED>(deal, part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -137,11 +138,12 @@ template <int LOGN>
 cudaError_t launch_share32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, const u32* parties_dev,
                            u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u32* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_share32_fft<LOGN>, smem32<LOGN>());
+  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 1);
+  const auto kernel = deal.whole ? k_share32_fft<LOGN, true> : k_share32_fft<LOGN, false>;
+  const cudaError_t e = set_smem(kernel, smem32<LOGN>());
   if (e != cudaSuccess) return e;
-  const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 2);
-  k_share32_fft<LOGN><<<n_units * v.L * split, G::T, smem32<LOGN>(), s>>>(
-      v, lp, agg, parties_dev, n_parties, n_cts, unit_first, reinterpret_cast<const uint4*>(noise), shares, split);
+  kernel<<<deal.blocks, G::T, smem32<LOGN>(), s>>>(
+      v, lp, agg, parties_dev, n_parties, n_cts, unit_first, reinterpret_cast<const uint4*>(noise), shares, deal);
   return cudaGetLastError();
 }
 template <int LOGN>

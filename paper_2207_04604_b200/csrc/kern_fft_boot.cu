@@ -8,15 +8,16 @@ namespace {
 // One thread block = one (recipient, ciphertext, limb) and component; it walks over its part of the parties.  The
 // component's fixed factor (c_1, or -alpha) stays in tensor memory, as in the share kernel.
 // alpha: [units][L][N] residues; noise: the bytes of e_0, e_1, N each per share; masks: M_k, N words per share.
-// grid = n_units * L * 2 * split
-template <int LOGN>
+// grid: fft_deal, rows = n_units * L * 2
+template <int LOGN, bool MIXED>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_boot_fft(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ agg,
                const u32* __restrict__ parties, u32 n_parties, u32 n_cts, u32 unit_first, const u64* __restrict__ alpha,
-               const uint4* __restrict__ noise, const u32* __restrict__ masks, u64* __restrict__ shares, u32 split) {
+               const uint4* __restrict__ noise, const u32* __restrict__ masks, u64* __restrict__ shares, FftDeal deal) {
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
-  const u32 part = blockIdx.x % split, comp = (blockIdx.x / split) & 1u, rest = blockIdx.x / split / 2;
+  u32 part, split;
+  const u32 row_comp = fft_dealt<MIXED>(deal, part, split), comp = row_comp & 1u, rest = row_comp / 2;
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -80,12 +81,13 @@ cudaError_t launch_boot(const DevView& v, const LimbParams& lp, cudaStream_t s, 
                         u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const u64* alpha, const void* noise,
                         const u32* masks, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_boot_fft<LOGN>, G::smem_bytes(1));
+  const FftDeal deal = fft_deal(v, n_units * v.L * 2, G::CTAS, n_parties, 2);
+  const auto kernel = deal.whole ? k_boot_fft<LOGN, true> : k_boot_fft<LOGN, false>;
+  const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
-  const u32 split = fft_party_split(v, n_units * v.L * 2, G::CTAS, n_parties, 2);
-  k_boot_fft<LOGN><<<n_units * v.L * 2 * split, G::T, G::smem_bytes(1), s>>>(
+  kernel<<<deal.blocks, G::T, G::smem_bytes(1), s>>>(
       v, lp, agg, parties_dev, n_parties, n_cts, unit_first, alpha, reinterpret_cast<const uint4*>(noise), masks, shares,
-      split);
+      deal);
   return cudaGetLastError();
 }
 

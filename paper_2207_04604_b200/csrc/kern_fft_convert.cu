@@ -9,16 +9,17 @@ namespace {
 // One thread block = one (recipient, ciphertext, limb); it walks over its part of the parties.  The transforms of both
 // parts of c_1 stay in tensor memory; those of s_k, mu_k (made once per share by k_fft_samples) and the recipient's
 // public key come from L2: h_0 is one inverse transform per part, of the sum of two products.
-// noise: the bytes of mu, e_0, e_1, N each per share.   grid = n_units * L * split
-template <int LOGN>
+// noise: the bytes of mu, e_0, e_1, N each per share.   grid: fft_deal, rows = n_units * L
+template <int LOGN, bool MIXED>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_convert_fft(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ agg,
                   const u32* __restrict__ recipients, const u32* __restrict__ parties, u32 n_parties, u32 n_cts,
                   u32 unit_first, const double2* __restrict__ mu_fft, const uint4* __restrict__ noise,
-                  u64* __restrict__ shares, u32 split) {
+                  u64* __restrict__ shares, FftDeal deal) {
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
-  const u32 block_part = blockIdx.x % split, rest = blockIdx.x / split;
+  u32 block_part, split;
+  const u32 rest = fft_dealt<MIXED>(deal, block_part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (block_part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -81,12 +82,13 @@ cudaError_t launch_convert(const DevView& v, const LimbParams& lp, cudaStream_t 
                            const u32* recipients_dev, const u32* parties_dev, u32 n_parties, u32 n_cts, u32 unit_first,
                            u32 n_units, const double2* mu_fft, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_convert_fft<LOGN>, G::smem_bytes(2));
+  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 4);
+  const auto kernel = deal.whole ? k_convert_fft<LOGN, true> : k_convert_fft<LOGN, false>;
+  const cudaError_t e = set_smem(kernel, G::smem_bytes(2));
   if (e != cudaSuccess) return e;
-  const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 4);
-  k_convert_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes(2), s>>>(
+  kernel<<<deal.blocks, G::T, G::smem_bytes(2), s>>>(
       v, lp, agg, recipients_dev, parties_dev, n_parties, n_cts, unit_first, mu_fft,
-      reinterpret_cast<const uint4*>(noise), shares, split);
+      reinterpret_cast<const uint4*>(noise), shares, deal);
   return cudaGetLastError();
 }
 

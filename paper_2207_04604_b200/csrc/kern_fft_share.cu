@@ -14,17 +14,18 @@ namespace {
 // the end of the previous transform frees was slower: 46.8 k instead of 40.0 k clocks per share and limb at N = 16384,
 // 18.5 k instead of 17.3 k at N = 8192.)  The rounded low part waits in shared memory, thread by thread, for the high
 // part.  The shares are written with a streaming hint, so that the keys stay in L2.
-// grid = n_units * L * split; party a belongs to block a mod split of its unit.
+// grid: fft_deal, rows = n_units * L.
 // OWN: the products c_1 sk_i with user i's own key instead (parties: the users of the units' rows, one to a unit, no
 // noise), as BFV.Decrypt needs them.
-template <int LOGN, bool OWN>
+template <int LOGN, bool OWN, bool MIXED>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_share_fft(DevView v, const __grid_constant__ LimbParams lp, const u64* __restrict__ agg,
                 const u32* __restrict__ parties, u32 n_parties, u32 n_cts, u32 unit_first,
-                const uint4* __restrict__ noise, u64* __restrict__ shares, u32 split) {
+                const uint4* __restrict__ noise, u64* __restrict__ shares, FftDeal deal) {
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
-  const u32 part = blockIdx.x % split, rest = blockIdx.x / split;
+  u32 part, split;
+  const u32 rest = fft_dealt<MIXED>(deal, part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -83,11 +84,12 @@ template <int LOGN, bool OWN>
 cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
                          u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_share_fft<LOGN, OWN>, G::smem_bytes(1));
+  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 2);
+  const auto kernel = deal.whole ? k_share_fft<LOGN, OWN, true> : k_share_fft<LOGN, OWN, false>;
+  const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
-  const u32 split = fft_party_split(v, n_units * v.L, G::CTAS, n_parties, 2);
-  k_share_fft<LOGN, OWN><<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
-                                                              reinterpret_cast<const uint4*>(noise), shares, split);
+  kernel<<<deal.blocks, G::T, G::smem_bytes(1), s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
+                                                              reinterpret_cast<const uint4*>(noise), shares, deal);
   return cudaGetLastError();
 }
 

@@ -1617,3 +1617,25 @@ def test_32_bit_products_at_the_limits(d2, log2_n, bits, L, K, C):
     assert np.array_equal(d2.to_u32_numpy(shares).astype(np.uint64), o.partial_decrypt(agg, [K - 1], parties, 5))
     assert np.array_equal(d2.to_u32_numpy(ct).astype(np.uint64), o.encrypt(pk, parties, 9, plain))
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits,L,K,C", [(12, 54, 1, 7, 90), (13, 54, 1, 5, 62), (14, 54, 1, 4, 41), (14, 29, 1, 4, 41)])
+def test_shares_of_just_over_a_wave_of_blocks(d2, log2_n, bits, L, K, C):
+    """A full wave of thread blocks takes whole units, the units that are left are split over one more."""
+    n, parties = 1 << log2_n, list(range(K))
+    moduli = wl.ntt_primes(bits, 2 * n, L)
+    ctx, o = d2.Context(log2_n, moduli, K, seed=91), make_oracle(log2_n, moduli, seed=91)
+    ctx.keygen_share(parties)
+    agg = wl.random_polys(moduli, log2_n, K * C * 2, seed=5).reshape(K, C, 2, L, n)
+    want = o.partial_decrypt(agg, parties, parties, 3)
+    if bits > 30:
+        shares = ctx.empty_u64(K, K, C, L, n)
+        ctx.partial_decrypt(d2.from_u64_numpy(agg, ctx.device), parties, parties, 3, C, shares)
+        ctx.sync()
+        assert np.array_equal(d2.to_u64_numpy(shares), want)
+    else:
+        shares = ctx.empty_u32(K, K, C, L, n)
+        ctx.partial_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), parties, parties, 3, C, shares)
+        ctx.sync()
+        assert np.array_equal(d2.to_u32_numpy(shares), want.astype(np.uint32))
+    ctx.close()

@@ -150,7 +150,10 @@ __global__ void __launch_bounds__(COLS * GROUPS)
 // decides.  L + 1 products per coefficient instead of L (L + 7) / 2 and no array of digits: the kernel is left with its
 // loads.  (The digits for every coefficient, one coefficient per thread: 48 us for 70 units of 10 shares at N = 8192,
 // L = 4 and 73 us for 40 of one share at N = 16384, L = 8; 42 and 46 us now.)
-// grid = (n_rec * n_cts, N / 64), 32 L threads.
+// grid = n_rec * n_cts * N / 32 V, 32 L threads: the blocks of a unit side by side, so that the loads in flight fall into
+// long runs of a few units' rows (with the units side by side 81.7 us for 99 units of nine shares at N = 8192, L = 6, now
+// 78.0; 130 units of ten, L = 4: 76.1 and 71.6).  Words of 32 bits four at a time, 16 bytes as for 64 bits: 130 units of ten,
+// L = 7: 91.6 and 74.5 us.  That takes registers for at most 12 warps a block: two at a time beyond 12 limbs.
 // ---------------------------------------------------------------------------
 
 // mixed-radix (Garner) digits d_i of w' = t v + (q-1)/2 in [0, q);  w' mod t = sum d_i prod_{j<i} q_j mod t;
@@ -175,29 +178,38 @@ __device__ __noinline__ u32 round_exact(const DevView& v, Acc acc) {
   return (u32)shoup_full(diff * v.round.qinv_mod_t, 1, tsh, t);
 }
 
-template <class W>
-struct Pair2;
+// V residues of W as one load
+template <class W, u32 V>
+struct Residues;
 template <>
-struct Pair2<u64> {
-  typedef ulonglong2 type;
+struct Residues<u64, 2> {
+  ulonglong2 q = {0, 0};
+  __device__ __forceinline__ u64 get(u32 i) const { return i ? q.y : q.x; }
 };
 template <>
-struct Pair2<u32> {
-  typedef uint2 type;
+struct Residues<u32, 2> {
+  uint2 q = {0, 0};
+  __device__ __forceinline__ u64 get(u32 i) const { return i ? q.y : q.x; }
+};
+template <>
+struct Residues<u32, 4> {
+  uint4 q = {0, 0, 0, 0};
+  __device__ __forceinline__ u64 get(u32 i) const { return i == 0 ? q.x : i == 1 ? q.y : i == 2 ? q.z : q.w; }
 };
 
 // W = u64, or u32 for the 32-bit-word messages (same arithmetic on the loaded residues).
-// One warp per limb: a thread sums the shares of two coefficients of its limb, all of its loads independent of one
+// One warp per limb, at most LIMBS of them: a thread sums the shares of V coefficients of its limb, all of its loads independent of one
 // another, and the block adds up the limbs' terms through shared memory.  (All limbs in one thread, one after another,
 // had too few loads in flight: 59 us for the 70 units above.)
-template <class W>
-__global__ void __launch_bounds__(32 * D2MHE_MAX_LIMBS)
+template <class W, u32 V, int LIMBS>
+__global__ void __launch_bounds__(32 * LIMBS)
     k_combine(const __grid_constant__ DevView v, const W* __restrict__ agg, const W* __restrict__ shares, u32 n_shares,
               u32 share_comps, u32 n_cts, u32* __restrict__ plain) {
-  typedef typename Pair2<W>::type P2;
-  __shared__ u64 terms[D2MHE_MAX_LIMBS][64];
-  const u32 unit = blockIdx.x, irec = unit / n_cts, cl = unit % n_cts;
-  const u32 lane = threadIdx.x & 31u, wl = threadIdx.x >> 5, L = v.L, j0 = blockIdx.y * 64u, jj = j0 + 2 * lane;
+  typedef Residues<W, V> R;
+  constexpr u32 COLS = 32 * V;
+  __shared__ u64 terms[LIMBS][COLS];
+  const u32 chunks = (v.n + COLS - 1) / COLS, unit = blockIdx.x / chunks, irec = unit / n_cts, cl = unit % n_cts;
+  const u32 lane = threadIdx.x & 31u, wl = threadIdx.x >> 5, L = v.L, j0 = blockIdx.x % chunks * COLS, jj = j0 + V * lane;
   const size_t poly = (size_t)L * v.n;
   const W* c0 = agg + (size_t)unit * 2 * poly;
   const W* sh = shares + ((size_t)irec * n_shares * n_cts + cl) * share_comps * poly;
@@ -210,32 +222,39 @@ __global__ void __launch_bounds__(32 * D2MHE_MAX_LIMBS)
     const u64 p = lt->p, w = lt->crt, ws = lt->crt_sh, fr = lt->frac;
     const u32 fs = lt->frac_shift;
     const size_t at = (size_t)wl * v.n + jj;
-    const P2 c = __ldg(reinterpret_cast<const P2*>(c0 + at));
-    u64 a0 = c.x, a1 = c.y;
+    auto load = [](const W* p) {
+      R r;
+      r.q = __ldg(reinterpret_cast<const decltype(r.q)*>(p));
+      return r;
+    };
+    const R c = load(c0 + at);
+    u64 a[V];
+#pragma unroll
+    for (u32 i = 0; i < V; ++i) a[i] = c.get(i);
     const W* s = sh + at;
     // Ten shares at a time, predicated, so that the loads of a remainder are in flight together too.  (Four at a time from 120
     // shares on: 130 recipients of 130 shares at N = 2048, L = 2 100 us, 92 us like this.)
     auto add = [&](auto sum) {
       for (u32 k0 = 0; k0 < n_shares; k0 += 10) {
-        P2 h[10];
+        R h[10];
 #pragma unroll
-        for (u32 k = 0; k < 10; ++k) {
-          h[k].x = 0, h[k].y = 0;
-          if (k0 + k < n_shares) h[k] = __ldg(reinterpret_cast<const P2*>(s + (k0 + k) * kstride));
-        }
+        for (u32 k = 0; k < 10; ++k)
+          if (k0 + k < n_shares) h[k] = load(s + (k0 + k) * kstride);
 #pragma unroll
-        for (u32 k = 0; k < 10; ++k) a0 = sum(a0, h[k].x), a1 = sum(a1, h[k].y);
+        for (u32 k = 0; k < 10; ++k)
+#pragma unroll
+          for (u32 i = 0; i < V; ++i) a[i] = sum(a[i], h[k].get(i));
       }
     };
     if (lazy)
       add([](u64 x, u64 y) { return x + y; });
     else
       add([p](u64 x, u64 y) { return addmod(x, y, p); });
-    terms[wl][2 * lane] = mulhi_u64(shoup_full(a0, w, ws, p) << fs, fr);
-    terms[wl][2 * lane + 1] = mulhi_u64(shoup_full(a1, w, ws, p) << fs, fr);
+#pragma unroll
+    for (u32 i = 0; i < V; ++i) terms[wl][V * lane + i] = mulhi_u64(shoup_full(a[i], w, ws, p) << fs, fr);
   }
   __syncthreads();
-  for (u32 i = threadIdx.x; i < 64u && j0 + i < v.n; i += blockDim.x) {
+  for (u32 i = threadIdx.x; i < COLS && j0 + i < v.n; i += blockDim.x) {
     const u32 F = v.round.frac_bits;
     u64 sum = (u64)1 << (F - 1);
     for (u32 l = 0; l < L; ++l) sum += terms[l][i];
@@ -436,9 +455,14 @@ cudaError_t aggregate(const DevView& v, cudaStream_t s, const u64* ct, u32 n_row
 template <class W>
 static cudaError_t combine_words(const DevView& v, cudaStream_t s, const W* agg, const W* shares, u32 n_rec,
                                  u32 n_shares, u32 share_comps, u32 n_cts, u32* plain) {
-  dim3 grid(n_rec * n_cts, (v.n + 63) / 64);
-  k_combine<W><<<grid, 32 * v.L, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
-  return cudaGetLastError();
+  const u32 units = n_rec * n_cts;
+  auto launch = [&](auto kernel, u32 cols) {
+    kernel<<<units * ((v.n + cols - 1) / cols), 32 * v.L, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
+    return cudaGetLastError();
+  };
+  if constexpr (sizeof(W) == 4)
+    if (v.L <= 12) return launch(k_combine<W, 4, 12>, 128);
+  return launch(k_combine<W, 2, D2MHE_MAX_LIMBS>, 64);
 }
 cudaError_t combine(const DevView& v, cudaStream_t s, const u64* agg, const u64* shares, u32 n_rec,
                     u32 n_shares, u32 share_comps, u32 n_cts, u32* plain) {

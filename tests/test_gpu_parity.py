@@ -1639,3 +1639,23 @@ def test_shares_of_just_over_a_wave_of_blocks(d2, log2_n, bits, L, K, C):
         ctx.sync()
         assert np.array_equal(d2.to_u32_numpy(shares), want.astype(np.uint32))
     ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,L,K", [(3, 12, 3), (3, 13, 3), (8, 12, 11), (8, 13, 11)])
+def test_32_bit_combination_on_both_sides_of_twelve_limbs(d2, log2_n, L, K):
+    """Four residues to a thread up to twelve limbs, two beyond."""
+    n = 1 << log2_n
+    moduli = small_moduli(log2_n, 30, L)
+    q, rng = q_of(moduli), np.random.default_rng(L)
+    ctx = d2.Context(log2_n, moduli, K, seed=93)
+    ctx.keygen_share(list(range(K)))
+    ctx.collective_pk(list(range(K)))
+    p = np.array(moduli, dtype=np.uint64)[:, None]
+    agg, shares = rng.integers(0, 1 << 62, (1, 2, 2, L, n), dtype=np.uint64) % p, rng.integers(0, 1 << 62, (1, K, 2, L, n), dtype=np.uint64) % p
+    out = ctx.empty_u32(1, 2, n)
+    ctx.combine_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), d2.from_u32_numpy(shares.astype(np.uint32), ctx.device), 1, K, 2, out)
+    ctx.sync()
+    for c in range(2):
+        total = agg[0, c, 0].astype(object) + shares[0, :, c].astype(object).sum(axis=0)
+        assert d2.to_u32_numpy(out)[0, c].tolist() == [((2 * T * v + q) // (2 * q)) % T for v in to_big(total, moduli)]
+    ctx.close()

@@ -582,6 +582,41 @@ __device__ __forceinline__ u32 fft_dealt(const FftDeal& deal, u32& first, u32& s
   return (MIXED ? deal.whole : 0u) + b / deal.split;
 }
 
+__device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer
+  return __hiloint2double(0x43300000, v ^ (int)0x80000000u) - __hiloint2double(0x43300000, (int)0x80000000u);
+}
+
+// The transform of a sampled polynomial, from its bytes in the order of the double-precision kernels.
+template <int LOGN, int STASH>
+__device__ __forceinline__ void fft_samples_forward(const FftSmem<LOGN, STASH>& sm, const FftTab& ft, const uint4* poly,
+                                                    double* xr, double* xi) {
+  using G = FftGeo<LOGN>;
+  // number i of thread t is coefficient fft_coef(i): a column's coefficients are this thread's, or (two groups) this
+  // thread's and the one's at the same place of the other group
+  u32 w[G::GR * 8];
+#pragma unroll
+  for (int g = 0; g < G::GR; ++g)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint4 a = __ldg(poly + sm.tg + g * G::TG + h * G::T);
+      w[8 * g + 4 * h] = a.x, w[8 * g + 4 * h + 1] = a.y, w[8 * g + 4 * h + 2] = a.z, w[8 * g + 4 * h + 3] = a.w;
+    }
+  auto value = [&](int word, int byte) {
+    return small_to_double((int)__byte_perm(w[word], 0, 0x4440 | byte) - D2MHE_GAUSS_B);
+  };
+  fft_forward_at<LOGN>(sm, ft, xr, xi, [&](auto c_, auto j_, auto h_) {
+    // digit j of column c; h: the upper half of the coefficients below n (two groups)
+    constexpr int j = decltype(j_)::value;
+    if constexpr (G::GR == 2) {  // i = (j & 7) + 8 (h + 2 imaginary) of group j / 8
+      constexpr int base = 8 * (j / 8) + 2 * decltype(h_)::value + (j & 7) / 4;
+      return cpx{value(base, j & 3), value(base + 4, j & 3)};
+    } else {  // i = 2R c + j + R imaginary
+      constexpr int i = 2 * G::R * decltype(c_)::value + j;
+      return cpx{value(i / 4, i & 3), value((i + G::R) / 4, i & 3)};
+    }
+  });
+}
+
 // How many thread blocks share the two components of a ciphertext: two when that is no more work for the slowest SM.
 inline u32 fft_component_split(const DevView& v, u32 base, u32 ctas) {
   const u32 resident = v.sms * ctas;
@@ -639,9 +674,6 @@ __device__ __forceinline__ void fft_finish(const FftSmem<LOGN, STASH>& sm, const
   }
 }
 
-__device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer
-  return __hiloint2double(0x43300000, v ^ (int)0x80000000u) - __hiloint2double(0x43300000, (int)0x80000000u);
-}
 // part `half` of coefficients j and j + n of a residue row mod p, split at 2^h
 __device__ __forceinline__ cpx fft_split_pair(const u64* row, u32 j, u32 n, u32 half, u64 p, u32 h) {
   int a0, a1, b0, b1;

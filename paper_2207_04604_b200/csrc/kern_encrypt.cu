@@ -104,12 +104,9 @@ cudaError_t encrypt(const DevView& v, const LimbParams& lp, cudaStream_t s, cons
                     u32* launches) {
   const size_t per_unit = 3 * (size_t)v.n;
   const u32 n_units = n_parties * n_cts;
-  // Double-precision products wherever they apply, except for the smallest calls at N = 4096 (up to an eighth of the
-  // thread blocks that the GPU holds): there the 512-thread modular transforms below have the shorter latency and one
-  // launch less (24 blocks: 24.9 us against 28.8; 48: 26.5 against 28.7; 96: 36.2 against 28.4; N = 8192, 4 blocks:
-  // 40.3 against 30.5).
-  const bool smallest = v.logn == 12 && n_units * v.L * 8 <= resident_ctas(v);
-  if (v.fft_on && !smallest && launches && scratch_bytes >= 11 * (size_t)v.n) {
+  // Double-precision products wherever they apply.  (The smallest calls at N = 4096 took the 512-thread modular transforms
+  // below as long as the transform of u had a launch of its own: 24 blocks 18.7 us with their samples, 14.9 us now.)
+  if (v.fft_on && launches && scratch_bytes >= 11 * (size_t)v.n) {
     *launches = 0;
     return encrypt_fft(v, lp, s, parties_dev, ct_first, n_cts, n_units, plain, ct, scratch, scratch_bytes, launches);
   }

@@ -9,7 +9,7 @@ namespace {
 // depend on the limb: it is made once per (party, ciphertext) by k_fft_samples, comes from L2 and stays in tensor
 // memory for all four products (two components, two parts of the key).  Bound like the share kernel.
 // noise: the bytes of u, e_0 and e_1, N each per unit.   grid = n_units * L * split
-template <int LOGN>
+template <int LOGN, bool OWN_U>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_encrypt_fft(DevView v, const __grid_constant__ LimbParams lp, u32 unit_first, const double2* __restrict__ u_fft,
                   const uint4* __restrict__ noise, const u32* __restrict__ plain, u64* __restrict__ ct, u32 split) {
@@ -25,8 +25,13 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   __syncthreads();
   const u32 tbase = *sm.slot, tm = tmem_thread_base(tbase, G::WORDS);
   double xr[16], xi[16];
-  fft_load(sm, u_fft + (size_t)ulocal * n, xr, xi);
-  fft_loaded_to_tmem(tm, xr, xi);
+  if (!OWN_U) {
+    fft_load(sm, u_fft + (size_t)ulocal * n, xr, xi);
+    fft_loaded_to_tmem(tm, xr, xi);
+  } else {
+    fft_samples_forward(sm, v.fft, noise + (size_t)ulocal * 3 * (v.n / 16), xr, xi);
+    fft_to_tmem(tm, xr, xi);
+  }
   tmem_store_done();
   const u32* m = plain + (size_t)unit * v.n;
   const u32 end = split > 1 ? 2 * part + 2 : 4;
@@ -57,10 +62,11 @@ template <int LOGN>
 cudaError_t launch_encrypt(const DevView& v, const LimbParams& lp, cudaStream_t s, u32 unit_first, u32 n_units,
                            const double2* u_fft, const void* noise, const u32* plain, u64* ct) {
   using G = FftGeo<LOGN>;
-  cudaError_t e = set_smem(k_encrypt_fft<LOGN>, G::smem_bytes(1));
+  const auto kernel = u_fft ? k_encrypt_fft<LOGN, false> : k_encrypt_fft<LOGN, true>;
+  const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   const u32 split = fft_component_split(v, n_units * v.L, G::CTAS);
-  k_encrypt_fft<LOGN><<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, unit_first, u_fft,
+  kernel<<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, unit_first, u_fft,
                                                                 reinterpret_cast<const uint4*>(noise), plain, ct, split);
   return cudaGetLastError();
 }
@@ -83,8 +89,15 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
     unsigned char* noise = reinterpret_cast<unsigned char*>(scratch) + (size_t)nu * 8 * v.n;
     cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, true, noise);
     if (e != cudaSuccess) return e;
-    e = fft_samples(v, s, noise, 3, nu, u_fft);
-    if (e != cudaSuccess) return e;
+    // One wave of blocks: each makes the transform of its u, which takes less time than a launch for it (105 blocks at
+    // N = 16384: 9.3 + 37.8 us in two launches, 42.2 in one); more waves would make it again and again.
+    const u32 ctas = v.logn == 12 ? FftGeo<12>::CTAS : v.logn == 13 ? FftGeo<13>::CTAS : FftGeo<14>::CTAS;
+    if (nu * v.L <= v.sms * ctas) {
+      u_fft = nullptr;
+    } else {
+      e = fft_samples(v, s, noise, 3, nu, u_fft);
+      if (e != cudaSuccess) return e;
+    }
     switch (v.logn) {
       case 12: e = launch_encrypt<12>(v, lp, s, first, nu, u_fft, noise, plain, ct); break;
       case 13: e = launch_encrypt<13>(v, lp, s, first, nu, u_fft, noise, plain, ct); break;
@@ -92,7 +105,7 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
       default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    *launches += 3;
+    *launches += u_fft ? 3 : 2;
   }
   return cudaSuccess;
 }

@@ -72,32 +72,8 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     k_fft_samples(DevView v, const uint4* __restrict__ src, u32 stride, double2* __restrict__ dst) {
   using G = FftGeo<LOGN>;
   const FftSmem<LOGN> sm(v);
-  const uint4* poly = src + (size_t)blockIdx.x * stride * (v.n / 16);
-  // number i of thread t is coefficient fft_coef(i): a column's coefficients are this thread's, or (two groups) this
-  // thread's and the one's at the same place of the other group
-  u32 w[G::GR * 8];
-#pragma unroll
-  for (int g = 0; g < G::GR; ++g)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint4 a = __ldg(poly + sm.tg + g * G::TG + h * G::T);
-      w[8 * g + 4 * h] = a.x, w[8 * g + 4 * h + 1] = a.y, w[8 * g + 4 * h + 2] = a.z, w[8 * g + 4 * h + 3] = a.w;
-    }
-  auto value = [&](int word, int byte) {
-    return small_to_double((int)__byte_perm(w[word], 0, 0x4440 | byte) - D2MHE_GAUSS_B);
-  };
   double xr[16], xi[16];
-  fft_forward_at<LOGN>(sm, v.fft, xr, xi, [&](auto c_, auto j_, auto h_) {
-    // digit j of column c; h: the upper half of the coefficients below n (two groups)
-    constexpr int j = decltype(j_)::value;
-    if constexpr (G::GR == 2) {  // i = (j & 7) + 8 (h + 2 imaginary) of group j / 8
-      constexpr int base = 8 * (j / 8) + 2 * decltype(h_)::value + (j & 7) / 4;
-      return cpx{value(base, j & 3), value(base + 4, j & 3)};
-    } else {  // i = 2R c + j + R imaginary
-      constexpr int i = 2 * G::R * decltype(c_)::value + j;
-      return cpx{value(i / 4, i & 3), value((i + G::R) / 4, i & 3)};
-    }
-  });
+  fft_samples_forward(sm, v.fft, src + (size_t)blockIdx.x * stride * (v.n / 16), xr, xi);
   fft_store(sm, dst + (size_t)blockIdx.x * G::n, xr, xi);
 }
 

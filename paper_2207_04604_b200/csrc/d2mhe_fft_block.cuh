@@ -517,6 +517,19 @@ __device__ __forceinline__ u64 fft_sum(u64 low, u64 hi, u32 e0, const FftSplit& 
   return s + low;
 }
 
+// The canonical residue of s, which fft_sum left 2^b too large: with s = (k + 1) 2^b + rem, u = rem + (k + 1) d = r + d for
+// r = s - 2^b mod p below 2p, and bit b of u says whether r >= p = 2^b - d: then r - p is u without that bit, else r = u - d.
+// (The subtraction by a multiple of that bit goes to the multiplier; a comparison and two selections cost two more
+// instructions on the logic pipe, which this part of the kernels keeps busy: refresh shares at N = 8192 1604 -> 1568 us, shares
+// at N = 16384 1710 -> 1702 us, at N = 4096 331 -> 328 us.)
+__device__ __forceinline__ u64 fft_canon(u64 s, const LimbTab& lt) {
+  u32 s0, s1, u0, u1;
+  split64(s, s0, s1);
+  const u32 mask = (1u << lt.sf_shift) - 1u;
+  split64(madwide(s1 >> lt.sf_shift, lt.sf_d, join64(s0, s1 & mask)), u0, u1);
+  return join64(u0, u1 & mask) - madlo(u1 >> lt.sf_shift, 0u - lt.sf_d, lt.sf_d);
+}
+
 __device__ __forceinline__ u32 lo_nibbles(u64 a, u64 b, u64 c, u64 d) {  // low half of byte 6 of four rounded values
   return ((u32)(a >> 48) & 15u) | ((u32)(b >> 44) & 0xf0u) | ((u32)(c >> 40) & 0xf00u) | ((u32)(d >> 36) & 0xf000u);
 }

@@ -325,7 +325,7 @@ d2mhe_status build_tables(d2mhe_ctx* c) {
       sp.fmask = ~((1u << f) - 1u);
       sp.magic = 1.5 * (double)((u64)1 << (52 - f)) + 0.5;
       const u64 h0 = ((u64)(1075 - f) << 20) + ((u64)1 << 19);  // high word of the magic number
-      sp.k0 = 64 * p - offset - D2MHE_GAUSS_B - gap * h0;
+      sp.k0 = ((u64)1 << bits) + 64 * p - offset - D2MHE_GAUSS_B - gap * h0;
       return error + fft_pow2(-(int)std::min(f, 8u)) < 0.5;
     };
     const u32 h = std::min((bits + 1) / 2, 40 - logn), h_conv = (bits + 1) / 2, high = std::max(h, bits - h);

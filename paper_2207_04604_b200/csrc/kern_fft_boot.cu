@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;
       const u64 dm = shoup_u32(__ldg(mask + j), lt.delta, lt.delta_sh, lt.np);  // Lambda M_k, below 2p
-      __stcs(out + j, canon8<true>(s + (comp ? dm : lt.twop - dm), lt));
+      __stcs(out + j, fft_canon(s + (comp ? dm : lt.twop - dm), lt));
     });
     key = next;
     if (high) a += split;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
       if (high) nz.load(noise + ((share * 3 + 1 + comp) * v.n) / 16, v.chk);
     });
     fft_finish<LOGN>(sm, lt, lt.fftc, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
-      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
+      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, fft_canon(s, lt));
     });
     i = (i + 1) & 3u;
     if (i == 0) a += split;

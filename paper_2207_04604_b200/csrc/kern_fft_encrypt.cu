@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
     fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
       if (!D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) return;
       if (comp == 0) s += shoup_u32(__ldg(m + j), lt.delta, lt.delta_sh, lt.np);  // Lambda m, below 2p
-      out[j] = canon8<true>(s, lt);
+      out[j] = fft_canon(s, lt);
     });
   }
   __syncthreads();

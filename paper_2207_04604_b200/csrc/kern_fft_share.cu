@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
         if (high) nz.load(noise + (((size_t)ulocal * n_parties + a) * v.n) / 16, v.chk);
     });
     fft_finish<LOGN>(sm, lt, lt.fft, tw, xr, xi, high, nz, [&](u32 j, u64 s) {
-      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, canon8<true>(s, lt));
+      if (D2MHE_CHK(v.chk, j, v.n, SITE_STORE)) __stcs(out + j, fft_canon(s, lt));
     });
     key = next;
     if (high) a += split;

@@ -88,6 +88,7 @@ void d2mhe_destroy(d2mhe_ctx* ctx);
 d2mhe_status d2mhe_set_stream(d2mhe_ctx* ctx, void* cuda_stream);
 /* Waits for the stream; returns the first asynchronous error, D2MHE_ERR_DEVICE_CHECK if a kernel of
  * a context created with D2MHE_FLAG_DEVICE_CHECKS recorded an index violation since the last sync,
+ * or a wait inside a kernel ran into its limit (a defect; the results are then wrong),
  * or D2MHE_ERR_RANGE if d2mhe_encode saw a value outside [-(t-1)/2, (t-1)/2] since the last sync
  * (either record is cleared by the call that reports it). */
 d2mhe_status d2mhe_sync(d2mhe_ctx* ctx);

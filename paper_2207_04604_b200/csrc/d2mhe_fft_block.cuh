@@ -65,8 +65,9 @@ struct FftSmem {
   // The exchange area is free for the next transform when every warp has read the last one's columns.  A warp arrives
   // when it has, and waits only when it writes there again, most of a transform later: nothing stalls where a block
   // barrier made every warp wait for the slowest one.  Shares at N = 8192 716 -> 679 us, at N = 16384 1852 -> 1709 us,
-  // Conversion at N = 16384 4247 -> 3888 us (1480 rows of ten parties); not in the encryption kernels, whose two to four
-  // transforms a block don't repay it (N = 8192: 152 us with block barriers, 161 us).
+  // Conversion at N = 16384 4247 -> 3888 us (1480 rows of ten parties); not in the encryption kernels from N = 8192
+  // on, whose two to four transforms a block don't repay it (370 ciphertexts, L = 4, block barriers against this: N = 4096
+  // 83.9 / 77.0 us, N = 8192 153.8 / 161.8, N = 16384 352 / 359).
   __device__ __forceinline__ void init() const {  // one thread, ahead of a block barrier
     slot[1] = 0;
     asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(bar()), "r"(G::T / 32) : "memory");

@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal, tid = threadIdx.x;
   const LimbTab& lt = lp.limbs[l];
   FftSmem<LOGN> sm(v);
-  sm.announce = false;
+  sm.announce = LOGN == 12;
   if (tid == 0) sm.init();
   if (tid < 32) tmem_alloc(sm.slot, G::tmem_cols(1));
   __syncthreads();

@@ -153,7 +153,8 @@ __global__ void __launch_bounds__(COLS * GROUPS)
 // grid = n_rec * n_cts * N / 32 V, 32 L threads: the blocks of a unit side by side, so that the loads in flight fall into
 // long runs of a few units' rows (with the units side by side 81.7 us for 99 units of nine shares at N = 8192, L = 6, now
 // 78.0; 130 units of ten, L = 4: 76.1 and 71.6).  Words of 32 bits four at a time, 16 bytes as for 64 bits: 130 units of ten,
-// L = 7: 91.6 and 74.5 us.  That takes registers for at most 12 warps a block: two at a time beyond 12 limbs.
+// L = 7: 91.6 and 74.5 us, in an instance for blocks of at most eight warps, 64 registers a thread (for twelve warps it took
+// 122 registers, and that round 67 us more); two at a time beyond eight limbs.
 // ---------------------------------------------------------------------------
 
 // mixed-radix (Garner) digits d_i of w' = t v + (q-1)/2 in [0, q);  w' mod t = sum d_i prod_{j<i} q_j mod t;
@@ -461,7 +462,7 @@ static cudaError_t combine_words(const DevView& v, cudaStream_t s, const W* agg,
     return cudaGetLastError();
   };
   if constexpr (sizeof(W) == 4)
-    if (v.L <= 12) return launch(k_combine<W, 4, 12>, 128);
+    if (v.L <= 8) return launch(k_combine<W, 4, 8>, 128);
   return launch(k_combine<W, 2, D2MHE_MAX_LIMBS>, 64);
 }
 cudaError_t combine(const DevView& v, cudaStream_t s, const u64* agg, const u64* shares, u32 n_rec,

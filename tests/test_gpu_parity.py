@@ -1641,9 +1641,9 @@ def test_shares_of_just_over_a_wave_of_blocks(d2, log2_n, bits, L, K, C):
     ctx.close()
 
 
-@pytest.mark.parametrize("log2_n,L,K", [(3, 12, 3), (3, 13, 3), (8, 12, 11), (8, 13, 11)])
-def test_32_bit_combination_on_both_sides_of_twelve_limbs(d2, log2_n, L, K):
-    """Four residues to a thread up to twelve limbs, two beyond."""
+@pytest.mark.parametrize("log2_n,L,K", [(3, 8, 3), (3, 9, 3), (8, 8, 11), (8, 9, 11)])
+def test_32_bit_combination_on_both_sides_of_eight_limbs(d2, log2_n, L, K):
+    """Four residues to a thread up to eight limbs, two beyond."""
     n = 1 << log2_n
     moduli = small_moduli(log2_n, 30, L)
     q, rng = q_of(moduli), np.random.default_rng(L)

@@ -20,7 +20,8 @@ struct FftGeo {
   static constexpr int RS = 271;
   static constexpr size_t ex_bytes = (size_t)GR * R * RS * 16;
   __host__ __device__ static constexpr size_t smem_bytes(int stash) {
-    return ex_bytes + (stash ? (size_t)n * (9 + stash) : 0) + 16;  // + the word of tcgen05.alloc, one for a wait that ran out, and the barrier
+    // 16: the word of tcgen05.alloc, one for a wait that ran out, and the barrier
+    return ex_bytes + (stash ? (size_t)n * (9 + stash) : 0) + 16;
   }
   // Words of tensor memory per thread for one transform, and columns for `k` of them: warp w of a block
   // reaches the lanes 32 (w mod 4) .. + 31 only, so warps w, w + 4, .. share lanes and split the columns.

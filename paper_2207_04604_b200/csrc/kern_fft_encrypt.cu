@@ -6,8 +6,9 @@
 namespace {
 
 // One thread block = one (party, ciphertext, limb), or one component of it (split = 2).  The transform of u does not
-// depend on the limb: it is made once per (party, ciphertext) by k_fft_samples, comes from L2 and stays in tensor
-// memory for all four products (two components, two parts of the key).  Bound like the share kernel.
+// depend on the limb: it is made once per (party, ciphertext) by k_fft_samples and comes from L2, or (OWN_U, calls of one
+// wave of blocks) every block makes it from the samples; it stays in tensor memory for all four products (two components,
+// two parts of the key).  Bound like the share kernel.
 // noise: the bytes of u, e_0 and e_1, N each per unit.   grid = n_units * L * split
 template <int LOGN, bool OWN_U>
 __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
@@ -67,7 +68,7 @@ cudaError_t launch_encrypt(const DevView& v, const LimbParams& lp, cudaStream_t 
   if (e != cudaSuccess) return e;
   const u32 split = fft_component_split(v, n_units * v.L, G::CTAS);
   kernel<<<n_units * v.L * split, G::T, G::smem_bytes(1), s>>>(v, lp, unit_first, u_fft,
-                                                                reinterpret_cast<const uint4*>(noise), plain, ct, split);
+                                                               reinterpret_cast<const uint4*>(noise), plain, ct, split);
   return cudaGetLastError();
 }
 

@@ -89,7 +89,7 @@ cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s,
   const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   kernel<<<deal.blocks, G::T, G::smem_bytes(1), s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,
-                                                              reinterpret_cast<const uint4*>(noise), shares, deal);
+                                                     reinterpret_cast<const uint4*>(noise), shares, deal);
   return cudaGetLastError();
 }
 

@@ -46,6 +46,7 @@
 // exchange with its butterfly joins the two results.  (One group of 256 threads with 32 points each: eight warps
 // per SM hide too little of the latencies.)
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <type_traits>
@@ -381,4 +382,48 @@ D2MHE_HD void fft_split(unsigned long long c, unsigned long long p, unsigned h, 
   const int l = (int)((unsigned)(unsigned long long)v << (32 - h)) >> (32 - h);
   lo = l;
   hi = (int)((v - l) >> h);
+}
+
+// How a launch's products are dealt out: `rows` fixed factors (a limb of a unit's c_1), each with the products of all
+// parties.  The first `whole` rows get a block each, the others `split` blocks, each of which transforms the fixed factor for
+// itself.
+struct FftDeal {
+  unsigned whole, split, blocks;
+};
+// Part transforms of a block: of its fixed factor, and for each of its parties.  A 64-bit residue has two parts, a 32-bit one
+// is one (taken for two there, 176 rows of ten at N = 8192 stayed whole: 71.4 us, in five blocks a row 57.7; 88 rows at
+// N = 16384 79.4 and 68.1; 455 rows of twenty at N = 4096 121.8 and 108.1).
+struct FftWork {
+  unsigned fixed, per_party;
+};
+constexpr FftWork FFT_WORK_SHARE = {2, 2}, FFT_WORK_SHARE32 = {1, 1}, FFT_WORK_BOOT = {2, 2}, FFT_WORK_CONVERT = {2, 4};
+// The deal with the shortest schedule, counted in part transforms over waves of `places` blocks: whole rows for as many full
+// waves as there are and the rest split over one wave, or all rows split alike.
+// (594 rows of nine on 296 places: three blocks to a row took seven waves of three parties; 592 whole rows and two rows split
+// nine ways take two waves of nine and one of one: 320 -> 264 us at N = 8192.)
+inline FftDeal fft_deal(unsigned places, unsigned rows, unsigned n_parties, FftWork work) {
+  const unsigned full = rows / places * places, rest = rows - full, all = work.fixed + work.per_party * n_parties;
+  FftDeal deal = {0, 1, rows};
+  unsigned long long best = (unsigned long long)((rows + places - 1) / places) * all;
+  auto consider = [&](unsigned whole, unsigned split, unsigned long long waves) {
+    const unsigned long long cost =
+        (unsigned long long)(whole / places) * all + waves * (work.fixed + work.per_party * ((n_parties + split - 1) / split));
+    if (cost < best) best = cost, deal = FftDeal{whole, split, whole + (rows - whole) * split};
+  };
+  if (full && rest) consider(full, std::max(1u, std::min(n_parties, places / rest)), 1);
+  for (unsigned c = 2; c <= n_parties && c <= 16u; ++c) consider(0, c, ((unsigned long long)rows * c + places - 1) / places);
+  if (!full) consider(0, std::max(1u, std::min(n_parties, places / std::max(rows, 1u))), 1);
+  return deal;
+}
+// A block's row and its part of the parties: first, first + step, ..  MIXED: some rows are whole, others not (an
+// instance of its own: a step that is not a launch constant takes a register that the kernels do not have).
+template <bool MIXED>
+D2MHE_HD unsigned fft_dealt(const FftDeal& deal, unsigned block, unsigned& first, unsigned& step) {
+  if (MIXED && block < deal.whole) {
+    first = 0, step = 1;
+    return block;
+  }
+  const unsigned b = MIXED ? block - deal.whole : block;
+  first = b % deal.split, step = deal.split;
+  return (MIXED ? deal.whole : 0u) + b / deal.split;
 }

@@ -561,42 +561,6 @@ struct FftNoNoise {
   }
 };
 
-// How a launch's products are dealt out: `rows` fixed factors (a limb of a unit's c_1), each with the products of all
-// parties.  The first `whole` rows get a block each, the others `split` blocks, each of which transforms the fixed factor for
-// itself.
-struct FftDeal {
-  u32 whole, split, blocks;
-};
-// The deal with the shortest schedule, counted in part transforms (2 forward and per_party for each party) over waves of
-// blocks: whole rows for as many full waves as there are and the rest split over one wave, or all rows split alike.
-// (594 rows of nine on 296 places: three blocks to a row took seven waves of three parties; 592 whole rows and two rows split
-// nine ways take two waves of nine and one of one: 320 -> 264 us at N = 8192.)
-inline FftDeal fft_deal(const DevView& v, u32 rows, u32 ctas, u32 n_parties, u32 per_party) {
-  const u32 places = v.sms * ctas, full = rows / places * places, rest = rows - full;
-  FftDeal deal = {0, 1, rows};
-  u64 best = (u64)((rows + places - 1) / places) * (2 + per_party * n_parties);
-  auto consider = [&](u32 whole, u32 split, u64 waves) {
-    const u64 cost = (u64)(whole / places) * (2 + per_party * n_parties) + waves * (2 + per_party * ((n_parties + split - 1) / split));
-    if (cost < best) best = cost, deal = FftDeal{whole, split, whole + (rows - whole) * split};
-  };
-  if (full && rest) consider(full, std::max(1u, std::min(n_parties, places / rest)), 1);
-  for (u32 c = 2; c <= n_parties && c <= 16u; ++c) consider(0, c, ((u64)rows * c + places - 1) / places);
-  if (!full) consider(0, std::max(1u, std::min(n_parties, places / std::max(rows, 1u))), 1);
-  return deal;
-}
-// This block's row and its part of the parties: first, first + step, ..  MIXED: some rows are whole, others not (an
-// instance of its own: a step that is not a launch constant takes a register that the kernels do not have).
-template <bool MIXED>
-__device__ __forceinline__ u32 fft_dealt(const FftDeal& deal, u32& first, u32& step) {
-  if (MIXED && blockIdx.x < deal.whole) {
-    first = 0, step = 1;
-    return blockIdx.x;
-  }
-  const u32 b = MIXED ? blockIdx.x - deal.whole : blockIdx.x;
-  first = b % deal.split, step = deal.split;
-  return (MIXED ? deal.whole : 0u) + b / deal.split;
-}
-
 __device__ __forceinline__ double small_to_double(int v) {  // exact for any 32-bit integer
   return __hiloint2double(0x43300000, v ^ (int)0x80000000u) - __hiloint2double(0x43300000, (int)0x80000000u);
 }

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
   u32 part, split;
-  const u32 rest = fft_dealt<MIXED>(deal, part, split);
+  const u32 rest = fft_dealt<MIXED>(deal, blockIdx.x, part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -138,7 +138,7 @@ template <int LOGN>
 cudaError_t launch_share32(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* agg, const u32* parties_dev,
                            u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u32* shares) {
   using G = FftGeo<LOGN>;
-  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 1);
+  const FftDeal deal = fft_deal(v.sms * G::CTAS, n_units * v.L, n_parties, FFT_WORK_SHARE32);
   const auto kernel = deal.whole ? k_share32_fft<LOGN, true> : k_share32_fft<LOGN, false>;
   const cudaError_t e = set_smem(kernel, smem32<LOGN>());
   if (e != cudaSuccess) return e;

@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
   u32 part, split;
-  const u32 row_comp = fft_dealt<MIXED>(deal, part, split), comp = row_comp & 1u, rest = row_comp / 2;
+  const u32 row_comp = fft_dealt<MIXED>(deal, blockIdx.x, part, split), comp = row_comp & 1u, rest = row_comp / 2;
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -81,7 +81,7 @@ cudaError_t launch_boot(const DevView& v, const LimbParams& lp, cudaStream_t s, 
                         u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const u64* alpha, const void* noise,
                         const u32* masks, u64* shares) {
   using G = FftGeo<LOGN>;
-  const FftDeal deal = fft_deal(v, n_units * v.L * 2, G::CTAS, n_parties, 2);
+  const FftDeal deal = fft_deal(v.sms * G::CTAS, n_units * v.L * 2, n_parties, FFT_WORK_BOOT);
   const auto kernel = deal.whole ? k_boot_fft<LOGN, true> : k_boot_fft<LOGN, false>;
   const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;

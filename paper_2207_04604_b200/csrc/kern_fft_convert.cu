@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
   u32 block_part, split;
-  const u32 rest = fft_dealt<MIXED>(deal, block_part, split);
+  const u32 rest = fft_dealt<MIXED>(deal, blockIdx.x, block_part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (block_part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -82,7 +82,7 @@ cudaError_t launch_convert(const DevView& v, const LimbParams& lp, cudaStream_t 
                            const u32* recipients_dev, const u32* parties_dev, u32 n_parties, u32 n_cts, u32 unit_first,
                            u32 n_units, const double2* mu_fft, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 4);
+  const FftDeal deal = fft_deal(v.sms * G::CTAS, n_units * v.L, n_parties, FFT_WORK_CONVERT);
   const auto kernel = deal.whole ? k_convert_fft<LOGN, true> : k_convert_fft<LOGN, false>;
   const cudaError_t e = set_smem(kernel, G::smem_bytes(2));
   if (e != cudaSuccess) return e;

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(FftGeo<LOGN>::T, FftGeo<LOGN>::CTAS)
   using G = FftGeo<LOGN>;
   constexpr int n = G::n;
   u32 part, split;
-  const u32 rest = fft_dealt<MIXED>(deal, part, split);
+  const u32 rest = fft_dealt<MIXED>(deal, blockIdx.x, part, split);
   const u32 l = rest % v.L, ulocal = rest / v.L, unit = unit_first + ulocal;
   if (part >= n_parties) return;
   const u32 irec = unit / n_cts, cl = unit % n_cts, tid = threadIdx.x;
@@ -84,7 +84,7 @@ template <int LOGN, bool OWN>
 cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s, const u64* agg, const u32* parties_dev,
                          u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
-  const FftDeal deal = fft_deal(v, n_units * v.L, G::CTAS, n_parties, 2);
+  const FftDeal deal = fft_deal(v.sms * G::CTAS, n_units * v.L, n_parties, FFT_WORK_SHARE);
   const auto kernel = deal.whole ? k_share_fft<LOGN, OWN, true> : k_share_fft<LOGN, OWN, false>;
   const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;

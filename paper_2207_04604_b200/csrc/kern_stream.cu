@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(COLS * GROUPS)
 // long runs of a few units' rows (with the units side by side 81.7 us for 99 units of nine shares at N = 8192, L = 6, now
 // 78.0; 130 units of ten, L = 4: 76.1 and 71.6).  Words of 32 bits four at a time, 16 bytes as for 64 bits: 130 units of ten,
 // L = 7: 91.6 and 74.5 us, in an instance for blocks of at most eight warps, 64 registers a thread (for twelve warps it took
-// 122 registers, and that round 67 us more); two at a time beyond eight limbs.
+// 122 registers, and that round 67 us more); combine_words has the rule.
 // ---------------------------------------------------------------------------
 
 // mixed-radix (Garner) digits d_i of w' = t v + (q-1)/2 in [0, q);  w' mod t = sum d_i prod_{j<i} q_j mod t;
@@ -461,8 +461,12 @@ static cudaError_t combine_words(const DevView& v, cudaStream_t s, const W* agg,
     kernel<<<units * ((v.n + cols - 1) / cols), 32 * v.L, 0, s>>>(v, agg, shares, n_shares, share_comps, n_cts, plain);
     return cudaGetLastError();
   };
+  // Four words to a thread leave half the blocks, which pays once the launch fills the chip: from a dozen warps per
+  // multiprocessor on (four units of twenty, N = 8192, L = 8, 14 warps: 6.5 and 4.7 us; 40 of ten, L = 7: 28.6 and 23.4; eight
+  // of ten, L = 3, 10 warps: 3.8 and 3.8; nine of fifty at N = 2048, L = 3, 3 warps: 4.9 and 5.9; one of ten at N = 8192,
+  // L = 3: 2.5 and 3.0).  Below N = 128 half the lanes would idle (1600 units of four at N = 64: 4.6 and 5.8 us).
   if constexpr (sizeof(W) == 4)
-    if (v.L <= 8) return launch(k_combine<W, 4, 8>, 128);
+    if (v.L <= 8 && v.n >= 128 && (u64)units * (v.n / 128) * v.L >= 12 * (u64)v.sms) return launch(k_combine<W, 4, 8>, 128);
   return launch(k_combine<W, 2, D2MHE_MAX_LIMBS>, 64);
 }
 cudaError_t combine(const DevView& v, cudaStream_t s, const u64* agg, const u64* shares, u32 n_rec,

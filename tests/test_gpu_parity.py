@@ -1,6 +1,7 @@
 """GPU parity: every output of the CUDA library against the CPU oracle, bit for bit,
 through the C ABI (via the thin ctypes binding)."""
 import gc
+import math
 import threading
 
 import numpy as np
@@ -1643,7 +1644,21 @@ def test_shares_of_just_over_a_wave_of_blocks(d2, log2_n, bits, L, K, C):
 
 @pytest.mark.parametrize("log2_n,L,K", [(3, 8, 3), (3, 9, 3), (8, 8, 11), (8, 9, 11)])
 def test_32_bit_combination_on_both_sides_of_eight_limbs(d2, log2_n, L, K):
-    """Four residues to a thread up to eight limbs, two beyond."""
+    """Small calls, two residues to a thread."""
+    _check_combination32(d2, log2_n, L, K, 2)
+
+
+@pytest.mark.parametrize("log2_n,L,K,fill", [(6, 8, 2, 2.0), (7, 8, 3, 0.999), (7, 8, 3, 1.0), (9, 3, 12, 0.999), (9, 3, 12, 1.0), (8, 9, 2, 1.1),
+                                             (12, 8, 2, 1.2)])
+def test_32_bit_combination_on_both_sides_of_the_fill(d2, log2_n, L, K, fill):
+    """Four residues to a thread from twelve warps per multiprocessor on, up to eight limbs and from N = 128 up."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    warps = max(1, (1 << log2_n) // 128) * L
+    units = int(fill * 12 * sms) // warps if fill < 1 else math.ceil(fill * 12 * sms / warps)
+    _check_combination32(d2, log2_n, L, K, units)
+
+
+def _check_combination32(d2, log2_n, L, K, units):
     n = 1 << log2_n
     moduli = small_moduli(log2_n, 30, L)
     q, rng = q_of(moduli), np.random.default_rng(L)
@@ -1651,11 +1666,12 @@ def test_32_bit_combination_on_both_sides_of_eight_limbs(d2, log2_n, L, K):
     ctx.keygen_share(list(range(K)))
     ctx.collective_pk(list(range(K)))
     p = np.array(moduli, dtype=np.uint64)[:, None]
-    agg, shares = rng.integers(0, 1 << 62, (1, 2, 2, L, n), dtype=np.uint64) % p, rng.integers(0, 1 << 62, (1, K, 2, L, n), dtype=np.uint64) % p
-    out = ctx.empty_u32(1, 2, n)
-    ctx.combine_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), d2.from_u32_numpy(shares.astype(np.uint32), ctx.device), 1, K, 2, out)
+    agg, shares = rng.integers(0, 1 << 62, (1, units, 2, L, n), dtype=np.uint64) % p, rng.integers(0, 1 << 62, (1, K, units, L, n), dtype=np.uint64) % p
+    out = ctx.empty_u32(1, units, n)
+    ctx.combine_decrypt32(d2.from_u32_numpy(agg.astype(np.uint32), ctx.device), d2.from_u32_numpy(shares.astype(np.uint32), ctx.device), 1, K, units, out)
     ctx.sync()
-    for c in range(2):
+    got = d2.to_u32_numpy(out)[0]
+    for c in range(units):
         total = agg[0, c, 0].astype(object) + shares[0, :, c].astype(object).sum(axis=0)
-        assert d2.to_u32_numpy(out)[0, c].tolist() == [((2 * T * v + q) // (2 * q)) % T for v in to_big(total, moduli)]
+        assert got[c].tolist() == [((2 * T * v + q) // (2 * q)) % T for v in to_big(total, moduli)]
     ctx.close()

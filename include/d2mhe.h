@@ -88,9 +88,10 @@ void d2mhe_destroy(d2mhe_ctx* ctx);
 d2mhe_status d2mhe_set_stream(d2mhe_ctx* ctx, void* cuda_stream);
 /* Waits for the stream; returns the first asynchronous error, D2MHE_ERR_DEVICE_CHECK if a kernel of
  * a context created with D2MHE_FLAG_DEVICE_CHECKS recorded an index violation since the last sync,
- * or a wait inside a kernel ran into its limit (a defect; the results are then wrong),
- * or D2MHE_ERR_RANGE if d2mhe_encode saw a value outside [-(t-1)/2, (t-1)/2] since the last sync
- * (either record is cleared by the call that reports it). */
+ * or a wait inside a kernel of any context ran into its limit of about a second (a defect; the
+ * results are then wrong), or D2MHE_ERR_RANGE if d2mhe_encode saw a value outside [-(t-1)/2, (t-1)/2] since
+ * the last sync (each record is cleared by the call that reports it: where there are several, the
+ * next calls report the others). */
 d2mhe_status d2mhe_sync(d2mhe_ctx* ctx);
 const char* d2mhe_strerror(d2mhe_status status);
 
@@ -303,7 +304,8 @@ d2mhe_status d2mhe_combine_decrypt32(d2mhe_ctx* ctx, const uint32_t* agg_dev, co
  * d2mhe_round_device takes device values/sums.  d2mhe_round_host takes HOST values/sums
  * (pinned memory recommended), copies each sub-chunk in and out on the stream that
  * computes it and returns after all of it has finished; it returns D2MHE_ERR_RANGE (sums then
- * unspecified) if a value was outside [-(t-1)/2, (t-1)/2].  If a launch or copy fails part-way,
+ * unspecified) if a value was outside [-(t-1)/2, (t-1)/2], and D2MHE_ERR_DEVICE_CHECK, before
+ * that, if a wait inside a kernel ran into its limit (see d2mhe_sync).  If a launch or copy fails part-way,
  * the internal streams are still joined back into the context's stream before the call returns.
  */
 size_t d2mhe_round_workspace_bytes(const d2mhe_ctx* ctx, uint32_t chunk_cts);
@@ -358,12 +360,18 @@ d2mhe_status d2mhe_round_device_static(d2mhe_ctx* ctx, const int32_t* values_dev
 /* Test hooks. */
 /* The violation that d2mhe_sync last reported as D2MHE_ERR_DEVICE_CHECK:
  * info = {site (1 load, 2 store, 3 octet, 4 shared-memory offset, 5 twiddle index, 6 party number,
- * 7 limb, 8 streaming element, 9 staged bytes, 15 self-test), index, limit, thread block}. */
+ * 7 limb, 8 streaming element, 9 staged bytes, 10 a wait that ran out, 15 self-test), index, limit,
+ * thread block} (zeros after the site for a wait, which d2mhe_round_host may have reported too). */
 d2mhe_status d2mhe_debug_last_device_check(const d2mhe_ctx* ctx, uint32_t info[4]);
 /* Launches one thread that runs the checked build's index test on the index 1 with limit 1 (it
  * touches no memory): with D2MHE_FLAG_DEVICE_CHECKS the next d2mhe_sync returns
  * D2MHE_ERR_DEVICE_CHECK with site 15, without the flag nothing happens. */
 d2mhe_status d2mhe_debug_check_selftest(d2mhe_ctx* ctx);
+/* Launches one thread block in which a warp never announces that it has read the block's exchange
+ * area, so that the waits run into their limit, here of `tries` (1 .. 2^18, which is what the
+ * products' kernels have): the kernel ends normally and the next d2mhe_sync returns
+ * D2MHE_ERR_DEVICE_CHECK with site 10. */
+d2mhe_status d2mhe_debug_wait_selftest(d2mhe_ctx* ctx, uint32_t tries);
 /* s_k as int8 [N] on the HOST (needs a key share for `party`): the key that the device stores (in
  * the transform domain) is inverse-transformed on the GPU, limb by limb, and copied back;
  * D2MHE_ERR_DEVICE_CHECK if the limbs disagree or a coefficient is not in {-1, 0, 1}.  Allocates a

@@ -71,6 +71,7 @@ enum : u32 {
   SITE_LIMB = 7,       // limb number
   SITE_ELEMENT = 8,    // element index of a streaming kernel
   SITE_STAGED = 9,     // offset into staged bytes in shared memory
+  SITE_WAIT = 10,      // a wait inside a kernel ran out (every build; noted by the host)
   SITE_SELFTEST = 15   // raised on purpose by the self-test hook
 };
 #ifdef D2MHE_CHECKED

@@ -39,8 +39,10 @@ struct FftSmem {
   unsigned short* nibbles;
   u32* chk;  // device check words (read by the checked kernel build only)
   u32 tg;
-  u32 phase = 0;         // of the barrier in the last transform
-  bool announce = true;  // false: a block barrier instead (a constant in every kernel)
+  static constexpr int WAIT_TRIES = 1 << 18;
+  u32 phase = 0;           // of the barrier in the last transform
+  int tries = WAIT_TRIES;  // left to this thread's waits
+  bool announce = true;    // false: a block barrier instead (a constant in every kernel)
   __device__ __forceinline__ explicit FftSmem(const DevView& v) {
     chk = v.chk;
     const u32 g = group();
@@ -82,16 +84,19 @@ struct FftSmem {
     __syncwarp();
     if ((threadIdx.x & 31u) == 0) asm volatile("{.reg .b64 t; mbarrier.arrive.shared.b64 t, [%0];}" ::"r"(bar()) : "memory");
   }
-  // The wait has a limit (a second or more), after which the call is reported as failed (finish).
+  // A try that fails takes 4 us on this GPU (5000 of them in the self-test's kernel 20 ms, with and without a time hint), and
+  // all the waits of a thread have WAIT_TRIES failing ones between them: a block loses about a second, whatever is wrong, and
+  // its call is reported as failed (finish).
   __device__ __forceinline__ void acquire() {
     if (!announce) {
       __syncthreads();
       return;
     }
     u32 done = 0;
-    for (int i = 0; !done && i < (1 << 20); ++i)
+    for (; !done && tries; --tries)
       asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
                    : "=r"(done) : "r"(bar()), "r"(phase ^ 1u) : "memory");
+    tries += (int)done;  // the one that succeeded
     if (!done) slot[1] = 1;
     phase ^= 1u;
   }

@@ -742,6 +742,18 @@ d2mhe_status d2mhe_set_stream(d2mhe_ctx* c, void* stream) {
   return D2MHE_OK;
 }
 
+// Reports what the kernels left in the range word: first a wait that ran out, then, by the next call, a value out of range.
+static d2mhe_status report_range_word(d2mhe_ctx* c, u32 flag) {
+  const bool wait = (flag & RANGE_FLAG_WAIT) != 0;
+  const u32 left = wait ? flag & ~(u32)RANGE_FLAG_WAIT : 0;
+  const cudaError_t e = cudaMemcpy(c->view.range_flag, &left, sizeof(u32), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return fail_cuda(c, e);
+  if (!wait) return D2MHE_ERR_RANGE;
+  const u32 words[4] = {SITE_WAIT, 0, 0, 0};
+  std::memcpy(c->last_check, words, sizeof(words));
+  return D2MHE_ERR_DEVICE_CHECK;
+}
+
 d2mhe_status d2mhe_sync(d2mhe_ctx* c) {
   if (!c) return D2MHE_ERR_INVALID_ARG;
   DeviceGuard guard(c->device);
@@ -758,16 +770,10 @@ d2mhe_status d2mhe_sync(d2mhe_ctx* c) {
       std::memcpy(c->last_check, words, sizeof(words));
       e = cudaMemset(c->view.chk, 0, sizeof(words));
       if (e != cudaSuccess) return fail_cuda(c, e);
-      if (flag) (void)cudaMemset(c->view.range_flag, 0, sizeof(u32));
       return D2MHE_ERR_DEVICE_CHECK;
     }
   }
-  if (flag) {
-    e = cudaMemset(c->view.range_flag, 0, sizeof(u32));
-    if (e != cudaSuccess) return fail_cuda(c, e);
-    return flag & RANGE_FLAG_WAIT ? D2MHE_ERR_DEVICE_CHECK : D2MHE_ERR_RANGE;
-  }
-  return D2MHE_OK;
+  return flag ? report_range_word(c, flag) : D2MHE_OK;
 }
 
 d2mhe_status d2mhe_debug_last_device_check(const d2mhe_ctx* c, uint32_t info[4]) {
@@ -780,6 +786,15 @@ d2mhe_status d2mhe_debug_check_selftest(d2mhe_ctx* c) {
   if (!c) return D2MHE_ERR_INVALID_ARG;
   DeviceGuard guard(c->device);
   cudaError_t e = L_(check_selftest)(c->view, c->stream);
+  if (e != cudaSuccess) return fail_cuda(c, e);
+  c->launches += 1;
+  return D2MHE_OK;
+}
+
+d2mhe_status d2mhe_debug_wait_selftest(d2mhe_ctx* c, u32 tries) {
+  if (!c || tries == 0 || tries > (1u << 18)) return D2MHE_ERR_INVALID_ARG;
+  DeviceGuard guard(c->device);
+  cudaError_t e = L_(wait_selftest)(c->view, c->stream, tries);
   if (e != cudaSuccess) return fail_cuda(c, e);
   c->launches += 1;
   return D2MHE_OK;
@@ -1514,10 +1529,7 @@ static d2mhe_status round_impl(d2mhe_ctx* c, const int32_t* values, bool host_io
     u32 flag = 0;
     if ((e = cudaMemcpy(&flag, c->view.range_flag, sizeof(u32), cudaMemcpyDeviceToHost)) != cudaSuccess)
       return fail_cuda(c, e);
-    if (flag) {
-      if ((e = cudaMemset(c->view.range_flag, 0, sizeof(u32))) != cudaSuccess) return fail_cuda(c, e);
-      return flag & RANGE_FLAG_WAIT ? D2MHE_ERR_DEVICE_CHECK : D2MHE_ERR_RANGE;
-    }
+    if (flag) return report_range_word(c, flag);
   }
   return D2MHE_OK;
 }

@@ -178,7 +178,8 @@ struct d2mhe_ctx {
 // n_parties 6 N + 8 N L); combine sums the first of share_comps polynomials per
 // (recipient, party, ciphertext); int_probe synchronises the stream; export_secret turns key rows
 // [L][N] (transform domain, Montgomery form) into int8 coefficients [L][N] (127 = not ternary);
-// check_selftest makes one thread of the checked build raise SITE_SELFTEST (no memory access).
+// check_selftest makes one thread of the checked build raise SITE_SELFTEST (no memory access);
+// wait_selftest runs one block whose waits for its exchange area run into the limit.
 #define D2MHE_LAUNCHER_DECLS \
 cudaError_t keygen(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties); \
 cudaError_t collective_pk(const DevView& v, const LimbParams& lp, cudaStream_t s, const u32* parties_dev, u32 n_parties, \
@@ -230,6 +231,7 @@ cudaError_t secret_product(const DevView& v, const LimbParams& lp, cudaStream_t 
 cudaError_t muladd(const DevView& v, cudaStream_t s, const u64* a, const u64* b, const u64* c, \
                    u64* d, u32 batch); \
 cudaError_t check_selftest(const DevView& v, cudaStream_t s); \
+cudaError_t wait_selftest(const DevView& v, cudaStream_t s, u32 tries); \
 cudaError_t sample_streams(const DevView& v, cudaStream_t s, const u32* recipients_dev, const u32* parties_dev, \
                            u32 n_parties, u32 ct_first, u32 n_cts, u32 unit_first, u32 n_units, SampleKinds kinds, \
                            bool fft_order, void* out); \

@@ -106,6 +106,20 @@ __global__ void __launch_bounds__(KEY_THREADS)
   });
 }
 
+// Test hook: warp 0 does not announce that it has read the exchange area, so the second wait runs into the limit, and those
+// after it give up at once.  No copies in flight, no tensor memory.
+__global__ void __launch_bounds__(FftGeo<12>::T) k_wait_selftest(DevView v, int tries) {
+  FftSmem<12, 0> sm(v);
+  sm.tries = tries;
+  if (threadIdx.x == 0) sm.init();
+  __syncthreads();
+  sm.acquire();
+  if (threadIdx.x >= 32) sm.release();
+  for (int i = 0; i < 4; ++i) sm.acquire();
+  __syncthreads();
+  if (threadIdx.x == 0) sm.finish(v);
+}
+
 template <int LOGN>
 cudaError_t launch_secret(const DevView& v, cudaStream_t s, const u32* parties_dev, u32 n_parties, u32 tag, double2* dst) {
   cudaError_t e = set_smem(k_fft_secret<LOGN>, key_smem<LOGN>());
@@ -142,6 +156,14 @@ cudaError_t fft_secret(const DevView& v, cudaStream_t s, const u32* parties_dev,
     case 14: return launch_secret<14>(v, s, parties_dev, n_parties, tag, dst);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t wait_selftest(const DevView& v, cudaStream_t s, u32 tries) {
+  const size_t smem = FftGeo<12>::smem_bytes(0);
+  const cudaError_t e = set_smem(k_wait_selftest, smem);
+  if (e != cudaSuccess) return e;
+  k_wait_selftest<<<1, FftGeo<12>::T, smem, s>>>(v, (int)tries);
+  return cudaGetLastError();
 }
 
 // every stride-th of the polynomials in src; dst: [polys][n]

@@ -34,7 +34,7 @@ EXPORTS = [
     "d2mhe_combine_decrypt32", "d2mhe_round_workspace_bytes", "d2mhe_round_plan", "d2mhe_round_device",
     "d2mhe_round_host", "d2mhe_round_device_static", "d2mhe_user_keygen", "d2mhe_convert_share",
     "d2mhe_convert_combine", "d2mhe_decrypt", "d2mhe_bootstrap_share", "d2mhe_bootstrap_combine", "d2mhe_debug_export_user_secret", "d2mhe_debug_export_secret", "d2mhe_debug_int_throughput", "d2mhe_debug_last_device_check",
-    "d2mhe_debug_check_selftest", "d2mhe_get_root", "d2mhe_get_plain_root",
+    "d2mhe_debug_check_selftest", "d2mhe_debug_wait_selftest", "d2mhe_get_root", "d2mhe_get_plain_root",
     "d2mhe_launch_count", "d2mhe_sample_scratch_bytes",
 ]
 
@@ -116,6 +116,7 @@ def load():
         lib.d2mhe_debug_int_throughput.argtypes = [vp, u32, u32, ctypes.POINTER(ctypes.c_double)]
         lib.d2mhe_debug_last_device_check.argtypes = [vp, vp]
         lib.d2mhe_debug_check_selftest.argtypes = [vp]
+        lib.d2mhe_debug_wait_selftest.argtypes = [vp, u32]
         lib.d2mhe_get_root.argtypes = [vp, u32, ctypes.POINTER(u64)]
         lib.d2mhe_get_plain_root.argtypes = [vp, ctypes.POINTER(u64)]
         lib.d2mhe_launch_count.argtypes = [vp]
@@ -391,6 +392,9 @@ class Context:
 
     def debug_check_selftest(self):
         self._check(load().d2mhe_debug_check_selftest(self._h), "d2mhe_debug_check_selftest")
+
+    def debug_wait_selftest(self, tries):
+        self._check(load().d2mhe_debug_wait_selftest(self._h, tries), "d2mhe_debug_wait_selftest")
 
     def get_root(self, limb):
         v = ctypes.c_uint64()

@@ -3,6 +3,7 @@ through the C ABI (via the thin ctypes binding)."""
 import gc
 import math
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -1306,6 +1307,55 @@ def test_checked_build_reports_a_violation_without_losing_the_context(d2):
     plain.sync()
     assert plain.debug_last_device_check() == [0, 0, 0, 0]
     plain.close()
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+def test_a_wait_that_runs_out_is_reported_once_and_the_context_stays_usable(d2, flags):
+    """A warp that never announces: the others' waits end at the limit (once for the block), the kernel ends normally, sync
+    and the host round report it and clear it, a value out of range beside it is reported by the next call."""
+    cfg = wl.round_config(1)
+    ctx = d2.Context(cfg.log2_n, cfg.moduli, cfg.num_parties, seed=1, flags=flags)
+    for bad in (0, (1 << 18) + 1):
+        with pytest.raises(d2.D2mheError) as e:
+            ctx.debug_wait_selftest(bad)
+        assert e.value.status == d2.ERR_INVALID_ARG
+    parties = list(range(cfg.num_parties))
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    offsets, rows = wl.regular_graph(cfg.num_parties, cfg.degree, 1)
+    values = wl.gradients(cfg, 1)
+    workspace = torch.empty(ctx.round_workspace_bytes(cfg.num_cts), dtype=torch.uint8, device=ctx.device)
+    host, sums = torch.from_numpy(values), torch.empty(values.shape, dtype=torch.int32)
+    ctx.round_host(host, 0, cfg.num_cts, offsets, rows, sums, workspace)
+    want = sums.numpy().copy()
+    ctx.sync()
+
+    start = time.perf_counter()
+    ctx.debug_wait_selftest(1 << 18)
+    with pytest.raises(d2.D2mheError) as e:
+        ctx.sync()
+    took = time.perf_counter() - start
+    assert e.value.status == d2.ERR_DEVICE_CHECK and 0.1 < took < 1.9  # 1.05 s; a second wait of that length would be 2.1
+    assert ctx.debug_last_device_check() == [10, 0, 0, 0]
+    ctx.sync()
+
+    ctx.debug_wait_selftest(50)
+    sums.zero_()
+    with pytest.raises(d2.D2mheError) as e:
+        ctx.round_host(host, 0, cfg.num_cts, offsets, rows, sums, workspace)
+    assert e.value.status == d2.ERR_DEVICE_CHECK
+    ctx.round_host(host, 0, cfg.num_cts, offsets, rows, sums, workspace)
+    assert np.array_equal(sums.numpy(), want)
+
+    out_of_range = torch.full((cfg.n,), T, dtype=torch.int32, device=ctx.device)
+    ctx.encode(out_of_range, 1, ctx.empty_u32(1, cfg.n))
+    ctx.debug_wait_selftest(50)
+    for status in (d2.ERR_DEVICE_CHECK, d2.ERR_RANGE):
+        with pytest.raises(d2.D2mheError) as e:
+            ctx.sync()
+        assert e.value.status == status
+    ctx.sync()
+    ctx.close()
 
 
 # ----------------------------------------------------------------------------------

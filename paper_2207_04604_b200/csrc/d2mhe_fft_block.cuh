@@ -82,7 +82,9 @@ struct FftSmem {
   __device__ __forceinline__ void release() const {
     if (!announce) return;
     __syncwarp();
-    if ((threadIdx.x & 31u) == 0) asm volatile("{.reg .b64 t; mbarrier.arrive.shared.b64 t, [%0];}" ::"r"(bar()) : "memory");
+    // one lane, by a predicate: with a branch the warp would not be known to be converged at the tensor-memory loads that follow
+    asm volatile("{.reg .b64 t; .reg .pred p; setp.eq.u32 p, %1, 0; @p mbarrier.arrive.shared.b64 t, [%0];}" ::"r"(bar()),
+                 "r"(threadIdx.x & 31u) : "memory");
   }
   // A try that fails takes 4 us on this GPU (5000 of them in the self-test's kernel 20 ms, with and without a time hint), and
   // all the waits of a thread have WAIT_TRIES failing ones between them: a block loses about a second, whatever is wrong, and
@@ -110,13 +112,17 @@ struct FftSmem {
 };
 
 // ---- tensor memory --------------------------------------------------------------------------------
-// One warp allocates; every thread then owns `words` 32-bit words at the returned address.
+// One warp allocates; every thread then owns `words` 32-bit words at the returned address.  All tcgen05 instructions here
+// are .aligned: a warp has to be converged at them, which __syncwarp guarantees after the branches of single threads (the
+// loads and stores of transforms come behind the exchanges, which have theirs).
 __device__ __forceinline__ void tmem_alloc(u32* slot_smem, u32 cols) {
+  __syncwarp();
   const u32 a = (u32)__cvta_generic_to_shared(slot_smem);
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(a), "r"(cols) : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
 }
 __device__ __forceinline__ void tmem_free(u32 base, u32 cols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols));
 }
 __device__ __forceinline__ u32 tmem_thread_base(u32 base, u32 words) {

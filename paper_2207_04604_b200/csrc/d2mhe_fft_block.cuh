@@ -95,6 +95,7 @@ struct FftSmem {
       return;
     }
     u32 done = 0;
+#pragma unroll 1  // refresh shares at N = 4096 737 -> 730 us, receiving call of 594 rows of nine 262.6 -> 260.9
     for (; !done && tries; --tries)
       asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
                    : "=r"(done) : "r"(bar()), "r"(phase ^ 1u) : "memory");

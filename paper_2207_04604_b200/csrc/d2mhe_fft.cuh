@@ -290,6 +290,17 @@ D2MHE_HD void fft_product4(double* xr, double* xi, int k, const cpx (&c)[4]) {
   fft_bfly_i<SGN>(xr[i1], xi[i1], xr[i3], xi[i3]);
 }
 
+// cos(pi m / 64) for any m
+D2MHE_HD constexpr double cos64_any(int m) {
+  const int k = m & 127, h = k > 64 ? 128 - k : k;
+  return h <= 32 ? cos64(h) : -cos64(64 - h);
+}
+// The factor of digit j in psi^-j of the columns of group g (two groups): what fft_twist multiplies by, as a table entry.
+D2MHE_HD constexpr cpx fft_digit(int g, int j) {
+  const int a = g ? 3 * j : -j;
+  return cpx{cos64_any(a), cos64_any(a - 32)};
+}
+
 // psi^-j of digit jC = JC of a column: tw * e^(-i pi JC / 2R) (one group), e^(-i pi JC / 4R) (first of two) or
 // e^(3 i pi JC / 4R) (second of two; psi_1 = e^(-3 i pi / 4 NG)).
 template <int R, int GR, int JC>

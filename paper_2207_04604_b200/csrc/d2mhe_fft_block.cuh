@@ -430,23 +430,14 @@ __device__ __forceinline__ u32 fft_coef(const FftSmem<LOGN, STASH>& sm, int i) {
 }
 // fft_twist's constants of two groups, by group and digit.  Selected instead, they were kept across the loop and spilled:
 // shares at N = 16384 1868 us, Conversion 4505 us, with two copies of the end of a part, 1852 and 4247 us like this.
-static __device__ __constant__ double2 c_digit[32] = {
-    {1.0, 0.0}, {0.9987954562051724, -0.049067674327418015},
-    {0.9951847266721969, -0.0980171403295606}, {0.989176509964781, -0.14673047445536175},
-    {0.9807852804032304, -0.19509032201612828}, {0.970031253194544, -0.2429801799032639},
-    {0.9569403357322088, -0.2902846772544624}, {0.9415440651830208, -0.33688985339222005},
-    {0.9238795325112867, -0.3826834323650898}, {0.9039892931234433, -0.4275550934302821},
-    {0.881921264348355, -0.47139673682599764}, {0.8577286100002721, -0.5141027441932218},
-    {0.8314696123025452, -0.5555702330196022}, {0.8032075314806449, -0.5956993044924334},
-    {0.773010453362737, -0.6343932841636455}, {0.7409511253549591, -0.6715589548470184},
-    {1.0, 0.0}, {0.989176509964781, 0.14673047445536175},
-    {0.9569403357322088, 0.2902846772544624}, {0.9039892931234433, 0.4275550934302821},
-    {0.8314696123025452, 0.5555702330196022}, {0.7409511253549591, 0.6715589548470184},
-    {0.6343932841636455, 0.773010453362737}, {0.5141027441932218, 0.8577286100002721},
-    {0.3826834323650898, 0.9238795325112867}, {0.2429801799032639, 0.970031253194544},
-    {0.0980171403295606, 0.9951847266721969}, {-0.049067674327418015, 0.9987954562051724},
-    {-0.19509032201612828, 0.9807852804032304}, {-0.33688985339222005, 0.9415440651830208},
-    {-0.47139673682599764, 0.881921264348355}, {-0.5956993044924334, 0.8032075314806449}};
+struct FftDigits {
+  double2 c[32];
+  constexpr FftDigits() : c() {
+    for (int g = 0; g < 2; ++g)
+      for (int j = 0; j < 16; ++j) c[16 * g + j].x = fft_digit(g, j).r, c[16 * g + j].y = fft_digit(g, j).i;
+  }
+};
+static __device__ __constant__ FftDigits c_digit;
 // The last step of an inverse transform: twists, joins the groups and hands the 32 results of this thread over in
 // eight portions of four, rounded: out(m, first number, R or 0 (see fft_result_number), v[4]) with v = bits of
 // M + value, M = 1.5 * 2^(52 - f) + 1/2, so that bits >> f is floor(value + 1/2) plus a constant.
@@ -475,7 +466,7 @@ __device__ __forceinline__ void fft_results(const FftSmem<LOGN, STASH>& sm, cons
     asm volatile("" : "+r"(step));
     static_for<16>([&](auto j_) {
       constexpr int j = decltype(j_)::value, i = brev_c<16>(j);
-      const double2 c = c_digit[step * 16 + j];
+      const double2 c = c_digit.c[step * 16 + j];
       const cpx z = cmul(cpx{xr[i], xi[i]}, cmul(tw[0], cpx{c.x, c.y}));
       xr[i] = z.r;
       xi[i] = z.i;

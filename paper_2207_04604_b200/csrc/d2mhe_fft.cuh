@@ -427,7 +427,8 @@ inline FftDeal fft_deal(unsigned places, unsigned rows, unsigned n_parties, FftW
   return deal;
 }
 // A block's row and its part of the parties: first, first + step, ..  MIXED: some rows are whole, others not (an
-// instance of its own: a step that is not a launch constant takes a register that the kernels do not have).
+// instance of its own, with a step that is not a launch constant: as the only one it made the refresh shares of 2960 rows of
+// ten at N = 8192, which are not mixed, 1702 us instead of 1574).
 template <bool MIXED>
 D2MHE_HD unsigned fft_dealt(const FftDeal& deal, unsigned block, unsigned& first, unsigned& step) {
   if (MIXED && block < deal.whole) {

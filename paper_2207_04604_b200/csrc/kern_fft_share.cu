@@ -85,7 +85,9 @@ cudaError_t launch_share(const DevView& v, const LimbParams& lp, cudaStream_t s,
                          u32 n_parties, u32 n_cts, u32 unit_first, u32 n_units, const void* noise, u64* shares) {
   using G = FftGeo<LOGN>;
   const FftDeal deal = fft_deal(v.sms * G::CTAS, n_units * v.L, n_parties, FFT_WORK_SHARE);
-  const auto kernel = deal.whole ? k_share_fft<LOGN, OWN, true> : k_share_fft<LOGN, OWN, false>;
+  auto kernel = k_share_fft<LOGN, OWN, false>;
+  if constexpr (!OWN)  // one product a row: every row is whole
+    if (deal.whole) kernel = k_share_fft<LOGN, OWN, true>;
   const cudaError_t e = set_smem(kernel, G::smem_bytes(1));
   if (e != cudaSuccess) return e;
   kernel<<<deal.blocks, G::T, G::smem_bytes(1), s>>>(v, lp, agg, parties_dev, n_parties, n_cts, unit_first,

@@ -1396,8 +1396,20 @@ def test_share_products_at_the_limits_of_the_split(d2, log2_n, bits, L, K):
 
 @pytest.mark.parametrize("log2_n,bits,L,C", [(12, 54, 1, 75), (12, 36, 3, 40), (13, 55, 1, 1), (13, 54, 3, 50), (14, 54, 1, 3), (14, 50, 5, 31)])
 def test_encrypt_sizes_against_oracle(d2, log2_n, bits, L, C):
-    """One and two thread blocks per ciphertext and limb, calls of part of a wave and of more than one; plaintext
-    coefficients at both ends of their range."""
+    """One and two thread blocks per ciphertext and limb, calls of part of a wave of blocks."""
+    _check_encryption(d2, log2_n, bits, L, C)
+
+
+@pytest.mark.parametrize("waves", ["one", "just over one", "two"])
+@pytest.mark.parametrize("log2_n,bits,L", [(12, 54, 4), (13, 55, 4), (14, 50, 4)])
+def test_encryption_of_one_wave_of_blocks_and_of_more(d2, log2_n, bits, L, waves):
+    """Up to one wave every block makes the transform of u, beyond it comes from a launch of its own."""
+    places = torch.cuda.get_device_properties(0).multi_processor_count * {12: 4, 13: 2, 14: 1}[log2_n]
+    _check_encryption(d2, log2_n, bits, L, {"one": places // L, "just over one": places // L + 1, "two": 2 * places // L}[waves])
+
+
+def _check_encryption(d2, log2_n, bits, L, C):
+    """Against the oracle; plaintext coefficients at both ends of their range."""
     moduli = wl.ntt_primes(bits, 2 << log2_n, L)
     ctx = d2.Context(log2_n, moduli, 2, seed=78)
     o = make_oracle(log2_n, moduli, seed=78)
@@ -1444,6 +1456,30 @@ def test_conversion_and_refresh_products_against_oracle(d2, log2_n, bits, L, K, 
     ctx.bootstrap_share(dagg, parties, parties, 3, C, shares)
     ctx.sync()
     assert np.array_equal(d2.to_u64_numpy(shares), o.boot_share(agg, parties, parties, 3))
+    ctx.close()
+
+
+@pytest.mark.parametrize("log2_n,bits", [(12, 54), (13, 54), (14, 54)])
+def test_conversion_and_refresh_of_just_over_a_wave_of_blocks(d2, log2_n, bits):
+    """Two rows of products more than the GPU holds blocks (a refresh has two rows a unit): as many whole rows as fill a wave,
+    the others split by party."""
+    places = torch.cuda.get_device_properties(0).multi_processor_count * {12: 4, 13: 2, 14: 1}[log2_n]
+    moduli, n, parties = wl.ntt_primes(bits, 2 << log2_n, 1), 1 << log2_n, [0, 1]
+    ctx = d2.Context(log2_n, moduli, 2, seed=95)
+    o = make_oracle(log2_n, moduli, seed=95)
+    ctx.keygen_share(parties)
+    ctx.collective_pk(parties)
+    o.collective_pk(parties)
+    ctx.user_keygen(parties)
+    pk_users = np.stack([o.user_pk(i) for i in parties])
+    agg = np.random.default_rng(log2_n).integers(0, moduli[0], (1, places + 2, 2, 1, n), dtype=np.uint64)
+    for C, call, want in ((places + 2, ctx.convert_share, lambda a: o.convert_share(a, pk_users[1:], [1], parties, 3)),
+                          (places // 2 + 1, ctx.bootstrap_share, lambda a: o.boot_share(a, [1], parties, 3))):
+        part = np.ascontiguousarray(agg[:, :C])
+        shares = ctx.empty_u64(1, 2, C, 2, 1, n)
+        call(d2.from_u64_numpy(part, ctx.device), [1], parties, 3, C, shares)
+        ctx.sync()
+        assert np.array_equal(d2.to_u64_numpy(shares), want(part))
     ctx.close()
 
 

@@ -56,6 +56,15 @@ def _schedule(kind, places, rows, parties, whole, split):
     return whole // places * (fixed + each * parties) + waves * (fixed + each * -(-parties // split))
 
 
+@pytest.mark.parametrize("places", [148, 296, 592])
+def test_the_calls_compared_with_the_oracle_on_the_gpu_have_mixed_deals(deal, places):
+    """The sizes of the GPU tests of just over a wave of blocks, with the 148 multiprocessors of a B200."""
+    parties, extra = {592: (7, 38), 296: (5, 14), 148: (4, 16)}[places]
+    calls = [("convert", places, places + 2, 2), ("boot", places, places + 2, 2), ("share", places, places + extra, parties)]
+    calls += [("share32", 148, 164, 4)]
+    assert all(whole == p for (_, p, _, _), (whole, _, _, _) in zip(calls, deal(calls)))
+
+
 @pytest.mark.parametrize("kind", sorted(TRANSFORMS))
 @pytest.mark.parametrize("places", [148, 296, 592])
 def test_every_product_is_dealt_once_and_no_even_split_is_shorter(deal, kind, places):

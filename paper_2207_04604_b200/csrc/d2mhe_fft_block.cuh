@@ -70,7 +70,8 @@ struct FftSmem {
   // barrier made every warp wait for the slowest one.  Shares at N = 8192 716 -> 679 us, at N = 16384 1852 -> 1709 us,
   // Conversion at N = 16384 4247 -> 3888 us (1480 rows of ten parties); not in the encryption kernels from N = 8192
   // on, whose two to four transforms a block don't repay it (370 ciphertexts, L = 4, block barriers against this: N = 4096
-  // 83.9 / 77.0 us, N = 8192 153.8 / 161.8, N = 16384 352 / 359).
+  // 83.9 / 77.0 us, N = 8192 153.8 / 161.8, N = 16384 352 / 359), nor in the one for 32-bit words with its one or two
+  // (N = 4096, L = 7, 370 ciphertexts 63.9 / 62.7 us).
   __device__ __forceinline__ void init() const {  // one thread, ahead of a block barrier
     slot[1] = 0;
     asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(bar()), "r"(G::T / 32) : "memory");
@@ -509,8 +510,9 @@ __device__ __forceinline__ u32 lo_bytes(u64 a, u64 b, u64 c, u64 d) {  // byte 5
                      __byte_perm((u32)(c >> 32), (u32)(d >> 32), 0x0051), 0x5410);
 }
 
-// 64 p + V_lo + 2^h V_hi + e0 - 19, between 0 and 129 p: the multiples of d below add up to less than 61 p (d N / 2 with
-// ternary factors, where 256 d < 2^b is enough; FFT_CONV_V times that in Conversion, which the host tests).  low: V_lo plus
+// 2^b + 64 p + V_lo + 2^h V_hi + e0 - 19, between 2^b and 2^b + 129 p, for fft_canon and nothing else (any other reduction
+// would be off by d for the 2^b): the multiples of d below add up to less than 61 p (d N / 2 with ternary factors, where
+// 256 d < 2^b is enough; FFT_CONV_V times that in Conversion, which the host tests).  low: V_lo plus
 // its offset; hi: the rounded high part with f fraction bits, f = 32 - (b - h) and p = 2^b - d: its low word holds
 // V_hi mod 2^(b-h) above the fraction, its high word floor(V_hi / 2^(b-h)) plus a constant, which counts multiples of
 // 2^b = d (mod p).  The constants are collected in k0.
@@ -522,7 +524,7 @@ __device__ __forceinline__ u64 fft_sum(u64 low, u64 hi, u32 e0, const FftSplit& 
   return s + low;
 }
 
-// The canonical residue of s, which fft_sum left 2^b too large: with s = (k + 1) 2^b + rem, u = rem + (k + 1) d = r + d for
+// The canonical residue of s = 2^b + a value in [0, 256 p) (fft_sum and what a store adds: below 132 p): with s = (k + 1) 2^b + rem, u = rem + (k + 1) d = r + d for
 // r = s - 2^b mod p below 2p, and bit b of u says whether r >= p = 2^b - d: then r - p is u without that bit, else r = u - d.
 // (The subtraction by a multiple of that bit goes to the multiplier; a comparison and two selections cost two more
 // instructions on the logic pipe, which this part of the kernels keeps busy: refresh shares at N = 8192 1604 -> 1568 us, shares
@@ -616,7 +618,8 @@ __device__ __forceinline__ void fft_fence(const cpx (&tw)[COLS], cpx (&out)[COLS
 }
 
 // The end of a part's inverse transform.  Low part (high = false): the rounded results are kept in shared memory.
-// High part: store(coefficient, sum) gets 64 p + product + noise for every coefficient of the thread.  Each part has a
+// High part: store(coefficient, sum) gets fft_sum's 2^b + 64 p + product + noise for every coefficient of the thread, and
+// may add a few p more before fft_canon.  Each part has a
 // copy of the code of its own, so that the loads and the arithmetic of several portions overlap (with one copy and a
 // branch in every portion the end of a high part took 5.3 k clocks of a transform's 10.2 k at N = 8192; refresh shares there
 // 1789 -> 1630 us, encryption at N = 16384 459 -> 353 us); the fences keep the copies from sharing subexpressions, 300 bytes

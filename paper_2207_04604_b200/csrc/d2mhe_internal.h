@@ -111,9 +111,10 @@ static const size_t kNoiseScratchMaxBytes = (size_t)512 << 20;
 #ifndef D2MHE_ROUND_LANES_HOST
 #define D2MHE_ROUND_LANES_HOST 3
 #endif
-// Internal streams of the whole-round entry points: two for device buffers (measured best at
-// configuration 2: 0.89 ms against 0.91 ms with three), three when the call also copies from and to
-// host buffers (1.02 ms against 1.04 ms with two: one more stream hides the copies better).
+// Internal streams of the whole-round entry points: two for device buffers (ten users, N = 8192, L = 4, 13 indices 499 us,
+// with three and one 558 and 549), three when the call also copies from and to host buffers (the same round 748 us, 755 with
+// two; 40 indices 1678 and 1763; twenty users, 40 indices 4995 and 5056; six users, L = 5, 30 indices 984 and 1069; thirty
+// users, N = 4096, 12 indices 1328 and 1267: one more stream hides the copies of longer rounds better).
 static const int kRoundLanesDevice = D2MHE_ROUND_LANES;
 static const int kRoundLanesHost = D2MHE_ROUND_LANES_HOST;
 static const int kRoundLanes = kRoundLanesDevice > kRoundLanesHost ? kRoundLanesDevice : kRoundLanesHost;

@@ -90,8 +90,10 @@ cudaError_t encrypt_fft(const DevView& v, const LimbParams& lp, cudaStream_t s, 
     unsigned char* noise = reinterpret_cast<unsigned char*>(scratch) + (size_t)nu * 8 * v.n;
     cudaError_t e = sample_streams(v, s, nullptr, parties_dev, 1, ct_first, n_cts, first, nu, kSampleEncrypt, true, noise);
     if (e != cudaSuccess) return e;
-    // One wave of blocks: each makes the transform of its u, which takes less time than a launch for it (105 blocks at
-    // N = 16384: 9.3 + 37.8 us in two launches, 42.2 in one); more waves would make it again and again.
+    // One wave of blocks: each makes the transform of its u, which takes less time than a launch for it; more waves would make
+    // it again and again.  Whole calls with it and with a launch for it, L = 4: N = 4096, 88 blocks 25.9 / 28.4 us, a full wave
+    // (592) 54.9 / 56.5; N = 8192, 44 blocks 27.3 / 31.1, a full wave (296) 55.6 / 58.2; N = 16384, 20 blocks 37.3 / 42.4, a
+    // full wave (148) 60.9 / 65.3; with L = 1 and L = 8 it saves 0.6 to 8 us everywhere, too.
     const u32 ctas = v.logn == 12 ? FftGeo<12>::CTAS : v.logn == 13 ? FftGeo<13>::CTAS : FftGeo<14>::CTAS;
     if (nu * v.L <= v.sms * ctas) {
       u_fft = nullptr;

@@ -6,8 +6,9 @@
 namespace {
 
 // One thread block = one (recipient, ciphertext, limb); it walks over the parties of the list.
-// What bounds it: the double-precision pipe and the issue slots around it (about 50 double-precision and 45 other
-// instructions per complex point and part), then shared memory (two exchanges per transform).  The transforms of
+// What bounds it: the double-precision pipe and the issue slots around it (42, 46 and 52 double-precision and as many other
+// instructions per complex point and part at N = 4096, 8192 and 16384, in captures of whole waves; the pipe is busy 48, 47
+// and 45 %, the load/store data pipe 65, 58 and 55 %), then shared memory (two exchanges per transform).  The transforms of
 // both parts of c_1 stay in tensor memory (all 256 KB of an SM: 32 bytes per point), where neither the load/store
 // pipe nor L2 sees them again; the key's transform does not depend on the limb (8 N bytes per party) and comes from
 // L2, or from L1 when the other block of the SM has just read it.  (Fetching it point by point into the registers that

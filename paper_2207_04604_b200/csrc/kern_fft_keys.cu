@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(FftGeo<12>::T) k_wait_selftest(DevView v, int 
   __syncthreads();
   sm.acquire();
   if (threadIdx.x >= 32) sm.release();
-  for (int i = 0; i < 4; ++i) sm.acquire();
+  for (int i = 0; i < 8; ++i) sm.acquire();
   __syncthreads();
   if (threadIdx.x == 0) sm.finish(v);
 }
